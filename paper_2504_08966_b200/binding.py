@@ -106,11 +106,13 @@ def _check(ctx, status: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    """Address of a tensor (ctypes takes plain integers for the pointer arguments and fields), None for None."""
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of the current stream of the current device."""
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dt(dtype) -> int:
@@ -213,6 +215,7 @@ class Context:
         self.d, self.n_qh, self.n_kvh, self.d_h = d, n_qh, n_kvh, d_h
         _check(None, self._L.pact_create(C.byref(self.handle), d, n_qh, n_kvh, d_h, _dt(in_dtype), _dt(out_dtype)))
         self.ws = None
+        self._need = {}                      # (max_batch, max_N) -> workspace bytes, asked from the library once
 
     def close(self):
         if self.handle:
@@ -229,13 +232,17 @@ class Context:
         return int(self._L.pact_workspace_bytes(self.handle, max_batch, max_N))
 
     def ensure_workspace(self, max_batch, max_N):
-        need = self.workspace_bytes(max_batch, max_N)
+        need = self._need.get((max_batch, max_N))
+        if need is None:
+            if len(self._need) >= 4096:
+                self._need.clear()
+            need = self._need[(max_batch, max_N)] = self.workspace_bytes(max_batch, max_N)
         if self.ws is None or self.ws.numel() < need:
             self.ws = torch.empty(need, dtype=torch.uint8, device="cuda")
         return self.ws
 
     def _ws(self):
-        return C.c_void_p(self.ws.data_ptr()), C.c_size_t(self.ws.numel())
+        return self.ws.data_ptr(), self.ws.numel()
 
     # ---- stage calls ------------------------------------------------------------------
     def pact_importance(self, im: DeviceImage, params: Params, score: torch.Tensor):
@@ -345,4 +352,4 @@ class Context:
                       _ptr(host.get("logw_out")))
         w, n = self._ws()
         _check(self.handle, self._L.pact_reduce_host(self.handle, C.byref(d), C.byref(params),
-                                                     _ptr(staging), C.c_size_t(staging.numel()), w, n, _stream()))
+                                                     _ptr(staging), staging.numel(), w, n, _stream()))

@@ -59,9 +59,7 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   const int Wp = Np / 32;
   m.Np = Np;
   m.Wp = Wp;
-  cv.take(m.cnt, (size_t)(kCntInts + kTickInts) * sizeof(int32_t));
-  if (m.cnt) m.tick = m.cnt + kCntInts;
-  cv.take(m.qpart, (size_t)kQPartRows * c->n_qcols * sizeof(double));
+  cv.take(m.cnt, (size_t)kCntInts * sizeof(int32_t));
   cv.take(m.qg, (size_t)c->n_qcols * sizeof(double));
   cv.take(m.E, (size_t)N * c->n_qh * sizeof(double));
   cv.take(m.part, (size_t)((N + kRowsPerCta - 1) / kRowsPerCta) * c->n_qh * 2 * sizeof(double));
@@ -232,7 +230,7 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
   const int v = in == PACT_BF16 ? 8 : 4;
   if (d % 8 != 0 || d_h % v != 0) return PACT_ERR_UNSUPPORTED;
   if (d > kMergeMaxD || n_qh > 256) return PACT_ERR_UNSUPPORTED;
-  if ((n_qh * d_h / v + 7) / 8 > kTickInts) return PACT_ERR_UNSUPPORTED;   // one ticket per 128-byte column group of Q
+  if ((n_qh * d_h / v + 7) / 8 > kMaxColGroups) return PACT_ERR_UNSUPPORTED;
   pact_ctx *c = new (std::nothrow) pact_ctx;
   if (!c) return PACT_ERR_INVALID_ARG;
   memset(c, 0, sizeof(*c));
@@ -242,9 +240,9 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
   pact_ctx *ctx = c;
   cudaError_t e = cudaGetDevice(&c->device);
   if (e == cudaSuccess) {
-    cudaDeviceProp pr;
-    e = cudaGetDeviceProperties(&pr, c->device);
-    if (e == cudaSuccess && pr.major != 10) { delete c; return PACT_ERR_UNSUPPORTED; }
+    int major = 0;                        // (cudaGetDeviceProperties takes milliseconds)
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
+    if (e == cudaSuccess && major != 10) { delete c; return PACT_ERR_UNSUPPORTED; }
   }
   if (e == cudaSuccess) e = euti_configure(c->n_qcols, c->n_qh);
   if (e == cudaSuccess) e = cluster_configure(&c->ccfg);
@@ -328,7 +326,6 @@ pact_status pact_importance(pact_ctx *ctx, const pact_image *img, const pact_par
   m.score_user = score;
   set_params(m, p, img->N);
   point_counts_at_workspace(m);
-  CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
   CK(launch_euti(bt, img->N, ctx->in == PACT_BF16, 1, st));
   ctx->launches += euti_kernels(1);
   CK(cudaGetLastError());
@@ -354,11 +351,10 @@ pact_status pact_prune(pact_ctx *ctx, const float *score, int N, const pact_para
   point_counts_at_workspace(m);
   m.score = const_cast<float *>(score);
   m.keep = keep; m.kept_idx = kept_idx; m.pruned_idx = pruned_idx;
-  launch_select_gather(bt, N, true, false, st);
+  m.counts_user = counts;
+  CK(launch_split(bt, N, st));
   ctx->launches += 1;
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(counts, m.cnt + PACT_CNT_Q, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-  CK(cudaMemcpyAsync(counts + 1, m.cnt + PACT_CNT_M, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return PACT_OK;
 }
 
@@ -386,14 +382,13 @@ pact_status pact_dbdpc(pact_ctx *ctx, const void *K, int64_t ldK, int N, const i
   m.kept_idx = const_cast<int32_t *>(idx);
   m.q_ptr = q_dev;
   m.rho_user = rho; m.center_idx_user = center_idx; m.C_user = C_dev; m.label_user = label;
-  CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
-  launch_keynorm_gather(bt, N, bf, false, st);
+  CK(launch_keynorm_gather(bt, N, bf, st));
   if (ctx->umma) CK(launch_gram_umma(bt, N, ctx->ccfg, st));
-  else launch_gram(bt, N, bf, ctx->ccfg, st);
+  else CK(launch_gram(bt, N, bf, ctx->ccfg, st));
   CK(launch_centers(bt, N, bf, ctx->ccfg, ctx->sweep_limit, st));
   if (ctx->umma) CK(launch_assign_umma(bt, N, true, ctx->ccfg, st));
-  else launch_assign(bt, N, bf, ROWS_KEPT_LIST, ctx->ccfg, st);
-  launch_label(bt, N, bf, ROWS_KEPT_LIST, st);
+  else CK(launch_assign(bt, N, bf, ROWS_KEPT_LIST, ctx->ccfg, st));
+  CK(launch_label(bt, N, bf, ROWS_KEPT_LIST, st));
   ctx->launches += 5;
   CK(cudaGetLastError());
   if (counters)
@@ -425,12 +420,11 @@ pact_status pact_key_spread(pact_ctx *ctx, const void *const *K_layers, int n_la
       carve_image(ctx, N, (char *)ws + (size_t)b * per_img, &m);
       m.N = N; m.Kc = K_layers[base + b]; m.ldKc = ldK;
       point_counts_at_workspace(m);
-      CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
     }
-    launch_key_rnorm(bt, N, bf, st);
+    CK(launch_key_rnorm(bt, N, bf, st));
     if (ctx->umma) CK(launch_spread_umma(bt, N, ctx->ccfg, st));
-    else launch_spread(bt, N, bf, ctx->ccfg, st);
-    launch_spread_finish(bt, max_dist, layer_out, base, threshold, st);
+    else CK(launch_spread(bt, N, bf, ctx->ccfg, st));
+    CK(launch_spread_finish(bt, max_dist, layer_out, base, threshold, st));
     ctx->launches += 3;
     CK(cudaGetLastError());
   }
@@ -461,22 +455,15 @@ pact_status pact_reincorporate(pact_ctx *ctx, const void *K, int64_t ldK, int N,
   m.pruned_idx = const_cast<int32_t *>(pruned_idx);
   m.m_ptr = m_dev; m.C_ptr = C_dev; m.cidx_ptr = center_idx;
   m.label = label;                      // updated in place
-  CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
-  if (ctx->umma) {
-    // the rows x centres pass on the tensor cores covers every token (the survivors' distances are computed
-    // and not used), so every token needs its inverse key norm
-    launch_key_rnorm(bt, N, bf, st);
-    launch_center_key_gather(bt, N, bf, st);
-    CK(launch_assign_umma(bt, N, false, ctx->ccfg, st));
-    ctx->launches += 1;
-  } else {
-    launch_center_key_gather(bt, N, bf, st);
-    launch_assign(bt, N, bf, ROWS_PRUNED_LIST, ctx->ccfg, st);
-  }
-  launch_label(bt, N, bf, ROWS_PRUNED_LIST, st);
+  m.r_user = r_dev;
+  // the rows x centres pass on the tensor cores covers every token (the survivors' distances are computed
+  // and not used), so every token needs its inverse key norm
+  CK(launch_center_key_gather(bt, N, bf, ctx->umma, st));
+  if (ctx->umma) CK(launch_assign_umma(bt, N, false, ctx->ccfg, st));
+  else CK(launch_assign(bt, N, bf, ROWS_PRUNED_LIST, ctx->ccfg, st));
+  CK(launch_label(bt, N, bf, ROWS_PRUNED_LIST, st));
   ctx->launches += 3;
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(r_dev, m.cnt + PACT_CNT_R, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   if (counters)
     CK(cudaMemcpyAsync(counters, m.cnt, PACT_N_COUNTERS * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return PACT_OK;
@@ -502,15 +489,11 @@ pact_status pact_merge(pact_ctx *ctx, const pact_image *img, const int32_t *labe
   point_counts_at_workspace(m);
   m.label = const_cast<int32_t *>(label);
   m.C_ptr = C_dev; m.cidx_ptr = center_idx;
-  CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
-  CK(cudaMemsetAsync(m.csize, 0, (size_t)m.Np * sizeof(int32_t), st));
-  CK(cudaMemsetAsync(m.cticket, 0, (size_t)m.Np * sizeof(int32_t), st));
-  CK(cudaMemsetAsync(m.cnt_cb, 0, (size_t)m.Np * m.nbp * sizeof(uint16_t), st));
+  CK(launch_list_clear(bt, st));
   CK(launch_lists(bt, img->N, ctx->in == PACT_BF16, false, ctx->spin_limit, st));
   CK(launch_merge(bt, ctx->in == PACT_BF16, ctx->out == PACT_BF16, ctx->ccfg, st));
-  ctx->launches += lists_kernels(img->N, 1) + 1;
+  ctx->launches += lists_kernels(img->N, 1) + 2;
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(img->counters, m.cnt, PACT_N_COUNTERS * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return PACT_OK;
 }
 
@@ -547,7 +530,6 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
       cmaxN = g->N > cmaxN ? g->N : cmaxN;
       const int qest = g->N - m.m_target + 64 < g->N ? g->N - m.m_target + 64 : g->N;   // survivors, with room for ties
       cmaxQ = qest > cmaxQ ? qest : cmaxQ;
-      CK(cudaMemsetAsync(m.cnt, 0, (kCntInts + kTickInts) * sizeof(int32_t), st));
     }
     int stage = 0;
     auto mark = [&]() -> cudaError_t {
@@ -562,7 +544,7 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     };
     CK(launch_euti(bt, cmaxN, bf, 0, st, ctx->prof_on ? &MarkFn::call : nullptr, &mark));  CK(mark());
     if (ctx->umma) CK(launch_gram_umma(bt, cmaxN, ctx->ccfg, st, cmaxQ));
-    else launch_gram(bt, cmaxN, bf, ctx->ccfg, st);
+    else CK(launch_gram(bt, cmaxN, bf, ctx->ccfg, st));
     CK(mark());
     CK(launch_centers(bt, cmaxQ, bf, ctx->ccfg, ctx->sweep_limit, st));  CK(mark());
     // On the tensor-core path with little work per SM (one image) the labels and member counts are formed as
@@ -571,7 +553,7 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, nb, ctx->ccfg);
     const bool fused_labels = ctx->umma && !pairs;
     if (ctx->umma) CK(launch_assign_umma(bt, cmaxN, false, ctx->ccfg, st, fused_labels, pairs));
-    else launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->ccfg, st);
+    else CK(launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->ccfg, st));
     CK(mark());
     if (fused_labels) CK(launch_members(bt, cmaxN, st));
     else CK(launch_lists(bt, cmaxN, bf, true, ctx->spin_limit, st));
@@ -579,9 +561,6 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->ccfg, st));  CK(mark());
     ctx->launches += euti_kernels(0) + 4 + (fused_labels ? 1 : lists_kernels(cmaxN, nb));
     CK(cudaGetLastError());
-    for (int b = 0; b < nb; ++b)
-      CK(cudaMemcpyAsync(bt.img[b].counters_user, bt.img[b].cnt, PACT_N_COUNTERS * sizeof(int32_t),
-                         cudaMemcpyDeviceToDevice, st));
   }
   return PACT_OK;
 }

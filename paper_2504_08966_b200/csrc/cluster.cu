@@ -2,7 +2,7 @@
 // distance tiles with the density and the d <= d_c adjacency fused into their epilogue, density
 // rank, centre selection, tokens-by-centres nearest-centre pass, labels.
 //
-// This file holds the SIMT tile kernels (any element type and key width); the tcgen05 tile
+// This file holds the double-precision tile kernels (any element type and key width); the tcgen05 tile
 // kernels for bf16 keys live in gram_umma.cu and share the epilogue arithmetic of common.cuh.
 #include <cooperative_groups.h>
 
@@ -16,71 +16,64 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
   return v;
 }
 
-// ---- inverse key norms, survivor gather, per-call initialisation -----------------------------
-// grid (ceil(maxN / 8), B), 256 threads, one warp per work item.
-//  all_tokens = 1: item = token i (inverse norm of every token; survivors are copied to Kp[slot])
-//  all_tokens = 0: item = list position r (token kept_idx[r]); only listed rows are touched
+// ---- inverse key norms, survivor gather, per-call initialisation (stage calls) ------------------------
+// grid (ceil(maxN / 8), B), 256 threads, one warp per list position r (token kept_idx[r]).
 template <typename T>
-__global__ void __launch_bounds__(256) k_keynorm_gather(const __grid_constant__ Batch bt, int all_tokens) {
+__global__ void __launch_bounds__(256) k_keynorm_gather(const __grid_constant__ Batch bt) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
   constexpr int V = Vec<T>::N;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
   const int lane = threadIdx.x & 31;
-  const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int q = all_tokens ? 0 : *im.q_ptr;
-  // per-call initialisation of the arrays later kernels accumulate into
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int q = *im.q_ptr;
+  // arrays later kernels accumulate into
   {
     const int gt = blockIdx.x * 256 + threadIdx.x, gs = gridDim.x * 256;
-    for (int r = gt; r < im.Np; r += gs) im.rho_fix[r] = 0ull;
+    for (int k = gt; k < im.Np; k += gs) im.rho_fix[k] = 0ull;
     for (int wd = gt; wd < im.Wp; wd += gs) { im.cmask[wd] = 0u; im.rmask[wd] = 0u; }
     for (int i = gt; i < im.N; i += gs) {
       im.best[i] = kBestInit;
-      if (!all_tokens) {
-        im.label[i] = -1;
-        if (im.label_user) im.label_user[i] = -1;
-      }
+      if (im.label_user) im.label_user[i] = -1;
     }
+    if (gt < kCntInts) im.cnt[gt] = 0;
   }
-  int i, r;
-  if (all_tokens) {
-    i = item;
-    if (i >= im.N) return;
-    r = im.slot[i];
-  } else {
-    r = item;
-    if (r >= q) return;
-    i = im.kept_idx[r];
-  }
+  if (r >= q) return;
+  const int i = im.kept_idx[r];
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
   const rn_t rn = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
   if (lane == 0) {
     rn_tok<D>(im)[i] = rn;
-    if (r >= 0) rn_kept<D>(im)[r] = rn;
+    rn_kept<D>(im)[r] = rn;
   }
-  if (r >= 0) {
-    T *dst = reinterpret_cast<T *>(im.Kp) + (size_t)r * bt.d_k;
-    for (int v = lane; v * V < bt.d_k; v += 32)
-      reinterpret_cast<uint4 *>(dst)[v] = reinterpret_cast<const uint4 *>(row)[v];
-  }
+  T *dst = reinterpret_cast<T *>(im.Kp) + (size_t)r * bt.d_k;
+  for (int v = lane; v * V < bt.d_k; v += 32)
+    reinterpret_cast<uint4 *>(dst)[v] = reinterpret_cast<const uint4 *>(row)[v];
 }
 
-// centre keys from a list of token indices (reincorporation as a stage of its own)
+// Centre keys from a list of token indices (reincorporation as a stage of its own), inverse norms of all rows
+// (all_rows) or of the listed pruned rows, per-call initialisation.  One warp per centre and row.
 template <typename T>
-__global__ void __launch_bounds__(256) k_center_key_gather(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(256) k_center_key_gather(const __grid_constant__ Batch bt, int all_rows) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
   constexpr int V = Vec<T>::N;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
   const int lane = threadIdx.x & 31;
   const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
   {
     const int gt = blockIdx.x * 256 + threadIdx.x, gs = gridDim.x * 256;
     for (int i = gt; i < im.N; i += gs) im.best[i] = kBestInit;
+    if (gt < kCntInts) im.cnt[gt] = 0;
+    if (gt == 0) *im.r_user = 0;
   }
-  if (c < *im.m_ptr) {                       // inverse norm of the c-th pruned row
-    const int i = im.pruned_idx[c];
+  if (c < (all_rows ? im.N : *im.m_ptr)) {   // inverse norm of row c, or of the c-th pruned row
+    const int i = all_rows ? c : im.pruned_idx[c];
     const double ss = row_sumsq<T>(reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc, bt.d_k, lane);
     if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
   }
@@ -94,113 +87,161 @@ __global__ void __launch_bounds__(256) k_center_key_gather(const __grid_constant
     reinterpret_cast<uint4 *>(dst)[v] = reinterpret_cast<const uint4 *>(row)[v];
 }
 
-// ---- 64 x 64 tile of dot products, 256 threads, thread (ty, tx) owns a 4 x 4 block -----------
-constexpr int TS = 64;   // tile side
-constexpr int KC = 32;   // key elements staged per step
+// ---- 32 x 32 tile of dot products in double, 128 threads -----------------------------------------
+// fp32 keys (and bf16 keys of a width the tcgen05 tiles do not take) get their dot products from the double-precision
+// tensor instruction (m8n8k4): the products of fp32 values are exact in double and the sums carry its full precision.
+// Warp (wy, wx) owns the 16 x 16 quarter at rows 16 wy, columns 16 wx as 2 x 2 fragments; lane l holds of fragment
+// (a, b) the row 8 a + l / 4 and the columns 8 b + 2 (l % 4) + {0, 1}.  Small tiles on purpose: these matrices are
+// small (a thumbnail has 138 survivors), so the tiles have to be many for the SMs to share them.  The operands are
+// widened once when they are staged; the next slab is on its way from the L2 while this one is multiplied.
+// One scalar FMA per product with 64 x 64 tiles, widening at every use, took 23 us for 138 x 138 x 128.
+constexpr int TS = 32;        // tile side
+constexpr int KC = 64;        // key elements staged per step
+constexpr int KST = KC + 4;   // row stride of a staged slab in doubles: fragment loads meet no bank twice
+constexpr int kTileThreads = 128;
 
-template <typename T, typename acc_t, typename RowA, typename RowB>
-__device__ __forceinline__ void tile_dots(RowA rowA, RowB rowB, int d_k, float (*As)[TS + 4],
-                                          float (*Bs)[TS + 4], acc_t (&acc)[4][4]) {
+template <typename T, typename RowA, typename RowB>
+__device__ __forceinline__ void tile_dots(RowA rowA, RowB rowB, int d_k, double (*As)[KST], double (*Bs)[KST],
+                                          double (&acc)[2][2][2]) {
   constexpr int V = Vec<T>::N;
-  constexpr int VPR = KC / V;                 // vectors per row per step
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+  constexpr int VPR = KC / V;                          // vectors per row of a slab
+  constexpr int NV = 2 * TS * VPR / kTileThreads;      // vectors per thread: the first half A, the second half B
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = (acc_t)0;
+    for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
+  uint4 buf[NV];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int v = (u % (NV / 2)) * kTileThreads + t, row = v / VPR, k = k0 + (v % VPR) * V;
+      const T *p = u < NV / 2 ? rowA(row) : rowB(row);
+      buf[u] = p && k < d_k ? *reinterpret_cast<const uint4 *>(p + k) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  fetch(0);
   for (int k0 = 0; k0 < d_k; k0 += KC) {
-    for (int v = t; v < TS * VPR; v += 256) {
-      const int row = v / VPR, kv = (v % VPR) * V;
-      float x[V], y[V];
-      const T *pa = rowA(row), *pb = rowB(row);
-      const bool inb = k0 + kv < d_k;
-      if (pa && inb) load_vec<T>(pa + k0 + kv, x);
-      else {
+    __syncthreads();                                   // the slab before has been read
 #pragma unroll
-        for (int k = 0; k < V; ++k) x[k] = 0.f;
-      }
-      if (pb && inb) load_vec<T>(pb + k0 + kv, y);
-      else {
+    for (int u = 0; u < NV; ++u) {
+      const int v = (u % (NV / 2)) * kTileThreads + t, row = v / VPR, k = (v % VPR) * V;
+      double *dst = (u < NV / 2 ? As[row] : Bs[row]) + k;
+      float x[V];
+      widen_vec<T>(buf[u], x);
 #pragma unroll
-        for (int k = 0; k < V; ++k) y[k] = 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < V; ++k) { As[kv + k][row] = x[k]; Bs[kv + k][row] = y[k]; }
+      for (int e = 0; e < V; e += 2) *reinterpret_cast<double2 *>(dst + e) = make_double2((double)x[e], (double)x[e + 1]);
     }
     __syncthreads();
+    if (k0 + KC < d_k) fetch(k0 + KC);
 #pragma unroll 8
-    for (int k = 0; k < KC; ++k) {
-      const float4 a4 = *reinterpret_cast<const float4 *>(&As[k][ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[k][tx * 4]);
-      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+    for (int k = 0; k < KC; k += 4) {
+      double a[2], b[2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int f = 0; f < 2; ++f) {
+        a[f] = As[wy * 16 + f * 8 + (lane >> 2)][k + (lane & 3)];
+        b[f] = Bs[wx * 16 + f * 8 + (lane >> 2)][k + (lane & 3)];
+      }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (sizeof(acc_t) == 8) acc[i][j] = fma((acc_t)a[i], (acc_t)b[j], acc[i][j]);
-          else acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+              : "+d"(acc[i][j][0]), "+d"(acc[i][j][1]) : "d"(a[i]), "d"(b[j]));
     }
-    __syncthreads();
   }
 }
 
+// tile `t` of the nt (nt + 1) / 2 tiles on and above the diagonal, row by row
+__device__ __forceinline__ void upper_tile(int t, int nt, int &tm, int &tn) {
+  const double b = 2.0 * nt + 1.0;
+  int i = (int)((b - sqrt(fmax(b * b - 8.0 * t, 0.0))) * 0.5);
+  i = max(0, min(i, nt - 1));
+  while (i > 0 && i * nt - i * (i - 1) / 2 > t) --i;
+  while (i + 1 < nt && (i + 1) * nt - (i + 1) * i / 2 <= t) ++i;
+  tm = i;
+  tn = i + (t - (i * nt - i * (i - 1) / 2));
+}
+
 // ---- Eq. 5-6: all pairs of survivors; density and adjacency in the epilogue --------------------
-// grid (n_ctas, B) persistent over the tiles of the q x q matrix; nothing of it is stored except
-// one bit per pair (d <= d_c) and one integer density per row.
+// grid (n_ctas, B) persistent over the tiles on and above the diagonal of the q x q matrix; nothing of it is stored
+// except one bit per pair (d <= d_c) and one integer density per row.  A tile above the diagonal serves its rows and
+// its columns; the two inverse norms are multiplied first, so that a pair has the same distance from both sides and
+// duplicate keys keep exactly equal densities.
 template <typename T>
-__global__ void __launch_bounds__(256) k_gram_simt(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(kTileThreads) k_gram_f64(const __grid_constant__ Batch bt) {
   using D = typename DistOf<T>::type;
-  using acc_t = typename D::acc_t;
+  using dist_t = typename D::acc_t;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
+  TL_SCOPE(im, 4);
   const int q = *im.q_ptr;
   const int nt = (q + TS - 1) / TS;
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-  __shared__ __align__(16) float As[KC][TS + 4];
-  __shared__ __align__(16) float Bs[KC][TS + 4];
-  __shared__ unsigned long long rowsum[TS];
-  __shared__ uint32_t adjw[TS][2];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
+  __shared__ __align__(16) double As[TS][KST];
+  __shared__ __align__(16) double Bs[TS][KST];
+  __shared__ unsigned long long rsum[2][TS], csum[2][TS];   // by column half of the rows, by row half of the columns
+  __shared__ uint32_t rbits[2][TS], cbits[2][TS];
   const T *Kp = reinterpret_cast<const T *>(im.Kp);
   const auto *rnk = rn_kept<D>(im);
   int band = 0;
-  for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
-    const int tm = tile / nt, tn = tile % nt;
-    if (t < TS) { rowsum[t] = 0ull; adjw[t][0] = 0u; adjw[t][1] = 0u; }
-    acc_t acc[4][4];
-    tile_dots<T, acc_t>(
+  for (int tile = blockIdx.x; tile < nt * (nt + 1) / 2; tile += gridDim.x) {
+    int tm, tn;
+    upper_tile(tile, nt, tm, tn);
+    double acc[2][2][2];
+    tile_dots<T>(
         [&](int r) { const int g = tm * TS + r; return g < q ? Kp + (size_t)g * bt.d_k : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < q ? Kp + (size_t)g * bt.d_k : (const T *)nullptr; },
         bt.d_k, As, Bs, acc);
+    unsigned long long rs[2] = {0ull, 0ull}, cs[2][2] = {};
+    uint32_t rb[2] = {0u, 0u}, cb[2][2] = {};
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int gi = tm * TS + ty * 4 + a;
-      if (gi >= q) continue;
-      const auto rni = rnk[gi];
-      unsigned long long s = 0ull;
-      uint32_t bits = 0u;
+    for (int a = 0; a < 2; ++a) {
+      const int li = wy * 16 + a * 8 + (lane >> 2), gi = tm * TS + li;
+      const double rni = gi < q ? (double)rnk[gi] : 0.0;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int gj = tn * TS + tx * 4 + b;
-        if (gj >= q) continue;
-        auto dd = D::dist(acc[a][b], rni, rnk[gj]);
-        if (gi == gj) dd = 0;
-        s += D::term(dd, im);
-        if (D::within(dd, im)) bits |= 1u << b;
-        if (gi < gj && D::in_band(dd, im)) ++band;
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int lj = wx * 16 + b * 8 + 2 * (lane & 3) + e, gj = tn * TS + lj;
+          if (gi >= q || gj >= q) continue;
+          dist_t dd = (dist_t)fmin(fmax(1.0 - acc[a][b][e] * (rni * (double)rnk[gj]), 0.0), 2.0);
+          if (gi == gj) dd = 0;
+          const unsigned long long term = D::term(dd, im);
+          rs[a] += term;
+          cs[b][e] += term;
+          if (D::within(dd, im)) { rb[a] |= 1u << lj; cb[b][e] |= 1u << li; }
+          if (gi < gj && D::in_band(dd, im)) ++band;
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {                      // rows: the four lanes that hold parts of one
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        rs[a] += __shfl_xor_sync(0xffffffffu, rs[a], o);
+        rb[a] |= __shfl_xor_sync(0xffffffffu, rb[a], o);
       }
-      atomicAdd(&rowsum[ty * 4 + a], s);
-      if (bits) atomicOr(&adjw[ty * 4 + a][tx >> 3], bits << ((tx & 7) * 4));
+      if ((lane & 3) == 0) { rsum[wx][wy * 16 + a * 8 + (lane >> 2)] = rs[a]; rbits[wx][wy * 16 + a * 8 + (lane >> 2)] = rb[a]; }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {                    // columns: the eight lanes
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+          cs[a][e] += __shfl_xor_sync(0xffffffffu, cs[a][e], o);
+          cb[a][e] |= __shfl_xor_sync(0xffffffffu, cb[a][e], o);
+        }
+        if (lane < 4) { csum[wy][wx * 16 + a * 8 + 2 * lane + e] = cs[a][e]; cbits[wy][wx * 16 + a * 8 + 2 * lane + e] = cb[a][e]; }
+      }
     }
     __syncthreads();
-    if (t < TS) {
-      const int gi = tm * TS + t;
-      if (gi < q) atomicAdd(&im.rho_fix[gi], rowsum[t]);
-    } else if (t < 3 * TS) {
-      const int r = (t - TS) >> 1, wd = (t - TS) & 1;
-      const int gi = tm * TS + r;
-      if (gi < q) im.adj[(size_t)gi * im.Wp + tn * 2 + wd] = adjw[r][wd];
+    if (t < 2 * TS) {                                  // (the barrier inside the next tile_dots comes before these are rewritten)
+      const int l = t & (TS - 1), side = t / TS;       // 0: rows, 1: columns (above the diagonal only)
+      const int g = (side ? tn : tm) * TS + l;
+      if (g < q && !(side && tm == tn)) {
+        atomicAdd(&im.rho_fix[g], side ? csum[0][l] + csum[1][l] : rsum[0][l] + rsum[1][l]);
+        im.adj[(size_t)g * im.Wp + (side ? tm : tn)] = side ? (cbits[0][l] | cbits[1][l]) : (rbits[0][l] | rbits[1][l]);
+      }
     }
-    __syncthreads();
   }
   if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
 }
@@ -213,9 +254,12 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_key_rnorm(const __grid_constant__ Batch bt) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i == 0 && lane == 0) im.cnt[kCntSpread] = 0;
   if (i >= im.N) return;
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
@@ -223,46 +267,52 @@ __global__ void __launch_bounds__(256) k_key_rnorm(const __grid_constant__ Batch
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_spread_simt(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(kTileThreads) k_spread_f64(const __grid_constant__ Batch bt) {
   using D = typename DistOf<T>::type;
   using acc_t = typename D::acc_t;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
   const int N = im.N;
   const int nt = (N + TS - 1) / TS;
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-  __shared__ __align__(16) float As[KC][TS + 4];
-  __shared__ __align__(16) float Bs[KC][TS + 4];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
+  __shared__ __align__(16) double As[TS][KST];
+  __shared__ __align__(16) double Bs[TS][KST];
   const T *K = reinterpret_cast<const T *>(im.Kc);
   const auto *rn = rn_tok<D>(im);
   float mx = 0.f;
-  for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
-    const int tm = tile / nt, tn = tile % nt;
-    if (tn < tm) continue;                         // every unordered pair once (uniform)
-    acc_t acc[4][4];
-    tile_dots<T, acc_t>(
+  for (int tile = blockIdx.x; tile < nt * (nt + 1) / 2; tile += gridDim.x) {   // every unordered pair once
+    int tm, tn;
+    upper_tile(tile, nt, tm, tn);
+    double acc[2][2][2];
+    tile_dots<T>(
         [&](int r) { const int g = tm * TS + r; return g < N ? K + (size_t)g * im.ldKc : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < N ? K + (size_t)g * im.ldKc : (const T *)nullptr; },
         bt.d_k, As, Bs, acc);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int gi = tm * TS + ty * 4 + a;
+    for (int a = 0; a < 2; ++a) {
+      const int gi = tm * TS + wy * 16 + a * 8 + (lane >> 2);
       if (gi >= N) continue;
       const auto rni = rn[gi];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int gj = tn * TS + tx * 4 + b;
-        if (gj >= N || gj == gi) continue;
-        mx = fmaxf(mx, (float)D::dist(acc[a][b], rni, rn[gj]));
-      }
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int gj = tn * TS + wx * 16 + b * 8 + 2 * (lane & 3) + e;
+          if (gj >= N || gj == gi) continue;
+          mx = fmaxf(mx, (float)D::dist((acc_t)acc[a][b][e], rni, rn[gj]));
+        }
     }
   }
-  const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));   // distances are >= 0
-  if ((t & 31) == 0 && w) atomicMax(reinterpret_cast<unsigned *>(&im.cnt[kCntSpread]), w);
+  const unsigned wmx = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));   // distances are >= 0
+  if (lane == 0 && wmx) atomicMax(reinterpret_cast<unsigned *>(&im.cnt[kCntSpread]), wmx);
 }
 
 // one warp: max_dist[l] of the layers of this batch, and the earliest layer at or above the threshold
 __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dist, int32_t *layer_out,
                                 int layer_base, float threshold) {
+  pdl_wait();
+  pdl_trigger();
   const int l = threadIdx.x;
   float v = -1.f;
   if (l < bt.B) {
@@ -527,21 +577,24 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
 }
 
 // ---- nearest centre of every row (Algorithm 2 assignment; Eq. 8 argmin) ---------------------------
-// grid (n_ctas, B) persistent over 64 x 64 tiles of rows x centres; the running minimum of a row
+// grid (n_ctas, B) persistent over 32 x 32 tiles of rows x centres; the running minimum of a row
 // is one 64-bit word (distance bits, cluster id) reduced with atomicMin, so ties go to the lower id.
 template <typename T>
-__global__ void __launch_bounds__(256) k_assign_simt(const __grid_constant__ Batch bt, int mode) {
+__global__ void __launch_bounds__(kTileThreads) k_assign_f64(const __grid_constant__ Batch bt, int mode) {
   using D = typename DistOf<T>::type;
   using acc_t = typename D::acc_t;
+  pdl_wait();
+  pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
+  TL_SCOPE(im, 6);
   const int C = *im.C_ptr;
   const int nrows = mode == ROWS_ALL ? im.N : (mode == ROWS_KEPT_LIST ? *im.q_ptr : *im.m_ptr);
   const int32_t *list = mode == ROWS_KEPT_LIST ? im.kept_idx : im.pruned_idx;
   const int ntm = (nrows + TS - 1) / TS, ntn = (C + TS - 1) / TS;
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-  __shared__ __align__(16) float As[KC][TS + 4];
-  __shared__ __align__(16) float Bs[KC][TS + 4];
-  __shared__ unsigned long long rowbest[TS];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
+  __shared__ __align__(16) double As[TS][KST];
+  __shared__ __align__(16) double Bs[TS][KST];
+  __shared__ unsigned long long rowbest[2][TS];
   __shared__ int rowtok[TS];
   const T *Kc = reinterpret_cast<const T *>(im.Kc);
   const T *Kcen = reinterpret_cast<const T *>(im.Kcen);
@@ -549,36 +602,41 @@ __global__ void __launch_bounds__(256) k_assign_simt(const __grid_constant__ Bat
   const auto *rnc = rn_cen<D>(im);
   for (int tile = blockIdx.x; tile < ntm * ntn; tile += gridDim.x) {
     const int tm = tile / ntn, tn = tile % ntn;
+    __syncthreads();                                   // the tile before has written its minima
     if (t < TS) {
-      rowbest[t] = kBestInit;
       const int g = tm * TS + t;
       rowtok[t] = g < nrows ? (mode == ROWS_ALL ? g : list[g]) : -1;
     }
     __syncthreads();
-    acc_t acc[4][4];
-    tile_dots<T, acc_t>(
+    double acc[2][2][2];
+    tile_dots<T>(
         [&](int r) { const int tok = rowtok[r]; return tok >= 0 ? Kc + (size_t)tok * im.ldKc : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < C ? Kcen + (size_t)g * bt.d_k : (const T *)nullptr; },
         bt.d_k, As, Bs, acc);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int tok = rowtok[ty * 4 + a];
-      if (tok < 0) continue;
-      const auto rni = rnt[tok];
+    for (int a = 0; a < 2; ++a) {
+      const int l = wy * 16 + a * 8 + (lane >> 2), tok = rowtok[l];
+      const auto rni = tok >= 0 ? rnt[tok] : 0;
       unsigned long long bestv = kBestInit;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = tn * TS + tx * 4 + b;
-        if (c >= C) continue;
-        const float dd = (float)D::dist(acc[a][b], rni, rnc[c]);
-        const unsigned long long pk = ((unsigned long long)__float_as_uint(dd) << 32) | (unsigned)c;
-        bestv = pk < bestv ? pk : bestv;
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int c = tn * TS + wx * 16 + b * 8 + 2 * (lane & 3) + e;
+          if (c >= C) continue;
+          const float dd = (float)D::dist((acc_t)acc[a][b][e], rni, rnc[c]);
+          const unsigned long long pk = ((unsigned long long)__float_as_uint(dd) << 32) | (unsigned)c;
+          bestv = pk < bestv ? pk : bestv;
+        }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, bestv, o);
+        bestv = y < bestv ? y : bestv;
       }
-      atomicMin(&rowbest[ty * 4 + a], bestv);
+      if ((lane & 3) == 0) rowbest[wx][l] = bestv;
     }
     __syncthreads();
-    if (t < TS && rowtok[t] >= 0) atomicMin(&im.best[rowtok[t]], rowbest[t]);
-    __syncthreads();
+    if (t < TS && rowtok[t] >= 0) atomicMin(&im.best[rowtok[t]], rowbest[0][t] < rowbest[1][t] ? rowbest[0][t] : rowbest[1][t]);
   }
 }
 
@@ -590,6 +648,8 @@ __global__ void __launch_bounds__(256) k_label(const __grid_constant__ Batch bt,
   using D = typename DistOf<T>::type;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 7);
+  pdl_wait();
+  pdl_trigger();
   const int nrows = mode == ROWS_ALL ? im.N : (mode == ROWS_KEPT_LIST ? *im.q_ptr : *im.m_ptr);
   int joined = 0, dropped = 0, band = 0;
   for (int g = blockIdx.x * 256 + threadIdx.x; g < nrows; g += gridDim.x * 256) {
@@ -617,7 +677,10 @@ __global__ void __launch_bounds__(256) k_label(const __grid_constant__ Batch bt,
     band += __shfl_xor_sync(0xffffffffu, band, o);
   }
   if ((threadIdx.x & 31) == 0) {
-    if (joined) { atomicAdd(&im.cnt[PACT_CNT_R], joined); }
+    if (joined) {
+      atomicAdd(&im.cnt[PACT_CNT_R], joined);
+      if (im.r_user) atomicAdd(im.r_user, joined);
+    }
     if (dropped) atomicAdd(&im.cnt[PACT_CNT_DISCARDED], dropped);
     if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_ADC], band);
   }
@@ -640,28 +703,24 @@ cudaError_t cluster_configure(ClusterCfg *cfg) {
   return cudaFuncSetAttribute(k_centers<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
 }
 
-#define PACT_DISPATCH(bf16, KERNEL, ...)                       \
-  do {                                                         \
-    if (bf16) KERNEL<__nv_bfloat16> __VA_ARGS__;               \
-    else KERNEL<float> __VA_ARGS__;                            \
-  } while (0)
+#define PACT_DISPATCH(bf16, KERNEL, grid, block, st, ...)                                      \
+  ((bf16) ? launch_k(KERNEL<__nv_bfloat16>, grid, dim3(block), 0, st, true, __VA_ARGS__)       \
+          : launch_k(KERNEL<float>, grid, dim3(block), 0, st, true, __VA_ARGS__))
 
-void launch_keynorm_gather(const Batch &bt, int maxN, bool bf16, bool all_tokens, cudaStream_t st) {
-  dim3 grid((maxN + 7) / 8, bt.B);
-  PACT_DISPATCH(bf16, k_keynorm_gather, <<<grid, 256, 0, st>>>(bt, all_tokens ? 1 : 0));
+cudaError_t launch_keynorm_gather(const Batch &bt, int maxN, bool bf16, cudaStream_t st) {
+  return PACT_DISPATCH(bf16, k_keynorm_gather, dim3((maxN + 7) / 8, bt.B), 256, st, bt);
 }
 
-void launch_center_key_gather(const Batch &bt, int maxN, bool bf16, cudaStream_t st) {
-  dim3 grid((maxN + 7) / 8, bt.B);
-  PACT_DISPATCH(bf16, k_center_key_gather, <<<grid, 256, 0, st>>>(bt));
+cudaError_t launch_center_key_gather(const Batch &bt, int maxN, bool bf16, bool all_rows, cudaStream_t st) {
+  return PACT_DISPATCH(bf16, k_center_key_gather, dim3((maxN + 7) / 8, bt.B), 256, st, bt, all_rows ? 1 : 0);
 }
 
 static int tile_grid(long long tiles, int cap) { return (int)(tiles < 1 ? 1 : (tiles > cap ? cap : tiles)); }
 
-void launch_gram(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_gram(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
-  dim3 grid(tile_grid(nt * nt, cfg.sm_count * 8), bt.B);
-  PACT_DISPATCH(bf16, k_gram_simt, <<<grid, 256, 0, st>>>(bt));
+  dim3 grid(tile_grid(nt * (nt + 1) / 2, cfg.sm_count * 5), bt.B);
+  return PACT_DISPATCH(bf16, k_gram_f64, grid, kTileThreads, st, bt);
 }
 
 cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int spin_limit, cudaStream_t st) {
@@ -673,40 +732,35 @@ cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCf
   int mask_cap = (maxQ + 31) / 32 + 1;
   if ((size_t)mask_cap * 8 > budget) mask_cap = 0;
   const size_t smem = (size_t)keys_cap * sizeof(unsigned long long) + (size_t)mask_cap * 8;
-  int per_sm = 0;
-  cudaError_t e = bf16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_centers<__nv_bfloat16>, kCenThreads, smem)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_centers<float>, kCenThreads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   return bf16 ? launch_coop(k_centers<__nv_bfloat16>, dim3(cfg.sm_count), dim3(kCenThreads), smem, st, true, bt, keys_cap, mask_cap, spin_limit)
               : launch_coop(k_centers<float>, dim3(cfg.sm_count), dim3(kCenThreads), smem, st, true, bt, keys_cap, mask_cap, spin_limit);
 }
 
-void launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const ClusterCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
-  dim3 grid(tile_grid(nt * nt, cfg.sm_count * 8), bt.B);
-  PACT_DISPATCH(bf16, k_assign_simt, <<<grid, 256, 0, st>>>(bt, (int)mode));
+  dim3 grid(tile_grid(nt * nt, cfg.sm_count * 5), bt.B);
+  return PACT_DISPATCH(bf16, k_assign_f64, grid, kTileThreads, st, bt, (int)mode);
 }
 
-void launch_key_rnorm(const Batch &bt, int maxN, bool bf16, cudaStream_t st) {
+cudaError_t launch_key_rnorm(const Batch &bt, int maxN, bool bf16, cudaStream_t st) {
   dim3 grid((maxN + 7) / 8, bt.B);
-  PACT_DISPATCH(bf16, k_key_rnorm, <<<grid, 256, 0, st>>>(bt));
+  return PACT_DISPATCH(bf16, k_key_rnorm, grid, 256, st, bt);
 }
 
-void launch_spread(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_spread(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
-  dim3 grid(tile_grid(nt * (nt + 1) / 2, cfg.sm_count * 8), bt.B);
-  PACT_DISPATCH(bf16, k_spread_simt, <<<grid, 256, 0, st>>>(bt));
+  dim3 grid(tile_grid(nt * (nt + 1) / 2, cfg.sm_count * 5), bt.B);
+  return PACT_DISPATCH(bf16, k_spread_f64, grid, kTileThreads, st, bt);
 }
 
-void launch_spread_finish(const Batch &bt, float *max_dist, int32_t *layer_out, int layer_base, float threshold,
+cudaError_t launch_spread_finish(const Batch &bt, float *max_dist, int32_t *layer_out, int layer_base, float threshold,
                           cudaStream_t st) {
-  k_spread_finish<<<1, 32, 0, st>>>(bt, max_dist, layer_out, layer_base, threshold);
+  return launch_k(k_spread_finish, dim3(1), dim3(32), 0, st, true, bt, max_dist, layer_out, layer_base, threshold);
 }
 
-void launch_label(const Batch &bt, int maxN, bool bf16, RowMode mode, cudaStream_t st) {
+cudaError_t launch_label(const Batch &bt, int maxN, bool bf16, RowMode mode, cudaStream_t st) {
   dim3 grid(tile_grid((maxN + 255) / 256, 1 << 16), bt.B);
-  PACT_DISPATCH(bf16, k_label, <<<grid, 256, 0, st>>>(bt, (int)mode));
+  return PACT_DISPATCH(bf16, k_label, grid, 256, st, bt, (int)mode);
 }
 
 }  // namespace pact

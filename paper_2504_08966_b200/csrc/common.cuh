@@ -16,8 +16,8 @@ constexpr int kCntSpread = 24;           // slot of cnt[]: largest key distance 
 constexpr int kSpinLimit = 1 << 20;      // default number of polls a bounded device wait makes before it gives up
 constexpr int kListBlock = 128;          // tokens per block of the member lists (128 measured 0.8 us faster per step than 256)
 constexpr int kMaxTokens = 1 << 18;      // most visual tokens per image
-constexpr int kCntInts = 64;             // counters and tickets at the head of an image's workspace ...
-constexpr int kTickInts = 1024;          // ... followed by the tickets of k_qsum; both are cleared when a call starts
+constexpr int kCntInts = 64;             // counters at the head of an image's workspace, cleared by the first kernel of a call
+constexpr int kMaxColGroups = 1024;      // most groups of eight 16-byte vectors in a row of Q
 
 // Per-image device pointers: the caller's buffers and the slices of the workspace.
 struct ImgDesc {
@@ -37,7 +37,6 @@ struct ImgDesc {
   double d_c64, inv_dn64, t_reinc64;
   unsigned flags;
   // workspace
-  double *qpart;         // [kQPartRows][n_qcols] partial column sums of Q
   double *qg;            // [n_qcols] global query
   double *E;             // [N][n_qh] exp(logit - CTA max)
   double *part;          // [G][n_qh][2] per-CTA (max, sum) of k_tokens, G = ceil(N / 32)
@@ -72,14 +71,14 @@ struct ImgDesc {
   int32_t *cticket;      // [Np] chunks of cluster c that are finished
   int32_t *rtick;        // [Wp] epilogue warps of the rows x centres pass that are done with a group of 32 tokens
   float *mpart;          // [2 * merge CTAs][d] sums of the clusters that a range boundary of k_merge cuts
-  int32_t *tick;         // [kTickInts] tickets of k_qsum, one per column group; zero when a call starts (cleared with cnt)
-  int32_t *cnt;          // [PACT_N_COUNTERS] + [16] ticket of the global query, [19] barrier of k_lists, [20] members of all clusters
+  int32_t *cnt;          // [PACT_N_COUNTERS] + [19] barrier of k_lists, [20] members of all clusters
   const int32_t *q_ptr;  // where the number of survivors lives (cnt[Q] or the caller's q_dev)
   const int32_t *m_ptr;  // where the number of pruned tokens lives
   const int32_t *C_ptr;  // where the number of clusters lives
   const int32_t *cidx_ptr;  // token index of centre c (workspace or caller)
   float *rho_user;       // optional outputs of the stage calls
   int32_t *center_idx_user, *C_user, *r_user;
+  int32_t *counts_user;  // [2] survivors and pruned tokens, for pact_prune
   unsigned long long *tl; // timeline buffer of the instrumented build (PACT_TIMELINE), else unused
   int Np, Wp;            // padded survivor capacity and words per adjacency row
   int nbp;               // entries per row of cnt_cb: token blocks, rounded up to a multiple of 8

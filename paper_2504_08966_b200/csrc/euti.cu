@@ -10,7 +10,7 @@
 //   k_select         every CTA selects the threshold (histogram bin, then radix passes inside the bin) and
 //                    counts the survivors before its tokens, then writes its share of the lists and gathers
 //                    its share of the survivor keys
-//   k_select_gather  the split for the stage call pact_prune (scores given, no histogram): radix select
+//   k_split          the split for the stage call pact_prune (scores given, no histogram): radix select
 //
 // The kernels are short chains of dependent memory round trips; each issues all the loads it can
 // before it consumes the first.
@@ -24,6 +24,19 @@ __device__ __forceinline__ double ld_cg_f64(const double *p) {
   return v;
 }
 
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the double at this shared-memory location of CTA `rank` of the cluster
+__device__ __forceinline__ double ld_cluster_f64(const double *p, int rank) {
+  uint32_t a;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+
 // sort key of a score: unsigned integers that order like the floats
 __device__ __forceinline__ uint32_t score_key(float s) {
   uint32_t b = __float_as_uint(s);
@@ -32,14 +45,14 @@ __device__ __forceinline__ uint32_t score_key(float s) {
 }
 
 // ---- Eq. 1: column sums of Q -----------------------------------------------------------------------------
-// grid (ncg RP, B), 512 threads at no more than 64 registers, on fewer than half of the SMs: a CTA leaves room
-// for one CTA of k_tokens beside it, and the other SMs take two, so that all of them start at once.  Work item
-// (column group of eight 16-byte vectors, block of rows): thread t takes vector t & 7 of the group and the rows
-// r0 + (t >> 3), + 64, ...; the four row lanes of a warp are added with shuffles, the warps through
-// shared memory.  The CTA that finishes a column group's last
-// row block adds the RP partial sums in block order and writes the group's part of the global query, so the
-// result does not depend on which CTA that is.  do_init: the grid also clears what later kernels accumulate
-// into.
+// grid (ncg RP, B) in clusters of RP CTAs, 512 threads at no more than 64 registers, on fewer than half of the
+// SMs where that is enough: a CTA leaves room for one CTA of k_tokens beside it, and the other SMs take two, so that
+// all of them start at once.  Work item (column group of eight 16-byte vectors, block of rows): thread t takes vector
+// t & 7 of the group and the rows r0 + (t >> 3), + 64, ...; the four row lanes of a warp are added with shuffles, the
+// warps through shared memory.  The RP row blocks of a column group are one cluster: its first CTA reads the
+// others' sums through distributed shared memory and adds them in block order.  (Partial sums in global memory
+// behind a ticket cost 2.6 us from the last row to the global query, and a cleared ticket before the kernel.)
+// do_init: the grid also clears what later kernels accumulate into.
 constexpr int kQsumThreads = 512;
 constexpr int kQsumRowLanes = kQsumThreads / 8;
 constexpr int kQsumWarps = kQsumThreads / 32;
@@ -49,6 +62,7 @@ __global__ void __launch_bounds__(kQsumThreads, 2) k_qsum(const __grid_constant_
   constexpr int V = Vec<T>::N;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 0);
+  pdl_wait();                                           // the work before this call, which may still use the workspace
   pdl_trigger();                                        // k_tokens may start: its first pass does not need the query
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, N = im.N, n_qcols = bt.n_qcols;
   if (do_init) {
@@ -60,13 +74,13 @@ __global__ void __launch_bounds__(kQsumThreads, 2) k_qsum(const __grid_constant_
     const int nq = im.Np * (im.nbp / 8);
     for (int i = gt; i < nq; i += gs) tab[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = gt; i < (1 << kHistBits); i += gs) im.ghist[i] = 0;
+    if (gt < kCntInts) im.cnt[gt] = 0;
   }
   if (!im.Q || (im.flags & PACT_FLAG_NORM_ONLY)) return;
-  const int nvq = n_qcols / V, ncg = (nvq + 7) / 8;
-  const int cg = blockIdx.x % ncg, rp = blockIdx.x / ncg;
-  if (rp >= RP) return;
+  const int nvq = n_qcols / V;
+  const int cg = blockIdx.x / RP, rp = blockIdx.x % RP; // rp = rank of the CTA in its cluster
   __shared__ double sm[kQsumWarps * 8 * V];
-  __shared__ int s_last;
+  __shared__ double s_part[8 * V];
   const int rchunk = (N + RP - 1) / RP;
   const int r0 = min(N, rp * rchunk), r1 = min(N, r0 + rchunk);
   const int v = cg * 8 + (t & 7);
@@ -112,31 +126,17 @@ __global__ void __launch_bounds__(kQsumThreads, 2) k_qsum(const __grid_constant_
 #pragma unroll
     for (int ww = 0; ww < kQsumWarps; ++ww) mine += sm[ww * 8 * V + t];
   }
-  if (RP == 1) {
-    if (col_ok) im.qg[col] = mine / (double)N;
-    return;
-  }
-  if (col_ok) im.qpart[(size_t)rp * n_qcols + col] = mine;
-  __threadfence();
-  __syncthreads();
-  if (t == 0) s_last = atomicAdd(&im.tick[cg], 1) == RP - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (col_ok) {
-    double s = 0.0;
+  if (t < 8 * V) s_part[t] = mine;
+  cluster_sync();
+  if (rp == 0 && col_ok) {
+    double pv[kQPartRows], s = 0.0;
 #pragma unroll
-    for (int u0 = 0; u0 < kQPartRows; u0 += 16) {       // sixteen partial sums in flight, added in block order
-      if (u0 < RP) {
-        double pv[16];
+    for (int u = 0; u < kQPartRows; ++u) pv[u] = u < RP ? ld_cluster_f64(&s_part[t], u) : 0.0;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) pv[u] = u0 + u < RP ? ld_cg_f64(&im.qpart[(size_t)(u0 + u) * n_qcols + col]) : 0.0;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) s += pv[u];
-      }
-    }
+    for (int u = 0; u < kQPartRows; ++u) s += pv[u];
     im.qg[col] = s / (double)N;
   }
+  cluster_sync();                                       // a CTA's sums may be read until here
 }
 
 // ---- Eq. 2, token pass: hidden-state norm, inverse key norm, logits, CTA-local softmax pieces ---------------
@@ -691,25 +691,20 @@ __global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant
   else euti_select<T, 0, false>(bt, im, skey_dyn, x, tok0, ntok, sh);
 }
 
-// ---- Eq. 3-4: order statistic, ordered compaction; survivor key gather ------------------------------
+// ---- Eq. 3-4 as a stage of its own (pact_prune): order statistic, ordered compaction ------------------
 
-// grid (X, B), 1024 threads; dynamic smem: own_cap token indices, then (KPT == 0 and keys_in_smem) N keys.
-// Every CTA computes the same threshold and the same list positions; CTA b writes the list entries of
-// its block of tokens, and (do_gather) copies its block of survivor rows into Kp and their inverse
-// norms into rnk, and clears its share of the arrays that later kernels accumulate into.
+// grid (1), 1024 threads; dynamic smem: N keys when KPT == 0 and keys_in_smem.
 // KPT > 0: thread t keeps the keys of tokens [t KPT, t KPT + KPT) in registers (N <= 1024 KPT);
 // KPT == 0: any N, keys in shared memory when they fit, else re-read from the scores.
-template <typename T, int KPT>
-__global__ void __launch_bounds__(1024) k_select_gather(const __grid_constant__ Batch bt, int do_gather,
-                                                        int keys_in_smem, int own_cap) {
-  using D = typename DistOf<T>::type;
+template <int KPT>
+__global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt, int keys_in_smem) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 3);
+  pdl_wait();
+  pdl_trigger();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int N = im.N;
-  extern __shared__ uint32_t dsm[];
-  int *own = reinterpret_cast<int *>(dsm);                  // [own_cap]
-  uint32_t *skey = dsm + own_cap;                           // [N] when KPT == 0 and keys_in_smem
+  extern __shared__ uint32_t skey[];                        // [N] when KPT == 0 and keys_in_smem
   __shared__ int hist[256];
   __shared__ int warp_tot[32];
   __shared__ uint32_t wmin[32], wmax[32];
@@ -730,15 +725,6 @@ __global__ void __launch_bounds__(1024) k_select_gather(const __grid_constant__ 
     for (int j = 0; j < KR; ++j) kreg[j] = score_key(sc[j]);
   } else if (keys_in_smem) {
     for (int i = t; i < N; i += 1024) skey[i] = score_key(im.score[i]);
-  }
-  if (do_gather) {   // per-call initialisation, spread over the grid
-    const int gt = blockIdx.x * 1024 + t, gs = gridDim.x * 1024;
-    for (int r = gt; r < im.Np; r += gs) { im.rho_fix[r] = 0ull; im.csize[r] = 0; im.cticket[r] = 0; }
-    for (int wd = gt; wd < im.Wp; wd += gs) { im.cmask[wd] = 0u; im.rmask[wd] = 0u; im.rtick[wd] = 0; }
-    for (int i = gt; i < N; i += gs) im.best[i] = kBestInit;
-    uint4 *tab = reinterpret_cast<uint4 *>(im.cnt_cb);
-    const int nq = im.Np * (im.nbp / 8);
-    for (int i = gt; i < nq; i += gs) tab[i] = make_uint4(0u, 0u, 0u, 0u);
   }
   if (t == 0) s_k = im.m_target;
   if (t < 256) hist[t] = 0;
@@ -856,51 +842,16 @@ __global__ void __launch_bounds__(1024) k_select_gather(const __grid_constant__ 
   __syncthreads();
   const int q = s_k;
   int before = warp_tot[w] + incl - mine;                   // survivors with a lower index
-  const int tpc = (N + gridDim.x - 1) / gridDim.x;          // tokens whose list entries this CTA writes
-  const int w0 = blockIdx.x * tpc, w1 = min(N, w0 + tpc);
-  const int rpc = (q + gridDim.x - 1) / gridDim.x;          // survivor rows this CTA gathers
-  const int g0 = min(q, (int)blockIdx.x * rpc), g1 = min(q, g0 + rpc);
-  const bool touches = (i0 < w1 && i1 > w0) || (do_gather && before < g1 && before + mine > g0);
-  if (touches) {
-    for (int j = 0; j < cnt_mine; ++j) {
-      const int i = i0 + j;
-      const bool kp = (KPT > 0 || CH <= 32) ? ((keptbits >> j) & 1u) != 0u : key(j) >= tau_key;
-      if (i >= w0 && i < w1) {
-        im.keep[i] = kp ? 1 : 0;
-        if (im.keep_user) im.keep_user[i] = kp ? 1 : 0;
-        if (kp) { im.kept_idx[before] = i; im.slot[i] = before; }
-        else { im.pruned_idx[i - before] = i; im.slot[i] = -1 - (i - before); }
-      }
-      if (kp) {
-        if (do_gather && before >= g0 && before < g1 && before - g0 < own_cap) own[before - g0] = i;
-        ++before;
-      }
-    }
+  for (int j = 0; j < cnt_mine; ++j) {
+    const int i = i0 + j;
+    const bool kp = (KPT > 0 || CH <= 32) ? ((keptbits >> j) & 1u) != 0u : key(j) >= tau_key;
+    im.keep[i] = kp ? 1 : 0;
+    if (kp) { im.kept_idx[before] = i; ++before; }
+    else im.pruned_idx[i - before] = i;
   }
-  if (blockIdx.x == 0 && t == 0) {
-    im.cnt[PACT_CNT_Q] = q;
-    im.cnt[PACT_CNT_M] = N - q;
-  }
-  if (!do_gather) return;
-  __syncthreads();
-  constexpr int V = Vec<T>::N;
-  const int nv = bt.d_k / V;
-  const T *Kc = reinterpret_cast<const T *>(im.Kc);
-  T *Kp = reinterpret_cast<T *>(im.Kp);
-  for (int rr = g0 + w; rr < g1; rr += 32) {
-    const int tok = own[rr - g0];
-    const uint4 *src = reinterpret_cast<const uint4 *>(Kc + (size_t)tok * im.ldKc);
-    uint4 *dst = reinterpret_cast<uint4 *>(Kp + (size_t)rr * bt.d_k);
-    for (int v0 = lane; v0 < nv; v0 += 128) {
-      uint4 buf[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (v0 + 32 * u < nv) buf[u] = __ldg(src + v0 + 32 * u);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (v0 + 32 * u < nv) dst[v0 + 32 * u] = buf[u];
-    }
-    if (lane == 0) rn_kept<D>(im)[rr] = rn_tok<D>(im)[tok];
+  if (t == 0) {
+    im.counts_user[0] = q;
+    im.counts_user[1] = N - q;
   }
 }
 
@@ -909,16 +860,15 @@ __global__ void __launch_bounds__(1024) k_select_gather(const __grid_constant__ 
 namespace {
 int g_sm_count = 148;
 size_t g_smem_optin = 48 * 1024;
-constexpr size_t kSelectReserve = 4096;      // static shared memory of k_select_gather, rounded up
+constexpr size_t kSplitReserve = 4096;       // static shared memory of k_split, rounded up
 }  // namespace
 
 static int qsum_row_blocks(int ncg, int B, int maxN) {
   // CTAs on 7/16 of the SMs (64 of 148) when that leaves a CTA no more than two rounds of loads (1024 rows),
-  // else as many row blocks as that takes: see k_qsum
-  int RP = g_sm_count * 7 / 16 / (ncg * B);
-  const int need = (maxN + 1023) / 1024;
-  if (RP < need) RP = need;
-  return RP < 1 ? 1 : (RP > kQPartRows ? kQPartRows : RP);
+  // else as many row blocks as that takes, up to a cluster of eight: see k_qsum
+  int RP = 1;
+  while (RP < kQPartRows && (ncg * B * RP * 2 <= g_sm_count * 7 / 16 || (maxN + RP - 1) / RP > 1024)) RP *= 2;
+  return RP;
 }
 
 template <typename T>
@@ -926,7 +876,9 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   constexpr int V = Vec<T>::N;
   const int ncg = (bt.n_qcols / V + 7) / 8;
   const int RP = qsum_row_blocks(ncg, bt.B, maxN);
-  cudaError_t e = launch_k(k_qsum<T>, dim3(ncg * RP, bt.B), dim3(kQsumThreads), 0, st, false, bt, RP, mode == 0 ? 1 : 0);
+  LaunchOpt opt;
+  opt.cluster = RP;
+  cudaError_t e = launch_opt(opt, k_qsum<T>, dim3(ncg * RP, bt.B), dim3(kQsumThreads), 0, st, bt, RP, mode == 0 ? 1 : 0);
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
   const size_t sm_tok = (size_t)(bt.n_qcols + kRowsPerCta * bt.n_qh) * sizeof(double);
@@ -957,31 +909,12 @@ cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStre
 
 int euti_kernels(int mode) { return mode == 0 ? 4 : 3; }
 
-template <typename T>
-static void launch_select_t(const Batch &bt, int maxN, bool gather, cudaStream_t st) {
-  int X = 1;
-  if (gather) {
-    X = g_sm_count / bt.B;
-    if (X < 1) X = 1;
-    const int cap = (maxN + 31) / 32;          // at least 32 survivor rows per CTA
-    if (X > cap) X = cap;
-  }
-  const int own_cap = gather ? (maxN + X - 1) / X + 1 : 0;
-  size_t sm = (size_t)own_cap * sizeof(int);
-  dim3 grid(X, bt.B);
-  const int g = gather ? 1 : 0;
-  if (maxN <= 8 * 1024) k_select_gather<T, 8><<<grid, 1024, sm, st>>>(bt, g, 0, own_cap);
-  else if (maxN <= 16 * 1024) k_select_gather<T, 16><<<grid, 1024, sm, st>>>(bt, g, 0, own_cap);
-  else {
-    const bool in_smem = sm + (size_t)maxN * 4 + kSelectReserve <= g_smem_optin;
-    if (in_smem) sm += (size_t)maxN * 4;
-    k_select_gather<T, 0><<<grid, 1024, sm, st>>>(bt, g, in_smem ? 1 : 0, own_cap);
-  }
-}
-
-void launch_select_gather(const Batch &bt, int maxN, bool bf16, bool gather, cudaStream_t st) {
-  if (bf16) launch_select_t<__nv_bfloat16>(bt, maxN, gather, st);
-  else launch_select_t<float>(bt, maxN, gather, st);
+cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st) {
+  if (N <= 8 * 1024) return launch_k(k_split<8>, dim3(1), dim3(1024), 0, st, true, bt, 0);
+  if (N <= 16 * 1024) return launch_k(k_split<16>, dim3(1), dim3(1024), 0, st, true, bt, 0);
+  const size_t sm = (size_t)N * sizeof(uint32_t);
+  const bool in_smem = sm + kSplitReserve <= g_smem_optin;
+  return launch_k(k_split<0>, dim3(1), dim3(1024), in_smem ? sm : 0, st, true, bt, in_smem ? 1 : 0);
 }
 
 cudaError_t select_configure() {
@@ -994,10 +927,7 @@ cudaError_t select_configure() {
   e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   g_smem_optin = (size_t)v;
-  const int dyn = (int)(g_smem_optin - kSelectReserve);
-  e = cudaFuncSetAttribute(k_select_gather<__nv_bfloat16, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_select_gather<float, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  return cudaFuncSetAttribute(k_split<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
 }
 
 cudaError_t euti_configure(int n_qcols, int n_qh) {

@@ -936,27 +936,14 @@ bool g_pair_gram_ok = false;                          // ... of its all-pairs fo
 bool g_pair_assign_ok = false;                        // ... of its rows x centres form
 
 template <int MODE, int EW>
-cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, int kept_rows, const ClusterCfg &cfg, bool pdl,
-                        cudaStream_t st) {
+cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, int kept_rows, const ClusterCfg &cfg, cudaStream_t st) {
   using PC = PairCfg<MODE, EW>;
   long long P = cfg.sm_count / 2;                     // one pair per two SMs
   if (P > tiles * bt.B) P = tiles * bt.B;
   if (P < 1) P = 1;
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)(2 * P));
-  lc.blockDim = dim3(PC::THREADS);
-  lc.dynamicSmemBytes = PC::SMEM;
-  lc.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = attr;
-  lc.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&lc, k_tiles_pair<MODE, EW>, bt, tm, kept_rows);
+  LaunchOpt opt;
+  opt.cluster = 2;
+  return launch_opt(opt, k_tiles_pair<MODE, EW>, dim3((unsigned)(2 * P)), dim3(PC::THREADS), PC::SMEM, st, bt, tm, kept_rows);
 }
 
 // can clusters of two CTAs of this kernel be launched at all?
@@ -1028,7 +1015,7 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, c
   const long long nq = (est_rows + BM - 1) / BM;
   if (g_pair_gram_ok && nq * (nq + 1) / 2 * bt.B >= 6LL * cfg.sm_count) {
     const long long n2 = (maxN + 2 * BM - 1) / (2 * BM);
-    return launch_pair<MODE_GRAM, 16>(bt, tm, n2 * (n2 + 1) / 2, 0, cfg, true, st);
+    return launch_pair<MODE_GRAM, 16>(bt, tm, n2 * (n2 + 1) / 2, 0, cfg, st);
   }
   const long long nb = (maxN + BM - 1) / BM;
   dim3 grid(umma_grid_x(nb * (nb + 1) / 2, bt.B, cfg.sm_count), bt.B);
@@ -1055,7 +1042,7 @@ cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const 
   }
   if (pairs && !kept_rows && g_pair_assign_ok) {
     const long long pt = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
-    return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, 0, cfg, true, st);
+    return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, 0, cfg, st);
   }
   const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kWideBN - 1) / kWideBN);
   dim3 grid(umma_grid_x(tiles, bt.B, cfg.sm_count), bt.B);
@@ -1072,11 +1059,11 @@ cudaError_t launch_spread_umma(const Batch &bt, int maxN, const ClusterCfg &cfg,
   }
   if (g_pair_ok) {
     const long long ptiles = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
-    return launch_pair<MODE_SPREAD, 8>(bt, tm, ptiles, 0, cfg, false, st);
+    return launch_pair<MODE_SPREAD, 8>(bt, tm, ptiles, 0, cfg, st);
   }
   const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kWideBN - 1) / kWideBN);
   dim3 grid(umma_grid_x(tiles, bt.B, cfg.sm_count), bt.B);
-  return launch_k(k_tiles_umma<MODE_SPREAD, kWideBN>, grid, dim3(THREADS), TileCfg<kWideBN>::SMEM, st, false, bt, tm, 0);
+  return launch_k(k_tiles_umma<MODE_SPREAD, kWideBN>, grid, dim3(THREADS), TileCfg<kWideBN>::SMEM, st, true, bt, tm, 0);
 }
 
 }  // namespace pact

@@ -383,6 +383,19 @@ __global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ 
   }
 }
 
+// What k_lists and k_merge accumulate into, and the counters (pact_merge; the whole step has k_qsum clear them).
+__global__ void __launch_bounds__(256) k_list_clear(const __grid_constant__ Batch bt) {
+  pdl_wait();
+  pdl_trigger();
+  const ImgDesc &im = bt.img[blockIdx.y];
+  const int gt = blockIdx.x * 256 + threadIdx.x, gs = gridDim.x * 256;
+  if (gt < kCntInts) im.cnt[gt] = 0;
+  for (int r = gt; r < im.Np; r += gs) { im.csize[r] = 0; im.cticket[r] = 0; }
+  uint4 *tab = reinterpret_cast<uint4 *>(im.cnt_cb);
+  const int nq = im.Np * (im.nbp / 8);
+  for (int i = gt; i < nq; i += gs) tab[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // ---- Eq. 10 ------------------------------------------------------------------------------------------
 // Grid (X, B), kMrgThreads threads, two CTAs per SM.  Work items are the member records in cluster order
 // followed by the text rows; CTA x takes items [x per, (x + 1) per).  A thread owns VPL groups of 8 columns
@@ -421,7 +434,8 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
   const int X = gridDim.x, x = blockIdx.x;
   const int per = (total + X - 1) / X;
   const int lo = min(total, x * per), hi = min(total, lo + per);
-  if (x == 0 && t == 0) im.cnt[PACT_CNT_N_OUT] = n_text + C;
+  // every other counter is final: this is the last kernel of the call
+  if (x == 0 && t < PACT_N_COUNTERS) im.counters_user[t] = t == PACT_CNT_N_OUT ? n_text + C : ld_cg_i32(&im.cnt[t]);
 
   float acc[VPL][8];
   int cur_c = -1, cur_off = 0, cur_size = 0, cur_dst = 0;
@@ -673,6 +687,12 @@ cudaError_t merge_configure() {
   if (e == cudaSuccess) e = merge_attr<float, float, 1>();
   if (e == cudaSuccess) e = merge_attr<float, float, V2>();
   return e;
+}
+
+cudaError_t launch_list_clear(const Batch &bt, cudaStream_t st) {
+  const long long words = (long long)bt.img[0].Np * (bt.img[0].nbp / 8);
+  const long long X = (words + 2047) / 2048;          // eight 16-byte stores per thread
+  return launch_k(k_list_clear, dim3((unsigned)(X < 1 ? 1 : (X > 1184 ? 1184 : X)), bt.B), dim3(256), 0, st, true, bt);
 }
 
 cudaError_t launch_merge(const Batch &bt, bool in_bf16, bool out_bf16, const ClusterCfg &cfg, cudaStream_t st) {

@@ -70,19 +70,11 @@ extern "C" pact_status pact_prune_static(const float *score, int N, const pact_p
   if (mt > N - 1) mt = N - 1;
   if (mt < 0) mt = 0;
   m.m_target = (int)mt;
-  m.slot = reinterpret_cast<int32_t *>(base);
-  m.cnt = reinterpret_cast<int32_t *>(base) + kStaticMaxN;
   m.score = const_cast<float *>(score);
   m.keep = keep;
   m.kept_idx = kept_idx;
   m.pruned_idx = pruned_idx;
-  // The array keeps whatever the previous call left: start the counters from zero.
-  if (cudaMemsetAsync(m.cnt, 0, kStaticCntInts * sizeof(int32_t), st) != cudaSuccess) return PACT_ERR_CUDA;
-  launch_select_gather(bt, N, true, false, st);
-  if (cudaGetLastError() != cudaSuccess) return PACT_ERR_CUDA;
-  if (cudaMemcpyAsync(counts, m.cnt + PACT_CNT_Q, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return PACT_ERR_CUDA;
-  if (cudaMemcpyAsync(counts + 1, m.cnt + PACT_CNT_M, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return PACT_ERR_CUDA;
+  m.counts_user = counts;
+  if (launch_split(bt, N, st) != cudaSuccess) return PACT_ERR_CUDA;
   return PACT_OK;
 }
