@@ -62,7 +62,7 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   cv.take(m.cnt, (size_t)kCntInts * sizeof(int32_t));
   cv.take(m.qg, (size_t)c->n_qcols * sizeof(double));
   cv.take(m.E, (size_t)N * c->n_qh * sizeof(double));
-  cv.take(m.part, (size_t)((N + kRowsPerCta - 1) / kRowsPerCta) * c->n_qh * 2 * sizeof(double));
+  cv.take(m.part, (size_t)((N + kMinPiece - 1) / kMinPiece) * c->n_qh * 2 * sizeof(double));
   cv.take(m.ghist, ((size_t)1 << kHistBits) * sizeof(int32_t));
   cv.take(m.nrm, (size_t)N * sizeof(double));
   cv.take(m.score, (size_t)N * sizeof(float));
@@ -95,8 +95,7 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   cv.take(m.csize, (size_t)Np * sizeof(int32_t));
   cv.take(m.cticket, (size_t)Np * sizeof(int32_t));
   cv.take(m.rtick, (size_t)Wp * sizeof(int32_t));
-  // two partial sums per CTA of k_merge (a range boundary cuts at most two clusters)
-  cv.take(m.mpart, (size_t)2 * merge_ctas(c->ccfg.sm_count, 1) * c->d * sizeof(float));
+  cv.take(m.mpart, merge_scratch_rows() * c->d * sizeof(float));
   return cv.off;
 }
 
@@ -244,7 +243,7 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
     if (e == cudaSuccess && major != 10) { delete c; return PACT_ERR_UNSUPPORTED; }
   }
-  if (e == cudaSuccess) e = euti_configure(c->n_qcols, c->n_qh);
+  if (e == cudaSuccess) e = euti_configure(c->n_qcols);
   if (e == cudaSuccess) e = cluster_configure(&c->ccfg);
   if (e == cudaSuccess) e = merge_configure();
   if (e == cudaSuccess && in == PACT_BF16) e = umma_configure();

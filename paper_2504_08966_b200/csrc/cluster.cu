@@ -6,6 +6,7 @@
 // kernels for bf16 keys live in gram_umma.cu and share the epilogue arithmetic of common.cuh.
 #include <cooperative_groups.h>
 
+#include "f64_tiles.cuh"
 #include "kernels.cuh"
 
 namespace pact {
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(256) k_keynorm_gather(const __grid_constant__ 
   const int i = im.kept_idx[r];
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  const rn_t rn = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
+  const rn_t rn = (rn_t)(inv_norm(ss));
   if (lane == 0) {
     rn_tok<D>(im)[i] = rn;
     rn_kept<D>(im)[r] = rn;
@@ -75,92 +76,16 @@ __global__ void __launch_bounds__(256) k_center_key_gather(const __grid_constant
   if (c < (all_rows ? im.N : *im.m_ptr)) {   // inverse norm of row c, or of the c-th pruned row
     const int i = all_rows ? c : im.pruned_idx[c];
     const double ss = row_sumsq<T>(reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc, bt.d_k, lane);
-    if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
+    if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(inv_norm(ss));
   }
   if (c >= *im.C_ptr) return;
   const int i = im.cidx_ptr[c];
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  if (lane == 0) rn_cen<D>(im)[c] = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
+  if (lane == 0) rn_cen<D>(im)[c] = (rn_t)(inv_norm(ss));
   T *dst = reinterpret_cast<T *>(im.Kcen) + (size_t)c * bt.d_k;
   for (int v = lane; v * V < bt.d_k; v += 32)
     reinterpret_cast<uint4 *>(dst)[v] = reinterpret_cast<const uint4 *>(row)[v];
-}
-
-// ---- 32 x 32 tile of dot products in double, 128 threads -----------------------------------------
-// fp32 keys (and bf16 keys of a width the tcgen05 tiles do not take) get their dot products from the double-precision
-// tensor instruction (m8n8k4): the products of fp32 values are exact in double and the sums carry its full precision.
-// Warp (wy, wx) owns the 16 x 16 quarter at rows 16 wy, columns 16 wx as 2 x 2 fragments; lane l holds of fragment
-// (a, b) the row 8 a + l / 4 and the columns 8 b + 2 (l % 4) + {0, 1}.  Small tiles on purpose: these matrices are
-// small (a thumbnail has 138 survivors), so the tiles have to be many for the SMs to share them.  The operands are
-// widened once when they are staged; the next slab is on its way from the L2 while this one is multiplied.
-// One scalar FMA per product with 64 x 64 tiles, widening at every use, took 23 us for 138 x 138 x 128.
-constexpr int TS = 32;        // tile side
-constexpr int KC = 64;        // key elements staged per step
-constexpr int KST = KC + 4;   // row stride of a staged slab in doubles: fragment loads meet no bank twice
-constexpr int kTileThreads = 128;
-
-template <typename T, typename RowA, typename RowB>
-__device__ __forceinline__ void tile_dots(RowA rowA, RowB rowB, int d_k, double (*As)[KST], double (*Bs)[KST],
-                                          double (&acc)[2][2][2]) {
-  constexpr int V = Vec<T>::N;
-  constexpr int VPR = KC / V;                          // vectors per row of a slab
-  constexpr int NV = 2 * TS * VPR / kTileThreads;      // vectors per thread: the first half A, the second half B
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
-  uint4 buf[NV];
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = (u % (NV / 2)) * kTileThreads + t, row = v / VPR, k = k0 + (v % VPR) * V;
-      const T *p = u < NV / 2 ? rowA(row) : rowB(row);
-      buf[u] = p && k < d_k ? *reinterpret_cast<const uint4 *>(p + k) : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  fetch(0);
-  for (int k0 = 0; k0 < d_k; k0 += KC) {
-    __syncthreads();                                   // the slab before has been read
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = (u % (NV / 2)) * kTileThreads + t, row = v / VPR, k = (v % VPR) * V;
-      double *dst = (u < NV / 2 ? As[row] : Bs[row]) + k;
-      float x[V];
-      widen_vec<T>(buf[u], x);
-#pragma unroll
-      for (int e = 0; e < V; e += 2) *reinterpret_cast<double2 *>(dst + e) = make_double2((double)x[e], (double)x[e + 1]);
-    }
-    __syncthreads();
-    if (k0 + KC < d_k) fetch(k0 + KC);
-#pragma unroll 8
-    for (int k = 0; k < KC; k += 4) {
-      double a[2], b[2];
-#pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        a[f] = As[wy * 16 + f * 8 + (lane >> 2)][k + (lane & 3)];
-        b[f] = Bs[wx * 16 + f * 8 + (lane >> 2)][k + (lane & 3)];
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-          asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-              : "+d"(acc[i][j][0]), "+d"(acc[i][j][1]) : "d"(a[i]), "d"(b[j]));
-    }
-  }
-}
-
-// tile `t` of the nt (nt + 1) / 2 tiles on and above the diagonal, row by row
-__device__ __forceinline__ void upper_tile(int t, int nt, int &tm, int &tn) {
-  const double b = 2.0 * nt + 1.0;
-  int i = (int)((b - sqrt(fmax(b * b - 8.0 * t, 0.0))) * 0.5);
-  i = max(0, min(i, nt - 1));
-  while (i > 0 && i * nt - i * (i - 1) / 2 > t) --i;
-  while (i + 1 < nt && (i + 1) * nt - (i + 1) * i / 2 <= t) ++i;
-  tm = i;
-  tn = i + (t - (i * nt - i * (i - 1) / 2));
 }
 
 // ---- Eq. 5-6: all pairs of survivors; density and adjacency in the epilogue --------------------
@@ -171,18 +96,16 @@ __device__ __forceinline__ void upper_tile(int t, int nt, int &tm, int &tn) {
 template <typename T>
 __global__ void __launch_bounds__(kTileThreads) k_gram_f64(const __grid_constant__ Batch bt) {
   using D = typename DistOf<T>::type;
-  using dist_t = typename D::acc_t;
   pdl_wait();
   pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 4);
   const int q = *im.q_ptr;
   const int nt = (q + TS - 1) / TS;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
+  const int t = threadIdx.x;
   __shared__ __align__(16) double As[TS][KST];
   __shared__ __align__(16) double Bs[TS][KST];
-  __shared__ unsigned long long rsum[2][TS], csum[2][TS];   // by column half of the rows, by row half of the columns
-  __shared__ uint32_t rbits[2][TS], cbits[2][TS];
+  __shared__ F64Sums sums;
   const T *Kp = reinterpret_cast<const T *>(im.Kp);
   const auto *rnk = rn_kept<D>(im);
   int band = 0;
@@ -191,57 +114,10 @@ __global__ void __launch_bounds__(kTileThreads) k_gram_f64(const __grid_constant
     upper_tile(tile, nt, tm, tn);
     double acc[2][2][2];
     tile_dots<T>(
-        [&](int r) { const int g = tm * TS + r; return g < q ? Kp + (size_t)g * bt.d_k : (const T *)nullptr; },
+        t, [&](int r) { const int g = tm * TS + r; return g < q ? Kp + (size_t)g * bt.d_k : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < q ? Kp + (size_t)g * bt.d_k : (const T *)nullptr; },
-        bt.d_k, As, Bs, acc);
-    unsigned long long rs[2] = {0ull, 0ull}, cs[2][2] = {};
-    uint32_t rb[2] = {0u, 0u}, cb[2][2] = {};
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const int li = wy * 16 + a * 8 + (lane >> 2), gi = tm * TS + li;
-      const double rni = gi < q ? (double)rnk[gi] : 0.0;
-#pragma unroll
-      for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int lj = wx * 16 + b * 8 + 2 * (lane & 3) + e, gj = tn * TS + lj;
-          if (gi >= q || gj >= q) continue;
-          dist_t dd = (dist_t)fmin(fmax(1.0 - acc[a][b][e] * (rni * (double)rnk[gj]), 0.0), 2.0);
-          if (gi == gj) dd = 0;
-          const unsigned long long term = D::term(dd, im);
-          rs[a] += term;
-          cs[b][e] += term;
-          if (D::within(dd, im)) { rb[a] |= 1u << lj; cb[b][e] |= 1u << li; }
-          if (gi < gj && D::in_band(dd, im)) ++band;
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {                      // rows: the four lanes that hold parts of one
-#pragma unroll
-      for (int o = 1; o < 4; o <<= 1) {
-        rs[a] += __shfl_xor_sync(0xffffffffu, rs[a], o);
-        rb[a] |= __shfl_xor_sync(0xffffffffu, rb[a], o);
-      }
-      if ((lane & 3) == 0) { rsum[wx][wy * 16 + a * 8 + (lane >> 2)] = rs[a]; rbits[wx][wy * 16 + a * 8 + (lane >> 2)] = rb[a]; }
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {                    // columns: the eight lanes
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-          cs[a][e] += __shfl_xor_sync(0xffffffffu, cs[a][e], o);
-          cb[a][e] |= __shfl_xor_sync(0xffffffffu, cb[a][e], o);
-        }
-        if (lane < 4) { csum[wy][wx * 16 + a * 8 + 2 * lane + e] = cs[a][e]; cbits[wy][wx * 16 + a * 8 + 2 * lane + e] = cb[a][e]; }
-      }
-    }
-    __syncthreads();
-    if (t < 2 * TS) {                                  // (the barrier inside the next tile_dots comes before these are rewritten)
-      const int l = t & (TS - 1), side = t / TS;       // 0: rows, 1: columns (above the diagonal only)
-      const int g = (side ? tn : tm) * TS + l;
-      if (g < q && !(side && tm == tn)) {
-        atomicAdd(&im.rho_fix[g], side ? csum[0][l] + csum[1][l] : rsum[0][l] + rsum[1][l]);
-        im.adj[(size_t)g * im.Wp + (side ? tm : tn)] = side ? (cbits[0][l] | cbits[1][l]) : (rbits[0][l] | rbits[1][l]);
-      }
-    }
+        bt.d_k, As, Bs, acc, []() { __syncthreads(); });
+    gram_epilogue_f64<D>(t, tm, tn, q, acc, [&](int g) { return (double)rnk[g]; }, im, sums, band, []() { __syncthreads(); });
   }
   if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
 }
@@ -263,7 +139,7 @@ __global__ void __launch_bounds__(256) k_key_rnorm(const __grid_constant__ Batch
   if (i >= im.N) return;
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
+  if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(inv_norm(ss));
 }
 
 template <typename T>
@@ -286,9 +162,9 @@ __global__ void __launch_bounds__(kTileThreads) k_spread_f64(const __grid_consta
     upper_tile(tile, nt, tm, tn);
     double acc[2][2][2];
     tile_dots<T>(
-        [&](int r) { const int g = tm * TS + r; return g < N ? K + (size_t)g * im.ldKc : (const T *)nullptr; },
+        t, [&](int r) { const int g = tm * TS + r; return g < N ? K + (size_t)g * im.ldKc : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < N ? K + (size_t)g * im.ldKc : (const T *)nullptr; },
-        bt.d_k, As, Bs, acc);
+        bt.d_k, As, Bs, acc, []() { __syncthreads(); });
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
       const int gi = tm * TS + wy * 16 + a * 8 + (lane >> 2);
@@ -582,7 +458,6 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
 template <typename T>
 __global__ void __launch_bounds__(kTileThreads) k_assign_f64(const __grid_constant__ Batch bt, int mode) {
   using D = typename DistOf<T>::type;
-  using acc_t = typename D::acc_t;
   pdl_wait();
   pdl_trigger();
   const ImgDesc &im = bt.img[blockIdx.y];
@@ -591,7 +466,7 @@ __global__ void __launch_bounds__(kTileThreads) k_assign_f64(const __grid_consta
   const int nrows = mode == ROWS_ALL ? im.N : (mode == ROWS_KEPT_LIST ? *im.q_ptr : *im.m_ptr);
   const int32_t *list = mode == ROWS_KEPT_LIST ? im.kept_idx : im.pruned_idx;
   const int ntm = (nrows + TS - 1) / TS, ntn = (C + TS - 1) / TS;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, wy = w >> 1, wx = w & 1;
+  const int t = threadIdx.x;
   __shared__ __align__(16) double As[TS][KST];
   __shared__ __align__(16) double Bs[TS][KST];
   __shared__ unsigned long long rowbest[2][TS];
@@ -610,31 +485,11 @@ __global__ void __launch_bounds__(kTileThreads) k_assign_f64(const __grid_consta
     __syncthreads();
     double acc[2][2][2];
     tile_dots<T>(
-        [&](int r) { const int tok = rowtok[r]; return tok >= 0 ? Kc + (size_t)tok * im.ldKc : (const T *)nullptr; },
+        t, [&](int r) { const int tok = rowtok[r]; return tok >= 0 ? Kc + (size_t)tok * im.ldKc : (const T *)nullptr; },
         [&](int r) { const int g = tn * TS + r; return g < C ? Kcen + (size_t)g * bt.d_k : (const T *)nullptr; },
-        bt.d_k, As, Bs, acc);
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const int l = wy * 16 + a * 8 + (lane >> 2), tok = rowtok[l];
-      const auto rni = tok >= 0 ? rnt[tok] : 0;
-      unsigned long long bestv = kBestInit;
-#pragma unroll
-      for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int c = tn * TS + wx * 16 + b * 8 + 2 * (lane & 3) + e;
-          if (c >= C) continue;
-          const float dd = (float)D::dist((acc_t)acc[a][b][e], rni, rnc[c]);
-          const unsigned long long pk = ((unsigned long long)__float_as_uint(dd) << 32) | (unsigned)c;
-          bestv = pk < bestv ? pk : bestv;
-        }
-#pragma unroll
-      for (int o = 1; o < 4; o <<= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, bestv, o);
-        bestv = y < bestv ? y : bestv;
-      }
-      if ((lane & 3) == 0) rowbest[wx][l] = bestv;
-    }
+        bt.d_k, As, Bs, acc, []() { __syncthreads(); });
+    assign_epilogue_f64<D>(t, tn * TS, C, acc, [&](int l) { return rowtok[l] >= 0 ? rnt[rowtok[l]] : (typename D::rn_t)0; },
+                           [&](int c) { return rnc[c]; }, rowbest);
     __syncthreads();
     if (t < TS && rowtok[t] >= 0) atomicMin(&im.best[rowtok[t]], rowbest[0][t] < rowbest[1][t] ? rowbest[0][t] : rowbest[1][t]);
   }
@@ -700,7 +555,8 @@ cudaError_t cluster_configure(ClusterCfg *cfg) {
   cfg->centers_smem_max = optin - 1024;
   e = cudaFuncSetAttribute(k_centers<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_centers<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
+  e = cudaFuncSetAttribute(k_centers<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
+  return e;
 }
 
 #define PACT_DISPATCH(bf16, KERNEL, grid, block, st, ...)                                      \

@@ -9,7 +9,7 @@
 namespace pact {
 
 constexpr int kMaxBatchPerLaunch = 16;   // images described by one kernel parameter block
-constexpr int kRowsPerCta = 32;          // visual tokens handled by one CTA of the EUTI kernels
+constexpr int kMinPiece = 8;             // fewest visual tokens in a softmax piece of k_tokens (at most 32)
 constexpr uint32_t kRhoShift = 30;       // density terms are summed as integers scaled by 2^30
 constexpr unsigned long long kBestInit = 0xFFFFFFFFFFFFFFFFull;
 constexpr int kCntSpread = 24;           // slot of cnt[]: largest key distance of a layer, as float bits
@@ -38,8 +38,8 @@ struct ImgDesc {
   unsigned flags;
   // workspace
   double *qg;            // [n_qcols] global query
-  double *E;             // [N][n_qh] exp(logit - CTA max)
-  double *part;          // [G][n_qh][2] per-CTA (max, sum) of k_tokens, G = ceil(N / 32)
+  double *E;             // [n_qh][N] exp(logit - largest of its piece)
+  double *part;          // [G][n_qh][2] (max, sum) of the pieces of k_tokens, G <= ceil(N / kMinPiece)
   int32_t *ghist;        // [2^kHistBits] scores per bin of their top key bits
   double *nrm;           // [N] hidden-state norms
   float *score;          // [N]
@@ -68,9 +68,9 @@ struct ImgDesc {
   uint16_t *cnt_cb;      // [Np][nbp] members of cluster c in token block b; zero before k_lists
   int4 *members;         // [N] {token, cluster, first member position of the cluster, cluster size}, cluster order
   int32_t *csize;        // [Np] members of cluster c
-  int32_t *cticket;      // [Np] chunks of cluster c that are finished
+  int32_t *cticket;      // [Np] tickets of the clusters that k_merge cuts: 8 (range of its first member) + column slice
   int32_t *rtick;        // [Wp] epilogue warps of the rows x centres pass that are done with a group of 32 tokens
-  float *mpart;          // [2 * merge CTAs][d] sums of the clusters that a range boundary of k_merge cuts
+  float *mpart;          // [2 * ranges][d] sums of the clusters that a range boundary of k_merge cuts
   int32_t *cnt;          // [PACT_N_COUNTERS] + [19] barrier of k_lists, [20] members of all clusters
   const int32_t *q_ptr;  // where the number of survivors lives (cnt[Q] or the caller's q_dev)
   const int32_t *m_ptr;  // where the number of pruned tokens lives
@@ -157,6 +157,15 @@ template <> __device__ __forceinline__ void load_vec<float>(const float *p, floa
 __device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float to_float(float v) { return v; }
 
+// Largest value over the warp: the order of doubles is that of their bits as integers (negative numbers flipped), upper
+// word first.  (Five rounds of shuffle and fmax take 700 clocks, the two reductions about 100.)
+__device__ __forceinline__ double warp_max(double v) {
+  const int hi = __double2hiint(v), s = hi >> 31, kh = hi ^ (s & 0x7fffffff);
+  const int mh = __reduce_max_sync(0xffffffffu, kh);
+  const uint32_t ml = __reduce_max_sync(0xffffffffu, kh == mh ? (uint32_t)(__double2loint(v) ^ s) : 0u);
+  const int ms = mh >> 31;
+  return __hiloint2double(mh ^ (ms & 0x7fffffff), (int)ml ^ ms);
+}
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -195,6 +204,52 @@ template <typename T> __device__ __forceinline__ void sumsq_accumulate(const uin
   }
 }
 
+template <typename O> __device__ __forceinline__ void store_vec8(O *p, const float (&x)[8]);
+template <> __device__ __forceinline__ void store_vec8<float>(float *p, const float (&x)[8]) {
+  reinterpret_cast<float4 *>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
+  reinterpret_cast<float4 *>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+}
+template <> __device__ __forceinline__ void store_vec8<__nv_bfloat16>(__nv_bfloat16 *p, const float (&x)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
+    w[i] = *reinterpret_cast<uint32_t *>(&h);
+  }
+  *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Eight consecutive elements of a row as loaded (not yet widened), so that many can be in flight.
+template <typename T> struct Raw8;
+template <> struct Raw8<__nv_bfloat16> {
+  uint4 a;
+  __device__ __forceinline__ void from_ring(const uint4 *p) { a = p[0]; }
+  __device__ __forceinline__ void add_to(float (&acc)[8]) const {
+    float x[8];
+    widen_vec<__nv_bfloat16>(a, x);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] += x[e];
+  }
+};
+template <> struct Raw8<float> {
+  uint4 a, b;
+  __device__ __forceinline__ void from_ring(const uint4 *p) { a = p[0]; b = p[1]; }
+  __device__ __forceinline__ void add_to(float (&acc)[8]) const {
+    float x[4], y[4];
+    widen_vec<float>(a, x);
+    widen_vec<float>(b, y);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { acc[e] += x[e]; acc[4 + e] += y[e]; }
+  }
+};
+
+// sort key of a score: unsigned integers that order like the floats
+__device__ __forceinline__ uint32_t score_key(float s) {
+  uint32_t b = __float_as_uint(s);
+  if (b == 0x80000000u) b = 0;                       // -0 orders as +0
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+
 // ---- programmatic dependent launch ----------------------------------------------------------------------
 // The step is a chain of short kernels.  A kernel launched with the programmatic-serialization attribute may
 // start while its predecessor in the stream is still running: pdl_wait() blocks until the predecessor has
@@ -205,73 +260,44 @@ template <typename T> __device__ __forceinline__ void sumsq_accumulate(const uin
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// ---- L2 eviction hints -------------------------------------------------------------------------
-// The hidden states are read twice, by the scoring pass and by the merge, with everything else of the step
-// in between; together that is more than the L2 keeps under its default policy.  The first pass asks for
-// its lines to be evicted last, streams that are read once ask to be evicted first.
-__device__ __forceinline__ unsigned long long policy_evict_last() {
-  unsigned long long p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
+// ---- thread-block clusters ------------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ __forceinline__ unsigned long long policy_evict_first() {
-  unsigned long long p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
 }
-__device__ __forceinline__ uint4 ldg_hint(const uint4 *p, unsigned long long policy) {
-  uint4 v;
-  asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
-  return v;
-}
-
-// The same with a compile-time byte offset folded into the instruction: a run of such loads from one base
-// needs one address register, not one per load.
-template <int OFF>
-__device__ __forceinline__ uint4 ldg_hint_off(const uint4 *p, unsigned long long policy) {
-  uint4 v;
-  asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4 + %6], %5;"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy), "n"(OFF));
-  return v;
-}
-
-// buf[u] = base[32 u] for the u with v0 + 32 u < nv, all from one address register
-template <int U, int I>
-__device__ __forceinline__ void load_run_hint(uint4 (&buf)[U], const uint4 *base, int v0, int nv, unsigned long long policy) {
-  if constexpr (I < U) {
-    if (v0 + 32 * I < nv) buf[I] = ldg_hint_off<32 * I * 16>(base, policy);
-    load_run_hint<U, I + 1>(buf, base, v0, nv, policy);
-  }
+// stores to this shared-memory location of CTA `rank` of the cluster
+__device__ __forceinline__ void st_cluster_f64(double *p, int rank, double v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
 // This lane's share (vectors lane, lane + 32, ... in ascending order) of the sum of squares of a
-// row of n elements, starting at vector `from`.  Up to U loads per lane are in flight at once.
-template <typename T, int U, bool HINT = false>
-__device__ __forceinline__ double row_sumsq_lane(const T *row, int n, int lane, int from = 0,
-                                                 unsigned long long policy = 0ull) {
+// row of n elements.  Up to U loads per lane are in flight at once.
+template <typename T, int U>
+__device__ __forceinline__ double row_sumsq_lane(const T *row, int n, int lane) {
   const int nv = n / Vec<T>::N;
   const uint4 *p = reinterpret_cast<const uint4 *>(row);
   double acc = 0.0;
-  for (int v0 = from + lane; v0 < nv; v0 += 32 * U) {
+  for (int v0 = lane; v0 < nv; v0 += 32 * U) {
     uint4 buf[U];
-    if (HINT) {
-      load_run_hint<U, 0>(buf, p + v0, v0, nv, policy);
-    } else {
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (v0 + 32 * u < nv) buf[u] = __ldg(p + v0 + 32 * u);
-    }
+    for (int u = 0; u < U; ++u)
+      if (v0 + 32 * u < nv) buf[u] = __ldg(p + v0 + 32 * u);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
+    for (int u = 0; u < U; ++u)
       if (v0 + 32 * u < nv) sumsq_accumulate<T>(buf[u], acc);
-      // one vector after the other: left to itself the compiler widens all U vectors at once for the sake of
-      // instruction-level parallelism and spills the loaded data, which serialises the loads
-      if (u + 1 < U) asm volatile("" : "+r"(buf[u + 1].x), "+d"(acc));
-    }
   }
   return acc;
 }
+
+// 1 / |row| from the sum of squares
+__device__ __forceinline__ double inv_norm(double ss) { return rsqrt(fmax(ss, 1e-40)); }
 
 // Sum of squares of one row by one warp.
 template <typename T>

@@ -3,9 +3,10 @@
 // in double so that the float32 score the library returns is the correctly rounded value in all but
 // rare double-rounding cases.
 //
-//   k_qsum           column sums of Q -> global query; also clears what later kernels accumulate into
+//   k_qsum           column sums of Q -> global query
 //   k_tokens         one pass over the hidden states and the keys: |h_i|, 1 / |k_i|, k_i . Qglobal per head,
-//                    CTA-local softmax pieces (HBM-bound, the first of two reads of H)
+//                    softmax pieces of up to 32 tokens (HBM-bound, the first of two reads of H); also clears what later
+//                    kernels accumulate into
 //   k_scores         merges the pieces, writes the float32 scores and the histogram of their top key bits
 //   k_select         every CTA selects the threshold (histogram bin, then radix passes inside the bin) and
 //                    counts the survivors before its tokens, then writes its share of the lists and gathers
@@ -15,6 +16,7 @@
 // The kernels are short chains of dependent memory round trips; each issues all the loads it can
 // before it consumes the first.
 #include "kernels.cuh"
+#include "tma.cuh"
 
 namespace pact {
 
@@ -24,312 +26,421 @@ __device__ __forceinline__ double ld_cg_f64(const double *p) {
   return v;
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+// Widening to double by moving bits: the exponent field of the element becomes the low bits of the double's, i.e. the
+// double is the element times 2^-896, exactly, zeros and subnormal numbers included (the sum is multiplied by 2^896 at
+// the end).  The conversion unit takes 16 elements per clock and SM and was what bounded the sums over Q.
+constexpr double kWidenScale = 0x1p896;
+template <typename T> __device__ __forceinline__ void widen_scaled(const uint4 &v, double (&x)[Vec<T>::N]);
+__device__ __forceinline__ double scaled_hi(uint32_t w) { return __hiloint2double((int)w >> 3 & (int)0x8FFFE000, 0); }   // bf16 in the upper half
+template <> __device__ __forceinline__ void widen_scaled<__nv_bfloat16>(const uint4 &v, double (&x)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { x[2 * i] = scaled_hi(w[i] << 16); x[2 * i + 1] = scaled_hi(w[i]); }
 }
-// the double at this shared-memory location of CTA `rank` of the cluster
-__device__ __forceinline__ double ld_cluster_f64(const double *p, int rank) {
-  uint32_t a;
-  double v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
-  return v;
+template <> __device__ __forceinline__ void widen_scaled<float>(const uint4 &v, double (&x)[4]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = __hiloint2double((int)w[i] >> 3 & (int)0x8FFFFFFF, (int)(w[i] << 29));
 }
-
-// sort key of a score: unsigned integers that order like the floats
-__device__ __forceinline__ uint32_t score_key(float s) {
-  uint32_t b = __float_as_uint(s);
-  if (b == 0x80000000u) b = 0;                       // -0 orders as +0
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+// Sum of the 32 parts of each of the rows w, w + step, ... < n: eight lanes per row, four rows at a time.
+template <typename F>
+__device__ __forceinline__ void finish_row_sums(const double (*acc)[32], int w, int step, int n, F put_sum) {
+  const int lane = threadIdx.x & 31;
+  for (int i = 0; w + i * step < n; i += 4) {
+    const int r = w + (i + lane / 8) * step;
+    double s = 0.0;
+    if (r < n) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s += acc[r][(lane & 7) * 4 + k];
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (r < n && (lane & 7) == 0) put_sum(r, s);
+  }
+  __syncwarp();
 }
 
 // ---- Eq. 1: column sums of Q -----------------------------------------------------------------------------
-// grid (ncg RP, B) in clusters of RP CTAs, 512 threads at no more than 64 registers, on fewer than half of the
-// SMs where that is enough: a CTA leaves room for one CTA of k_tokens beside it, and the other SMs take two, so that
-// all of them start at once.  Work item (column group of eight 16-byte vectors, block of rows): thread t takes vector
-// t & 7 of the group and the rows r0 + (t >> 3), + 64, ...; the four row lanes of a warp are added with shuffles, the
-// warps through shared memory.  The RP row blocks of a column group are one cluster: its first CTA reads the
-// others' sums through distributed shared memory and adds them in block order.  (Partial sums in global memory
-// behind a ticket cost 2.6 us from the last row to the global query, and a cleared ticket before the kernel.)
-// do_init: the grid also clears what later kernels accumulate into.
-constexpr int kQsumThreads = 512;
-constexpr int kQsumRowLanes = kQsumThreads / 8;
+// grid (ncg RP, B) in clusters of RP CTAs, 256 threads at no more than 64 registers, at most about two CTAs per SM, which
+// leave room for k_tokens beside them.  Work item (column group of GV 16-byte vectors, block of rows): thread t takes
+// vector t % GV of the group and the rows r0 + t / GV, + 256 / GV, ...; the row lanes of a warp are added with shuffles, the
+// warps through shared memory.  The RP row blocks of a column group are one cluster: the CTAs store their sums into the
+// first one's shared memory, which adds them in block order (the others leave at once: fetching the sums took a second
+// barrier and 2 us more).  Bound by memory: 7.5 MB of one image's Q take 9 us with the start of the call, 48 MB of 16 images
+// 25 us beside the row stream of k_tokens.  (Partial sums in global memory behind a ticket cost 2.6 us from the last row to
+// the global query; with a conversion instruction per element instead of widen_scaled an SM took in 30 GB/s.)
+constexpr int kQsumThreads = 256;
 constexpr int kQsumWarps = kQsumThreads / 32;
 
-template <typename T>
-__global__ void __launch_bounds__(kQsumThreads, 2) k_qsum(const __grid_constant__ Batch bt, int RP, int do_init) {
-  constexpr int V = Vec<T>::N;
+template <typename T, int GV>
+__global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant__ Batch bt, int RP) {
+  constexpr int V = Vec<T>::N, LANES = kQsumThreads / GV;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 0);
   pdl_wait();                                           // the work before this call, which may still use the workspace
-  pdl_trigger();                                        // k_tokens may start: its first pass does not need the query
+  pdl_trigger();                                        // k_tokens may start: much of it does not need the query
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, N = im.N, n_qcols = bt.n_qcols;
-  if (do_init) {
-    const int gt = blockIdx.x * kQsumThreads + t, gs = gridDim.x * kQsumThreads;
-    for (int r = gt; r < im.Np; r += gs) { im.rho_fix[r] = 0ull; im.csize[r] = 0; im.cticket[r] = 0; }
-    for (int wd = gt; wd < im.Wp; wd += gs) { im.cmask[wd] = 0u; im.rmask[wd] = 0u; im.rtick[wd] = 0; }
-    for (int i = gt; i < N; i += gs) im.best[i] = kBestInit;
-    uint4 *tab = reinterpret_cast<uint4 *>(im.cnt_cb);
-    const int nq = im.Np * (im.nbp / 8);
-    for (int i = gt; i < nq; i += gs) tab[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = gt; i < (1 << kHistBits); i += gs) im.ghist[i] = 0;
-    if (gt < kCntInts) im.cnt[gt] = 0;
-  }
   if (!im.Q || (im.flags & PACT_FLAG_NORM_ONLY)) return;
+  if (RP > 1) cluster_arrive();                         // (every CTA of the cluster runs before one stores to another)
   const int nvq = n_qcols / V;
   const int cg = blockIdx.x / RP, rp = blockIdx.x % RP; // rp = rank of the CTA in its cluster
-  __shared__ double sm[kQsumWarps * 8 * V];
-  __shared__ double s_part[8 * V];
+  __shared__ double sm[kQsumWarps * GV * V];
+  __shared__ double s_part[kQPartRows][GV * V];
   const int rchunk = (N + RP - 1) / RP;
   const int r0 = min(N, rp * rchunk), r1 = min(N, r0 + rchunk);
-  const int v = cg * 8 + (t & 7);
-  const unsigned long long pol = policy_evict_first();   // Q is read once
-  const T *Q = reinterpret_cast<const T *>(im.Q);
+  const int v = cg * GV + (t % GV);
   double acc[V];
 #pragma unroll
   for (int k = 0; k < V; ++k) acc[k] = 0.0;
   if (v < nvq) {
     constexpr int UQ = 8;
-    const size_t coff = (size_t)v * V;
-    for (int r = r0 + (t >> 3); r < r1; r += kQsumRowLanes * UQ) {
+    const T *Q = reinterpret_cast<const T *>(im.Q) + (size_t)v * V;
+    for (int r = r0 + t / GV; r < r1; r += LANES * UQ) {
       uint4 buf[UQ];
 #pragma unroll
       for (int u = 0; u < UQ; ++u)
-        if (r + u * kQsumRowLanes < r1)
-          buf[u] = ldg_hint(reinterpret_cast<const uint4 *>(Q + (size_t)(r + u * kQsumRowLanes) * im.ldQ + coff), pol);
+        if (r + u * LANES < r1) buf[u] = __ldg(reinterpret_cast<const uint4 *>(Q + (size_t)(r + u * LANES) * im.ldQ));
 #pragma unroll
       for (int u = 0; u < UQ; ++u) {
-        if (r + u * kQsumRowLanes < r1) {
-          float x[V];
-          widen_vec<T>(buf[u], x);
+        if (r + u * LANES < r1) {
+          double x[V];
+          widen_scaled<T>(buf[u], x);
 #pragma unroll
-          for (int k = 0; k < V; ++k) acc[k] += (double)x[k];
+          for (int k = 0; k < V; ++k) acc[k] += x[k];
         }
       }
     }
   }
 #pragma unroll
-  for (int k = 0; k < V; ++k) {
-    acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 8);
-    acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 16);
-  }
-  if (lane < 8) {
+  for (int o = GV; o < 32; o <<= 1)
 #pragma unroll
-    for (int k = 0; k < V; ++k) sm[(w * 8 + lane) * V + k] = acc[k];
+    for (int k = 0; k < V; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+  if (lane < GV) {
+#pragma unroll
+    for (int k = 0; k < V; ++k) sm[(w * GV + lane) * V + k] = acc[k];
   }
   __syncthreads();
-  const bool col_ok = t < 8 * V && cg * 8 + t / V < nvq;
-  const size_t col = (size_t)cg * 8 * V + t;
+  const bool col_ok = t < GV * V && cg * GV + t / V < nvq;
+  const size_t col = (size_t)cg * GV * V + t;
   double mine = 0.0;
   if (col_ok) {
 #pragma unroll
-    for (int ww = 0; ww < kQsumWarps; ++ww) mine += sm[ww * 8 * V + t];
+    for (int ww = 0; ww < kQsumWarps; ++ww) mine += sm[ww * GV * V + t];
+    if (RP == 1) im.qg[col] = mine * kWidenScale / (double)N;
   }
-  if (t < 8 * V) s_part[t] = mine;
-  cluster_sync();
-  if (rp == 0 && col_ok) {
-    double pv[kQPartRows], s = 0.0;
-#pragma unroll
-    for (int u = 0; u < kQPartRows; ++u) pv[u] = u < RP ? ld_cluster_f64(&s_part[t], u) : 0.0;
-#pragma unroll
-    for (int u = 0; u < kQPartRows; ++u) s += pv[u];
-    im.qg[col] = s / (double)N;
+  if (RP == 1) return;
+  cluster_wait();
+  if (t < GV * V) st_cluster_f64(&s_part[rp][t], 0, mine);   // to the first CTA of the cluster
+  cluster_arrive();
+  if (rp != 0) return;
+  cluster_wait();
+  if (col_ok) {
+    double s = 0.0;
+    for (int u = 0; u < RP; ++u) s += s_part[u][t];
+    im.qg[col] = s * kWidenScale / (double)N;
   }
-  cluster_sync();                                       // a CTA's sums may be read until here
 }
 
-// ---- Eq. 2, token pass: hidden-state norm, inverse key norm, logits, CTA-local softmax pieces ---------------
-// grid (ceil(maxN / 32), B), 256 threads, two CTAs per SM; dynamic smem (n_qcols + 32 n_qh) doubles.
-// A CTA takes 32 tokens, a warp four of them.  First the rows, one token after the other: the 16-byte loads of
-// the token's clustering-key row and hidden-state row are all issued before the first is used (the
-// hidden-state lines are asked to stay in the L2 for the merge); |h_i| in double, 1 / |k_i|.  Then the logits
-// of the warp's four tokens together: k_i . Qglobal per head in double.  Then per head the largest logit of the
-// CTA's tokens, exp(l - that) per token and their sum.
-constexpr int kTokThreads = 256;
-constexpr int kTokWarps = kTokThreads / 32;
-constexpr int kTokPerWarp = kRowsPerCta / kTokWarps;
+// ---- Eq. 2, token pass: hidden-state norm, inverse key norm, logits, softmax pieces --------------------------------
+// Persistent: one CTA of 512 threads and at most 64 registers per SM (beside it a CTA of k_qsum still fits), units of
+// at most 32 tokens dealt out in turn over all images of the call.  Two groups of warps work side by side:
+//   norms    Every warp takes each eighth token of a unit.  The hidden-state rows run through two buffers of the warp's
+//            own in shared memory, one bulk copy per row (or per 8 KB of it), so that copies never wait for arithmetic.
+//            Sums of squares in float over a 16-byte vector and in double across.  Nothing here needs the global query.
+//   logits   Two teams of four warps take the units in turn; a team's scoring keys come through a buffer of its own, in
+//            flight before the global query is known: inverse key norms; k_i . Qglobal per head in double; per head the
+//            largest logit of the unit, exp(l - that) per token and their sum.  A lane is a token (with few tokens a
+//            part of its elements), a warp has up to four query heads of a key head at a time, and their global query
+//            comes from shared memory at one address per warp: with the lanes spread over the row the loads of the
+//            query were what took the time, and with the double-precision tensor instruction (m8n8k4, whose rate is
+//            that of the ordinary one) the seven idle heads of eight: 16 tokens of four heads took 4100 clocks a team.
+// As 16-byte loads of four tokens per warp, one token's row at a time and the logits between them, the pass took 4.2 TB/s
+// of HBM, and with 28 query heads on 4 key heads 31 us of 40 for a few hundred tokens.  Now 46656 tokens of 3584 (382 MB)
+// end 77 us after the call began, against 100 us; bound by memory, 5.6 TB/s with the queries.
+constexpr int kTokThreads = 512;
+constexpr int kTokGroup = 256;                          // threads of the norms group and of the logits group
+constexpr int kTokTeam = kTokGroup / 2;                 // threads of a logits team
+constexpr int kTokWarps = kTokGroup / 32;
+constexpr int kTeamWarps = kTokTeam / 32;
+constexpr int kTokMaxBuf = 2;                           // row buffers per warp
+constexpr int kTokSmem = 200 * 1024;
+
+struct TokCfg {
+  int rpp;                                              // tokens per unit (piece)
+  int chunk, nchunk;                                    // bytes of a hidden-state row per copy, copies per row
+  int nbuf;                                             // row buffers per warp
+  int keys;                                             // a key buffer per team (else the keys are read from global memory)
+};
+// stride of a key row in shared memory: an odd number of 16-byte vectors, so that a vector of 8 rows is in 8 different banks
+__host__ __device__ inline int tok_key_stride(int row_bytes) { return row_bytes | 16; }
+inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
+  return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)n_qcols * 8 + (size_t)c.rpp * 32 * 8;
+}
+
+// Logits of this lane's token (its vectors p, p + P, ... of nv) with nr <= RB heads of a key head, q at one address per part.
+template <typename T, int RB>
+__device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, int d_h, int p, int P, int nr, double (&l)[RB]) {
+  constexpr int V = Vec<T>::N, CH = 4 / RB;             // CH chains per head: an FMA takes nine clocks, two per warp can start
+  const int nv = d_h / V;
+  double acc[RB][CH];
+#pragma unroll
+  for (int j = 0; j < RB; ++j)
+#pragma unroll
+    for (int c = 0; c < CH; ++c) acc[j][c] = 0.0;
+#pragma unroll 2
+  for (int v = p; v < nv; v += P) {
+    double a[V];
+    widen_scaled<T>(*(reinterpret_cast<const uint4 *>(krow) + v), a);
+#pragma unroll
+    for (int j = 0; j < RB; ++j) {
+      const double2 *qj = reinterpret_cast<const double2 *>(q + (size_t)min(j, nr - 1) * d_h + v * V);
+#pragma unroll
+      for (int e = 0; e < V; e += 2) {
+        const double2 x = qj[e / 2];
+        acc[j][e % CH] = fma(a[e], x.x, acc[j][e % CH]);
+        acc[j][(e + 1) % CH] = fma(a[e + 1], x.y, acc[j][(e + 1) % CH]);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < RB; ++j) {
+    l[j] = acc[j][0];
+#pragma unroll
+    for (int c = 1; c < CH; ++c) l[j] += acc[j][c];
+    l[j] *= kWidenScale;
+  }
+  for (int o = 32 / P; o < 32; o <<= 1)
+#pragma unroll
+    for (int j = 0; j < RB; ++j) l[j] += __shfl_xor_sync(0xffffffffu, l[j], o);
+}
+
+// The same heads j0, j0 + 1, ...: logits (zero without a query), the piece's largest, exp and sum.  tl = 32 / P lanes are
+// the tokens of the unit, n of them real.
+template <typename T, int RB>
+__device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, const uint8_t *krow, const double *q, bool use_query, int P, int nr, int j0,
+                                           int r0, int n, int g) {
+  const int lane = threadIdx.x & 31, tl = 32 / P, r = lane & (tl - 1), p = lane / tl;
+  double l[RB];
+  if (use_query) head_dots<T, RB>(krow, q, bt.d_h, p, P, nr, l);
+  else {
+#pragma unroll
+    for (int j = 0; j < RB; ++j) l[j] = 0.0;
+  }
+  double m[RB], e[RB], sum[RB];
+#pragma unroll
+  for (int j = 0; j < RB; ++j) {
+    m[j] = warp_max(r < n ? l[j] : -1.0e300);
+    e[j] = r < n ? exp(l[j] - m[j]) : 0.0;
+    sum[j] = e[j];
+  }
+  for (int o = tl >> 1; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < RB; ++j) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+#pragma unroll
+  for (int j = 0; j < RB; ++j)
+    if (j < nr) {
+      if (r < n && p == 0) im.E[(size_t)(j0 + j) * im.N + r0 + r] = e[j];
+      if (lane == 0) *reinterpret_cast<double2 *>(im.part + ((size_t)g * bt.n_qh + j0 + j) * 2) = make_double2(m[j], sum[j]);
+    }
+}
 
 template <typename T>
-__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int do_init) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
   constexpr int V = Vec<T>::N;
-  constexpr int UK = 2;                                 // preloaded 16-byte vectors of the key row per lane
-  const ImgDesc &im = bt.img[blockIdx.y];
-  TL_SCOPE(im, 1);
-  const int g = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int N = im.N, n_qh = bt.n_qh, n_qcols = bt.n_qcols;
-  const int r0 = g * kRowsPerCta, r1 = min(N, r0 + kRowsPerCta);
-  if (r0 >= N) { pdl_wait(); return; }
-  extern __shared__ double smd[];
-  double *qT = smd;                                     // [n_qcols] global query, transposed (see below)
-  double *lg = smd + n_qcols;                           // [32][n_qh]
-  const bool use_query = !(im.flags & PACT_FLAG_NORM_ONLY) && im.Q != nullptr;
-  const int nv = bt.d_k / V, vph = bt.d_h / V, nvq = n_qcols / V;
-  const T *Ke = reinterpret_cast<const T *>(im.Ke);
-  const unsigned long long pol_keep = policy_evict_last();
-  // fast path of the logits: one query head per key head and a power-of-two number of vectors per head, all
-  // preloaded: the lanes that hold one head's vectors form a group, reduced with xor shuffles inside the group
-  const bool grouped = n_qh == bt.n_kvh && (vph & (vph - 1)) == 0 && vph <= 32 && nv <= 32 * UK;
+  TL_SCOPE(bt.img[0], 1);
+  const int lane = threadIdx.x & 31;
+  const bool norms = threadIdx.x < kTokGroup;
+  const int n_kvh = bt.n_kvh, d_h = bt.d_h, n_rep = bt.n_qh / n_kvh, rpp = cfg.rpp;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int ks = tok_key_stride(bt.d_k * (int)sizeof(T));
+  uint8_t *s_key = smem + (size_t)kTokWarps * cfg.nbuf * cfg.chunk;   // [2][rpp][ks], behind the row buffers
+  double *s_q = reinterpret_cast<double *>(s_key + (size_t)2 * cfg.keys * rpp * ks);     // [n_qh][d_h] global query
+  double(*s_acc)[32] = reinterpret_cast<double(*)[32]>(s_q + bt.n_qcols);                // [rpp][32] parts of the sums of squares
+  __shared__ int s_first[kMaxBatchPerLaunch + 1];                     // first unit of each image
+  __shared__ uint64_t s_rbar[kTokWarps][kTokMaxBuf], s_kbar[2];
+  __shared__ int s_abort, s_query;                                    // s_query: the global queries are complete
+  if (threadIdx.x == 0) {
+    s_query = 0;
+    int first = 0;
+    for (int b = 0; b < bt.B; ++b) { s_first[b] = first; first += (bt.img[b].N + rpp - 1) / rpp; }
+    s_first[bt.B] = first;
+    for (int k = 0; k < kTokWarps; ++k)
+      for (int i = 0; i < kTokMaxBuf; ++i) mbar_init(&s_rbar[k][i], 1);
+    mbar_init(&s_kbar[0], 1);
+    mbar_init(&s_kbar[1], 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const int units = s_first[bt.B];
+  // units of this CTA: neighbours, so that it meets few images (each brings another query)
+  const int u0 = (int)((long long)blockIdx.x * units / gridDim.x), u1 = (int)((long long)(blockIdx.x + 1) * units / gridDim.x);
+  auto image_of = [&](int u, int b) { while (u >= s_first[b + 1]) ++b; return b; };
 
-  // the global query is kept transposed, qT[k][vq] = Qglobal[vq * V + k], so that the lanes of a warp,
-  // which hold consecutive 16-byte vectors of the key row, read consecutive doubles
-  // the rows: |h_i| and 1 / |k_i| of one of the warp's tokens
-  auto row_pass = [&](int i) {
-    const int tok = r0 + w * kTokPerWarp + i;
-    if (tok >= r1) return;                              // the same for the whole warp
-    uint4 kb[UK];
-    const T *kcrow = im.Kc ? reinterpret_cast<const T *>(im.Kc) + (size_t)tok * im.ldKc : nullptr;
-    if (kcrow) {
+  if (norms) {
+    const int w = threadIdx.x >> 5, t = threadIdx.x;
+    uint8_t *s_rows = smem + (size_t)w * cfg.nbuf * cfg.chunk;        // this warp's row buffers
+    // the stream of this warp's row chunks, ahead of their use: unit, next row, rows left of the unit, chunk of the row
+    int lu = u0 - 1, lb = 0, lrows = 0, lc = 0, islot = 0;
+    const uint8_t *lsrc = nullptr;
+    size_t lstep = 0;
+    const int last = bt.d * (int)sizeof(T) - (cfg.nchunk - 1) * cfg.chunk;   // bytes of a row's last chunk
+    auto issue_row = [&]() {                            // lane 0: the next chunk of the stream into its buffer
+      while (lrows == 0) {
+        if (++lu >= u1) { lu = u1; return; }
+        lb = image_of(lu, lb);
+        const ImgDesc &im = bt.img[lb];
+        const int r0 = (lu - s_first[lb]) * rpp, n = min(rpp, im.N - r0);
+        if ((im.flags & PACT_FLAG_NO_NORM) || n <= w) continue;
+        lrows = (n - w + kTokWarps - 1) / kTokWarps;
+        lsrc = reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + r0 + w) * im.ldH);
+        lstep = (size_t)im.ldH * kTokWarps * sizeof(T);
+      }
+      const int bytes = lc == cfg.nchunk - 1 ? last : cfg.chunk;
+      mbar_arrive_expect_tx(&s_rbar[w][islot], bytes);
+      bulk_load(s_rows + (size_t)islot * cfg.chunk, lsrc + (size_t)lc * cfg.chunk, bytes, &s_rbar[w][islot]);
+      if (++islot == cfg.nbuf) islot = 0;
+      if (++lc == cfg.nchunk) { lc = 0; lsrc += lstep; --lrows; }
+    };
+    // One buffer per warp until k_qsum is done, all of them from then on: with more from the start this stream leaves k_qsum a
+    // third of the memory rate and the logits begin late (16 images of 2916 tokens: at 37 us), with none the memory
+    // idles towards the end of k_qsum.
+    if (lane == 0) issue_row();
+    bool all = false;
+    int slot = 0, b = 0;                                // buffer that is next
+    uint32_t par = 0;                                   // parity of each buffer's barrier
+    for (int u = u0; u < u1; ++u) {
+      b = image_of(u, b);
+      const ImgDesc &im = bt.img[b];
+      const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
+      if (im.flags & PACT_FLAG_NO_NORM) {
+        for (int r = t; r < n; r += kTokGroup) im.nrm[r0 + r] = 1.0;
+        continue;
+      }
+      for (int r = w; r < n; r += kTokWarps) {
+        double a0 = 0.0, a1 = 0.0;
+        for (int c = 0; c < cfg.nchunk; ++c) {
+          if (!mbar_wait_warp(&s_rbar[w][slot], (par >> slot) & 1)) s_abort = 1;
+          par ^= 1u << slot;
+          const uint4 *row = reinterpret_cast<const uint4 *>(s_rows + (size_t)slot * cfg.chunk);
+          const int nv = min(cfg.chunk, bt.d * (int)sizeof(T) - c * cfg.chunk) / 16;
+          int v = lane;
+          for (; v + 96 < nv; v += 128) {
+            uint4 x[4];
 #pragma unroll
-      for (int u = 0; u < UK; ++u)
-        if (lane + 32 * u < nv) kb[u] = __ldg(reinterpret_cast<const uint4 *>(kcrow) + lane + 32 * u);
-    }
-    double nn = 1.0;
-    if (!(im.flags & PACT_FLAG_NO_NORM)) {
-      const T *hrow = reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + tok) * im.ldH;
-      nn = sqrt(warp_sum(row_sumsq_lane<T, 16, true>(hrow, bt.d, lane, 0, pol_keep)));
-    }
-    if (lane == 0) im.nrm[tok] = nn;
-    if (kcrow) {
-      double a = 0.0;
-#pragma unroll
-      for (int u = 0; u < UK; ++u)
-        if (lane + 32 * u < nv) sumsq_accumulate<T>(kb[u], a);
-      if (nv > 32 * UK) a += row_sumsq_lane<T, 8>(kcrow, bt.d_k, lane, 32 * UK);
-      const double ss = warp_sum(a);
-      if (lane == 0) rn_tok<D>(im)[tok] = (rn_t)(1.0 / sqrt(fmax(ss, 1e-40)));
-    }
-  };
-  // first all but the last of the warp's tokens, one after the other
-#pragma unroll 1
-  for (int i = 0; i + 1 < kTokPerWarp; ++i) row_pass(i);
-  // the last token's hidden-state row is asked for now (into the L2) and read after the logits, which are
-  // formed while it is on its way
-  {
-    const int tok = r0 + w * kTokPerWarp + kTokPerWarp - 1;
-    if (tok < r1 && !(im.flags & PACT_FLAG_NO_NORM)) {
-      const char *hrow = reinterpret_cast<const char *>(reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + tok) * im.ldH);
-      const int bytes = bt.d * (int)sizeof(T);
-      for (int o = lane * 128; o < bytes; o += 32 * 128)
-        asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(hrow + o));
-    }
-  }
-  // the global query is kept transposed, qT[k][vq] = Qglobal[vq * V + k], so that the lanes of a warp,
-  // which hold consecutive 16-byte vectors of the key row, read consecutive doubles
-  pdl_wait();                                           // the global query is complete
-  pdl_trigger();
-  if (use_query)
-    for (int c = t; c < n_qcols; c += kTokThreads) qT[(c % V) * nvq + c / V] = ld_cg_f64(&im.qg[c]);
-  __syncthreads();
-  // then the logits: the key rows of the warp's tokens (read a moment ago when the two key matrices are one)
-  // are loaded together
-  {
-    uint4 kb[kTokPerWarp][UK];
-#pragma unroll
-    for (int i = 0; i < kTokPerWarp; ++i) {
-      const uint4 *krow = reinterpret_cast<const uint4 *>(Ke + (size_t)min(r0 + w * kTokPerWarp + i, N - 1) * im.ldKe);
-#pragma unroll
-      for (int u = 0; u < UK; ++u)
-        if (lane + 32 * u < nv) kb[i][u] = __ldg(krow + lane + 32 * u);
-    }
-    const int l0 = w * kTokPerWarp;                     // first token of the warp within the CTA
-    if (grouped) {
-      double acc[kTokPerWarp][UK];
-#pragma unroll
-      for (int u = 0; u < UK; ++u) {
-        const int v = lane + 32 * u;
-#pragma unroll
-        for (int i = 0; i < kTokPerWarp; ++i) acc[i][u] = 0.0;
-        if (use_query && v < nv) {
-          double qv[V];
-#pragma unroll
-          for (int k = 0; k < V; ++k) qv[k] = qT[k * nvq + v];
-#pragma unroll
-          for (int i = 0; i < kTokPerWarp; ++i) {
-            float x[V];
-            widen_vec<T>(kb[i][u], x);
-#pragma unroll
-            for (int k = 0; k < V; ++k) acc[i][u] = fma((double)x[k], qv[k], acc[i][u]);
+            for (int k = 0; k < 4; ++k) x[k] = row[v + 32 * k];
+            sumsq_accumulate<T>(x[0], a0); sumsq_accumulate<T>(x[1], a1);
+            sumsq_accumulate<T>(x[2], a0); sumsq_accumulate<T>(x[3], a1);
           }
-        }
-      }
-      for (int o = vph >> 1; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < kTokPerWarp; ++i)
-#pragma unroll
-          for (int u = 0; u < UK; ++u) acc[i][u] += __shfl_xor_sync(0xffffffffu, acc[i][u], o);
-      if ((lane & (vph - 1)) == 0) {
-#pragma unroll
-        for (int i = 0; i < kTokPerWarp; ++i)
-#pragma unroll
-          for (int u = 0; u < UK; ++u)
-            if (lane + 32 * u < nv) lg[(l0 + i) * n_qh + (lane + 32 * u) / vph] = acc[i][u];
-      }
-    } else {
-      for (int j = 0; j < n_qh; ++j) {
-        double acc[kTokPerWarp];
-#pragma unroll
-        for (int i = 0; i < kTokPerWarp; ++i) acc[i] = 0.0;
-        if (use_query) {
-          const int kv = (j * bt.n_kvh) / n_qh;
-          const int vshift = (j - kv) * vph;            // key-row vector v pairs with query vector v + vshift
-#pragma unroll
-          for (int u = 0; u < UK; ++u) {
-            const int v = lane + 32 * u;
-            if (v < nv && v / vph == kv) {
-#pragma unroll
-              for (int i = 0; i < kTokPerWarp; ++i) {
-                float x[V];
-                widen_vec<T>(kb[i][u], x);
-#pragma unroll
-                for (int k = 0; k < V; ++k) acc[i] = fma((double)x[k], qT[k * nvq + v + vshift], acc[i]);
-              }
+          for (; v < nv; v += 32) sumsq_accumulate<T>(row[v], a0);
+          __syncwarp();
+          if (lane == 0) {
+            issue_row();
+            if (!all && *const_cast<volatile int *>(&s_query)) {
+              all = true;
+              for (int k = 1; k < cfg.nbuf; ++k) issue_row();
             }
           }
-          for (int v = lane + 32 * UK; v < nv; v += 32) {   // rows wider than the preloaded part
-            if (v / vph == kv) {
-#pragma unroll
-              for (int i = 0; i < kTokPerWarp; ++i) {
-                const int rr = min(r0 + l0 + i, N - 1);
-                float x[V];
-                widen_vec<T>(__ldg(reinterpret_cast<const uint4 *>(Ke + (size_t)rr * im.ldKe) + v), x);
-#pragma unroll
-                for (int k = 0; k < V; ++k) acc[i] = fma((double)x[k], qT[k * nvq + v + vshift], acc[i]);
-              }
+          if (++slot == cfg.nbuf) slot = 0;
+        }
+        s_acc[r][lane] = a0 + a1;
+      }
+      __syncwarp();
+      finish_row_sums(s_acc, w, kTokWarps, n, [&](int r, double s) { im.nrm[r0 + r] = sqrt(s); });
+    }
+    pdl_wait();
+  } else {
+    const int team = threadIdx.x >= kTokGroup + kTokTeam, t = threadIdx.x & (kTokTeam - 1), w = t >> 5;   // within the team
+    const int P = rpp <= 8 ? 4 : rpp <= 16 ? 2 : 1;     // lanes per token
+    uint8_t *s_mine = s_key + (size_t)team * rpp * ks;
+    auto issue_keys = [&](int u) {                      // lane 0 of every warp: its share of the scoring keys of unit u
+      if (u >= u1) return;
+      const int b = image_of(u, 0);
+      const ImgDesc &im = bt.img[b];
+      const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
+      if (w == 0) mbar_arrive_expect_tx(&s_kbar[team], n * bt.d_k * (int)sizeof(T));
+      for (int r = w; r < n; r += kTeamWarps)
+        bulk_load(s_mine + (size_t)r * ks, reinterpret_cast<const T *>(im.Ke) + (size_t)(r0 + r) * im.ldKe, bt.d_k * (int)sizeof(T), &s_kbar[team]);
+    };
+    if (cfg.keys && lane == 0) issue_keys(u0 + team);
+    auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTokTeam) : "memory"); };
+    auto sync_both = []() { asm volatile("bar.sync 3, %0;" ::"n"(kTokGroup) : "memory"); };
+    if (do_init) {                                      // what later kernels accumulate into
+      const int gt = blockIdx.x * kTokGroup + threadIdx.x - kTokGroup, gs = gridDim.x * kTokGroup;
+      for (int i = 0; i < bt.B; ++i) {
+        const ImgDesc &im = bt.img[i];
+        for (int r = gt; r < im.Np; r += gs) { im.rho_fix[r] = 0ull; im.csize[r] = 0; im.cticket[r] = 0; }
+        for (int wd = gt; wd < im.Wp; wd += gs) { im.cmask[wd] = 0u; im.rmask[wd] = 0u; im.rtick[wd] = 0; }
+        for (int r = gt; r < im.N; r += gs) im.best[r] = kBestInit;
+        uint4 *tab = reinterpret_cast<uint4 *>(im.cnt_cb);
+        for (int r = gt; r < im.Np * (im.nbp / 8); r += gs) tab[r] = make_uint4(0u, 0u, 0u, 0u);
+        for (int r = gt; r < (1 << kHistBits); r += gs) im.ghist[r] = 0;
+        if (gt < kCntInts) im.cnt[gt] = 0;
+      }
+    }
+    int b = 0, loaded = -1;                             // loaded: image whose query is in s_q
+    uint32_t par = 0;
+    for (int u = u0; u < u1; ++u) {
+      b = image_of(u, b);
+      const ImgDesc &im = bt.img[b];
+      const bool mine = ((u - u0) & 1) == team;
+      const int g = u - s_first[b], r0 = g * rpp, n = min(rpp, im.N - r0);
+      const uint8_t *keys = cfg.keys ? s_mine : reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.Ke) + (size_t)r0 * im.ldKe);
+      const size_t kstride = cfg.keys ? (size_t)ks : (size_t)im.ldKe * sizeof(T);
+      if (mine) {
+        if (cfg.keys && !mbar_wait_warp(&s_kbar[team], par)) s_abort = 1;
+        par ^= 1u;
+        if (im.Kc) {                                     // inverse norms: eight lanes per row, four rows at a time
+          const bool same = cfg.keys && im.Kc == im.Ke;
+          const uint8_t *kc = same ? keys : reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.Kc) + (size_t)r0 * im.ldKc);
+          const size_t cs = same ? kstride : (size_t)im.ldKc * sizeof(T);
+          const int nv = bt.d_k / V;
+          for (int rb = w * 4; rb < n; rb += kTeamWarps * 4) {
+            const int r = rb + lane / 8;
+            double a = 0.0;
+            if (r < n) {
+#pragma unroll 4
+              for (int v = lane & 7; v < nv; v += 8) sumsq_accumulate<T>(*(reinterpret_cast<const uint4 *>(kc + (size_t)r * cs) + v), a);
             }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (r < n && (lane & 7) == 0) rn_tok<D>(im)[r0 + r] = (rn_t)inv_norm(a);
           }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int i = 0; i < kTokPerWarp; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-        if (lane == 0) {
-#pragma unroll
-          for (int i = 0; i < kTokPerWarp; ++i) lg[(l0 + i) * n_qh + j] = acc[i];
-        }
+      }
+      if (u == u0) {
+        pdl_wait();                                      // the global queries are complete
+        s_query = 1;
+        pdl_trigger();
+      }
+      const bool use_query = !(im.flags & PACT_FLAG_NORM_ONLY) && im.Q != nullptr;
+      if (use_query && loaded != b) {                    // both teams come by here for every image of the CTA's units
+        if (loaded >= 0) sync_both();
+        for (int c = threadIdx.x - kTokGroup; c < bt.n_qcols; c += kTokGroup) s_q[c] = ld_cg_f64(&im.qg[c]);
+        loaded = b;
+        sync_both();
+      }
+      if (!mine) continue;
+      const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
+      const int nblk = (n_rep + 3) / 4;                  // blocks of up to four query heads per key head
+      for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
+        const int kv = it / nblk, j = (it - kv * nblk) * 4, nr = min(4, n_rep - j), j0 = kv * n_rep + j;
+        const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
+        if (nr >= 3) head_piece<T, 4>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else if (nr == 2) head_piece<T, 2>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else head_piece<T, 1>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+      }
+      if (cfg.keys && u + 2 < u1) {
+        sync();                                          // the keys have been read
+        if (lane == 0) issue_keys(u + 2);
       }
     }
   }
-  row_pass(kTokPerWarp - 1);
   __syncthreads();
-  // per head: CTA max, exp, CTA sum; lane = token within the CTA
-  for (int j = w; j < n_qh; j += kTokWarps) {
-    const int rr = r0 + lane;
-    const bool ok = rr < r1;
-    const double l = ok ? lg[lane * n_qh + j] : -1.0e300;
-    double m = l;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const double e = ok ? exp(l - m) : 0.0;
-    if (ok) im.E[(size_t)rr * n_qh + j] = e;
-    const double sum = warp_sum(e);
-    if (lane == 0) {
-      im.part[((size_t)g * n_qh + j) * 2] = m;
-      im.part[((size_t)g * n_qh + j) * 2 + 1] = sum;
-    }
-  }
+  if (threadIdx.x == 0 && s_abort)
+    for (int i = 0; i < bt.B; ++i) atomicMin(&bt.img[i].cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
 }
 
 __device__ __forceinline__ void ld_cg_f64x2(const double *p, double &a, double &b) {
@@ -338,97 +449,116 @@ __device__ __forceinline__ void ld_cg_f64x2(const double *p, double &a, double &
 
 // ---- Eq. 2, second half: merge the pieces (M = max, Z = sum S_g exp(M_g - M), fixed order), scores --------
 // grid (ceil(maxN / 256), B), 256 threads.  Every CTA merges all G pieces itself: the warps share out the
-// heads (and, with fewer heads than warps, the pieces of a head), four loads per lane in flight.  with_hist:
+// heads (and, with fewer heads than warps, the pieces of a head), eight loads per lane in flight; what turns a term into
+// a share, exp(M_g - M) / (Z n_qh), is formed once per piece and head of the CTA's tokens.  with_hist:
 // every score also counts in the histogram of its top key bits, the first level of the threshold selection.
 constexpr int kScoreWarps = 8;
+constexpr int kScoreHeads = 32;                         // heads whose factors are in shared memory at a time
+constexpr int kScorePieces = 256 / kMinPiece + 1;       // most pieces that 256 tokens belong to
 
-__global__ void __launch_bounds__(256) k_scores(const __grid_constant__ Batch bt, int with_hist) {
+__global__ void __launch_bounds__(256) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 2);
   pdl_wait();
   pdl_trigger();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int N = im.N, n_qh = bt.n_qh;
-  if ((int)blockIdx.x * 256 >= N) return;
-  const int G = (N + kRowsPerCta - 1) / kRowsPerCta;
+  const int N = im.N, n_qh = bt.n_qh, i0 = blockIdx.x * 256;
+  if (i0 >= N) return;
+  const int G = (N + rpp - 1) / rpp, g0 = i0 / rpp, np = (min(N, i0 + 256) - 1) / rpp - g0 + 1;   // pieces of the CTA's tokens
   __shared__ double sM[256], sInv[256];
   __shared__ double pmx[kScoreWarps], pz[kScoreWarps];
-  const int i = blockIdx.x * 256 + t;
-  // this token's terms, requested before the merge so that they arrive meanwhile
+  __shared__ double s_fac[kScorePieces * kScoreHeads];
+  const int i = i0 + t;
+  // this token's terms and the first of the CTA's pieces, requested before the merge so that they arrive meanwhile
   constexpr int EP = 4;
-  double e_pre[EP], nrm_i = 0.0;
-  const bool pre = n_qh <= EP && i < N;
-  if (pre) {
+  double e_pre[EP], nrm_i = 0.0, m_pre = 0.0;
+  if (i < N) {
 #pragma unroll
-    for (int j = 0; j < EP; ++j) e_pre[j] = j < n_qh ? im.E[(size_t)i * n_qh + j] : 0.0;
+    for (int j = 0; j < EP; ++j) e_pre[j] = j < n_qh ? im.E[(size_t)j * N + i] : 0.0;
+    nrm_i = im.nrm[i];
   }
-  if (i < N) nrm_i = im.nrm[i];
+  const int nf0 = np * min(n_qh, kScoreHeads);
+  if (t < nf0) m_pre = im.part[((size_t)(g0 + t % np) * n_qh + t / np) * 2];
   const int wph = n_qh >= kScoreWarps ? 1 : kScoreWarps / n_qh;   // warps per head
   const int hpp = kScoreWarps / wph;                    // heads per pass
+  constexpr int U = 8;
   const int step = 32 * wph;
-  const int nbatch = (G + 4 * step - 1) / (4 * step);
+  const int nbatch = (G + U * step - 1) / (U * step);
   for (int j0 = 0; j0 < n_qh; j0 += hpp) {
     const int j = j0 + w / wph, sub = w % wph;
     const bool mine = j < n_qh && w / wph < hpp;
-    auto load4 = [&](int b, double (&pm)[4], double (&ps)[4]) {
+    auto load = [&](int b, double (&pm)[U], double (&ps)[U]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int h = sub * 32 + lane + step * (4 * b + u);
+      for (int u = 0; u < U; ++u) {
+        const int h = sub * 32 + lane + step * (U * b + u);
         pm[u] = -1.0e300;
         ps[u] = 0.0;
         if (mine && h < G) ld_cg_f64x2(im.part + ((size_t)h * n_qh + j) * 2, pm[u], ps[u]);
       }
     };
-    double pm0[4], ps0[4];
-    load4(0, pm0, ps0);
-    double m = fmax(fmax(pm0[0], pm0[1]), fmax(pm0[2], pm0[3]));
+    double pm0[U], ps0[U], m = -1.0e300;
+    load(0, pm0, ps0);
+#pragma unroll
+    for (int u = 0; u < U; ++u) m = pm0[u] > m ? pm0[u] : m;
     for (int b = 1; b < nbatch; ++b) {
-      double pm[4], ps[4];
-      load4(b, pm, ps);
-      m = fmax(m, fmax(fmax(pm[0], pm[1]), fmax(pm[2], pm[3])));
+      double pm[U], ps[U];
+      load(b, pm, ps);
+#pragma unroll
+      for (int u = 0; u < U; ++u) m = pm[u] > m ? pm[u] : m;
     }
+    m = warp_max(m);
+    if (wph > 1) {
+      __syncthreads();
+      if (lane == 0) pmx[w] = m;
+      __syncthreads();
+      if (mine)
+        for (int k = 0; k < wph; ++k) { const double o = pmx[w - sub + k]; m = o > m ? o : m; }
+    }
+    double z = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __syncthreads();
-    if (lane == 0) pmx[w] = m;
-    __syncthreads();
-    if (mine)
-      for (int k = 0; k < wph; ++k) m = fmax(m, pmx[w - sub + k]);
-    double z = 0.0;                                     // an empty slot adds 0 * exp(-huge) = 0
-#pragma unroll
-    for (int u = 0; u < 4; ++u) z += ps0[u] * exp(pm0[u] - m);
+    for (int u = 0; u < U; ++u)
+      if (step * u < G) z += ps0[u] * exp(pm0[u] - m);  // (an empty slot adds 0 * exp(-huge) = 0)
     for (int b = 1; b < nbatch; ++b) {
-      double pm[4], ps[4];
-      load4(b, pm, ps);
+      double pm[U], ps[U];
+      load(b, pm, ps);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) z += ps[u] * exp(pm[u] - m);
+      for (int u = 0; u < U; ++u) z += ps[u] * exp(pm[u] - m);
     }
     z = warp_sum(z);
-    if (lane == 0) pz[w] = z;
-    __syncthreads();
+    if (wph > 1) {
+      if (lane == 0) pz[w] = z;
+      __syncthreads();
+    }
     if (mine && sub == 0 && lane == 0) {
-      double zz = 0.0;
-      for (int k = 0; k < wph; ++k) zz += pz[w + k];
+      if (wph > 1) {
+        z = 0.0;
+        for (int k = 0; k < wph; ++k) z += pz[w + k];
+      }
       sM[j] = m;
-      sInv[j] = 1.0 / (zz * (double)n_qh);
+      sInv[j] = 1.0 / (z * (double)n_qh);
     }
   }
-  __syncthreads();
-  if (i >= N) return;
-  const int g = i / kRowsPerCta;
   double s = 0.0;
-  for (int j = 0; j < n_qh; ++j) {
-    const double fac = exp(im.part[((size_t)g * n_qh + j) * 2] - sM[j]) * sInv[j];
-    double e;
-    if (pre) {
-      e = e_pre[0];
-#pragma unroll
-      for (int q = 1; q < EP; ++q) if (j == q) e = e_pre[q];
-    } else {
-      e = im.E[(size_t)i * n_qh + j];
+  for (int h0 = 0; h0 < n_qh; h0 += kScoreHeads) {
+    const int nh = min(kScoreHeads, n_qh - h0);
+    __syncthreads();
+    for (int f = t; f < np * nh; f += 256) {            // factor f: head h0 + f / np, piece f % np
+      const int j = h0 + f / np;
+      const double mg = h0 == 0 && f == t ? m_pre : im.part[((size_t)(g0 + f % np) * n_qh + j) * 2];
+      s_fac[f] = exp(mg - sM[j]) * sInv[j];
     }
-    s = fma(e, fac, s);
+    __syncthreads();
+    if (i < N) {
+      const double *fac = s_fac + (i / rpp - g0);
+      int j = 0;
+      if (h0 == 0) {
+#pragma unroll
+        for (; j < EP; ++j) if (j < nh) s = fma(e_pre[j], fac[j * np], s);
+      }
+      for (; j < nh; ++j) s = fma(im.E[(size_t)(h0 + j) * N + i], fac[j * np], s);
+    }
   }
+  if (i >= N) return;
   const float sf = (float)(s * nrm_i);
   im.score[i] = sf;
   if (im.score_user) im.score_user[i] = sf;
@@ -455,7 +585,7 @@ struct SelShared {
   int own_tok[kSelThreads], own_slot[kSelThreads];
 };
 
-// The key of the (m_target + 1)-th smallest score.  the key of the (m_target + 1)-th smallest score.  The histogram of the top kHistBits key
+// The key of the (m_target + 1)-th smallest score.  The histogram of the top kHistBits key
 // bits, filled by k_scores, gives the bin of the threshold and its rank inside that bin; radix passes
 // over the bits below, kSelBits at a time, finish the selection (only the keys of that bin take part, so the
 // shared-memory counters see little contention; the bins of a pass are scanned by all threads).  KPT > 0: thread t holds the keys t, t + 512, ... in
@@ -863,29 +993,63 @@ size_t g_smem_optin = 48 * 1024;
 constexpr size_t kSplitReserve = 4096;       // static shared memory of k_split, rounded up
 }  // namespace
 
-static int qsum_row_blocks(int ncg, int B, int maxN) {
-  // CTAs on 7/16 of the SMs (64 of 148) when that leaves a CTA no more than two rounds of loads (1024 rows),
-  // else as many row blocks as that takes, up to a cluster of eight: see k_qsum
-  int RP = 1;
-  while (RP < kQPartRows && (ncg * B * RP * 2 <= g_sm_count * 7 / 16 || (maxN + RP - 1) / RP > 1024)) RP *= 2;
-  return RP;
+template <typename T>
+static cudaError_t launch_qsum(const Batch &bt, cudaStream_t st) {
+  // column groups of four vectors where that does not take more CTAs than two per SM, else of eight; then as many row
+  // blocks (CTAs of a cluster) as keep the grid within two CTAs per SM
+  const int nvq = bt.n_qcols / Vec<T>::N;
+  const bool narrow = (nvq + 3) / 4 * bt.B * kQPartRows <= 2 * g_sm_count;
+  const int ncg = narrow ? (nvq + 3) / 4 : (nvq + 7) / 8;
+  LaunchOpt opt;
+  opt.cluster = 1;
+  while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 2 * g_sm_count) opt.cluster *= 2;
+  const dim3 grid(ncg * opt.cluster, bt.B), block(kQsumThreads);
+  return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster);
+}
+
+// Tokens per unit: the fewest rounds of units of `most` tokens over the SMs, then as few tokens as that many rounds allow
+// (but eight), so that the rounds are full.
+template <typename T> static TokCfg tokens_config(const Batch &bt) {
+  TokCfg c;
+  long long total = 0;
+  for (int b = 0; b < bt.B; ++b) total += bt.img[b].N;
+  const int rowb = bt.d * (int)sizeof(T), keyb = bt.d_k * (int)sizeof(T);
+  c.nchunk = (rowb + 8191) / 8192;
+  c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
+  c.nbuf = kTokMaxBuf;
+  c.keys = 1;
+  const auto fits = [&]() { return tok_smem(c, keyb, bt.n_qcols) <= (size_t)kTokSmem; };
+  for (int most = 32; most >= kMinPiece; most /= 2) {
+    const long long rounds = (total + (long long)most * g_sm_count - 1) / ((long long)most * g_sm_count);
+    const long long rpp = (total + rounds * g_sm_count - 1) / (rounds * g_sm_count);
+    c.rpp = (int)(rpp < kMinPiece ? kMinPiece : rpp);
+    if (fits()) return c;
+  }
+  c.keys = 0;                                                             // very wide keys or queries
+  while (!fits() && c.chunk > 1024) {
+    c.nchunk *= 2;
+    c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
+  }
+  return c;
+}
+static int tokens_grid(const Batch &bt, int rpp) {
+  long long units = 0;
+  for (int b = 0; b < bt.B; ++b) units += (bt.img[b].N + rpp - 1) / rpp;
+  return (int)(units < g_sm_count ? units : g_sm_count);
 }
 
 template <typename T>
-static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream_t st, StageMark mark, void *mark_arg) {
-  constexpr int V = Vec<T>::N;
-  const int ncg = (bt.n_qcols / V + 7) / 8;
-  const int RP = qsum_row_blocks(ncg, bt.B, maxN);
-  LaunchOpt opt;
-  opt.cluster = RP;
-  cudaError_t e = launch_opt(opt, k_qsum<T>, dim3(ncg * RP, bt.B), dim3(kQsumThreads), 0, st, bt, RP, mode == 0 ? 1 : 0);
+static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
+  cudaError_t e = launch_qsum<T>(bt, st);
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
-  const size_t sm_tok = (size_t)(bt.n_qcols + kRowsPerCta * bt.n_qh) * sizeof(double);
-  e = launch_k(k_tokens<T>, dim3((maxN + kRowsPerCta - 1) / kRowsPerCta, bt.B), dim3(kTokThreads), sm_tok, st, true, bt);
+  const TokCfg tc = tokens_config<T>(bt);
+  e = launch_k(k_tokens<T>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, true, bt, tc, mode != 1 ? 1 : 0);
   if (e != cudaSuccess) return e;
+  if (rpp) *rpp = tc.rpp;
+  if (mode == 2) return cudaSuccess;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
-  e = launch_k(k_scores, dim3((maxN + 255) / 256, bt.B), dim3(256), 0, st, true, bt, mode == 0 ? 1 : 0);
+  e = launch_k(k_scores, dim3((maxN + 255) / 256, bt.B), dim3(256), 0, st, true, bt, tc.rpp, mode == 0 ? 1 : 0);
   if (e != cudaSuccess) return e;
   if (mode == 0) {
     if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
@@ -902,12 +1066,12 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark, void *mark_arg) {
-  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, mark, mark_arg)
-              : launch_euti_t<float>(bt, maxN, mode, st, mark, mark_arg);
+cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
+  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, mark, mark_arg, rpp)
+              : launch_euti_t<float>(bt, maxN, mode, st, mark, mark_arg, rpp);
 }
 
-int euti_kernels(int mode) { return mode == 0 ? 4 : 3; }
+int euti_kernels(int mode) { return mode == 0 ? 4 : mode == 1 ? 3 : 2; }
 
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st) {
   if (N <= 8 * 1024) return launch_k(k_split<8>, dim3(1), dim3(1024), 0, st, true, bt, 0);
@@ -927,22 +1091,30 @@ cudaError_t select_configure() {
   e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   g_smem_optin = (size_t)v;
-  return cudaFuncSetAttribute(k_split<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
+  e = cudaFuncSetAttribute(k_split<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
+  if (e != cudaSuccess) return e;
+  return e;
 }
 
-cudaError_t euti_configure(int n_qcols, int n_qh) {
+cudaError_t euti_configure(int n_qcols) {
   cudaError_t e = select_configure();
   if (e != cudaSuccess) return e;
-  const size_t sm = (size_t)(n_qcols + kRowsPerCta * n_qh) * sizeof(double);
-  if (sm > g_smem_optin - 1024) return cudaErrorInvalidConfiguration;
-  e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // the widest query and the narrowest of everything else have to fit
+  if ((size_t)n_qcols * 8 + kMinPiece * 32 * 8 + kTokWarps * 1040 + 64 > g_smem_optin - 4096)
+    return cudaErrorInvalidConfiguration;
+  const int tok = (int)(g_smem_optin - 2048);
+  e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_tokens<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  e = cudaFuncSetAttribute(k_tokens<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok);
   if (e != cudaSuccess) return e;
   const int dyn = 96 * 1024;
   e = cudaFuncSetAttribute(k_select<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_select<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  e = cudaFuncSetAttribute(k_select<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  if (e != cudaSuccess) return e;
+  // k_tokens can only begin beside k_qsum if both run under the same split of the SM's memory (with the default it waited
+  // for k_qsum to drain, 9 us at 6272 tokens); for the other kernels the default is as good or better (16384-token images: 10 us)
+  return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16>, k_tokens<float>);
 }
 
 }  // namespace pact

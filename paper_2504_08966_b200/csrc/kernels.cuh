@@ -56,6 +56,13 @@ inline cudaError_t launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   return launch_opt(o, kernel, grid, block, smem, st, args...);
 }
 
+// The largest shared-memory carve-out for these kernels.
+template <typename... K> inline cudaError_t prefer_shared(K... kernel) {
+  cudaError_t e = cudaSuccess;
+  ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) : e), ...);
+  return e;
+}
+
 constexpr int kMergeMaxD = 256 * 4 * 8;   // widest hidden state the merge kernel holds in registers
 
 // how a kernel finds its rows
@@ -66,15 +73,15 @@ constexpr int kQPartRows = 8;             // most row blocks the column sums of 
 constexpr int kHistBits = 12;             // key bits of the first-level histogram of the threshold selection
 constexpr int kHistShift = 32 - kHistBits; // a key's bin in that histogram is key >> kHistShift
 // Algorithm 1.  mode 0: scores, threshold, lists, survivor keys (four kernels; the first also clears what later
-// kernels accumulate into); mode 1: scores only (three kernels).
+// kernels accumulate into); mode 1: scores only (three kernels); mode 2: mode 0 up to the token pass (two kernels).
 // mark (optional) is called between the kernels of the group (the per-kernel timing of a profiled call)
 typedef cudaError_t (*StageMark)(void *);
 cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark = nullptr,
-                        void *mark_arg = nullptr);
+                        void *mark_arg = nullptr, int *rpp = nullptr);   // rpp: receives the tokens per softmax piece
 int euti_kernels(int mode);
 // threshold + ordered compaction of given scores (pact_prune, one image)
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st);
-cudaError_t euti_configure(int n_qcols, int n_qh);
+cudaError_t euti_configure(int n_qcols);
 cudaError_t select_configure();            // what launch_split needs, once per device
 
 // cluster.cu
@@ -117,6 +124,6 @@ int lists_kernels(int maxN, int B);        // kernels launch_lists launches (1, 
 cudaError_t launch_list_clear(const Batch &bt, cudaStream_t st);   // csize, cticket, cnt_cb and the counters
 cudaError_t launch_merge(const Batch &bt, bool in_bf16, bool out_bf16, const ClusterCfg &cfg, cudaStream_t st);
 cudaError_t merge_configure();
-int merge_ctas(int sm_count, int B);       // CTAs per image of k_merge (sizes its scratch)
+size_t merge_scratch_rows();               // rows of partial sums k_merge may need per image
 
 }  // namespace pact

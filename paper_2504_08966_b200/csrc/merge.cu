@@ -6,55 +6,17 @@
 //            cluster id: every block of 128 tokens sorts its own, an image-wide barrier, and every
 //            token writes one 16-byte record {token, cluster, first member position, cluster size}
 //            at its place in the cluster-sorted member array.  Also P', sizes and log sizes.
-//   k_merge  the member array (followed by the text rows) is cut into one contiguous range per CTA;
-//            a CTA streams the rows of its range with many loads in flight and no look-ups, keeps the
-//            running cluster in registers and writes a row out whenever the cluster id changes.
-//            Clusters cut by a range boundary leave partial sums; the last CTA to arrive adds them in
+//   k_merge  the member array (followed by the text rows) is cut into contiguous ranges;
+//            a CTA streams its columns of the rows of a range with many loads in flight and no look-ups, keeps
+//            the running cluster in registers and writes a row out whenever the cluster id changes.
+//            Large clusters cut by a range boundary leave partial sums; the last CTA to arrive adds them in
 //            range order, so the result does not depend on timing.
 #include <cooperative_groups.h>
 
 #include "kernels.cuh"
+#include "tma.cuh"
 
 namespace pact {
-
-template <typename O> __device__ __forceinline__ void store_vec8(O *p, const float (&x)[8]);
-template <> __device__ __forceinline__ void store_vec8<float>(float *p, const float (&x)[8]) {
-  reinterpret_cast<float4 *>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
-  reinterpret_cast<float4 *>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
-}
-template <> __device__ __forceinline__ void store_vec8<__nv_bfloat16>(__nv_bfloat16 *p, const float (&x)[8]) {
-  uint32_t w[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
-    w[i] = *reinterpret_cast<uint32_t *>(&h);
-  }
-  *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// Eight consecutive elements of a row as loaded (not yet widened), so that many can be in flight.
-template <typename T> struct Raw8;
-template <> struct Raw8<__nv_bfloat16> {
-  uint4 a;
-  __device__ __forceinline__ void from_ring(const uint4 *p) { a = p[0]; }
-  __device__ __forceinline__ void add_to(float (&acc)[8]) const {
-    float x[8];
-    widen_vec<__nv_bfloat16>(a, x);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] += x[e];
-  }
-};
-template <> struct Raw8<float> {
-  uint4 a, b;
-  __device__ __forceinline__ void from_ring(const uint4 *p) { a = p[0]; b = p[1]; }
-  __device__ __forceinline__ void add_to(float (&acc)[8]) const {
-    float x[4], y[4];
-    widen_vec<float>(a, x);
-    widen_vec<float>(b, y);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { acc[e] += x[e]; acc[4 + e] += y[e]; }
-  }
-};
 
 __device__ __forceinline__ int ld_cg_i32(const int *p) {
   int v;
@@ -397,208 +359,223 @@ __global__ void __launch_bounds__(256) k_list_clear(const __grid_constant__ Batc
 }
 
 // ---- Eq. 10 ------------------------------------------------------------------------------------------
-// Grid (X, B), kMrgThreads threads, two CTAs per SM.  Work items are the member records in cluster order
-// followed by the text rows; CTA x takes items [x per, (x + 1) per).  A thread owns VPL groups of 8 columns
-// and adds the rows of the running cluster in float.  The rows arrive through a ring of DEPTH rows in shared
-// memory filled with asynchronous 16-byte copies (every thread copies and later reads its own columns, so
-// the ring needs no barrier): DEPTH rows are in flight per SM whatever the registers hold.  A cluster that
-// lies inside the range is divided and stored when the next one begins.  A range boundary cuts at most two clusters per CTA: the one that began before the range (its
-// sum is set aside when it ends) and the one that goes on after it.  Their sums go to scratch (slot 0 and
-// slot 1 of the CTA) with a ticket each; the CTA that draws a cluster's last ticket adds the sums in range
-// order and stores the row, so the result does not depend on which CTA that is.
-constexpr int kMrgThreads = 512;
-constexpr int kMrgTile = 256;                       // records staged in shared memory at a time
-constexpr int kMrgCtasPerSm = 2;
-constexpr int kMrgRingBytes = 160 * 1024 / kMrgCtasPerSm;   // rows in flight per CTA
+// Grid (ranges x slices, B), 128 threads, eight CTAs per SM.  Work items are the member records in cluster order
+// followed by the text rows; a CTA takes one range of `per` of them and one slice of the columns, a thread VPL groups of
+// eight columns, and adds the rows of the running cluster in float.  The rows arrive through two half rings in shared
+// memory, one bulk copy per row and one barrier per half: while one half is added the other is on its way.
+//
+// A cluster of at most `whole` members is done by the range it begins in, however far it reaches past the range's
+// end: a cut costs a chain of three trips through the L2 at the end of a CTA (about 2.5 us).  Larger clusters are cut at
+// the range boundaries: their sums go to scratch with a ticket, and the CTA that draws a cluster's last ticket adds the
+// sums in range order and stores the row, so the result does not depend on which CTA that is.
+//
+// Instructions count here: 46000 rows of 7 KB through 16-byte copies of every thread's own took 85 warp instructions per
+// 512 bytes and with them 83 us at 0.54 of the memory rate; with bulk copies a thread only adds, and they take 62 us.
+constexpr int kMrgThreads = 128;
+constexpr int kMrgCtasPerSm = 8;
+constexpr int kMrgRanges = 296;                     // most ranges per image (sizes the scratch)
+constexpr int kMrgRingBytes = 24 * 1024;            // rows in flight per CTA when an SM has eight, more when it has fewer
+constexpr int kMrgRingMost = 192 * 1024;
+constexpr int kMrgMaxHalf = 32;                     // rows in a half ring
 
-template <typename T, typename O, int VPL, int DEPTH>
-__global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __grid_constant__ Batch bt) {
+template <typename T, typename O, int VPL>
+__global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __grid_constant__ Batch bt, int per, int whole, int slices, int ring_bytes) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 9);
-  // final since the centre selection, which is complete before any kernel after it can start
-  const int C = min(ld_cg_i32(im.C_ptr), im.Np);
+  extern __shared__ uint4 ring[];
+  __shared__ uint64_t s_bar[2];
+  __shared__ int s_abort;
+  if (threadIdx.x == 0) {
+    mbar_init(&s_bar[0], 1);
+    mbar_init(&s_bar[1], 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   pdl_wait();
   pdl_trigger();
   const int t = threadIdx.x;
-  __shared__ int4 s_rec[kMrgTile];                  // {row of H, cluster, first member position, size}
-  __shared__ int s_dst[kMrgTile];                   // output row
-  __shared__ float s_inv[kMrgTile];                 // 1 / size (1 for text rows and centre-only merging)
+  __shared__ int s_row[kMrgThreads], s_cluster[kMrgThreads], s_dst[kMrgThreads];   // row of H, cluster, output row of an item
+  __shared__ float s_inv[kMrgThreads];              // 1 / size (1 for text rows and centre-only merging)
   __shared__ int s_last;
-  const int n_text = im.n_total - im.N;
-  const int d = bt.d, ng = d / 8;
+  const int n_text = im.n_total - im.N, d = bt.d, ng = d / 8;
   const bool center_only = (im.flags & PACT_FLAG_CENTER_ONLY) != 0;
-  const T *H = reinterpret_cast<const T *>(im.H);
-  O *Ho = reinterpret_cast<O *>(im.H_out);
-  const int n_mem = center_only ? C : min(max(ld_cg_i32(&im.cnt[20]), 0), im.N);
-  const int total = n_mem + n_text;
-  const int X = gridDim.x, x = blockIdx.x;
-  const int per = (total + X - 1) / X;
-  const int lo = min(total, x * per), hi = min(total, lo + per);
+  const int x = blockIdx.x / slices, sl = blockIdx.x - x * slices;
+  // this slice's groups of eight columns: gn from g0 on; thread t takes g0 + t, g0 + t + nth
+  const int gps = (ng + slices - 1) / slices, g0 = sl * gps, gn = min(ng, g0 + gps) - g0, nth = (gn + VPL - 1) / VPL;
+  bool mine[VPL];
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) mine[v] = t < nth && t + v * nth < gn;
+  const int lo = x * per;
+  // everything the range needs to know in one trip to the L2: the counts, the records of its first items and of its last
+  auto fetch = [&](int p) { return center_only ? make_int4(__ldcg(im.cidx_ptr + min(p, im.N - 1)), p, p, 1) : __ldcg(im.members + min(p, im.N - 1)); };
+  const int C_raw = ld_cg_i32(im.C_ptr), n_all = ld_cg_i32(&im.cnt[20]);
+  const int4 rec_lo = fetch(lo), rec_hi = fetch(lo + per - 1), rec_t = fetch(lo + t);
+  const int C = min(C_raw, im.Np), n_mem = center_only ? C : min(max(n_all, 0), im.N);
+  const int hi = min(n_mem + n_text, lo + per);
   // every other counter is final: this is the last kernel of the call
-  if (x == 0 && t < PACT_N_COUNTERS) im.counters_user[t] = t == PACT_CNT_N_OUT ? n_text + C : ld_cg_i32(&im.cnt[t]);
+  if (blockIdx.x == 0 && t < PACT_N_COUNTERS) im.counters_user[t] = t == PACT_CNT_N_OUT ? n_text + C : ld_cg_i32(&im.cnt[t]);
+  if (lo >= hi) return;
+  // {token, cluster, first member, size} of a member; in bounds whatever an aborted earlier stage left in the records
+  auto checked = [&](int4 r, int p) {
+    r.x = min(max(r.x, 0), im.N - 1);
+    r.y = min(max(r.y, 0), C - 1);
+    r.z = min(max(r.z, 0), p);
+    r.w = min(max(r.w, p - r.z + 1), n_mem - r.z);
+    return r;
+  };
+  int start = lo, stop = hi;
+  int cut_head = -1, cut_tail = -1;                 // first member of the cut cluster the range begins / ends with
+  int cut_head_n = 0, cut_tail_n = 0;
+  if (lo < n_mem) {
+    const int4 a = checked(rec_lo, lo);
+    if (a.z < lo) {
+      if (a.w <= whole) start = a.z + a.w;          // done by the range it begins in
+      else { cut_head = a.z; cut_head_n = a.w; }
+    }
+    if (hi < n_mem) {
+      const int4 b = checked(rec_hi, hi - 1);
+      if (b.z + b.w > hi) {
+        if (b.w > whole) { cut_tail = b.z; cut_tail_n = b.w; }
+        else if (b.z >= lo) stop = b.z + b.w;       // the last cluster of the range goes on a little
+        else stop = lo;                             // (the whole range belongs to a cluster that began before it)
+      }
+    }
+    if (start >= stop) return;
+  }
 
+  const T *H = reinterpret_cast<const T *>(im.H) + (size_t)g0 * 8;
+  O *Ho = reinterpret_cast<O *>(im.H_out) + (size_t)(g0 + t) * 8;
   float acc[VPL][8];
-  int cur_c = -1, cur_off = 0, cur_size = 0, cur_dst = 0;
-  float cur_inv = 1.f;
-  bool head_open = false;                           // the running cluster began before this range
+  auto zero = [&]() {
 #pragma unroll
-  for (int v = 0; v < VPL; ++v)
+    for (int v = 0; v < VPL; ++v)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[v][e] = 0.f;
-
-  auto store_row = [&](const float (&a)[VPL][8], float inv, int dst) {
+      for (int e = 0; e < 8; ++e) acc[v][e] = 0.f;
+  };
+  auto store_row = [&](float inv, int dst) {
+    O *o = Ho + (size_t)dst * im.ldHo;
 #pragma unroll
     for (int v = 0; v < VPL; ++v) {
-      const int g = t + v * kMrgThreads;
-      if (g < ng) {
-        float y[8];
+      float y[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) y[e] = a[v][e] * inv;
-        store_vec8<O>(Ho + (size_t)dst * im.ldHo + g * 8, y);
-      }
+      for (int e = 0; e < 8; ++e) y[e] = acc[v][e] * inv;
+      if (mine[v]) store_vec8<O>(o + (size_t)v * nth * 8, y);
     }
   };
   // a cluster cut by a range boundary: sum to scratch, ticket, and the last one adds the sums in range order
-  auto cut = [&](float (&a)[VPL][8], int c, int off, int size, float inv, int dst, int slot) {
-    float *part = im.mpart + ((size_t)x * 2 + slot) * d;
+  auto cut = [&](int first, int size, float inv, int dst, int slot) {
+    float *part = im.mpart + (size_t)(g0 + t) * 8;
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int g = t + v * kMrgThreads;
-      if (g < ng) {
-        reinterpret_cast<float4 *>(part + g * 8)[0] = make_float4(a[v][0], a[v][1], a[v][2], a[v][3]);
-        reinterpret_cast<float4 *>(part + g * 8)[1] = make_float4(a[v][4], a[v][5], a[v][6], a[v][7]);
+    for (int v = 0; v < VPL; ++v)
+      if (mine[v]) {
+        float4 *p = reinterpret_cast<float4 *>(part + ((size_t)x * 2 + slot) * d + (size_t)v * nth * 8);
+        p[0] = make_float4(acc[v][0], acc[v][1], acc[v][2], acc[v][3]);
+        p[1] = make_float4(acc[v][4], acc[v][5], acc[v][6], acc[v][7]);
       }
-    }
-    const int x0 = off / per, x1 = (off + size - 1) / per;
+    const int x0 = first / per, x1 = (first + size - 1) / per;
+    int32_t *ticket = &im.cticket[x0 * 8 + sl];     // (at most one cluster goes on after a range; a range has eight members or more)
     __threadfence();
     __syncthreads();
-    if (t == 0) s_last = (atomicAdd(&im.cticket[c], 1) == x1 - x0);
+    if (t == 0) s_last = (atomicAdd(ticket, 1) == x1 - x0);
     __syncthreads();
     const bool last = s_last != 0;
     __syncthreads();                                 // s_last may be rewritten by the second cut cluster
     if (!last) return;
     __threadfence();
+    zero();
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) a[v][e] = 0.f;
-    for (int xx = x0; xx <= x1; ++xx) {
-      const float *p = im.mpart + ((size_t)xx * 2 + (xx < x1 ? 1 : 0)) * d;
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        const int g = t + v * kMrgThreads;
-        if (g < ng) {
-          const float4 u = ld_cg_f4(p + g * 8), w = ld_cg_f4(p + g * 8 + 4);
-          a[v][0] += u.x; a[v][1] += u.y; a[v][2] += u.z; a[v][3] += u.w;
-          a[v][4] += w.x; a[v][5] += w.y; a[v][6] += w.z; a[v][7] += w.w;
+      if (mine[v])
+#pragma unroll 4
+        for (int xx = x0; xx <= x1; ++xx) {
+          const float *p = part + ((size_t)xx * 2 + (xx == x0 ? 1 : 0)) * d + (size_t)v * nth * 8;
+          const float4 u = ld_cg_f4(p), w = ld_cg_f4(p + 4);
+          acc[v][0] += u.x; acc[v][1] += u.y; acc[v][2] += u.z; acc[v][3] += u.w;
+          acc[v][4] += w.x; acc[v][5] += w.y; acc[v][6] += w.z; acc[v][7] += w.w;
         }
-      }
-    }
-    if (t == 0) im.cticket[c] = 0;
-    store_row(a, inv, dst);
+    if (t == 0) *ticket = 0;
+    store_row(inv, dst);
   };
 
-  constexpr int Q16 = (int)sizeof(T) * 8 / 16;        // 16-byte pieces of a group of 8 columns
-  constexpr int kSlot = VPL * kMrgThreads * Q16;      // 16-byte pieces per ring slot
-  extern __shared__ uint4 ring[];                     // [DEPTH][kSlot]
-  auto issue = [&](int j, int tn) {                   // row j of the tile -> slot j % DEPTH; one group per call
-    if (j < tn) {
-      const T *row = H + (size_t)s_rec[j].x * im.ldH;
-      uint4 *slot = ring + (size_t)(j % DEPTH) * kSlot;
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        const int g = t + v * kMrgThreads;
-        if (g < ng) {
-#pragma unroll
-          for (int pc = 0; pc < Q16; ++pc) {
-            const unsigned dsta = (unsigned)__cvta_generic_to_shared(slot + (size_t)g * Q16 + pc);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dsta), "l"(row + g * 8 + pc * (16 / (int)sizeof(T))) : "memory");
-          }
-        }
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  auto consume = [&](int j) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(DEPTH - 1) : "memory");
-    const int4 rec = s_rec[j];
-    if (rec.y != cur_c) {                            // the next cluster begins (the same for all threads)
-      if (cur_c >= 0) {
-        if (head_open) {                               // the cluster that began before this range ends here
-          cut(acc, cur_c, cur_off, cur_size, cur_inv, cur_dst, 0);
-          head_open = false;
-        } else {
-          store_row(acc, cur_inv, cur_dst);
-        }
-      } else {
-        head_open = rec.z < lo;
-      }
-#pragma unroll
-      for (int v = 0; v < VPL; ++v)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[v][e] = 0.f;
-      cur_c = rec.y; cur_off = rec.z; cur_size = rec.w;
-      cur_dst = s_dst[j]; cur_inv = s_inv[j];
-    }
-    const uint4 *slot = ring + (size_t)(j % DEPTH) * kSlot;
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int g = t + v * kMrgThreads;
-      if (g < ng) {
-        Raw8<T> x;
-        x.from_ring(slot + (size_t)g * Q16);
-        x.add_to(acc[v]);
-      }
-    }
-  };
-  for (int t0 = lo; t0 < hi; t0 += kMrgTile) {
-    const int tn = min(kMrgTile, hi - t0);
-    __syncthreads();                                 // the previous tile's records are no longer needed
+  const uint32_t rowb = (uint32_t)gn * 8 * (uint32_t)sizeof(T);
+  const int half = min(kMrgMaxHalf, ring_bytes / 2 / (int)rowb);   // rows in a half ring (at least three)
+  int h = 0, cur = -1, cur_dst = 0;                   // h: the half that is next
+  uint32_t par = 0;
+  bool first_cut = cut_head >= 0;                     // the running cluster is the one the range begins with
+  float cur_inv = 1.f;
+  for (int t0 = lo; t0 < stop; t0 += kMrgThreads) {
+    const int tn = min(kMrgThreads, stop - t0);
+    if (t0 > lo) __syncthreads();                     // the previous tile's records are no longer needed
     if (t < tn) {
-      const int g = t0 + t;
-      int4 rec;
-      int dst;
-      float inv = 1.f;
-      if (g < n_mem) {
-        if (center_only) rec = make_int4(im.cidx_ptr[g], g, g, 1);
-        else rec = __ldcg(im.members + g);
-        // in bounds whatever an aborted earlier stage left in the records
-        rec.x = min(max(rec.x, 0), im.N - 1) + im.vis_start;     // row of H
-        rec.y = min(max(rec.y, 0), C - 1);
-        rec.z = min(max(rec.z, 0), g);
-        rec.w = min(max(rec.w, g - rec.z + 1), n_mem - rec.z);
-        dst = im.vis_start + rec.y;
-        if (!center_only) inv = 1.0f / (float)rec.w;
-      } else {                                       // a text row: a cluster of its own, numbered after the real ones
-        const int tr = g - n_mem;
-        const int src = tr < im.vis_start ? tr : tr + im.N;
-        dst = tr < im.vis_start ? tr : tr + C;
-        rec = make_int4(src, C + tr, g, 1);
-        im.P_out[dst] = im.P[src];
-        im.size_out[dst] = 1;
-        if (im.logw_out) im.logw_out[dst] = 0.f;
+      const int p = t0 + t;
+      if (p < n_mem) {
+        const int4 r = checked(t0 == lo ? rec_t : fetch(p), p);
+        s_row[t] = im.vis_start + r.x;
+        s_cluster[t] = r.y;
+        s_dst[t] = im.vis_start + r.y;
+        s_inv[t] = 1.0f / (float)r.w;
+      } else {                                        // a text row: a cluster of its own, numbered after the real ones
+        const int tr = p - n_mem, src = tr < im.vis_start ? tr : tr + im.N, dst = tr < im.vis_start ? tr : tr + C;
+        s_row[t] = src;
+        s_cluster[t] = C + tr;
+        s_dst[t] = dst;
+        s_inv[t] = 1.f;
+        if (sl == 0) {
+          im.P_out[dst] = im.P[src];
+          im.size_out[dst] = 1;
+          if (im.logw_out) im.logw_out[dst] = 0.f;
+        }
       }
-      s_rec[t] = rec;
-      s_dst[t] = dst;
-      s_inv[t] = inv;
     }
     __syncthreads();
     TL_POINT(im, 15);
-    for (int j = 0; j < DEPTH; ++j) issue(j, tn);
+    // rows j .. of the tile into half hh (the rows shared out among the warps: issuing one takes a warp about 90 ns)
+    auto issue = [&](int j, int hh) {
+      const int n = min(half, tn - j);
+      if (n <= 0) return;
+      if (t == 0) mbar_arrive_expect_tx(&s_bar[hh], (uint32_t)n * rowb);
+      if ((t & 31) == 0)
+        for (int k = t >> 5; k < n; k += kMrgThreads / 32)
+          bulk_load(reinterpret_cast<uint8_t *>(ring) + (size_t)(hh * half + k) * rowb, H + (size_t)s_row[j + k] * im.ldH, rowb, &s_bar[hh]);
+    };
+    const int j0 = max(start - t0, 0);                // (a first tile may begin with items of the range before)
+    issue(j0, h);
+    issue(j0 + half, h ^ 1);
 #pragma unroll 1
-    for (int j = 0; j < tn; ++j) {
-      consume(j);
-      issue(j + DEPTH, tn);
+    for (int jh = j0; jh < tn; jh += half) {
+      if (!mbar_wait_warp(&s_bar[h], (par >> h) & 1)) s_abort = 1;
+      par ^= 1u << h;
+      const uint8_t *buf = reinterpret_cast<const uint8_t *>(ring) + (size_t)(h * half) * rowb + (size_t)t * 8 * sizeof(T);
+      const int je = min(jh + half, tn);
+#pragma unroll 1
+      for (int j = jh; j < je; ++j, buf += rowb) {
+        const int c = s_cluster[j];
+        if (c != cur) {                               // the next cluster begins (the same for all threads)
+          if (cur >= 0) {
+            if (first_cut) cut(cut_head, cut_head_n, cur_inv, cur_dst, 0);
+            else store_row(cur_inv, cur_dst);
+            first_cut = false;
+          }
+          zero();
+          cur = c; cur_dst = s_dst[j]; cur_inv = s_inv[j];
+        }
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+          if (mine[v]) {
+            Raw8<T> xr;
+            xr.from_ring(reinterpret_cast<const uint4 *>(buf + (size_t)v * nth * 8 * sizeof(T)));
+            xr.add_to(acc[v]);
+          }
+      }
+      __syncthreads();                                // this half has been read
+      issue(jh + 2 * half, h);
+      h ^= 1;
     }
   }
-  if (cur_c < 0) return;                             // an empty range
-  const bool goes_on = cur_off + cur_size > hi;
-  if (head_open) {                                   // one cluster covers the whole range
-    cut(acc, cur_c, cur_off, cur_size, cur_inv, cur_dst, goes_on ? 1 : 0);
-    return;
-  }
-  if (goes_on) cut(acc, cur_c, cur_off, cur_size, cur_inv, cur_dst, 1);
-  else store_row(acc, cur_inv, cur_dst);
+  if (first_cut) cut(cut_head, cut_head_n, cur_inv, cur_dst, 0);
+  else if (cut_tail >= 0) cut(cut_tail, cut_tail_n, cur_inv, cur_dst, 1);
+  else store_row(cur_inv, cur_dst);
+  if (t == 0 && s_abort) atomicMin(&im.counters_user[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
 }
 
 // ---- launchers -----------------------------------------------------------------------------------
@@ -635,30 +612,49 @@ int lists_kernels(int maxN, int B) {
   return (long long)((maxN + kListBlock - 1) / kListBlock) * B <= g_lists_resident ? 1 : 2;
 }
 
-int merge_ctas(int sm_count, int B) {
-  const int X = kMrgCtasPerSm * sm_count / B;
-  return X < 1 ? 1 : X;
+// items per range: at least sixteen (with few items as many ranges as that gives are in flight at once), no more than
+// eight rounds of CTAs over the GPU, and no more ranges than the scratch has room for
+static int merge_per(int n_items, int slices, int B, int sm_count) {
+  const long long most = 8LL * kMrgCtasPerSm * sm_count;
+  long long r = (n_items + 15) / 16;
+  if (r * slices * B > most) r = most / ((long long)slices * B);
+  if (r > kMrgRanges) r = kMrgRanges;
+  if (r < 1) r = 1;
+  return (int)((n_items + r - 1) / r);
 }
+size_t merge_scratch_rows() { return 2 * kMrgRanges; }
 
 template <typename T, typename O, int VPL>
-static cudaError_t launch_merge_v(const Batch &bt, dim3 grid, cudaStream_t st) {
-  constexpr int kSlotBytes = VPL * kMrgThreads * 8 * (int)sizeof(T);
-  constexpr int DEPTH = kMrgRingBytes / kSlotBytes;
-  return launch_k(k_merge<T, O, VPL, DEPTH>, grid, dim3(kMrgThreads), (size_t)DEPTH * kSlotBytes, st, true, bt);
+static cudaError_t launch_merge_v(const Batch &bt, int n_items, int slices, const ClusterCfg &cfg, cudaStream_t st) {
+  const int per = merge_per(n_items, slices, bt.B, cfg.sm_count), ranges = (n_items + per - 1) / per;
+  const long long per_sm = ((long long)ranges * slices * bt.B + cfg.sm_count - 1) / cfg.sm_count;
+  int ring = per_sm >= kMrgCtasPerSm ? kMrgRingBytes : (int)(kMrgCtasPerSm * kMrgRingBytes / per_sm);
+  if (ring > kMrgRingMost) ring = kMrgRingMost;
+  // One round of CTAs: the longest range counts, so only clusters that leave it within what the ring holds at once stay
+  // whole.  Several rounds: the bytes count.
+  const int row = ((bt.d / 8 + slices - 1) / slices) * 8 * (int)sizeof(T), most = 2 * kMrgMaxHalf, room = (ring / row < most ? ring / row : most) - per;
+  const int whole = per_sm > kMrgCtasPerSm ? per : room < 8 ? 8 : room;
+  return launch_k(k_merge<T, O, VPL>, dim3(ranges * slices, bt.B), dim3(kMrgThreads), (size_t)ring, st, true, bt, per, whole, slices, ring);
 }
 
 template <typename T, typename O>
 static cudaError_t launch_merge_t(const Batch &bt, const ClusterCfg &cfg, cudaStream_t st) {
-  dim3 grid(merge_ctas(cfg.sm_count, bt.B), bt.B);
-  if (bt.d <= kMrgThreads * 8) return launch_merge_v<T, O, 1>(bt, grid, st);
-  return launch_merge_v<T, O, kMergeMaxD / 8 / kMrgThreads>(bt, grid, st);
+  int n_items = 1;
+  for (int b = 0; b < bt.B; ++b) n_items = bt.img[b].n_total > n_items ? bt.img[b].n_total : n_items;
+  const int s1 = (bt.d / 8 + kMrgThreads - 1) / kMrgThreads, s2 = (bt.d / 8 + 2 * kMrgThreads - 1) / (2 * kMrgThreads);
+  // Two groups of columns per thread halve the instructions per byte, which counts when the GPU has several rounds of
+  // CTAs to do (46000 rows of 7 KB: 4 us of 75); with less, narrower slices spread the rows over more CTAs (7300 rows:
+  // 2 us of 20 the other way).  Rows of fp32 stay at one group: 4 KB per row and slice.
+  if constexpr (sizeof(T) == 2)
+    if ((long long)n_items * s1 * bt.B >= 64LL * kMrgCtasPerSm * cfg.sm_count) return launch_merge_v<T, O, 2>(bt, n_items, s2, cfg, st);
+  return launch_merge_v<T, O, 1>(bt, n_items, s1, cfg, st);
 }
 
-template <typename T, typename O, int VPL>
-static cudaError_t merge_attr() {
-  constexpr int kSlotBytes = VPL * kMrgThreads * 8 * (int)sizeof(T);
-  constexpr int DEPTH = kMrgRingBytes / kSlotBytes;
-  return cudaFuncSetAttribute(k_merge<T, O, VPL, DEPTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEPTH * kSlotBytes);
+template <typename T, typename O> static cudaError_t merge_attr() {
+  cudaError_t e = cudaFuncSetAttribute(k_merge<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMrgRingMost);
+  if constexpr (sizeof(T) == 2)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_merge<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMrgRingMost);
+  return e;
 }
 
 cudaError_t merge_configure() {
@@ -677,15 +673,10 @@ cudaError_t merge_configure() {
   if (e != cudaSuccess) return e;
   m = per_sm < m ? per_sm : m;
   g_lists_resident = m * sms;
-  constexpr int V2 = kMergeMaxD / 8 / kMrgThreads;
-  e = merge_attr<__nv_bfloat16, __nv_bfloat16, 1>();
-  if (e == cudaSuccess) e = merge_attr<__nv_bfloat16, __nv_bfloat16, V2>();
-  if (e == cudaSuccess) e = merge_attr<__nv_bfloat16, float, 1>();
-  if (e == cudaSuccess) e = merge_attr<__nv_bfloat16, float, V2>();
-  if (e == cudaSuccess) e = merge_attr<float, __nv_bfloat16, 1>();
-  if (e == cudaSuccess) e = merge_attr<float, __nv_bfloat16, V2>();
-  if (e == cudaSuccess) e = merge_attr<float, float, 1>();
-  if (e == cudaSuccess) e = merge_attr<float, float, V2>();
+  e = merge_attr<__nv_bfloat16, __nv_bfloat16>();
+  if (e == cudaSuccess) e = merge_attr<__nv_bfloat16, float>();
+  if (e == cudaSuccess) e = merge_attr<float, __nv_bfloat16>();
+  if (e == cudaSuccess) e = merge_attr<float, float>();
   return e;
 }
 

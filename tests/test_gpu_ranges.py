@@ -1,0 +1,92 @@
+"""Sizes at which a kernel's split of the work has its edges: ranges of the merge, units of the token pass, images of
+the one-cluster step and of the kernels that take over from it."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2504_08966_b200 import workloads
+from tests.helpers import compare_image, fragile_report, gpu_reduce, oracle_image
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,C,T,d,dtype", [
+    (1, 1, 0, 3584, torch.bfloat16), (17, 1, 0, 3584, torch.bfloat16), (31, 31, 2, 520, torch.bfloat16),
+    (300, 1, 5, 896, torch.float32),          # one cluster over all ranges
+    (1184, 9, 3, 1032, torch.float32),        # a last slice of one vector
+    (2909, 37, 64, 3584, torch.bfloat16), (4737, 2, 0, 8192, torch.bfloat16),
+    (7301, 700, 64, 8, torch.bfloat16),
+    (20011, 41, 7, 3584, torch.bfloat16),     # two vectors per thread
+])
+def test_merge_ranges(N, C, T, d, dtype):
+    """Clusters that end inside a range of members, cross one boundary, or cover many; some tokens in no cluster."""
+    from paper_2504_08966_b200 import binding as pb
+    g = torch.Generator(device="cuda").manual_seed(N)
+    H = torch.randn(N + T, d, device="cuda", generator=g).to(dtype)
+    label = torch.randint(-1 if N > 40 else 0, C, (N,), device="cuda", generator=g, dtype=torch.int32)
+    label[label == C // 2] = 0                # one large cluster, one without members but its centre
+    cidx = torch.arange(C, dtype=torch.int32, device="cuda")
+    label[:C] = cidx
+    n = N + T
+    z = lambda m, dt: torch.zeros(m, dtype=dt, device="cuda")   # noqa: E731
+    K = z((N, 64), dtype)
+    im = pb.DeviceImage(H, K, K, K, torch.arange(n, dtype=torch.int32, device="cuda"), T // 2, N, z((n, d), torch.float32), z(n, torch.int32),
+                        z(n, torch.int32), z(N, torch.int32), z(N, torch.float32), z(N, torch.uint8), z(pb.N_COUNTERS, torch.int32), z(n, torch.float32))
+    ctx = pb.Context(d, 1, 1, 64, dtype, torch.float32)
+    for _ in range(2):                        # the tickets of the first call must not be left over
+        ctx.pact_merge(im, label, cidx, torch.tensor([C], dtype=torch.int32, device="cuda"), pb.make_params())
+    torch.cuda.synchronize()
+    v0, lab = T // 2, label.long()
+    keep = lab >= 0
+    size = torch.bincount(lab[keep], minlength=C)
+    want = torch.zeros(C, d, dtype=torch.float64, device="cuda").index_add_(0, lab[keep], H[v0:v0 + N][keep].double()) / size[:, None]
+    assert int(im.counters[0]) == C + T and int(im.counters[pb.CNT["status"]]) == 0
+    assert torch.equal(im.size_out[v0:v0 + C].long(), size)
+    err = (im.H_out[v0:v0 + C].double() - want).abs().amax(1) / want.abs().amax(1)
+    assert float(err.max()) < 2e-5
+    text = torch.cat([im.H_out[:v0], im.H_out[v0 + C:C + T]])
+    assert torch.equal(text, torch.cat([H[:v0], H[v0 + N:]]).float())
+
+
+def _workload(N, n_qh, n_kvh, d_h, d, dtype, seed, scale=1.0, rope=False, T=3):
+    rng = np.random.default_rng(seed)
+    dk = n_kvh * d_h
+    t = lambda x: torch.from_numpy(np.ascontiguousarray(x)).to(torch.float32).to(dtype)   # noqa: E731
+    blobs = rng.standard_normal((max(1, N // 12), dk))
+    z = blobs[rng.integers(0, blobs.shape[0], N)] + 0.25 * rng.standard_normal((N, dk))
+    R = rng.standard_normal((dk, n_qh * d_h)) / np.sqrt(dk)
+    K = t(scale * z)
+    img = workloads.Image(H=t(rng.standard_normal((N + T, d)) * np.exp(0.5 * rng.standard_normal((N + T, 1)))), K=K, Q=t(z @ R), P=torch.arange(N + T, dtype=torch.int32),
+                          n_total=N + T, vis_start=1, N=N, K_clu=t(z + 0.05 * rng.standard_normal((N, dk))) if rope else None)
+    return workloads.Workload("edge", [img], d, n_qh, n_kvh, d_h, dtype, 0.5, 0.3)
+
+
+def _check(wl, out_dtype):
+    outs, _ = gpu_reduce(wl, out_dtype)
+    for img, g in zip(wl.images, outs):
+        o = oracle_image(wl, img)
+        bad = compare_image(o, g, img, out_dtype == torch.bfloat16)
+        assert not bad, f"{bad}; fragile: {fragile_report(o, wl.d_c, wl.alpha)}"
+
+
+@pytest.mark.parametrize("N,n_qh,n_kvh,d_h,d,dtype,scale,rope", [
+    (1, 1, 1, 8, 8, torch.bfloat16, 1.0, False), (7, 2, 2, 64, 896, torch.float32, 1.0, False),
+    (9, 3, 1, 40, 72, torch.bfloat16, 1.0, True),                 # three heads of one key head, five vectors per head
+    (1185, 5, 1, 96, 136, torch.bfloat16, 1.0, False),            # units of nine tokens; heads in blocks of four and one
+    (2369, 14, 2, 64, 896, torch.bfloat16, 4.0, False),           # seventeen tokens; four and three heads; steep softmax
+    (4737, 28, 4, 128, 512, torch.bfloat16, 1.0, True),
+    (1500, 4, 4, 36, 4104, torch.float32, 1.0, False),            # rows in three copies
+    (4800, 2, 2, 12, 264, torch.float32, 1.0, True),
+    (1200, 40, 40, 64, 1024, torch.bfloat16, 1.0, False),         # more heads than one block of the scoring kernel
+])
+def test_token_units(N, n_qh, n_kvh, d_h, d, dtype, scale, rope):
+    _check(_workload(N, n_qh, n_kvh, d_h, d, dtype, N, scale, rope), torch.float32)
+
+
+def test_no_norm_and_norm_only():
+    """Both forms of the score without one of its factors, over several units of the token pass."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = _workload(5000, 4, 2, 64, 256, torch.bfloat16, 5)
+    for flags, kw in ((pb.FLAG_NO_NORM, {"use_norm": False}), (pb.FLAG_NORM_ONLY, {"use_query": False})):
+        outs, _ = gpu_reduce(wl, torch.float32, params=pb.make_params(lam=0.5, d_c=0.3, flags=flags))
+        assert not compare_image(oracle_image(wl, wl.images[0], **kw), outs[0], wl.images[0], False)
