@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpact.so")
 LIB_TIMELINE = os.path.join(HERE, "libpact_timeline.so")   # instrumented build (per-CTA timestamps), see timeline.py
-SOURCES = ["api.cu", "euti.cu", "cluster.cu", "gram_umma.cu", "merge.cu", "prune_static.cu"]
+SOURCES = ["api.cu", "euti.cu", "cluster.cu", "gram_umma.cu", "merge.cu", "small.cu", "prune_static.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

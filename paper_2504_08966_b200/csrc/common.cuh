@@ -15,6 +15,7 @@ constexpr unsigned long long kBestInit = 0xFFFFFFFFFFFFFFFFull;
 constexpr int kCntSpread = 24;           // slot of cnt[]: largest key distance of a layer, as float bits
 constexpr int kSpinLimit = 1 << 20;      // default number of polls a bounded device wait makes before it gives up
 constexpr int kListBlock = 128;          // tokens per block of the member lists (128 measured 0.8 us faster per step than 256)
+constexpr int kSmallMaxN = 1024;         // images of at most this many tokens take the one-kernel step (small.cu)
 constexpr int kMaxTokens = 1 << 18;      // most visual tokens per image
 constexpr int kCntInts = 64;             // counters at the head of an image's workspace, cleared by the first kernel of a call
 constexpr int kMaxColGroups = 1024;      // most groups of eight 16-byte vectors in a row of Q

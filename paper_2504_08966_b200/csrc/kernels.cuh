@@ -116,6 +116,11 @@ bool umma_pairs_for_assign(int maxN, int B, const ClusterCfg &cfg);
 cudaError_t launch_members(const Batch &bt, int maxN, cudaStream_t st);
 cudaError_t launch_spread_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, cudaStream_t st);
 
+// small.cu: scores to member lists in one kernel, a cluster per image
+cudaError_t small_configure();
+bool small_fits(const Batch &bt, int maxN, bool umma);
+cudaError_t launch_small(const Batch &bt, bool in_bf16, bool umma, int rpp, int sweep_limit, cudaStream_t st);
+
 // merge.cu
 // member records in cluster order from label[] (from_best: labels are first formed from the nearest-centre
 // pass, all tokens); csize, cticket and cnt_cb must be zero.  spin_limit bounds the wait of its barrier.

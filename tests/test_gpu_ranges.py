@@ -83,6 +83,21 @@ def test_token_units(N, n_qh, n_kvh, d_h, d, dtype, scale, rope):
     _check(_workload(N, n_qh, n_kvh, d_h, d, dtype, N, scale, rope), torch.float32)
 
 
+@pytest.mark.parametrize("dtype,n_qh,n_kvh,d_h", [(torch.bfloat16, 4, 2, 64), (torch.bfloat16, 3, 3, 24), (torch.float32, 2, 2, 20)])
+@pytest.mark.parametrize("N", [1, 2, 15, 17, 127, 129, 511, 513, 1023, 1024, 1025])
+def test_small_images(N, dtype, n_qh, n_kvh, d_h):
+    """Around the tiles and the limits of the one-cluster step; widths that the tensor cores take and others."""
+    _check(_workload(N, n_qh, n_kvh, d_h, 256, dtype, 7 * N + 1), torch.float32)
+
+
+@pytest.mark.parametrize("B", [2, 9, 16])
+def test_small_batches(B):
+    """As many images as clusters fit on the GPU at once, and more."""
+    wls = [_workload(max(1, 300 - 19 * b), 4, 2, 64, 256, torch.bfloat16, 900 + b) for b in range(B)]
+    wl = workloads.Workload("edge", [w.images[0] for w in wls], 256, 4, 2, 64, torch.bfloat16, 0.5, 0.3)
+    _check(wl, torch.bfloat16)
+
+
 def test_no_norm_and_norm_only():
     """Both forms of the score without one of its factors, over several units of the token pass."""
     from paper_2504_08966_b200 import binding as pb
