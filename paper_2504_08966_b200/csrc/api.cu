@@ -389,7 +389,7 @@ pact_status pact_dbdpc(pact_ctx *ctx, const void *K, int64_t ldK, int N, const i
   if (ctx->umma) CK(launch_assign_umma(bt, N, true, ctx->ccfg, st));
   else CK(launch_assign(bt, N, bf, ROWS_KEPT_LIST, ctx->ccfg, st));
   CK(launch_label(bt, N, bf, ROWS_KEPT_LIST, st));
-  ctx->launches += 5;
+  ctx->launches += 6;
   CK(cudaGetLastError());
   if (counters)
     CK(cudaMemcpyAsync(counters, m.cnt, PACT_N_COUNTERS * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
@@ -568,7 +568,7 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     else CK(launch_lists(bt, cmaxN, bf, true, ctx->spin_limit, st));
     CK(mark());
     CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->ccfg, st));  CK(mark());
-    ctx->launches += euti_kernels(0) + 4 + (fused_labels ? 1 : lists_kernels(cmaxN, nb));
+    ctx->launches += euti_kernels(0) + 5 + (fused_labels ? 1 : lists_kernels(cmaxN, nb));
     CK(cudaGetLastError());
   }
   return PACT_OK;

@@ -4,10 +4,9 @@
 //
 // This file holds the double-precision tile kernels (any element type and key width); the tcgen05 tile
 // kernels for bf16 keys live in gram_umma.cu and share the epilogue arithmetic of common.cuh.
-#include <cooperative_groups.h>
-
 #include "f64_tiles.cuh"
 #include "kernels.cuh"
+#include "tma.cuh"
 
 namespace pact {
 
@@ -45,7 +44,7 @@ __global__ void __launch_bounds__(256) k_keynorm_gather(const __grid_constant__ 
   const int i = im.kept_idx[r];
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  const rn_t rn = (rn_t)(inv_norm(ss));
+  const rn_t rn = (rn_t)inv_norm(ss);
   if (lane == 0) {
     rn_tok<D>(im)[i] = rn;
     rn_kept<D>(im)[r] = rn;
@@ -76,13 +75,13 @@ __global__ void __launch_bounds__(256) k_center_key_gather(const __grid_constant
   if (c < (all_rows ? im.N : *im.m_ptr)) {   // inverse norm of row c, or of the c-th pruned row
     const int i = all_rows ? c : im.pruned_idx[c];
     const double ss = row_sumsq<T>(reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc, bt.d_k, lane);
-    if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(inv_norm(ss));
+    if (lane == 0) rn_tok<D>(im)[i] = (rn_t)inv_norm(ss);
   }
   if (c >= *im.C_ptr) return;
   const int i = im.cidx_ptr[c];
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  if (lane == 0) rn_cen<D>(im)[c] = (rn_t)(inv_norm(ss));
+  if (lane == 0) rn_cen<D>(im)[c] = (rn_t)inv_norm(ss);
   T *dst = reinterpret_cast<T *>(im.Kcen) + (size_t)c * bt.d_k;
   for (int v = lane; v * V < bt.d_k; v += 32)
     reinterpret_cast<uint4 *>(dst)[v] = reinterpret_cast<const uint4 *>(row)[v];
@@ -139,7 +138,7 @@ __global__ void __launch_bounds__(256) k_key_rnorm(const __grid_constant__ Batch
   if (i >= im.N) return;
   const T *row = reinterpret_cast<const T *>(im.Kc) + (size_t)i * im.ldKc;
   const double ss = row_sumsq<T>(row, bt.d_k, lane);
-  if (lane == 0) rn_tok<D>(im)[i] = (rn_t)(inv_norm(ss));
+  if (lane == 0) rn_tok<D>(im)[i] = (rn_t)inv_norm(ss);
 }
 
 template <typename T>
@@ -208,247 +207,240 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 // schedule that only takes final decisions reproduces it (the argument of Appendix D.2).  A row becomes
 //   removed  once an earlier neighbour is a centre,
 //   a centre once every earlier neighbour is removed.
-// Both facts are monotone bits, so rows are resolved asynchronously from two bit masks in global memory.
-// The masks are a few hundred bytes that every row depends on: thousands of warps polling them directly
-// queue up at the same few L2 lines.  Instead a CTA copies both masks to shared memory once per sweep,
-// its warps decide what they can from the copy and publish decisions with atomics; a decision reaches the
-// other CTAs with their next copy.
+// Both facts are monotone bits of two masks in global memory, so rows are resolved asynchronously and a decision may reach
+// others late.  A new centre removes its neighbours itself: it sets its adjacency words in the mask of removed rows (an
+// earlier neighbour is in it already).  A row keeps one earlier neighbour that is not removed as its witness and looks at
+// its adjacency words again only when the witness has been removed; without another one it is a centre.  (A row whose
+// witness is a centre waits for its own bit.)  Most rows are looked at once or twice; with every row's earlier neighbours
+// filtered first and every open row tested against both masks in every sweep, 16 images of 1458 survivors took 23 us for
+// the same decisions.
 //
-// One cooperative kernel (every CTA resident), one CTA of 1024 threads per SM, three parts:
-//  1. "earlier" is decided from the integer densities themselves (no rank array): the densities of an
-//     image are staged in shared memory, each warp masks the adjacency words of its rows down to the
-//     earlier neighbours (the first row's words stay in registers, further rows are written back);
-//  2. sweeps (bounded) until no row of the CTA is pending;
-//  3. after a grid-wide barrier: cluster ids (number of centres with a lower index), centre list,
-//     centre keys and inverse norms.
-constexpr int kAdjRegs = 8;      // adjacency words per lane kept in registers: rows of up to 8192 survivors
+// k_centers: one CTA of 1024 threads per SM, the CTAs shared out evenly among the images (the last image also takes the
+// remainder).  A CTA has a block of rows, their adjacency words and all densities of its image in shared memory (what does
+// not fit stays in the L2); lane k of warp w keeps the state of row w + 32 k.  In a sweep the CTA copies the mask of removed
+// rows to shared memory once (thousands of warps polling the same few L2 lines queue up there), and its warps decide what
+// they can from the copy.  Bound by latency, a trip to the L2 per sweep: 7 us for one image of 3645 survivors, 10 us for 16
+// of 1458, 15 us for 4 of 4916.
+// CTAs wait for one another's decisions but need not be resident together: after kCenSweeps sweeps a CTA leaves its open
+// rows to k_center_keys, where every CTA resolves what is open by itself.  (As a cooperative launch the kernel could not
+// begin beside the one before, which cost a call on a stream 4 us.  One cluster of 16 CTAs per image, with masks in each
+// other's shared memory, was no faster with 16 images and 18 us slower with one: 16 SMs are too few to take in the rows.)
+//
+// k_center_keys: cluster ids (number of centres with a lower index), centre list, centre keys and inverse norms.
 constexpr int kCenThreads = 1024;
 constexpr int kCenWarps = kCenThreads / 32;
+constexpr int kCenSweeps = 512;                          // sweeps of k_centers (about a microsecond each)
 
-template <typename T>
-__global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constant__ Batch bt, int keys_cap, int mask_cap,
-                                                            int spin_limit) {
-  using D = typename DistOf<T>::type;
-  constexpr int V = Vec<T>::N;
-  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+// One row against the removed rows, by a warp: an earlier neighbour that is not removed, or -1.
+__device__ __forceinline__ int open_earlier(const uint32_t *row, const uint32_t *removed, const unsigned long long *keys, int r, int nw, int lane) {
+  const unsigned long long mine = keys[r];
+  for (int base = 0; base < nw; base += 32) {
+    const int wd = base + lane;
+    uint32_t bits = wd < nw ? row[wd] & ~removed[wd] : 0u;
+    if (wd == (r >> 5)) bits &= ~(1u << (r & 31));
+    while (__any_sync(0xffffffffu, bits != 0u)) {        // a bit per lane at a time: nearly always the first will do
+      int found = -1;
+      if (bits) {
+        const int j = wd * 32 + __ffs(bits) - 1;
+        bits &= bits - 1;
+        const unsigned long long o = keys[j];
+        if (o > mine || (o == mine && j < r)) found = j;
+      }
+      const unsigned hits = __ballot_sync(0xffffffffu, found >= 0);
+      if (hits) return __shfl_sync(0xffffffffu, found, __ffs(hits) - 1);
+    }
+  }
+  return -1;
+}
+
+__global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constant__ Batch bt, int mask_cap, int keys_cap, int adj_bytes,
+                                                            int sweep_limit) {
   TL_SCOPE(bt.img[0], 5);
-  extern __shared__ unsigned long long skeys[];          // [keys_cap] densities of this CTA's image
-  uint32_t *cm_s = reinterpret_cast<uint32_t *>(skeys + keys_cap);   // [mask_cap] copy of the centre mask
-  uint32_t *rm_s = cm_s + mask_cap;                      // [mask_cap] copy of the removed mask
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // The CTAs are shared out evenly among the images (the last image also takes the remainder); a CTA
-  // works on one image throughout, so the images of a batch are resolved side by side.
+  extern __shared__ __align__(16) uint8_t cen_smem[];
+  uint32_t *rm = reinterpret_cast<uint32_t *>(cen_smem);              // [mask_cap] copy of the removed rows
+  unsigned long long *skeys = reinterpret_cast<unsigned long long *>(rm + mask_cap);   // [keys_cap] densities
+  uint4 *sadj = reinterpret_cast<uint4 *>(skeys + keys_cap);          // adjacency words of the first rows of the CTA
+  __shared__ uint64_t s_bar;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const int per = max(1, (int)gridDim.x / bt.B);
   const int b = min((int)blockIdx.x / per, bt.B - 1);
-  const int ncta = b == bt.B - 1 ? (int)gridDim.x - per * (bt.B - 1) : per;
-  const int nwarps = ncta * kCenWarps;
-  const int gw = ((int)blockIdx.x - b * per) * kCenWarps + wid;
+  const int ncta = b == bt.B - 1 ? (int)gridDim.x - per * (bt.B - 1) : per, rank = (int)blockIdx.x - b * per;
   const ImgDesc &im = bt.img[b];
+  if (t == 0) {
+    mbar_init(&s_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
-  const int q = *im.q_ptr, nw = (q + 31) >> 5;
-
-  // part 1: keep only the neighbours that come earlier in density order
-  uint32_t cached[kAdjRegs];
-  int cached_item = -1;
-  {
-    const bool in_smem = q <= keys_cap;
-    if (in_smem)
-      for (int r = threadIdx.x; r < q; r += kCenThreads) skeys[r] = im.rho_fix[r];
-    __syncthreads();
-    const unsigned long long *keys = in_smem ? skeys : im.rho_fix;
-    for (int r = gw; r < q; r += nwarps) {
-      const unsigned long long mine = keys[r];
-      uint32_t *row = im.adj + (size_t)r * im.Wp;
-      const bool keep_regs = cached_item < 0 && nw <= 32 * kAdjRegs;
-      uint32_t w_in[kAdjRegs];
-#pragma unroll
-      for (int u = 0; u < kAdjRegs; ++u) w_in[u] = (lane + 32 * u < nw) ? row[lane + 32 * u] : 0u;
-#pragma unroll
-      for (int u = 0; u < kAdjRegs; ++u) {
-        const int wd = lane + 32 * u;
-        uint32_t bits = w_in[u], out = 0u;
-        while (bits) {
-          const int bpos = __ffs(bits) - 1;
-          bits &= bits - 1;
-          const int j = wd * 32 + bpos;
-          const unsigned long long o = keys[j];
-          if (j != r && (o > mine || (o == mine && j < r))) out |= 1u << bpos;
-        }
-        if (wd < nw && !keep_regs) row[wd] = out;
-        if (keep_regs) cached[u] = out;
-      }
-      for (int wd = lane + 32 * kAdjRegs; wd < nw; wd += 32) {     // rows longer than the register part
-        uint32_t bits = row[wd], out = 0u;
-        while (bits) {
-          const int bpos = __ffs(bits) - 1;
-          bits &= bits - 1;
-          const int j = wd * 32 + bpos;
-          const unsigned long long o = keys[j];
-          if (j != r && (o > mine || (o == mine && j < r))) out |= 1u << bpos;
-        }
-        row[wd] = out;
-      }
-      if (keep_regs) cached_item = r;
-      if (lane == 0) {
-        const float rf = (float)((double)mine * (1.0 / (double)(1u << kRhoShift)));
-        im.rho[r] = rf;
-        if (im.rho_user) im.rho_user[r] = rf;
-      }
-    }
+  const int q = *im.q_ptr, nw = (q + 31) >> 5, nv = (nw + 3) >> 2;
+  const int rows = (q + ncta - 1) / ncta, r0 = min(q, rank * rows), n = min(q, r0 + rows) - r0;
+  if (n <= 0) return;
+  const bool in_smem = q <= keys_cap;
+  if (in_smem && t == 0) {
+    const uint32_t bytes = ((uint32_t)q * 8 + 15) & ~15u;
+    mbar_arrive_expect_tx(&s_bar, bytes);
+    bulk_load(skeys, im.rho_fix, bytes, &s_bar);
   }
+  const unsigned long long *keys = in_smem ? skeys : im.rho_fix;
+  const int nsm = min(n, adj_bytes / (nv * 16));
+  for (int l = wid; l < nsm; l += 4 * kCenWarps)
+    for (int v = lane; v < nv; v += 32) {
+      uint4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (l + u * kCenWarps < nsm) x[u] = __ldcg(reinterpret_cast<const uint4 *>(im.adj + (size_t)(r0 + l + u * kCenWarps) * im.Wp) + v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (l + u * kCenWarps < nsm) sadj[(size_t)(l + u * kCenWarps) * nv + v] = x[u];
+    }
+  for (int wd = t; wd < nw; wd += kCenThreads) rm[wd] = 0u;
+  if (in_smem && !mbar_wait_warp(&s_bar, 0) && lane == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+  __syncthreads();
   TL_POINT(bt.img[0], 10);
 
-  // part 2: resolve
-  const bool masks_in_smem = nw <= mask_cap;
+  int wit = -1;                                          // witness of row wid + 32 lane
+  bool done = false;                                     // that row is a centre
   int sweeps = 0;
-  bool cached_done = false;
   for (;;) {
-    if (masks_in_smem) {
-      __syncthreads();                                  // the previous sweep has read the copy
-      for (int wd = threadIdx.x; wd < nw; wd += kCenThreads) {
-        cm_s[wd] = ld_relaxed_u32(&im.cmask[wd]);
-        rm_s[wd] = ld_relaxed_u32(&im.rmask[wd]);
-      }
-      __syncthreads();
-    }
-    const uint32_t *cmL = masks_in_smem ? cm_s : im.cmask, *rmL = masks_in_smem ? rm_s : im.rmask;
-    auto ldm = [&](const uint32_t *p) { return masks_in_smem ? *p : ld_relaxed_u32(p); };
     int pending = 0;
     ++sweeps;
-    for (int r = gw; r < q; r += nwarps) {
-      const uint32_t mybit = 1u << (r & 31);
-      bool hit_center = false, alive = false;
-      if (r == cached_item) {                     // the masked adjacency of this row is in registers
-        if (cached_done) continue;
-#pragma unroll
-        for (int u = 0; u < kAdjRegs; ++u) {
-          if (cached[u] != 0u) {
-            hit_center |= (cached[u] & ldm(&cmL[lane + 32 * u])) != 0u;
-            alive |= (cached[u] & ~ldm(&rmL[lane + 32 * u])) != 0u;
-          }
+    for (int m = 0; m * kCenThreads < n; ++m) {
+      const int l = wid + 32 * (m * 32 + lane), r = r0 + l;
+      bool open = l < n && !(m == 0 && done) && !((rm[r >> 5] >> (r & 31)) & 1u);
+      if (m > 0 && open) open = !((ld_relaxed_u32(&im.cmask[r >> 5]) >> (r & 31)) & 1u);   // (blocks of more than 1024 rows)
+      const bool look = open && (m > 0 || wit < 0 || ((rm[wit >> 5] >> (wit & 31)) & 1u));
+      pending |= open && !look;
+      unsigned todo = __ballot_sync(0xffffffffu, look);
+      while (todo) {
+        const int k = __ffs(todo) - 1, ll = wid + 32 * (m * 32 + k), rr = r0 + ll;
+        todo &= todo - 1;
+        const uint32_t *row = ll < nsm ? reinterpret_cast<const uint32_t *>(sadj + (size_t)ll * nv) : im.adj + (size_t)rr * im.Wp;
+        const int f = open_earlier(row, rm, keys, rr, nw, lane);
+        if (f >= 0) {
+          pending = 1;
+          if (m == 0 && lane == k) wit = f;
+          continue;
         }
-      } else {
-        if ((ldm(&cmL[r >> 5]) | ldm(&rmL[r >> 5])) & mybit) continue;   // decided
-        const uint32_t *row = im.adj + (size_t)r * im.Wp;
         for (int wd = lane; wd < nw; wd += 32) {
-          const uint32_t e = row[wd];
-          if (e) {
-            hit_center |= (e & ldm(&cmL[wd])) != 0u;
-            alive |= (e & ~ldm(&rmL[wd])) != 0u;
+          uint32_t e = row[wd];
+          if (wd == (rr >> 5)) {
+            e &= ~(1u << (rr & 31));
+            atomicOr(&im.cmask[wd], 1u << (rr & 31));
           }
+          if (e) atomicOr(&im.rmask[wd], e);
         }
-      }
-      hit_center = __any_sync(0xffffffffu, hit_center);
-      alive = __any_sync(0xffffffffu, alive);
-      if (hit_center) {
-        if (lane == 0) atomicOr(&im.rmask[r >> 5], mybit);
-        if (r == cached_item) cached_done = true;
-      } else if (!alive) {
-        if (lane == 0) atomicOr(&im.cmask[r >> 5], mybit);
-        if (r == cached_item) cached_done = true;
-      } else {
-        pending = 1;
+        if (m == 0 && lane == k) done = true;
       }
     }
-    if (!__syncthreads_or(pending)) break;              // no row of this CTA is pending
-    if (sweeps >= spin_limit) {
-      if (threadIdx.x == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+    if (!__syncthreads_or(pending)) break;               // no row of this CTA is open
+    if (sweeps >= sweep_limit || sweeps >= kCenSweeps) {
+      if (t == 0 && sweeps >= sweep_limit) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
       break;
     }
-  }
-  if (threadIdx.x == 0 && gw < q) atomicMax(&im.cnt[PACT_CNT_SWEEPS], sweeps);
-
-  // part 3: every decision is final once all CTAs are here
-  TL_POINT(bt.img[0], 11);
-  __threadfence();
-  grid.sync();
-  TL_POINT(bt.img[0], 12);
-  // Cluster id of a centre = number of centres with a lower index.  The centre mask of an image is read
-  // once per CTA into shared memory with its running bit counts; images too large for the staging buffer
-  // take the words from global memory.
-  __shared__ int wsum3[kCenWarps];
-  __shared__ int s_carry3;
-  {
-    const bool staged = q <= keys_cap;              // nw words and nw counts fit where the densities were
-    uint32_t *cm = reinterpret_cast<uint32_t *>(skeys);
-    int *pref = reinterpret_cast<int *>(skeys) + nw;
+    for (int wd = t; wd < nw; wd += kCenThreads) rm[wd] = ld_relaxed_u32(&im.rmask[wd]);
     __syncthreads();
-    if (staged) {
-      if (threadIdx.x == 0) s_carry3 = 0;
-      __syncthreads();
-      for (int base = 0; base < nw; base += kCenThreads) {
-        const int wd = base + threadIdx.x;
-        const uint32_t m = wd < nw ? __ldcg(&im.cmask[wd]) : 0u;
-        const int pc = __popc(m);
-        int x = pc;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum3[wid] = x;
-        __syncthreads();
-        int off = s_carry3;
-        for (int k = 0; k < wid; ++k) off += wsum3[k];
-        if (wd < nw) { cm[wd] = m; pref[wd] = off + x - pc; }
-        __syncthreads();
-        if (threadIdx.x == kCenThreads - 1) s_carry3 = off + x;
-        __syncthreads();
-      }
-    }
-    for (int r = gw; r < q; r += nwarps) {
-      int c, all;
-      bool is_center;
-      if (staged) {
-        const uint32_t m = cm[r >> 5];
-        is_center = ((m >> (r & 31)) & 1u) != 0u;
-        c = pref[r >> 5] + __popc(m & ((1u << (r & 31)) - 1u));
-        all = s_carry3;
-      } else {
-        int below = 0;
-        all = 0;
-        uint32_t myword = 0u;
+  }
+  TL_POINT(bt.img[0], 11);
+  if (t == 0) atomicMax(&im.cnt[PACT_CNT_SWEEPS], sweeps);
+}
+
+// grid (X, B), 256 threads, dynamic smem: three words per 32 survivors.
+constexpr int kCenKeyThreads = 256;
+
+template <typename T>
+__global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_constant__ Batch bt, int mask_cap) {
+  using D = typename DistOf<T>::type;
+  constexpr int V = Vec<T>::N, kWarps = kCenKeyThreads / 32;
+  const ImgDesc &im = bt.img[blockIdx.y];
+  extern __shared__ __align__(16) uint8_t cen_smem[];
+  uint32_t *cm = reinterpret_cast<uint32_t *>(cen_smem), *rm = cm + mask_cap;   // [mask_cap] centres, removed rows
+  int *pref = reinterpret_cast<int *>(rm + mask_cap);                 // [mask_cap] centres before the word
+  __shared__ int wsum[kWarps], s_carry;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  if (t == 0) s_carry = 0;
+  pdl_wait();
+  pdl_trigger();
+  TL_POINT(bt.img[0], 12);
+  const int q = *im.q_ptr, nw = (q + 31) >> 5, gw = blockIdx.x * kWarps + wid, nwarps = gridDim.x * kWarps;
+  int open = 0;
+  for (int wd = t; wd < nw; wd += kCenKeyThreads) {
+    const uint32_t c = __ldcg(&im.cmask[wd]), r = __ldcg(&im.rmask[wd]);
+    cm[wd] = c;
+    rm[wd] = r;
+    open |= (c | r) != (wd * 32 + 32 <= q ? 0xffffffffu : (1u << (q & 31)) - 1u);
+  }
+  if (__syncthreads_or(open)) {
+    // Rows that k_centers left: every CTA resolves them, to the same end (the set is unique), against its own copies;
+    // the first CTA also writes the centres for later kernels.
+    do {
+      open = 0;
+      for (int r = wid; r < q; r += kWarps) {
+        const uint32_t bit = 1u << (r & 31);
+        const volatile uint32_t *vc = cm + (r >> 5), *vr = rm + (r >> 5);
+        if ((*vc | *vr) & bit) continue;
+        const uint32_t *row = im.adj + (size_t)r * im.Wp;
+        if (open_earlier(row, rm, im.rho_fix, r, nw, lane) >= 0) { open = 1; continue; }
         for (int wd = lane; wd < nw; wd += 32) {
-          const uint32_t m = __ldcg(&im.cmask[wd]);
-          const int pc = __popc(m);
-          all += pc;
-          if (wd < (r >> 5)) below += pc;
-          else if (wd == (r >> 5)) { below += __popc(m & ((1u << (r & 31)) - 1u)); myword = m; }
+          uint32_t e = row[wd];
+          if (wd == (r >> 5)) {
+            e &= ~bit;
+            atomicOr(&cm[wd], bit);
+            if (blockIdx.x == 0) atomicOr(&im.cmask[wd], bit);
+          }
+          if (e) atomicOr(&rm[wd], e);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          below += __shfl_xor_sync(0xffffffffu, below, o);
-          all += __shfl_xor_sync(0xffffffffu, all, o);
-          myword |= __shfl_xor_sync(0xffffffffu, myword, o);
-        }
-        c = below;
-        is_center = ((myword >> (r & 31)) & 1u) != 0u;
       }
-      if (r == 0 && lane == 0) {
-        im.cnt[PACT_CNT_C] = all;
-        if (im.C_user) *im.C_user = all;
-      }
-      if (!is_center) continue;
-      const T *src = reinterpret_cast<const T *>(im.Kp) + (size_t)r * bt.d_k;
-      const int nv = bt.d_k / V;
-      uint4 buf[4];
+    } while (__syncthreads_or(open));                    // ends: the earliest open row is decided in every pass
+  }
+  for (int base = 0; base < nw; base += kCenKeyThreads) {
+    const int wd = base + t, pc = wd < nw ? __popc(cm[wd]) : 0;
+    int x = pc;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (lane + 32 * u < nv) buf[u] = __ldcg(reinterpret_cast<const uint4 *>(src) + lane + 32 * u);
-      if (lane == 0) {
-        const int tok = im.kept_idx[r];
-        im.cid[r] = c;
-        im.center_idx[c] = tok;
-        if (im.center_idx_user) im.center_idx_user[c] = tok;
-        rn_cen<D>(im)[c] = rn_kept<D>(im)[r];
-      }
-      uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<T *>(im.Kcen) + (size_t)c * bt.d_k);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (lane + 32 * u < nv) dst[lane + 32 * u] = buf[u];
-      for (int v = lane + 128; v < nv; v += 32) dst[v] = __ldcg(reinterpret_cast<const uint4 *>(src) + v);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    int off = s_carry;
+    for (int k = 0; k < wid; ++k) off += wsum[k];
+    if (wd < nw) pref[wd] = off + x - pc;
+    __syncthreads();
+    if (t == kCenKeyThreads - 1) s_carry = off + x;
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && t == 0) {
+    im.cnt[PACT_CNT_C] = s_carry;
+    if (im.C_user) *im.C_user = s_carry;
+  }
+  for (int r = gw; r < q; r += nwarps) {
+    if (lane == 0) {
+      const float rf = (float)((double)__ldcg(&im.rho_fix[r]) * (1.0 / (double)(1u << kRhoShift)));
+      im.rho[r] = rf;
+      if (im.rho_user) im.rho_user[r] = rf;
+    }
+    const uint32_t m = cm[r >> 5];
+    if (!((m >> (r & 31)) & 1u)) continue;
+    const int c = pref[r >> 5] + __popc(m & ((1u << (r & 31)) - 1u));
+    const T *src = reinterpret_cast<const T *>(im.Kp) + (size_t)r * bt.d_k;
+    const int nvk = bt.d_k / V;
+    uint4 buf[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lane + 32 * u < nvk) buf[u] = __ldcg(reinterpret_cast<const uint4 *>(src) + lane + 32 * u);
+    if (lane == 0) {
+      const int tok = im.kept_idx[r];
+      im.cid[r] = c;
+      im.center_idx[c] = tok;
+      if (im.center_idx_user) im.center_idx_user[c] = tok;
+      rn_cen<D>(im)[c] = rn_kept<D>(im)[r];
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<T *>(im.Kcen) + (size_t)c * bt.d_k);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lane + 32 * u < nvk) dst[lane + 32 * u] = buf[u];
+    for (int v = lane + 128; v < nvk; v += 32) dst[v] = __ldcg(reinterpret_cast<const uint4 *>(src) + v);
   }
 }
 
@@ -553,9 +545,10 @@ cudaError_t cluster_configure(ClusterCfg *cfg) {
   if (e != cudaSuccess) return e;
   cfg->sm_count = sms;
   cfg->centers_smem_max = optin - 1024;
-  e = cudaFuncSetAttribute(k_centers<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_centers<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
+  e = cudaFuncSetAttribute(k_centers, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
+  constexpr int masks = (kMaxTokens / 32 + 4) * 12;
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_center_keys<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, masks);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_center_keys<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, masks);
   return e;
 }
 
@@ -579,17 +572,24 @@ cudaError_t launch_gram(const Batch &bt, int maxN, bool bf16, const ClusterCfg &
   return PACT_DISPATCH(bf16, k_gram_f64, grid, kTileThreads, st, bt);
 }
 
-cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int spin_limit, cudaStream_t st) {
-  // the densities of one image are staged in shared memory when they fit in half of it; maxQ is an estimate of
-  // the largest survivor count, an image with more reads them from global memory.  The two mask copies
-  // take a word per 32 survivors each.
-  const size_t budget = (size_t)cfg.centers_smem_max / 2;
-  int keys_cap = (size_t)maxQ * sizeof(unsigned long long) <= budget ? maxQ : 0;
-  int mask_cap = (maxQ + 31) / 32 + 1;
-  if ((size_t)mask_cap * 8 > budget) mask_cap = 0;
-  const size_t smem = (size_t)keys_cap * sizeof(unsigned long long) + (size_t)mask_cap * 8;
-  return bf16 ? launch_coop(k_centers<__nv_bfloat16>, dim3(cfg.sm_count), dim3(kCenThreads), smem, st, true, bt, keys_cap, mask_cap, spin_limit)
-              : launch_coop(k_centers<float>, dim3(cfg.sm_count), dim3(kCenThreads), smem, st, true, bt, keys_cap, mask_cap, spin_limit);
+cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int sweep_limit, cudaStream_t st) {
+  // maxQ is an estimate of the largest survivor count (ties can exceed it): the masks are sized for every token, densities
+  // and adjacency by the estimate, and what does not fit is read from global memory.
+  int maxN = 1;
+  for (int b = 0; b < bt.B; ++b) maxN = bt.img[b].N > maxN ? bt.img[b].N : maxN;
+  const int mask_cap = ((maxN + 31) / 32 + 3) & ~3, ncta = cfg.sm_count / bt.B > 1 ? cfg.sm_count / bt.B : 1;
+  const size_t room = (size_t)cfg.centers_smem_max - (size_t)mask_cap * 4;
+  const int keys_cap = (size_t)maxQ * 8 + 16 <= room / 2 ? (maxQ + 1) & ~1 : 0;
+  size_t adj = (size_t)((maxQ + ncta - 1) / ncta) * ((maxQ + 127) / 128) * 16;
+  if (adj > room - (size_t)keys_cap * 8) adj = room - (size_t)keys_cap * 8;
+  const size_t smem = (size_t)mask_cap * 4 + (size_t)keys_cap * 8 + adj;
+  const cudaError_t e = launch_k(k_centers, dim3(cfg.sm_count > bt.B ? cfg.sm_count : bt.B), dim3(kCenThreads), smem, st, true, bt, mask_cap, keys_cap, (int)adj, sweep_limit);
+  if (e != cudaSuccess) return e;
+  // a warp for two rows, but no more than eight CTAs per SM in all
+  const int most = 8 * cfg.sm_count / bt.B, want = (maxQ + 2 * kCenKeyThreads / 32 - 1) / (2 * kCenKeyThreads / 32), X = want < most ? want : most;
+  const dim3 grid(X > 0 ? X : 1, bt.B), block(kCenKeyThreads);
+  return bf16 ? launch_k(k_center_keys<__nv_bfloat16>, grid, block, (size_t)mask_cap * 12, st, true, bt, mask_cap)
+              : launch_k(k_center_keys<float>, grid, block, (size_t)mask_cap * 12, st, true, bt, mask_cap);
 }
 
 cudaError_t launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const ClusterCfg &cfg, cudaStream_t st) {

@@ -94,9 +94,9 @@ cudaError_t cluster_configure(ClusterCfg *cfg);
 cudaError_t launch_keynorm_gather(const Batch &bt, int maxN, bool bf16, cudaStream_t st);
 cudaError_t launch_center_key_gather(const Batch &bt, int maxN, bool bf16, bool all_rows, cudaStream_t st);
 cudaError_t launch_gram(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st);
-// density order, centre selection, cluster ids and centre keys in one cooperative kernel
-// maxQ: estimate of the largest number of survivors of an image (sizes the staging buffer only)
-cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int spin_limit, cudaStream_t st);
+// centre selection, cluster ids and centre keys (two kernels); maxQ: estimate of the largest number of survivors of an
+// image (sizes staging buffers only)
+cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int sweep_limit, cudaStream_t st);
 cudaError_t launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const ClusterCfg &cfg, cudaStream_t st);
 cudaError_t launch_label(const Batch &bt, int maxN, bool bf16, RowMode mode, cudaStream_t st);
 // layer choice: inverse norms of all keys of every layer, largest pair distance (any dtype), result

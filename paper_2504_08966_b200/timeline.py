@@ -23,7 +23,7 @@ from . import workloads
 
 KERNELS = {0: "k_qsum", 1: "k_tokens", 2: "k_scores", 3: "k_select", 4: "k_tiles_umma<gram>", 5: "k_centers",
            6: "k_tiles_umma<assign>", 7: "  k_select: threshold known", 8: "k_members / k_lists", 9: "k_merge",
-           10: "  k_centers: keys staged", 11: "  k_centers: sweeps done", 12: "  k_centers: after grid barrier",
+           10: "  k_centers: rows staged", 11: "  k_centers: sweeps done", 12: "  k_center_keys: start",
            13: "  members: labels read", 14: "  members: offsets known", 15: "  k_merge: records read"}
 SLOTS, CTAS = 16, 4096
 

@@ -98,6 +98,33 @@ def test_small_batches(B):
     _check(wl, torch.bfloat16)
 
 
+@pytest.mark.parametrize("case", ["many rows", "more survivors than estimated"])
+def test_centres_outside_shared_memory(case):
+    """Blocks of more than 1024 rows, adjacency words and densities that stay in global memory."""
+    if case == "many rows":                   # sixteen images, so nine CTAs for the large one
+        wls = [_workload(9400 if b == 3 else 5 + b, 1, 1, 8, 8, torch.bfloat16, 40 + b) for b in range(16)]
+        wl = workloads.Workload("edge", [w.images[0] for w in wls], 8, 1, 1, 8, torch.bfloat16, 0.0, 0.3)
+    else:                                     # six groups of equal scores; the threshold is in one of them
+        wl = _workload(1800, 4, 2, 64, 256, torch.bfloat16, 3)
+        img, pick = wl.images[0], torch.arange(1800) % 6
+        img.K.copy_(img.K[pick]); img.Q.copy_(img.Q[pick]); img.H[1:1801] = img.H[1:1801][pick]
+    _check(wl, torch.float32)
+
+
+def test_centres_left_open_are_resolved():
+    """Rows that the sweeps give up on are resolved by the kernel that lists the centres."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = workloads.single_image(seed=29, N=2000, T=8, n_blobs=50)
+    img = wl.images[0]
+    ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
+    im = pb.device_image(img, torch.float32)
+    ctx.set_wait_limits(center_sweeps=1)
+    ctx.pact_reduce([im], pb.make_params(lam=wl.lam, d_c=wl.d_c, d_n=wl.d_n, alpha=wl.alpha))
+    torch.cuda.synchronize()
+    assert int(im.counters[pb.CNT["status"]]) == -5
+    assert np.array_equal(im.label.cpu().numpy(), oracle_image(wl, img)["label"])
+
+
 def test_no_norm_and_norm_only():
     """Both forms of the score without one of its factors, over several units of the token pass."""
     from paper_2504_08966_b200 import binding as pb
