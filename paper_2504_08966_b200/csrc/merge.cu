@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // (No early trigger: with one the next call's first kernel is placed while this one still fills most SMs, all on the few
+  // that are free, and takes 4 to 12 us more from there.)
   pdl_wait();
-  pdl_trigger();
   const int t = threadIdx.x;
   __shared__ int s_row[kMrgThreads], s_cluster[kMrgThreads], s_dst[kMrgThreads];   // row of H, cluster, output row of an item
   __shared__ float s_inv[kMrgThreads];              // 1 / size (1 for text rows and centre-only merging)
