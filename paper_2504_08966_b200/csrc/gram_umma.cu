@@ -194,6 +194,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
     if (r4.y > kHuge) r4.y = 0.f;
     if (r4.z > kHuge) r4.z = 0.f;
     if (r4.w > kHuge) r4.w = 0.f;
+    r4.x *= -0.5f; r4.y *= -0.5f; r4.z *= -0.5f; r4.w *= -0.5f;   // see gram_chunk
   }
   __syncwarp();
   if (lane * 4 < HALF) reinterpret_cast<float4 *>(rn_col)[lane] = r4;
@@ -215,16 +216,15 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
     tmem_ld_wait();
     if (MODE == MODE_GRAM) {
       uint32_t bits, colbits = 0u;
+      float nearest;
       unsigned long long colsum = 0ull;
       if (above) {
         // every row of this block is a survivor (only the last block row is ragged, and it has no
         // block to its right); each pair (row, column) is also the pair (column, row)
-        int bnd = 0;
         if (c0 + 32 > ncols)
-          gram_chunk<true, true>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, bnd, colsum, colbits);
+          gram_chunk<true, true>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, nearest, colsum, colbits);
         else
-          gram_chunk<false, true>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, bnd, colsum, colbits);
-        band += bnd;                            // row < column throughout
+          gram_chunk<false, true>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, nearest, colsum, colbits);
         const int gj = c0 + lane;
         if (gj < ncols) {
           atomicAdd(&im.rho_fix[gj], colsum);
@@ -232,20 +232,22 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
         }
       } else {
         const bool edge = (c0 + 32 > ncols) || (c0 < r0 + 32 && c0 + 32 > r0);
-        if (edge) gram_chunk<true, false>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, band, colsum, colbits);
-        else {
-          int bnd = 0;
-          gram_chunk<false, false>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, bnd, colsum, colbits);
-          if (row < c0) band += bnd;            // each unordered pair once; the chunk lies wholly on one side
-        }
+        if (edge) gram_chunk<true, false>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, nearest, colsum, colbits);
+        else gram_chunk<false, false>(v, rn_col + ch * 32, rni, row, c0, ncols, d_c, neg_k, lane, tr, rowsum, bits, nearest, colsum, colbits);
+      }
+      if (__any_sync(0xffffffffu, nearest <= kNear)) {   // rare
+        tmem_ld32(taddr + ch * 32, v);
+        tmem_ld_wait();
+        band += gram_band(v, rn_col + ch * 32, rni, row, c0, ncols, d_c);
       }
       if (row_ok) im.adj[(size_t)row * im.Wp + (c0 >> 5)] = bits;
     } else if (MODE == MODE_SPREAD) {
       // The largest distance of the chunk belongs to its smallest cosine: d = clamp(1 - c) does not increase
-      // with c, in floating point either, so the cosines (dot * rn_i) * rn_j are compared and one distance is
-      // formed per chunk from the smallest.  Rows and columns past the end hold zero dot products,
+      // with c, in floating point either, so the products dot * rn_j are compared and one cosine and distance is
+      // formed per chunk from the smallest (the row's inverse norm is positive).  Rows and columns past the end hold zero dot products,
       // i.e. distance 1, and the pair (i, i) is not a pair: chunks that hold either take the checked loop.
-      float cmin = 4.0f;
+      constexpr float kNone = 3.0e38f;
+      float cmin = kNone;
       const bool plain = c0 + 32 <= ncols && r0 + 32 <= nrows && (c0 + 32 <= r0 || c0 >= r0 + 32);   // uniform
       if (plain) {
 #pragma unroll
@@ -253,7 +255,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
           const float4 rn4 = *reinterpret_cast<const float4 *>(rn_col + ch * 32 + k4);
           const float rnj[4] = {rn4.x, rn4.y, rn4.z, rn4.w};
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) cmin = fminf(cmin, (__uint_as_float(v[k4 + kk]) * rni) * rnj[kk]);
+          for (int kk = 0; kk < 4; ++kk) cmin = fminf(cmin, __uint_as_float(v[k4 + kk]) * rnj[kk]);
         }
       } else {
         const int lim = row_ok ? min(32, ncols - c0) : 0;
@@ -265,12 +267,12 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
             const int k = k4 + kk;
-            const float c = (__uint_as_float(v[k]) * rni) * rnj[kk];
+            const float c = __uint_as_float(v[k]) * rnj[kk];
             if (k < lim && k != self) cmin = fminf(cmin, c);
           }
         }
       }
-      if (cmin < 4.0f) mx = fmaxf(mx, fminf(fmaxf(1.0f - cmin, 0.0f), 2.0f));
+      if (cmin < kNone) mx = fmaxf(mx, fminf(fmaxf(1.0f - cmin * rni, 0.0f), 2.0f));
     } else {
       // the nearest centre of the chunk is the one with the largest cosine (dot * rn_i) * rn_j; the first of
       // equal cosines wins, i.e. the centre with the lowest index; the distance is formed once per tile

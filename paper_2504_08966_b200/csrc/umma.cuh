@@ -53,22 +53,36 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {   // clamped to [0, 1]
+  float y;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
 // One 32-column chunk of the epilogue of the all-pairs pass for one row (= one lane): distance
 // (Eq. 5), density term (Eq. 6) as an integer multiple of 2^-30, adjacency bit d <= d_c, band count.
 // EDGE adds the per-element checks that only edge chunks need (diagonal, columns past the end).
 // COLS (blocks above the diagonal) also hands every pair to its column: the warp's 32 x 32 terms go
 // through a shared-memory buffer `tr` (row stride 36 words: conflict-free stores, 16-byte loads), lane k
-// adds the 32 terms of column k, and a 32 x 32 bit transpose gives it the column's adjacency word.  The arithmetic is that of DistF (common.cuh) with the two inverse norms multiplied first,
-// written out so that three terms are summed in 32 bits.
+// adds the 32 terms of column k, and a 32 x 32 bit transpose gives it the column's adjacency word.
+//
+// Instructions are what this pass is bound by (2.2 issued per clock and SM, half of the tensor pipe idle), so the arithmetic
+// of DistF (common.cuh) is written for few of them, with the same results: all of it on half the distance, whose clamp to
+// [0, 1] is part of the multiply-add and whose scaling by two is exact (rn_col holds -1/2 of the columns' inverse norms);
+// the adjacency bit is the sign of h minus the number after d_c / 2; `nearest`, the smallest
+// magnitude of that, tells whether a pair may be within the band (see gram_band); three terms are summed in 32 bits.  BEFOREAFTER
 template <bool EDGE, bool COLS>
 __device__ __forceinline__ void gram_chunk(const uint32_t (&v)[32], const float *rn_col, float rni, int row, int c0,
                                            int ncols, float d_c, float neg_k, int lane, uint32_t *tr,
-                                           unsigned long long &rowsum, uint32_t &bits, int &band,
+                                           unsigned long long &rowsum, uint32_t &bits, float &nearest,
                                            unsigned long long &colsum, uint32_t &colbits) {
   uint32_t b = 0u;
   unsigned long long s = 0ull;
   uint32_t s3 = 0u;                                 // three terms, each at most 2^30, fit in 32 bits
-  int bnd = 0;
+  const float after = __uint_as_float(__float_as_uint(0.5f * d_c) + 1u), k2 = 2.0f * neg_k;   // (d_c is not negative)
+  float closest = 4.0f;
+  // rn_i * rn_j first: a pair must get the same distance whichever of the two is the row, so that
+  // duplicate keys keep exactly equal densities
 #pragma unroll
   for (int k4 = 0; k4 < 32; k4 += 4) {
     const float4 rn4 = *reinterpret_cast<const float4 *>(rn_col + k4);
@@ -76,33 +90,21 @@ __device__ __forceinline__ void gram_chunk(const uint32_t (&v)[32], const float 
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       const int k = k4 + kk;
-      // rn_i * rn_j first: a pair must get the same distance whichever of the two is the row, so that
-      // duplicate keys keep exactly equal densities
-      float dd = fminf(fmaxf(1.0f - __uint_as_float(v[k]) * (rni * rnj[kk]), 0.0f), 2.0f);
-      bool ok = true;
-      if (EDGE) {
-        const int gj = c0 + k;
-        if (gj == row) dd = 0.f;
-        ok = gj < ncols;
-      }
-      uint32_t term = __float2uint_rn(ex2_approx(dd * neg_k) * (float)(1u << kRhoShift));
-      bool within = dd <= d_c;
-      const bool inband = fabsf(dd - d_c) <= 1e-6f;
-      if (EDGE) {
-        if (!ok) { term = 0u; within = false; }
-        if (ok && inband && row < c0 + k) ++bnd;
-      } else {
-        if (inband) ++bnd;
-      }
+      const float h = EDGE && c0 + k == row ? 0.f : fma_sat(__uint_as_float(v[k]), rni * rnj[kk], 0.5f), t = h - after;
+      uint32_t term = __float2uint_rn(ex2_approx(h * k2) * (float)(1u << kRhoShift));
+      if (EDGE && c0 + k >= ncols) term = 0u;
+      b = __funnelshift_l(__float_as_uint(t), b, 1);
+      closest = fminf(closest, fabsf(t));
       s3 += term;
-      if (within) b |= 1u << k;
       if (k % 3 == 2 || k == 31) { s += s3; s3 = 0u; }   // a run of keys at distance 0 adds 2^30 each
       if (COLS) tr[k * 36 + lane] = term;
     }
   }
+  b = __brev(b);                                    // (column 0 went in first)
+  if (EDGE && c0 + 32 > ncols) b &= ncols > c0 ? (1u << (ncols - c0)) - 1u : 0u;
   rowsum += s;
   bits = b;
-  band += bnd;
+  nearest = closest;
   if (COLS) {
     __syncwarp();
     // lane k: the 32 terms of column k, three to a 32-bit partial sum as above
@@ -132,6 +134,16 @@ __device__ __forceinline__ void gram_chunk(const uint32_t (&v)[32], const float 
     colbits = w;
     __syncwarp();                                   // tr may be rewritten by the next chunk
   }
+}
+
+// Pairs (row, column after it) of the chunk within 1e-6 of d_c; called where the chunk's `nearest` is at most kNear.
+constexpr float kNear = 1e-6f;                      // half of the band, and the step to the number after d_c / 2
+__device__ __forceinline__ int gram_band(const uint32_t (&v)[32], const float *rn_col, float rni, int row, int c0, int ncols, float d_c) {
+  int n = 0;
+#pragma unroll
+  for (int k = 0; k < 32; ++k)
+    n += row < c0 + k && c0 + k < ncols && fabsf(2.0f * fma_sat(__uint_as_float(v[k]), rni * rn_col[k], 0.5f) - d_c) <= 1e-6f;
+  return n;
 }
 
 }  // namespace pact
