@@ -229,6 +229,7 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 // k_center_keys: cluster ids (number of centres with a lower index), centre list, centre keys and inverse norms.
 constexpr int kCenThreads = 1024;
 constexpr int kCenWarps = kCenThreads / 32;
+constexpr int kCenPasses = 1 << 13;                      // most passes of k_center_keys over open rows
 constexpr int kCenSweeps = 512;                          // sweeps of k_centers (about a microsecond each)
 
 // One row against the removed rows, by a warp: an earlier neighbour that is not removed, or -1.
@@ -373,6 +374,7 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
   if (__syncthreads_or(open)) {
     // Rows that k_centers left: every CTA resolves them, to the same end (the set is unique), against its own copies;
     // the first CTA also writes the centres for later kernels.
+    int passes = 0;
     do {
       open = 0;
       for (int r = wid; r < q; r += kWarps) {
@@ -380,6 +382,14 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
         const volatile uint32_t *vc = cm + (r >> 5), *vr = rm + (r >> 5);
         if ((*vc | *vr) & bit) continue;
         const uint32_t *row = im.adj + (size_t)r * im.Wp;
+        // (the neighbour of a centre is removed here as well: should an earlier stage have failed, the words need not be
+        // symmetric, and the earliest open row must still be decided)
+        int hit = 0;
+        for (int wd = lane; wd < nw; wd += 32) hit |= (row[wd] & *const_cast<volatile uint32_t *>(cm + wd)) != 0u;
+        if (__any_sync(0xffffffffu, hit)) {
+          if (lane == 0) atomicOr(&rm[r >> 5], bit);
+          continue;
+        }
         if (open_earlier(row, rm, im.rho_fix, r, nw, lane) >= 0) { open = 1; continue; }
         for (int wd = lane; wd < nw; wd += 32) {
           uint32_t e = row[wd];
@@ -391,7 +401,11 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
           if (e) atomicOr(&rm[wd], e);
         }
       }
-    } while (__syncthreads_or(open));                    // ends: the earliest open row is decided in every pass
+      if (++passes >= kCenPasses) {
+        if (t == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+        open = 0;
+      }
+    } while (__syncthreads_or(open));                    // (the earliest open row is decided in every pass)
   }
   for (int base = 0; base < nw; base += kCenKeyThreads) {
     const int wd = base + t, pc = wd < nw ? __popc(cm[wd]) : 0;
