@@ -3,6 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <atomic>
 #include <new>
 
 #include "kernels.cuh"
@@ -25,6 +26,10 @@ struct pact_ctx {
   int prof_on;             // record an event after every stage of pact_reduce
   int prof_n;              // stages recorded by the last profiled call
   cudaEvent_t ev[kProfStages + 1];
+  // pact_reduce_host: a stream for the copies in, used by one call at a time (another thread's call does without)
+  std::atomic_flag feed_busy = ATOMIC_FLAG_INIT;
+  cudaStream_t feed_stream = nullptr;
+  cudaEvent_t feed_start = nullptr, feed_keys = nullptr, feed_part[kFeedParts] = {};
 };
 
 struct pact_graph {
@@ -230,9 +235,8 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
   if (d % 8 != 0 || d_h % v != 0) return PACT_ERR_UNSUPPORTED;
   if (d > kMergeMaxD || n_qh > 256) return PACT_ERR_UNSUPPORTED;
   if ((n_qh * d_h / v + 7) / 8 > kMaxColGroups) return PACT_ERR_UNSUPPORTED;
-  pact_ctx *c = new (std::nothrow) pact_ctx;
+  pact_ctx *c = new (std::nothrow) pact_ctx();
   if (!c) return PACT_ERR_INVALID_ARG;
-  memset(c, 0, sizeof(*c));
   c->d = d; c->n_qh = n_qh; c->n_kvh = n_kvh; c->d_h = d_h;
   c->d_k = n_kvh * d_h; c->n_qcols = n_qh * d_h;
   c->in = in; c->out = o; c->elt = in == PACT_BF16 ? 2 : 4;
@@ -261,9 +265,30 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
   return PACT_OK;
 }
 
+static void release_feed(pact_ctx *ctx) {
+  for (cudaEvent_t *e : {&ctx->feed_start, &ctx->feed_keys, &ctx->feed_part[0], &ctx->feed_part[1]}) {
+    if (*e) cudaEventDestroy(*e);
+    *e = nullptr;
+  }
+  if (ctx->feed_stream) cudaStreamDestroy(ctx->feed_stream);
+  ctx->feed_stream = nullptr;
+}
+static bool prepare_feed(pact_ctx *ctx) {            // on the first call that uses it
+  if (ctx->feed_stream) return true;
+  bool ok = cudaStreamCreateWithFlags(&ctx->feed_stream, cudaStreamNonBlocking) == cudaSuccess;
+  for (cudaEvent_t *e : {&ctx->feed_start, &ctx->feed_keys, &ctx->feed_part[0], &ctx->feed_part[1]})
+    ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    (void)cudaGetLastError();
+    release_feed(ctx);
+  }
+  return ok;
+}
+
 pact_status pact_destroy(pact_ctx *ctx) {
   if (ctx && ctx->prof_on)
     for (int i = 0; i <= kProfStages; ++i) cudaEventDestroy(ctx->ev[i]);
+  if (ctx) release_feed(ctx);
   delete ctx;
   return PACT_OK;
 }
@@ -497,8 +522,8 @@ pact_status pact_merge(pact_ctx *ctx, const pact_image *img, const int32_t *labe
   return PACT_OK;
 }
 
-pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact_params *params,
-                        int params_stride, void *ws, size_t ws_bytes, void *stream) {
+static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, const pact_params *params,
+                                 int params_stride, void *ws, size_t ws_bytes, void *stream, const HostFeed *feed) {
   if (!ctx || !imgs || B < 1 || !params || (params_stride != 0 && params_stride != 1))
     return PACT_ERR_INVALID_ARG;
   int maxN = 0;
@@ -534,7 +559,8 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     // (a profiled call is launched kernel by kernel)
     if (!ctx->prof_on && small_fits(bt, cmaxN, ctx->umma)) {
       int rpp = 0;
-      CK(launch_euti(bt, cmaxN, bf, 2, st, nullptr, nullptr, &rpp));
+      if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 2, st, *feed, &rpp));
+      else CK(launch_euti(bt, cmaxN, bf, 2, st, nullptr, nullptr, &rpp));
       CK(launch_small(bt, bf, ctx->umma, rpp, ctx->sweep_limit, st));
       CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->ccfg, st));
       ctx->launches += euti_kernels(2) + 2;
@@ -551,7 +577,9 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     struct MarkFn {
       static cudaError_t call(void *p) { return (*static_cast<decltype(mark) *>(p))(); }
     };
-    CK(launch_euti(bt, cmaxN, bf, 0, st, ctx->prof_on ? &MarkFn::call : nullptr, &mark));  CK(mark());
+    if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 0, st, *feed, nullptr));
+    else CK(launch_euti(bt, cmaxN, bf, 0, st, ctx->prof_on ? &MarkFn::call : nullptr, &mark));
+    CK(mark());
     if (ctx->umma) CK(launch_gram_umma(bt, cmaxN, ctx->ccfg, st, cmaxQ));
     else CK(launch_gram(bt, cmaxN, bf, ctx->ccfg, st));
     CK(mark());
@@ -572,6 +600,11 @@ pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact
     CK(cudaGetLastError());
   }
   return PACT_OK;
+}
+
+pact_status pact_reduce(pact_ctx *ctx, const pact_image *imgs, int B, const pact_params *params,
+                        int params_stride, void *ws, size_t ws_bytes, void *stream) {
+  return reduce_images(ctx, imgs, B, params, params_stride, ws, ws_bytes, stream, nullptr);
 }
 
 pact_status pact_graph_create(pact_ctx *ctx, const pact_image *imgs, int B, const pact_params *params,
@@ -634,10 +667,62 @@ size_t pact_host_staging_bytes(const pact_ctx *ctx, int n_total, int N) {
   return b;
 }
 
+namespace {
+
+constexpr size_t kFeedBytes = 12u << 20;              // hidden states of at least this size arrive on a stream of their own
+
+// host memory that kernels can write to under its own address
+bool mapped(const void *p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeHost && at.devicePointer == p;
+}
+
+cudaError_t copy_small_inputs(const pact_image *img, const pact_image &dv, size_t bK, size_t bQ, bool alias, cudaStream_t st) {
+  cudaError_t e = cudaMemcpyAsync(const_cast<void *>(dv.Q_euti), img->Q_euti, bQ, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(const_cast<void *>(dv.K_euti), img->K_euti, bK, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && !alias) e = cudaMemcpyAsync(const_cast<void *>(dv.K_clu), img->K_clu, bK, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(const_cast<int32_t *>(dv.P), img->P, (size_t)img->n_total * 4, cudaMemcpyHostToDevice, st);
+  return e;
+}
+
+// The copies in on the context's stream, after what the caller's stream holds; pact_reduce on the caller's behind them.
+pact_status feed_and_reduce(pact_ctx *ctx, const pact_image *img, const pact_image *dv, const pact_params *p, size_t bH, size_t bK, size_t bQ,
+                            bool alias, void *ws, size_t ws_bytes, cudaStream_t st) {
+  HostFeed feed;
+  feed.keys = ctx->feed_keys;
+  // the last part is an eighth: its norms take 4 us after the last byte
+  const int tail = img->N / 8 + (img->n_total - img->N - img->vis_start);   // rows, text rows included
+  const int rows[kFeedParts] = {img->n_total - tail, tail};
+  feed.end[0] = img->N - img->N / 8;
+  feed.end[1] = img->N;
+  const size_t row = bH / img->n_total;
+  cudaStream_t in = ctx->feed_stream;
+  cudaError_t e = cudaEventRecord(ctx->feed_start, st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(in, ctx->feed_start, 0);
+  if (e == cudaSuccess) e = copy_small_inputs(img, *dv, bK, bQ, alias, in);
+  if (e == cudaSuccess) e = cudaEventRecord(feed.keys, in);
+  size_t done = 0;
+  for (int k = 0; e == cudaSuccess && k < kFeedParts; done += rows[k++] * row) {
+    feed.part[k] = ctx->feed_part[k];
+    e = cudaMemcpyAsync((char *)dv->H + done, (const char *)img->H + done, rows[k] * row, cudaMemcpyHostToDevice, in);
+    if (e == cudaSuccess) e = cudaEventRecord(feed.part[k], in);
+  }
+  pact_status s = e == cudaSuccess ? reduce_images(ctx, dv, 1, p, 0, ws, ws_bytes, st, &feed) : fail_cuda(ctx, e, "pact_reduce_host");
+  if (s == PACT_OK) ctx->launches += kFeedParts;
+  else (void)cudaStreamSynchronize(in);              // (the caller's stream need not have been ordered behind the copies)
+  return s;
+}
+
+}  // namespace
+
 pact_status pact_reduce_host(pact_ctx *ctx, const pact_image *img, const pact_params *p, void *dev_staging,
                              size_t staging_bytes, void *ws, size_t ws_bytes, void *stream) {
   if (!ctx || !img || !p || !dev_staging) return PACT_ERR_INVALID_ARG;
-  if (img->N < 1 || img->n_total < img->N) return PACT_ERR_INVALID_ARG;
+  if (img->N < 1 || img->vis_start < 0 || img->n_total < img->N || img->n_total - img->N < img->vis_start) return PACT_ERR_INVALID_ARG;
   if (staging_bytes < pact_host_staging_bytes(ctx, img->n_total, img->N)) return PACT_ERR_WORKSPACE;
   if ((reinterpret_cast<uintptr_t>(dev_staging) % kAlign) != 0) return PACT_ERR_WORKSPACE;
   if (!img->H || !img->K_euti || !img->Q_euti || !img->K_clu || !img->P || !img->H_out || !img->P_out ||
@@ -658,25 +743,37 @@ pact_status pact_reduce_host(pact_ctx *ctx, const pact_image *img, const pact_pa
   char *dHo = take(bHo), *dPo = take((size_t)nt * 4), *dSo = take((size_t)nt * 4), *dL = take((size_t)N * 4);
   char *dC = take(PACT_N_COUNTERS * 4);
   char *dLw = take((size_t)nt * 4);
-  CK(cudaMemcpyAsync(dH, img->H, bH, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(dKe, img->K_euti, bK, cudaMemcpyHostToDevice, st));
   const bool alias = img->K_clu == img->K_euti;
-  if (!alias) CK(cudaMemcpyAsync(dKc, img->K_clu, bK, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(dQ, img->Q_euti, bQ, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(dP, img->P, (size_t)nt * 4, cudaMemcpyHostToDevice, st));
   pact_image dv = *img;
   dv.H = dH; dv.K_euti = dKe; dv.K_clu = alias ? dKe : dKc; dv.Q_euti = dQ; dv.P = (const int32_t *)dP;
   dv.H_out = dHo; dv.P_out = (int32_t *)dPo; dv.size_out = (int32_t *)dSo; dv.label = (int32_t *)dL;
   dv.score = nullptr; dv.keep = nullptr; dv.counters = (int32_t *)dC;
   dv.logw_out = img->logw_out ? (float *)dLw : nullptr;
-  pact_status s = pact_reduce(ctx, &dv, 1, p, 0, ws, ws_bytes, stream);
+  // Results that the kernels can reach in host memory are written there by them: the number of rows depends on the data, and
+  // copies of exactly that many had to wait for it (two synchronisations and 40 us at 7290 tokens).
+  const bool direct = aligned16(img->H_out) && mapped(img->H_out) && mapped(img->P_out) && mapped(img->size_out) &&
+                      (!img->logw_out || mapped(img->logw_out)) && (!img->label || mapped(img->label));
+  if (direct) { dv.H_out = img->H_out; dv.P_out = img->P_out; dv.size_out = img->size_out; dv.label = img->label; dv.logw_out = img->logw_out; }
+  // The hidden states are most of what comes in: they come last, on a stream of their own, while the global query and the
+  // logits are formed, and their norms are formed part by part; what is left after the last byte is the split, the
+  // clustering and the merge.  (7290 tokens: 20 us of kernels hidden, 1474 -> 1465; 2916: 659 -> 657; with less to copy the
+  // events cost what that gives.)
+  const bool fed = bH >= kFeedBytes && !ctx->prof_on && !ctx->feed_busy.test_and_set(std::memory_order_acquire);
+  pact_status s = PACT_OK;
+  if (fed && prepare_feed(ctx)) {
+    s = feed_and_reduce(ctx, img, &dv, p, bH, bK, bQ, alias, ws, ws_bytes, st);
+  } else {
+    cudaError_t e = copy_small_inputs(img, dv, bK, bQ, alias, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dH, img->H, bH, cudaMemcpyHostToDevice, st);
+    s = e != cudaSuccess ? fail_cuda(ctx, e, "pact_reduce_host") : pact_reduce(ctx, &dv, 1, p, 0, ws, ws_bytes, stream);
+  }
+  if (fed) ctx->feed_busy.clear(std::memory_order_release);
   if (s != PACT_OK) return s;
-  // The number of valid output rows is data dependent: read the counters first, then copy
-  // exactly the rows that exist.
   CK(cudaMemcpyAsync(img->counters, dC, PACT_N_COUNTERS * 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   const int n_out = img->counters[PACT_CNT_N_OUT];
   if (n_out < 0 || n_out > nt) return PACT_ERR_INVALID_ARG;
+  if (direct) return PACT_OK;
   CK(cudaMemcpyAsync(img->H_out, dHo, (size_t)n_out * ctx->d * oe, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(img->P_out, dPo, (size_t)n_out * 4, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(img->size_out, dSo, (size_t)n_out * 4, cudaMemcpyDeviceToHost, st));

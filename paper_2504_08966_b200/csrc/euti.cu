@@ -154,9 +154,12 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
 //            comes from shared memory at one address per warp: with the lanes spread over the row the loads of the
 //            query were what took the time, and with the double-precision tensor instruction (m8n8k4, whose rate is
 //            that of the ordinary one) the seven idle heads of eight: 16 tokens of four heads took 4100 clocks a team.
+// `what` names the parts of the work (kTok...): hidden states that arrive from the host piece by piece have their norms
+// formed by launches of their own.
 // As 16-byte loads of four tokens per warp, one token's row at a time and the logits between them, the pass took 4.2 TB/s
 // of HBM, and with 28 query heads on 4 key heads 31 us of 40 for a few hundred tokens.  Now 46656 tokens of 3584 (382 MB)
 // end 77 us after the call began, against 100 us; bound by memory, 5.6 TB/s with the queries.
+constexpr int kTokInit = 1, kTokNorms = 2, kTokLogits = 4;
 constexpr int kTokThreads = 512;
 constexpr int kTokGroup = 256;                          // threads of the norms group and of the logits group
 constexpr int kTokTeam = kTokGroup / 2;                 // threads of a logits team
@@ -245,7 +248,7 @@ __device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, c
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int do_init) {
+__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int what) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
   constexpr int V = Vec<T>::N;
@@ -293,7 +296,7 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
         lb = image_of(lu, lb);
         const ImgDesc &im = bt.img[lb];
         const int r0 = (lu - s_first[lb]) * rpp, n = min(rpp, im.N - r0);
-        if ((im.flags & PACT_FLAG_NO_NORM) || n <= w) continue;
+        if ((im.flags & PACT_FLAG_NO_NORM) || !(what & kTokNorms) || n <= w) continue;
         lrows = (n - w + kTokWarps - 1) / kTokWarps;
         lsrc = reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + r0 + w) * im.ldH);
         lstep = (size_t)im.ldH * kTokWarps * sizeof(T);
@@ -311,7 +314,7 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
     bool all = false;
     int slot = 0, b = 0;                                // buffer that is next
     uint32_t par = 0;                                   // parity of each buffer's barrier
-    for (int u = u0; u < u1; ++u) {
+    for (int u = u0; u < u1 && (what & kTokNorms); ++u) {
       b = image_of(u, b);
       const ImgDesc &im = bt.img[b];
       const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
@@ -364,10 +367,10 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
       for (int r = w; r < n; r += kTeamWarps)
         bulk_load(s_mine + (size_t)r * ks, reinterpret_cast<const T *>(im.Ke) + (size_t)(r0 + r) * im.ldKe, bt.d_k * (int)sizeof(T), &s_kbar[team]);
     };
-    if (cfg.keys && lane == 0) issue_keys(u0 + team);
+    if (cfg.keys && (what & kTokLogits) && lane == 0) issue_keys(u0 + team);
     auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTokTeam) : "memory"); };
     auto sync_both = []() { asm volatile("bar.sync 3, %0;" ::"n"(kTokGroup) : "memory"); };
-    if (do_init) {                                      // what later kernels accumulate into
+    if (what & kTokInit) {                                      // what later kernels accumulate into
       const int gt = blockIdx.x * kTokGroup + threadIdx.x - kTokGroup, gs = gridDim.x * kTokGroup;
       for (int i = 0; i < bt.B; ++i) {
         const ImgDesc &im = bt.img[i];
@@ -382,7 +385,12 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
     }
     int b = 0, loaded = -1;                             // loaded: image whose query is in s_q
     uint32_t par = 0;
-    for (int u = u0; u < u1; ++u) {
+    if (!(what & kTokLogits)) {
+      pdl_wait();
+      s_query = 1;
+      pdl_trigger();
+    }
+    for (int u = u0; u < u1 && (what & kTokLogits); ++u) {
       b = image_of(u, b);
       const ImgDesc &im = bt.img[b];
       const bool mine = ((u - u0) & 1) == team;
@@ -1039,17 +1047,35 @@ static int tokens_grid(const Batch &bt, int rpp) {
 }
 
 template <typename T>
-static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
-  cudaError_t e = launch_qsum<T>(bt, st);
+static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, cudaStream_t st, int *rpp) {
+  const TokCfg tc = tokens_config<T>(bt);
+  if (rpp) *rpp = tc.rpp;
+  return launch_k(k_tokens<T>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
+}
+
+template <typename T>
+static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp_out, const HostFeed *feed) {
+  cudaError_t e = cudaSuccess;
+  if (feed && (e = cudaStreamWaitEvent(st, feed->keys, 0)) != cudaSuccess) return e;
+  e = launch_qsum<T>(bt, st);
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
-  const TokCfg tc = tokens_config<T>(bt);
-  e = launch_k(k_tokens<T>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, true, bt, tc, mode != 1 ? 1 : 0);
+  int rpp = 0;
+  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, st, &rpp);
   if (e != cudaSuccess) return e;
-  if (rpp) *rpp = tc.rpp;
+  for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
+    if (feed->end[k] <= first) continue;
+    Batch part = bt;
+    part.img[0].N = feed->end[k] - first;
+    part.img[0].vis_start += first;
+    part.img[0].nrm += first;
+    if ((e = cudaStreamWaitEvent(st, feed->part[k], 0)) != cudaSuccess) return e;
+    if ((e = launch_tokens<T>(part, kTokNorms, false, st, nullptr)) != cudaSuccess) return e;
+  }
+  if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
-  e = launch_k(k_scores, dim3((maxN + 255) / 256, bt.B), dim3(256), 0, st, true, bt, tc.rpp, mode == 0 ? 1 : 0);
+  e = launch_k(k_scores, dim3((maxN + 255) / 256, bt.B), dim3(256), 0, st, true, bt, rpp, mode == 0 ? 1 : 0);
   if (e != cudaSuccess) return e;
   if (mode == 0) {
     if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
@@ -1067,8 +1093,12 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
 }
 
 cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
-  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, mark, mark_arg, rpp)
-              : launch_euti_t<float>(bt, maxN, mode, st, mark, mark_arg, rpp);
+  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, mark, mark_arg, rpp, nullptr)
+              : launch_euti_t<float>(bt, maxN, mode, st, mark, mark_arg, rpp, nullptr);
+}
+cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, const HostFeed &feed, int *rpp) {
+  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, nullptr, nullptr, rpp, &feed)
+              : launch_euti_t<float>(bt, maxN, mode, st, nullptr, nullptr, rpp, &feed);
 }
 
 int euti_kernels(int mode) { return mode == 0 ? 4 : mode == 1 ? 3 : 2; }

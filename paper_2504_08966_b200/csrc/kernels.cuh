@@ -76,8 +76,17 @@ constexpr int kHistShift = 32 - kHistBits; // a key's bin in that histogram is k
 // kernels accumulate into); mode 1: scores only (three kernels); mode 2: mode 0 up to the token pass (two kernels).
 // mark (optional) is called between the kernels of the group (the per-kernel timing of a profiled call)
 typedef cudaError_t (*StageMark)(void *);
+// The inputs of one image on their way from the host: everything but the hidden states once `keys` has been recorded,
+// the rows up to end[k] (all of them for the last part) once part[k] has.
+constexpr int kFeedParts = 2;
+struct HostFeed {
+  cudaEvent_t keys, part[kFeedParts];
+  int end[kFeedParts];                     // visual tokens
+};
 cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark = nullptr,
                         void *mark_arg = nullptr, int *rpp = nullptr);   // rpp: receives the tokens per softmax piece
+// modes 0 and 2 for one image whose hidden states arrive in parts meanwhile (kFeedParts kernels more)
+cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, const HostFeed &feed, int *rpp);
 int euti_kernels(int mode);
 // threshold + ordered compaction of given scores (pact_prune, one image)
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st);

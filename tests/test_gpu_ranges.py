@@ -125,6 +125,37 @@ def test_centres_left_open_are_resolved():
     assert np.array_equal(im.label.cpu().numpy(), oracle_image(wl, img)["label"])
 
 
+@pytest.mark.parametrize("N,T,vis,d,rope,pinned", [
+    (3, 0, 0, 64, False, True),               # smaller than the parts
+    (780, 9, 2, 8192, False, True),           # just above the size that arrives in parts, one-cluster step
+    (760, 0, 0, 8192, True, True),            # just below it
+    (2309, 40, 40, 3584, True, True), (2309, 40, 0, 3584, False, False), (700, 5, 1, 64, False, False),
+])
+def test_host_buffers(N, T, vis, d, rope, pinned):
+    """Inputs in parts or not, results written to host memory by the kernels or copied."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = _workload(N, 4, 2, 64, d, torch.bfloat16, N + T, rope=rope, T=T)
+    img = wl.images[0]
+    img.vis_start = vis
+    ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
+    z = lambda m, dt: torch.full(m, 7, dtype=dt).pin_memory() if pinned else torch.full(m, 7, dtype=dt)   # noqa: E731
+    n = N + T
+    host = dict(H=img.H.pin_memory(), K_euti=img.K.pin_memory(), Q_euti=img.Q.pin_memory(), P=img.P.pin_memory(), vis_start=vis, N=N,
+                H_out=z((n, d), torch.float32), P_out=z((n,), torch.int32), size_out=z((n,), torch.int32), logw_out=z((n,), torch.float32),
+                label=z((N,), torch.int32), counters=z((16,), torch.int32))
+    host["K_clu"] = img.K_clu.pin_memory() if rope else host["K_euti"]
+    staging = torch.empty(ctx.host_staging_bytes(n, N), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        ctx.pact_reduce_host(host, pb.make_params(lam=wl.lam, d_c=wl.d_c), staging)
+    want = gpu_reduce(wl, torch.float32)[0][0]
+    n_out = int(host["counters"][0])
+    assert n_out == want["n_out"] and np.array_equal(host["label"].numpy(), want["label"])
+    for key in ("P_out", "size_out", "logw_out"):
+        assert np.array_equal(host[key][:n_out].numpy(), want[key])
+    assert torch.equal(host["H_out"][:n_out], want["H_out_raw"])
+    assert bool((host["H_out"][n_out:] == 7).all()) and bool((host["P_out"][n_out:] == 7).all())
+
+
 def test_no_norm_and_norm_only():
     """Both forms of the score without one of its factors, over several units of the token pass."""
     from paper_2504_08966_b200 import binding as pb
