@@ -156,7 +156,8 @@ long long pact_launch_count(const pact_ctx *ctx);
 /* With profiling on, pact_reduce records a CUDA event on `stream` after each of its kernels
  * (first parameter block of a call only).  pact_profile_read waits for the last one and writes
  * the duration of each kernel in milliseconds to ms[0..n), returning n (0 if nothing was
- * recorded).  pact_profile_stage_name(i) names the i-th kernel.  Off by default. */
+ * recorded).  pact_profile_stage_name(i) names the i-th kernel.  A profiled call is launched kernel by
+ * kernel whatever the size of its images.  Off by default. */
 pact_status pact_profile_enable(pact_ctx *ctx, int on);
 int pact_profile_read(pact_ctx *ctx, float *ms /*host*/, int cap);
 const char *pact_profile_stage_name(int i);
@@ -266,8 +267,9 @@ pact_status pact_graph_launch(pact_graph *graph, void *stream);
 pact_status pact_graph_destroy(pact_graph *graph);
 
 /* Same computation with HOST buffers for one image: copies the inputs to the device, runs
- * pact_reduce, copies H_out/P_out/size_out/label/counters back and synchronises.
- * dev_in / dev_out are device staging buffers the caller provides (sizes from
+ * pact_reduce, brings H_out/P_out/size_out/logw_out/label/counters back (results in mapped host memory are
+ * written there by the kernels) and synchronises.
+ * dev_staging is a device buffer the caller provides (size from
  * pact_host_staging_bytes); every pointer inside `img` is a host pointer here. */
 pact_status pact_reduce_host(pact_ctx *ctx, const pact_image *img /*host, host pointers*/,
                              const pact_params *p /*host*/, void *dev_staging, size_t staging_bytes,

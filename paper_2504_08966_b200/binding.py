@@ -111,8 +111,8 @@ def _ptr(t):
 
 
 def _stream():
-    """Handle of the current stream of the current device."""
-    return torch.cuda.current_stream().cuda_stream
+    """Handle of the current stream of the current device, without a Stream object around it (3 us of a call)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dt(dtype) -> int:
