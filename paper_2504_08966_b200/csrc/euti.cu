@@ -61,7 +61,7 @@ __device__ __forceinline__ void finish_row_sums(const double (*acc)[32], int w, 
 }
 
 // ---- Eq. 1: column sums of Q -----------------------------------------------------------------------------
-// grid (ncg RP, B) in clusters of RP CTAs, 256 threads at no more than 64 registers, at most about two CTAs per SM, which
+// grid (ncg RP, B) in clusters of RP CTAs, 256 threads at no more than 64 registers, two CTAs per SM or three, which
 // leave room for k_tokens beside them.  Work item (column group of GV 16-byte vectors, block of rows): thread t takes
 // vector t % GV of the group and the rows r0 + t / GV, + 256 / GV, ...; the row lanes of a warp are added with shuffles, the
 // warps through shared memory.  The RP row blocks of a column group are one cluster: the CTAs store their sums into the
@@ -1004,13 +1004,14 @@ constexpr size_t kSplitReserve = 4096;       // static shared memory of k_split,
 template <typename T>
 static cudaError_t launch_qsum(const Batch &bt, cudaStream_t st) {
   // column groups of four vectors where that does not take more CTAs than two per SM, else of eight; then as many row
-  // blocks (CTAs of a cluster) as keep the grid within two CTAs per SM
+  // blocks (CTAs of a cluster) as keep the grid within three CTAs per SM (three images with 28 query heads: 168 CTAs of
+  // very different length took 26 us, twice as many take 20; with five per SM k_tokens has no room beside them)
   const int nvq = bt.n_qcols / Vec<T>::N;
   const bool narrow = (nvq + 3) / 4 * bt.B * kQPartRows <= 2 * g_sm_count;
   const int ncg = narrow ? (nvq + 3) / 4 : (nvq + 7) / 8;
   LaunchOpt opt;
   opt.cluster = 1;
-  while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 2 * g_sm_count) opt.cluster *= 2;
+  while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 3 * g_sm_count) opt.cluster *= 2;
   const dim3 grid(ncg * opt.cluster, bt.B), block(kQsumThreads);
   return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster);
 }
