@@ -834,6 +834,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant
 // grid (1), 1024 threads; dynamic smem: N keys when KPT == 0 and keys_in_smem.
 // KPT > 0: thread t keeps the keys of tokens [t KPT, t KPT + KPT) in registers (N <= 1024 KPT);
 // KPT == 0: any N, keys in shared memory when they fit, else re-read from the scores.
+constexpr int kSplitBits = 11;
+
 template <int KPT>
 __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt, int keys_in_smem) {
   const ImgDesc &im = bt.img[blockIdx.y];
@@ -843,11 +845,11 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int N = im.N;
   extern __shared__ uint32_t skey[];                        // [N] when KPT == 0 and keys_in_smem
-  __shared__ int hist[256];
+  __shared__ __align__(8) int hist[1 << kSplitBits];
   __shared__ int warp_tot[32];
   __shared__ uint32_t wmin[32], wmax[32];
   __shared__ uint32_t s_prefix;
-  __shared__ int s_k;
+  __shared__ int s_k, s_cnt;
   constexpr int KR = KPT > 0 ? KPT : 1;
   const int CH = KPT > 0 ? KPT : (N + 1023) / 1024;         // tokens per thread, contiguous
   const int i0 = min(N, t * CH), i1 = min(N, i0 + CH);
@@ -865,7 +867,7 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
     for (int i = t; i < N; i += 1024) skey[i] = score_key(im.score[i]);
   }
   if (t == 0) s_k = im.m_target;
-  if (t < 256) hist[t] = 0;
+  reinterpret_cast<int2 *>(hist)[t] = make_int2(0, 0);
   __syncthreads();
   // j-th key of this thread (j < cnt_mine)
   auto key = [&](int j) -> uint32_t {
@@ -894,55 +896,59 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
   if (t == 0) s_prefix = 0u;
   __syncthreads();
 
-  // radix select of the (m_target + 1)-th smallest key over the varying bits, up to 8 bits per pass
-  for (int hi = top; hi > 0; hi -= 8) {
-    const int lo = hi > 8 ? hi - 8 : 0;
+  // Radix select of the (m_target + 1)-th smallest key over the varying bits, up to eleven bits per pass: the first pass
+  // leaves a few candidates, the second nearly always one (eight bits and one warp to scan the bins: four passes, 5 us of 11).
+  for (int hi = top; hi > 0; hi -= kSplitBits) {
+    const int lo = hi > kSplitBits ? hi - kSplitBits : 0;
     const uint32_t dmask = (1u << (hi - lo)) - 1u;
     const uint32_t above = hi >= 32 ? 0u : ~((1u << hi) - 1u);   // bits already fixed
     const uint32_t prefix = s_prefix;
+    const int k = s_k;
     if (KPT > 0) {
 #pragma unroll
       for (int j = 0; j < KR; ++j) {
         const uint32_t kk = kreg[j] - kbase;
-        if (j < cnt_mine && (kk & above) == (prefix & above)) atomicAdd(&hist[(kk >> lo) & dmask], 1);
+        if (j < cnt_mine && (kk & above) == prefix) atomicAdd(&hist[(kk >> lo) & dmask], 1);
       }
     } else {
       for (int j = 0; j < cnt_mine; ++j) {
         const uint32_t kk = key(j) - kbase;
-        if ((kk & above) == (prefix & above)) atomicAdd(&hist[(kk >> lo) & dmask], 1);
+        if ((kk & above) == prefix) atomicAdd(&hist[(kk >> lo) & dmask], 1);
       }
     }
     __syncthreads();
-    if (w == 0) {
-      int c[8], s = 0;
+    const int2 c = reinterpret_cast<const int2 *>(hist)[t];      // every thread takes two bins
+    reinterpret_cast<int2 *>(hist)[t] = make_int2(0, 0);
+    int incl = c.x + c.y;
 #pragma unroll
-      for (int b = 0; b < 8; ++b) { c[b] = hist[lane * 8 + b]; s += c[b]; }
-      int incl = s;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int k = s_k;
-      const unsigned has = __ballot_sync(0xffffffffu, incl > k);
-      const int L = has ? __ffs(has) - 1 : 31;   // the candidates always number more than k
-      if (lane == L) {
-        int kk = k - (incl - s), dgt = 7;
-        bool done = false;
-#pragma unroll
-        for (int b = 0; b < 7; ++b) {
-          if (!done) {
-            if (kk < c[b]) { dgt = b; done = true; }
-            else kk -= c[b];
-          }
-        }
-        s_k = kk;
-        s_prefix = prefix | ((uint32_t)(lane * 8 + dgt) << lo);
-      }
-#pragma unroll
-      for (int b = 0; b < 8; ++b) hist[lane * 8 + b] = 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_tot[w] = incl;
+    __syncthreads();
+    const int below = incl - c.x - c.y + __reduce_add_sync(0xffffffffu, lane < w ? warp_tot[lane] : 0);
+    if (below <= k && k < below + c.x + c.y) {                   // exactly one thread: the candidates number more than k
+      const bool second = k >= below + c.x;
+      s_k = k - below - (second ? c.x : 0);
+      s_cnt = second ? c.y : c.x;
+      s_prefix = prefix | ((uint32_t)(2 * t + (second ? 1 : 0)) << lo);
     }
     __syncthreads();
+    if (lo > 0 && s_cnt == 1) {                                  // one key left under the prefix: it is the threshold
+      const uint32_t fixed = ~((1u << lo) - 1u), pre = s_prefix;
+      __syncthreads();
+      if (KPT > 0) {
+#pragma unroll
+        for (int j = 0; j < KR; ++j)
+          if (j < cnt_mine && ((kreg[j] - kbase) & fixed) == pre) s_prefix = kreg[j] - kbase;
+      } else {
+        for (int j = 0; j < cnt_mine; ++j)
+          if (((key(j) - kbase) & fixed) == pre) s_prefix = key(j) - kbase;
+      }
+      __syncthreads();
+      break;
+    }
   }
   const uint32_t tau_key = s_prefix + kbase;
 
@@ -998,7 +1004,7 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
 namespace {
 int g_sm_count = 148;
 size_t g_smem_optin = 48 * 1024;
-constexpr size_t kSplitReserve = 4096;       // static shared memory of k_split, rounded up
+constexpr size_t kSplitReserve = 12288;      // static shared memory of k_split, rounded up
 }  // namespace
 
 template <typename T>
