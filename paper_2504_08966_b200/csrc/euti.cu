@@ -574,13 +574,14 @@ __global__ void __launch_bounds__(256) k_scores(const __grid_constant__ Batch bt
 }
 
 // ---- Eq. 3-4 in the whole step: threshold, ordered compaction, survivor keys (Eq. 7) ------------------------
-// grid (X, B), 512 threads, two CTAs per SM; dynamic smem: N sort keys when they fit.  CTA x owns the tokens
+// grid (X, B), 512 threads, one or two CTAs per SM; dynamic smem: N sort keys when they fit.  CTA x owns the tokens
 // [x tpc, (x + 1) tpc).  Every CTA selects the threshold itself (identical in all of them), counts the
 // survivors before its tokens, writes keep flags, lists and slots of its tokens and copies the clustering keys
 // of its survivors to their rows of K'.
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kHistPerThread = (1 << kHistBits) / kSelThreads;
+constexpr size_t kSelKeyBytes = 96 * 1024;     // most sort keys kept in shared memory
 constexpr int kSelBits = 10;                  // key bits per pass of the selection below the first-level histogram
 constexpr int kSelPerThread = (1 << kSelBits) / kSelThreads;
 static_assert(kHistPerThread % 4 == 0 && kHistPerThread * kSelThreads == (1 << kHistBits), "histogram split");
@@ -813,8 +814,10 @@ __device__ __forceinline__ void euti_select(const Batch &bt, const ImgDesc &im, 
   euti_compact<T, KPT, IN_SMEM>(bt, im, skey, kreg, tau_key, g, tok0, ntok, sh);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant__ Batch bt, int keys_in_smem) {
+// KPT > 0: N <= 512 KPT for every image.  (A kernel for each case: the code runs once, from a cold instruction cache, and
+// for images of up to 3072 tokens six keys per thread in place of sixteen take 2 us off the call.)
+template <typename T, int KPT, bool IN_SMEM>
+__global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant__ Batch bt) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 3);
   pdl_wait();
@@ -824,9 +827,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant
   const int N = im.N, X = gridDim.x, x = blockIdx.x;
   const int tpc = (N + X - 1) / X;
   const int tok0 = min(N, x * tpc), ntok = min(N, tok0 + tpc) - tok0;
-  if (keys_in_smem && N <= 16 * kSelThreads) euti_select<T, 16, true>(bt, im, skey_dyn, x, tok0, ntok, sh);
-  else if (keys_in_smem) euti_select<T, 0, true>(bt, im, skey_dyn, x, tok0, ntok, sh);
-  else euti_select<T, 0, false>(bt, im, skey_dyn, x, tok0, ntok, sh);
+  euti_select<T, KPT, IN_SMEM>(bt, im, skey_dyn, x, tok0, ntok, sh);
 }
 
 // ---- Eq. 3-4 as a stage of its own (pact_prune): order statistic, ordered compaction ------------------
@@ -1087,13 +1088,17 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   if (mode == 0) {
     if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
     size_t keys = (size_t)maxN * sizeof(uint32_t);
-    const int in_smem = keys <= 96 * 1024;
+    const bool in_smem = keys <= kSelKeyBytes;
     if (!in_smem) keys = 0;
-    int X = 2 * g_sm_count / bt.B;
+    // One CTA per SM while it has few tokens: all of them begin beside k_scores (with two a tenth waited for its end; one
+    // image of 7290 tokens: 1.9 us).  With more than 128 tokens the lists and rows of K' are what counts, and two share them.
+    int X = g_sm_count / bt.B;
+    if (X < 1 || (maxN + X - 1) / X > 128) X = 2 * g_sm_count / bt.B;
     const int want = (maxN + 15) / 16;         // at least sixteen tokens per CTA
     if (X > want) X = want;
     if (X < 1) X = 1;
-    e = launch_k(k_select<T>, dim3(X, bt.B), dim3(kSelThreads), keys, st, true, bt, in_smem);
+    const auto kernel = maxN <= 6 * kSelThreads ? k_select<T, 6, true> : maxN <= 16 * kSelThreads ? k_select<T, 16, true> : in_smem ? k_select<T, 0, true> : k_select<T, 0, false>;
+    e = launch_k(kernel, dim3(X, bt.B), dim3(kSelThreads), keys, st, true, bt);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
@@ -1144,11 +1149,8 @@ cudaError_t euti_configure(int n_qcols) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_tokens<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok);
   if (e != cudaSuccess) return e;
-  const int dyn = 96 * 1024;
-  e = cudaFuncSetAttribute(k_select<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_select<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-  if (e != cudaSuccess) return e;
+  for (const auto f : {k_select<__nv_bfloat16, 0, true>, k_select<float, 0, true>})   // (the others need less than the default)
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelKeyBytes)) != cudaSuccess) return e;
   // k_tokens can only begin beside k_qsum if both run under the same split of the SM's memory (with the default it waited
   // for k_qsum to drain, 9 us at 6272 tokens); for the other kernels the default is as good or better (16384-token images: 10 us)
   return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16>, k_tokens<float>);

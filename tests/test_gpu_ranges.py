@@ -98,6 +98,12 @@ def test_small_batches(B):
     _check(wl, torch.bfloat16)
 
 
+@pytest.mark.parametrize("N", [3072, 3073, 8192, 8193])
+def test_select_key_registers(N):
+    """The last size with the keys of the split in six, in sixteen registers per thread, and the first without."""
+    _check(_workload(N, 2, 1, 16, 32, torch.bfloat16, N), torch.float32)
+
+
 @pytest.mark.parametrize("case", ["many rows", "more survivors than estimated"])
 def test_centres_outside_shared_memory(case):
     """Blocks of more than 1024 rows, adjacency words and densities that stay in global memory."""
