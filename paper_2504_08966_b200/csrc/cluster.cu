@@ -599,8 +599,9 @@ cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCf
   const size_t smem = (size_t)mask_cap * 4 + (size_t)keys_cap * 8 + adj;
   const cudaError_t e = launch_k(k_centers, dim3(cfg.sm_count > bt.B ? cfg.sm_count : bt.B), dim3(kCenThreads), smem, st, true, bt, mask_cap, keys_cap, (int)adj, sweep_limit);
   if (e != cudaSuccess) return e;
-  // a warp for two rows, but no more than eight CTAs per SM in all
-  const int most = 8 * cfg.sm_count / bt.B, want = (maxQ + 2 * kCenKeyThreads / 32 - 1) / (2 * kCenKeyThreads / 32), X = want < most ? want : most;
+  // a warp for a row (two rows: 1 us more of one image), but no more than four CTAs per SM in all: each reads the masks of
+  // its image (with eight: 2 us more of 16 images)
+  const int most = 4 * cfg.sm_count / bt.B, want = (maxQ + kCenKeyThreads / 32 - 1) / (kCenKeyThreads / 32), X = want < most ? want : most;
   const dim3 grid(X > 0 ? X : 1, bt.B), block(kCenKeyThreads);
   return bf16 ? launch_k(k_center_keys<__nv_bfloat16>, grid, block, (size_t)mask_cap * 12, st, true, bt, mask_cap)
               : launch_k(k_center_keys<float>, grid, block, (size_t)mask_cap * 12, st, true, bt, mask_cap);
