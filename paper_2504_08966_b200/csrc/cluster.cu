@@ -229,6 +229,7 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 // k_center_keys: cluster ids (number of centres with a lower index), centre list, centre keys and inverse norms.
 constexpr int kCenThreads = 1024;
 constexpr int kCenWarps = kCenThreads / 32;
+static_assert(kCenWarps == 32, "lane k of warp w has row w + 32 k");
 constexpr int kCenPasses = 1 << 13;                      // most passes of k_center_keys over open rows
 constexpr int kCenSweeps = 512;                          // sweeps of k_centers (about a microsecond each)
 

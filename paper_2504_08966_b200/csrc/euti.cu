@@ -464,7 +464,8 @@ constexpr int kScoreWarps = 8;
 constexpr int kScoreHeads = 32;                         // heads whose factors are in shared memory at a time
 constexpr int kScorePieces = 256 / kMinPiece + 1;       // most pieces that 256 tokens belong to
 
-__global__ void __launch_bounds__(256) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist) {
+// (Three CTAs per SM: at 112 registers a call of three images with 28 heads took 1 us more.)
+__global__ void __launch_bounds__(256, 3) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 2);
   pdl_wait();
