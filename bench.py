@@ -31,15 +31,15 @@ N_COPIES = 4          # input copies rotated between steps so that no step finds
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under profiles/
 # (workload, kernel) -> bytes; absent = not captured for the kernel as it stands
 NCU_TRAFFIC: dict = {
-    ("single_image", "qsum"): 7.49e6,
-    ("single_image", "tokens"): 59.79e6 + 0.17e6,
-    ("single_image", "scores"): 0.34e6,
-    ("single_image", "select"): 3.86e6,
-    ("single_image", "gram_density"): 3.92e6,
-    ("single_image", "centers"): 2.74e6,
+    ("single_image", "qsum"): 7.48e6,
+    ("single_image", "tokens"): 59.80e6 + 0.23e6,
+    ("single_image", "scores"): 0.35e6,
+    ("single_image", "select"): 3.83e6,
+    ("single_image", "gram_density"): 3.91e6,
+    ("single_image", "centers"): 2.15e6 + 0.63e6,
     ("single_image", "assign"): 9.25e6,
     ("single_image", "label_lists"): 0.15e6,
-    ("single_image", "merge"): 52.33e6 + 0.35e6,
+    ("single_image", "merge"): 52.35e6 + 0.81e6,
 }
 
 
@@ -605,7 +605,7 @@ def main():
             "dtype": "bf16", "data": "synthetic",
             "config": {"workload": f"{wl.name} (LLaVA-OneVision-7B-shaped)", "images_per_step_per_gpu": B, "N": img0.N,
                        "text_tokens": T, "d": d, "d_k": d_k, "lambda": wl.lam, "d_c": wl.d_c, "alpha": wl.alpha,
-                       "d_n": wl.d_n, "out_dtype": "bf16", "launch": "CUDA graph replay of pact_reduce (pact_graph_launch): 9 kernels chained by programmatic dependent launch",
+                       "d_n": wl.d_n, "out_dtype": "bf16", "launch": "CUDA graph replay of pact_reduce (pact_graph_launch): 10 kernels chained by programmatic dependent launch",
                        "l2": f"{copies} input copies rotated between steps ({in_bytes * copies / 1e6:.0f} MB > 126 MB L2)"
                              + ("; per-kernel pass also writes a 512 MB flush buffer" if flush is not None else "")},
             "latency_us": ms_per_step * 1e3 / B, "step_times": step_times, "stream_launch_ms_per_step": plain_ms,
