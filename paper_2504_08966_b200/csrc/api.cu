@@ -712,7 +712,7 @@ pact_status feed_and_reduce(pact_ctx *ctx, const pact_image *img, const pact_ima
     if (e == cudaSuccess) e = cudaEventRecord(feed.part[k], in);
   }
   pact_status s = e == cudaSuccess ? reduce_images(ctx, dv, 1, p, 0, ws, ws_bytes, st, &feed) : fail_cuda(ctx, e, "pact_reduce_host");
-  if (s == PACT_OK) ctx->launches += kFeedParts;
+  if (s == PACT_OK) ctx->launches += 1 + (feed.end[1] > feed.end[0]);
   else (void)cudaStreamSynchronize(in);              // (the caller's stream need not have been ordered behind the copies)
   return s;
 }

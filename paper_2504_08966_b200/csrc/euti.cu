@@ -1073,12 +1073,13 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, st, &rpp);
   if (e != cudaSuccess) return e;
   for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
+    // (a part without visual tokens may still bring text rows, which k_merge copies)
+    if ((e = cudaStreamWaitEvent(st, feed->part[k], 0)) != cudaSuccess) return e;
     if (feed->end[k] <= first) continue;
     Batch part = bt;
     part.img[0].N = feed->end[k] - first;
     part.img[0].vis_start += first;
     part.img[0].nrm += first;
-    if ((e = cudaStreamWaitEvent(st, feed->part[k], 0)) != cudaSuccess) return e;
     if ((e = launch_tokens<T>(part, kTokNorms, false, st, nullptr)) != cudaSuccess) return e;
   }
   if (rpp_out) *rpp_out = rpp;

@@ -85,7 +85,7 @@ struct HostFeed {
 };
 cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark = nullptr,
                         void *mark_arg = nullptr, int *rpp = nullptr);   // rpp: receives the tokens per softmax piece
-// modes 0 and 2 for one image whose hidden states arrive in parts meanwhile (kFeedParts kernels more)
+// modes 0 and 2 for one image whose hidden states arrive in parts meanwhile (one kernel more for each part with visual tokens)
 cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, const HostFeed &feed, int *rpp);
 int euti_kernels(int mode);
 // threshold + ordered compaction of given scores (pact_prune, one image)

@@ -162,6 +162,39 @@ def test_host_buffers(N, T, vis, d, rope, pinned):
     assert bool((host["H_out"][n_out:] == 7).all()) and bool((host["P_out"][n_out:] == 7).all())
 
 
+def _host_call(wl, ctx, params=None):
+    """pact_reduce_host on pinned copies of the workload's image; the staging buffer holds nothing of an earlier call."""
+    from paper_2504_08966_b200 import binding as pb
+    img, n = wl.images[0], wl.images[0].n_total
+    z = lambda m, dt: torch.full(m, 7, dtype=dt).pin_memory()   # noqa: E731
+    host = dict(H=img.H.pin_memory(), K_euti=img.K.pin_memory(), Q_euti=img.Q.pin_memory(), P=img.P.pin_memory(), vis_start=img.vis_start, N=img.N,
+                H_out=z((n, wl.d), ctx.out_dtype), P_out=z((n,), torch.int32), size_out=z((n,), torch.int32), logw_out=z((n,), torch.float32),
+                label=z((img.N,), torch.int32), counters=z((16,), torch.int32))
+    host["K_clu"] = host["K_euti"]
+    staging = torch.full((ctx.host_staging_bytes(n, img.N),), 255, dtype=torch.uint8, device="cuda")
+    ctx.pact_reduce_host(host, params or pb.make_params(lam=wl.lam, d_c=wl.d_c), staging)
+    return host
+
+
+def _same_as_device(host, want):
+    n_out = int(host["counters"][0])
+    assert int(host["counters"][8]) == 0 and n_out == want["n_out"] and np.array_equal(host["label"].numpy(), want["label"])
+    for key in ("P_out", "size_out", "logw_out"):
+        assert np.array_equal(host[key][:n_out].numpy(), want[key])
+    assert torch.equal(host["H_out"][:n_out], want["H_out_raw"])
+
+
+@pytest.mark.parametrize("N", [1, 3, 7, 8, 9])
+def test_host_buffers_of_a_tiny_image_in_a_long_prompt(N):
+    """The part of the hidden states that holds no visual token still holds the text behind the image: 13 MB of it."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = _workload(N, 4, 2, 64, 3584, torch.bfloat16, N, T=1850)
+    ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
+    want = gpu_reduce(wl, torch.float32)[0][0]
+    for _ in range(3):
+        _same_as_device(_host_call(wl, ctx), want)
+
+
 def test_no_norm_and_norm_only():
     """Both forms of the score without one of its factors, over several units of the token pass."""
     from paper_2504_08966_b200 import binding as pb
