@@ -247,7 +247,7 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
     if (e == cudaSuccess && major != 10) { delete c; return PACT_ERR_UNSUPPORTED; }
   }
-  if (e == cudaSuccess) e = euti_configure(c->n_qcols);
+  if (e == cudaSuccess) e = euti_configure(c->n_qcols, n_qh);
   if (e == cudaSuccess) e = cluster_configure(&c->ccfg);
   if (e == cudaSuccess) e = merge_configure();
   if (e == cudaSuccess) e = small_configure();

@@ -200,11 +200,12 @@ struct TokCfg {
   int chunk, nchunk;                                    // bytes of a hidden-state row per copy, copies per row
   int nbuf;                                             // row buffers per warp
   int keys;                                             // a key buffer per team (else the keys are read from global memory)
+  int query;                                            // the global query in shared memory (else read from global memory)
 };
 // stride of a key row in shared memory: an odd number of 16-byte vectors, so that a vector of 8 rows is in 8 different banks
 __host__ __device__ inline int tok_key_stride(int row_bytes) { return row_bytes | 16; }
 inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
-  return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)n_qcols * 8 + (size_t)c.rpp * 32 * 8;
+  return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)c.query * n_qcols * 8 + (size_t)c.rpp * 32 * 8;
 }
 
 // Logits of this lane's token (its vectors p, p + P, ... of nv) with nr <= RB heads of a key head, q at one address per part.
@@ -303,7 +304,7 @@ __device__ __forceinline__ void plain_heads(const ImgDesc &im, int n_qh, const u
   }
 }
 
-template <typename T>
+template <typename T, bool QUERY>
 __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int what) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
   const int ks = tok_key_stride(bt.d_k * (int)sizeof(T));
   uint8_t *s_key = smem + (size_t)kTokWarps * cfg.nbuf * cfg.chunk;   // [2][rpp][ks], behind the row buffers
   double *s_q = reinterpret_cast<double *>(s_key + (size_t)2 * cfg.keys * rpp * ks);     // [n_qh][d_h] global query
-  double(*s_acc)[32] = reinterpret_cast<double(*)[32]>(s_q + bt.n_qcols);                // [rpp][32] parts of the sums of squares
+  double(*s_acc)[32] = reinterpret_cast<double(*)[32]>(s_q + (QUERY ? bt.n_qcols : 0));  // [rpp][32] parts of the sums of squares
   __shared__ int s_first[kMaxBatchPerLaunch + 1];                     // first unit of each image
   __shared__ uint64_t s_rbar[kTokWarps][kTokMaxBuf], s_kbar[2];
   __shared__ int s_abort, s_query;                                    // s_query: the global queries are complete
@@ -480,27 +481,28 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
         pdl_trigger();
       }
       const bool use_query = !(im.flags & PACT_FLAG_NORM_ONLY) && im.Q != nullptr;
-      if (use_query && loaded != b) {                    // both teams come by here for every image of the CTA's units
+      if (QUERY && use_query && loaded != b) {                  // both teams come by here for every image of the CTA's units
         if (loaded >= 0) sync_both();
         for (int c = threadIdx.x - kTokGroup; c < bt.n_qcols; c += kTokGroup) s_q[c] = ld_cg_f64(&im.qg[c]);
         loaded = b;
         sync_both();
       }
       if (!mine) continue;
+      const double *q = QUERY ? s_q : im.qg;
       const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
       const int nblk = (n_rep + 3) / 4;                  // blocks of up to four query heads per key head
       bool finite = true;
       for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
         const int kv = it / nblk, j = (it - kv * nblk) * 4, nr = min(4, n_rep - j), j0 = kv * n_rep + j;
         const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
-        if (nr >= 3) finite &= head_piece<T, 4>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else if (nr == 2) finite &= head_piece<T, 2>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else finite &= head_piece<T, 1>(bt, im, kh, s_q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        if (nr >= 3) finite &= head_piece<T, 4>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else if (nr == 2) finite &= head_piece<T, 2>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else finite &= head_piece<T, 1>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
       }
       if (__any_sync(0xffffffffu, !finite))
         for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
           const int kv = it / nblk, j = (it - kv * nblk) * 4, j0 = kv * n_rep + j;
-          plain_heads<T>(im, bt.n_qh, krow + (size_t)kv * d_h * sizeof(T), s_q + (size_t)j0 * d_h, d_h, P, min(4, n_rep - j), j0, r0, n, g);
+          plain_heads<T>(im, bt.n_qh, krow + (size_t)kv * d_h * sizeof(T), q + (size_t)j0 * d_h, d_h, P, min(4, n_rep - j), j0, r0, n, g);
         }
       if (cfg.keys && u + 2 < u1) {
         sync();                                          // the keys have been read
@@ -1069,6 +1071,7 @@ namespace {
 int g_sm_count = 148;
 size_t g_smem_optin = 48 * 1024;
 constexpr size_t kSplitReserve = 12288;      // static shared memory of k_split, rounded up
+constexpr size_t kTokReserve = 2048;         // of k_tokens
 }  // namespace
 
 template <typename T>
@@ -1087,7 +1090,8 @@ static cudaError_t launch_qsum(const Batch &bt, cudaStream_t st) {
 }
 
 // Tokens per unit: the fewest rounds of units of `most` tokens over the SMs, then as few tokens as that many rounds allow
-// (but eight), so that the rounds are full.
+// (but eight), so that the rounds are full.  Keys, then a part of the row buffers, then the global query (more than 26496
+// columns with the largest rows) go without shared memory where it is too small.
 template <typename T> static TokCfg tokens_config(const Batch &bt) {
   TokCfg c;
   long long total = 0;
@@ -1097,6 +1101,7 @@ template <typename T> static TokCfg tokens_config(const Batch &bt) {
   c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
   c.nbuf = kTokMaxBuf;
   c.keys = 1;
+  c.query = 1;
   const auto fits = [&]() { return tok_smem(c, keyb, bt.n_qcols) <= (size_t)kTokSmem; };
   for (int most = 32; most >= kMinPiece; most /= 2) {
     const long long rounds = (total + (long long)most * g_sm_count - 1) / ((long long)most * g_sm_count);
@@ -1109,6 +1114,7 @@ template <typename T> static TokCfg tokens_config(const Batch &bt) {
     c.nchunk *= 2;
     c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
   }
+  c.query = tok_smem(c, keyb, bt.n_qcols) <= g_smem_optin - kTokReserve;
   return c;
 }
 static int tokens_grid(const Batch &bt, int rpp) {
@@ -1121,7 +1127,7 @@ template <typename T>
 static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, cudaStream_t st, int *rpp) {
   const TokCfg tc = tokens_config<T>(bt);
   if (rpp) *rpp = tc.rpp;
-  return launch_k(k_tokens<T>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
+  return launch_k(tc.query ? k_tokens<T, true> : k_tokens<T, false>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
 }
 
 template <typename T>
@@ -1202,22 +1208,20 @@ cudaError_t select_configure() {
   return e;
 }
 
-cudaError_t euti_configure(int n_qcols) {
+cudaError_t euti_configure(int n_qcols, int n_qh) {
   cudaError_t e = select_configure();
   if (e != cudaSuccess) return e;
-  // the widest query and the narrowest of everything else have to fit
-  if ((size_t)n_qcols * 8 + kMinPiece * 32 * 8 + kTokWarps * 1040 + 64 > g_smem_optin - 4096)
-    return cudaErrorInvalidConfiguration;
-  const int tok = (int)(g_smem_optin - 2048);
-  e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_tokens<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok);
-  if (e != cudaSuccess) return e;
+  if ((size_t)(n_qcols + 32 * n_qh) * 8 > g_smem_optin - 1024) return cudaErrorInvalidConfiguration;   // the widest query
+  const int tok = (int)(g_smem_optin - kTokReserve);
+  if ((e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_tokens<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_tokens<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
   for (const auto f : {k_select<__nv_bfloat16, 0, true>, k_select<float, 0, true>})   // (the others need less than the default)
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelKeyBytes)) != cudaSuccess) return e;
   // k_tokens can only begin beside k_qsum if both run under the same split of the SM's memory (with the default it waited
   // for k_qsum to drain, 9 us at 6272 tokens); for the other kernels the default is as good or better (16384-token images: 10 us)
-  return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16>, k_tokens<float>);
+  return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16, true>, k_tokens<float, true>);
 }
 
 }  // namespace pact

@@ -90,7 +90,7 @@ cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cuda
 int euti_kernels(int mode);
 // threshold + ordered compaction of given scores (pact_prune, one image)
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st);
-cudaError_t euti_configure(int n_qcols);
+cudaError_t euti_configure(int n_qcols, int n_qh);
 cudaError_t select_configure();            // what launch_split needs, once per device
 
 // cluster.cu

@@ -236,3 +236,20 @@ def test_non_finite_queries_and_keys_reach_the_scores(N, n_qh, n_kvh, d_h, dtype
                 torch.cuda.synchronize()
                 assert bool(im.score.isnan().all()) and int(im.counters[pb.CNT["q"]]) == N and int(im.counters[pb.CNT["status"]]) == 0
         t[N - 2, col] = old
+
+
+@pytest.mark.parametrize("n_qh,n_kvh,d_h,d,dtype", [
+    (1, 1, 26496, 8192, torch.bfloat16),      # the last width whose query fits beside the smallest row buffers
+    (1, 1, 26504, 8192, torch.bfloat16), (1, 1, 28896, 64, torch.bfloat16), (32, 1, 872, 3584, torch.bfloat16), (1, 1, 28896, 2056, torch.float32),
+])
+def test_widest_queries(n_qh, n_kvh, d_h, d, dtype):
+    """Queries that leave little or no shared memory to the token pass; 28928 columns less 32 per head are the most that are taken."""
+    from paper_2504_08966_b200 import binding as pb
+    N = 43
+    g = torch.Generator().manual_seed(d_h)
+    t = lambda m, n: (0.1 * torch.randn(m, n, generator=g)).to(dtype)   # noqa: E731
+    img = workloads.Image(H=t(N, d), K=t(N, n_kvh * d_h), Q=t(N, n_qh * d_h), P=torch.arange(N, dtype=torch.int32), n_total=N, vis_start=0, N=N)
+    wl = workloads.Workload("wide", [img], d, n_qh, n_kvh, d_h, dtype, 0.5, 0.3)
+    _check(wl, torch.float32)
+    with pytest.raises(pb.PactError):
+        pb.Context(64, 1, 1, 28904, dtype, torch.float32)
