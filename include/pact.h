@@ -71,7 +71,8 @@ enum {
   PACT_CNT_C = 2,         /* clusters                                                           */
   PACT_CNT_R = 3,         /* pruned tokens that rejoined a cluster                              */
   PACT_CNT_DISCARDED = 4, /* pruned tokens that did not                                         */
-  PACT_CNT_SWEEPS = 5,    /* largest number of passes any row needed in the centre selection    */
+  PACT_CNT_SWEEPS = 5,    /* most sweeps over its rows any CTA made in the centre selection, and passes over
+                             rows left open after them; depends on timing                         */
   PACT_CNT_BAND_DC = 6,   /* unordered surviving pairs with |d - d_c| <= 1e-6                   */
   PACT_CNT_BAND_ADC = 7,  /* pruned tokens whose nearest-centre distance is within 1e-6 of alpha*d_c */
   PACT_CNT_STATUS = 8,    /* 0, or a negative pact_status raised on the device                  */
@@ -145,8 +146,9 @@ const char *pact_last_cuda_error(const pact_ctx *ctx);
  * and the member lists of Eq. 10 are built behind one barrier between CTAs).  When a bound is reached the
  * kernel stops waiting, writes PACT_ERR_TIMEOUT to counters[PACT_CNT_STATUS] of the image and carries on
  * within bounds; the call itself still returns PACT_OK and the outputs of that image are not valid.
- * barrier_polls: polls of the member-list barrier; center_sweeps: sweeps of the centre selection;
- * 0 restores the default (about a million).  Graphs recorded earlier keep the limits they were recorded with. */
+ * barrier_polls: polls of the member-list barrier; center_sweeps: sweeps of the centre selection (rows that are
+ * still open are then decided without waiting, in at most one pass per surviving token; the same happens, with no
+ * status, when no row has been removed for 512 sweeps); 0 restores the default (about a million).  Graphs recorded earlier keep the limits they were recorded with. */
 pact_status pact_set_wait_limits(pact_ctx *ctx, int barrier_polls, int center_sweeps);
 
 /* ---- instrumentation ---------------------------------------------------------------------- */

@@ -221,8 +221,10 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 // rows to shared memory once (thousands of warps polling the same few L2 lines queue up there), and its warps decide what
 // they can from the copy.  Bound by latency, a trip to the L2 per sweep: 7 us for one image of 3645 survivors, 10 us for 16
 // of 1458, 15 us for 4 of 4916.
-// CTAs wait for one another's decisions but need not be resident together: after kCenSweeps sweeps a CTA leaves its open
-// rows to k_center_keys, where every CTA resolves what is open by itself.  (As a cooperative launch the kernel could not
+// CTAs wait for one another's decisions but need not be resident together: after kCenIdle sweeps in which no row of the image
+// was removed a CTA leaves its open rows to k_center_keys, where every CTA resolves what is open by itself.  (Progress is
+// what counts, not the number of sweeps: 2600 rows whose decisions hang on one another in a chain of 1300 take 1300 sweeps
+// and more, and left to k_center_keys after 512 they took 175 ms.)  (As a cooperative launch the kernel could not
 // begin beside the one before, which cost a call on a stream 4 us.  One cluster of 16 CTAs per image, with masks in each
 // other's shared memory, was no faster with 16 images and 18 us slower with one: 16 SMs are too few to take in the rows.)
 //
@@ -230,8 +232,7 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 constexpr int kCenThreads = 1024;
 constexpr int kCenWarps = kCenThreads / 32;
 static_assert(kCenWarps == 32, "lane k of warp w has row w + 32 k");
-constexpr int kCenPasses = 1 << 13;                      // most passes of k_center_keys over open rows
-constexpr int kCenSweeps = 512;                          // sweeps of k_centers (about a microsecond each)
+constexpr int kCenIdle = 512;                            // sweeps of k_centers without a removed row (about a microsecond each)
 
 // One row against the removed rows, by a warp: an earlier neighbour that is not removed, or -1.
 __device__ __forceinline__ int open_earlier(const uint32_t *row, const uint32_t *removed, const unsigned long long *keys, int r, int nw, int lane) {
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
 
   int wit = -1;                                          // witness of row wid + 32 lane
   bool done = false;                                     // that row is a centre
-  int sweeps = 0;
+  int sweeps = 0, idle = 0;
   for (;;) {
     int pending = 0;
     ++sweeps;
@@ -336,12 +337,17 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
       }
     }
     if (!__syncthreads_or(pending)) break;               // no row of this CTA is open
-    if (sweeps >= sweep_limit || sweeps >= kCenSweeps) {
+    if (sweeps >= sweep_limit || idle >= kCenIdle) {
       if (t == 0 && sweeps >= sweep_limit) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
       break;
     }
-    for (int wd = t; wd < nw; wd += kCenThreads) rm[wd] = ld_relaxed_u32(&im.rmask[wd]);
-    __syncthreads();
+    int moved = 0;
+    for (int wd = t; wd < nw; wd += kCenThreads) {
+      const uint32_t x = ld_relaxed_u32(&im.rmask[wd]);
+      moved |= x != rm[wd];
+      rm[wd] = x;
+    }
+    idle = __syncthreads_or(moved) ? 0 : idle + 1;
   }
   TL_POINT(bt.img[0], 11);
   if (t == 0) atomicMax(&im.cnt[PACT_CNT_SWEEPS], sweeps);
@@ -374,7 +380,8 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
   }
   if (__syncthreads_or(open)) {
     // Rows that k_centers left: every CTA resolves them, to the same end (the set is unique), against its own copies;
-    // the first CTA also writes the centres for later kernels.
+    // the first CTA also writes the centres for later kernels.  The earliest open row is decided in every pass, so q passes
+    // are enough.
     int passes = 0;
     do {
       open = 0;
@@ -402,11 +409,12 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
           if (e) atomicOr(&rm[wd], e);
         }
       }
-      if (++passes >= kCenPasses) {
+      if (++passes > q) {
         if (t == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
         open = 0;
       }
-    } while (__syncthreads_or(open));                    // (the earliest open row is decided in every pass)
+    } while (__syncthreads_or(open));
+    if (blockIdx.x == 0 && t == 0) im.cnt[PACT_CNT_SWEEPS] += passes;
   }
   for (int base = 0; base < nw; base += kCenKeyThreads) {
     const int wd = base + t, pc = wd < nw ? __popc(cm[wd]) : 0;

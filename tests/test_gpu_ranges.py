@@ -253,3 +253,25 @@ def test_widest_queries(n_qh, n_kvh, d_h, d, dtype):
     _check(wl, torch.float32)
     with pytest.raises(pb.PactError):
         pb.Context(64, 1, 1, 28904, dtype, torch.float32)
+
+
+@pytest.mark.parametrize("N,limit", [(600, 0), (2601, 0), (600, 1)])
+def test_a_chain_of_centres(N, limit):
+    """Row k is a neighbour of rows k - 1 and k + 1 only and all densities but the ends' are equal: rows 1, 3, 5, ... become
+    centres one after the other, more of them than the sweeps a CTA may spend without seeing progress."""
+    from paper_2504_08966_b200 import binding as pb
+    d_k = (N + 64) // 64 * 64
+    i = torch.arange(N, device="cuda")
+    K = torch.zeros(N, d_k, dtype=torch.bfloat16, device="cuda")
+    K[i, i] = 1
+    K[i, i + 1] = 1                           # neighbours at distance 1/2, all others at 1
+    ctx = pb.Context(64, 1, 1, d_k, torch.bfloat16, torch.float32)
+    ctx.set_wait_limits(center_sweeps=limit)
+    z = lambda n, dt=torch.int32: torch.zeros(n, dtype=dt, device="cuda")   # noqa: E731
+    cidx, C, label, cnt = z(N), z(1), z(N), z(16)
+    ctx.pact_dbdpc(K, i.int(), torch.tensor([N], dtype=torch.int32, device="cuda"), pb.make_params(lam=0.0, d_c=0.75), z(N, torch.float32), cidx, C, label, cnt)
+    want = list(range(1, N - 1, 2)) + ([N - 1] if N % 2 == 0 else [])     # an end's density is the smallest
+    assert cidx[:int(C)].tolist() == want
+    assert label.tolist() == [max(0, (k - 1) // 2) for k in range(N)]
+    assert int(cnt[pb.CNT["status"]]) == (-5 if limit else 0)
+    assert int(cnt[pb.CNT["sweeps"]]) > (512 if N > 2000 else 1)
