@@ -64,6 +64,7 @@ template <typename T> struct SmallShared {
   int wsum[kSmWarps];
   int C;
   uint64_t acc_bar;
+  uint64_t done;                                       // after a wait that ran out: every MMA this CTA has issued is complete
   uint32_t tmem_base;
   int abort;
 };
@@ -94,15 +95,19 @@ __device__ __forceinline__ int pow2_ceil(int x) { return x <= 1 ? 1 : 1 << (32 -
 // One tile of dot products on the tensor core, rows of both operands gathered from K by token (a negative token gives
 // a row of zeros).  tokA: tokens of the rows t / 8 and t / 8 + 64 that this thread copies, tokB: token of row t / 8 of
 // the other operand (nB rows); same: the 128 rows against themselves.  The accumulator (tensor-memory columns 0 ..)
-// is complete on return.
+// is complete when the calling warp gets true; false: the wait for it ran out.  The CTA then goes on through its few tiles
+// (every wait is bounded, and the status word says that the results are not valid, whatever operands an MMA still read) and
+// finish_mmas() comes before it gives its tensor memory back.  (To leave the loops together takes an or-barrier or a flag per tile, 0.6 to 0.9 us
+// of an image of 729 tokens.)
 template <typename Sh>
-__device__ __forceinline__ void small_tile(Sh &sh, uint8_t *buf, uint32_t &phase, const __nv_bfloat16 *K, long long ldK, int d_k,
+__device__ __forceinline__ bool small_tile(Sh &sh, uint8_t *buf, uint32_t &phase, const __nv_bfloat16 *K, long long ldK, int d_k,
                                            const int (&tokA)[2], int tokB, int nB, bool same) {
   const int t = threadIdx.x, piece = t & 7, row0 = t >> 3;
   const uint32_t a0 = smem_u32(buf), b0 = same ? a0 : a0 + kSmSlabs * kSmABytes;
   const uint32_t at = row0 * 128 + ((piece ^ (row0 & 7)) << 4);          // 128-byte swizzle (rows + 64: the same)
   const __nv_bfloat16 *srcA0 = K + (long long)max(tokA[0], 0) * ldK + piece * 8, *srcA1 = K + (long long)max(tokA[1], 0) * ldK + piece * 8;
   const __nv_bfloat16 *srcB = K + (long long)max(tokB, 0) * ldK + piece * 8;
+  bool ok = true;
   for (int k0 = 0; k0 < d_k; k0 += kSmSlabs * kSmBK) {
     const int n = min(kSmSlabs, (d_k - k0) / kSmBK);
     // (through registers: twice the rate of 16-byte asynchronous copies, see bulk_load in tma.cuh)
@@ -141,10 +146,19 @@ __device__ __forceinline__ void small_tile(Sh &sh, uint8_t *buf, uint32_t &phase
           umma_bf16(sh.tmem_base, smem_desc(a0 + h * kSmABytes + k * 32), smem_desc(b0 + h * bstep + k * 32), idesc, (k0 | h | k) != 0);
       umma_commit(&sh.acc_bar);
     }
-    if (!mbar_wait_warp(&sh.acc_bar, phase)) sh.abort = 1;
+    ok = mbar_wait_warp(&sh.acc_bar, phase);
+    if (!ok) sh.abort = 1;
     phase ^= 1;
   }
   tc_fence_after();
+  return ok;
+}
+
+// No MMA may still be running when the tensor memory is given back.  (A call: code that hardly ever runs costs its place in
+// the instruction stream, 0.5 us of an image of 729 tokens.)
+__device__ __noinline__ void finish_mmas(uint64_t *done) {
+  umma_commit(done);
+  mbar_wait(done, 0);
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -228,6 +242,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   if constexpr (UMMA) { if (w == 0) tmem_alloc(&sh.tmem_base, 128); }
   if (t == 0) {
     mbar_init(&sh.acc_bar, 1);
+    mbar_init(&sh.done, 1);
     sh.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -351,9 +366,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         tokA[k] = ra < q ? sh.kept[ra] : -1;
       }
       const int rb = c00 + (t >> 3);
-      small_tile(sh, dyn, phase, Kc, im.ldKc, bt.d_k, tokA, rb < q ? (int)sh.kept[rb] : -1, kSmBN, diag);
+      const bool ok = small_tile(sh, dyn, phase, Kc, im.ldKc, bt.d_k, tokA, rb < q ? (int)sh.kept[rb] : -1, kSmBN, diag);
       const int qd = w & 3, k0 = (w >> 2) * 32, c0 = c00 + k0, r0 = tm * kSmBM + qd * 32, row = r0 + lane;
-      if (c0 < q && (diag || k0 < kSmBN)) {
+      if (ok && c0 < q && (diag || k0 < kSmBN)) {
         constexpr float kHuge = 1e19f;                 // a vanishing key: see epi_tile
         float rnj = c0 + lane < q ? (float)sh.rn[sh.kept[c0 + lane]] : 0.f, rni = row < q ? (float)sh.rn[sh.kept[row]] : 0.f;
         if (rnj > kHuge) rnj = 0.f;
@@ -519,9 +534,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         tokA[k] = ra < N ? ra : -1;
       }
       const int rb = cb + (t >> 3);
-      small_tile(sh, dyn, phase, Kc, im.ldKc, bt.d_k, tokA, rb < C ? (int)sh.cen[rb] : -1, CW, false);
+      const bool ok = small_tile(sh, dyn, phase, Kc, im.ldKc, bt.d_k, tokA, rb < C ? (int)sh.cen[rb] : -1, CW, false);
       const int qd = w & 3, row = blk * kSmBM + qd * 32 + lane, k0 = (w >> 2) * 32, c0 = cb + k0;
-      const int lim = min(min(32, CW - k0), C - c0);
+      const int lim = ok ? min(min(32, CW - k0), C - c0) : 0;
       if (lim > 0) {
         sh.rn_col[w][lane] = lane < lim ? (float)sh.rn[sh.cen[c0 + lane]] : 0.f;
         __syncwarp();
@@ -598,7 +613,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
     }
     if (t == 0 && sh.abort) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
   }
-  if constexpr (UMMA) { if (w == 0) tmem_dealloc(sh.tmem_base, 128); }
+  if constexpr (UMMA) {
+    if (w == 0) {
+      if (lane == 0 && sh.abort) finish_mmas(&sh.done);
+      __syncwarp();
+      tmem_dealloc(sh.tmem_base, 128);
+    }
+  }
   cluster_sync();
   TL_POINT(im, 10);
 
