@@ -350,6 +350,7 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
     idle = __syncthreads_or(moved) ? 0 : idle + 1;
   }
   TL_POINT(bt.img[0], 11);
+  if (in_smem && !mbar_try_wait(&s_bar, 0)) land_copies(&s_bar, 1);   // (only after a wait that ran out)
   if (t == 0) atomicMax(&im.cnt[PACT_CNT_SWEEPS], sweeps);
 }
 

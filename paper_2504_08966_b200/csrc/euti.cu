@@ -382,7 +382,10 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
       for (int r = w; r < n; r += kTokWarps) {
         double a0 = 0.0, a1 = 0.0;
         for (int c = 0; c < cfg.nchunk; ++c) {
-          if (!mbar_wait_warp(&s_rbar[w][slot], (par >> slot) & 1)) s_abort = 1;
+          if (!mbar_wait_warp(&s_rbar[w][slot], (par >> slot) & 1)) {
+            s_abort = 1;
+            goto norms_end;
+          }
           par ^= 1u << slot;
           const uint4 *row = reinterpret_cast<const uint4 *>(s_rows + (size_t)slot * cfg.chunk);
           const int nv = min(cfg.chunk, bt.d * (int)sizeof(T) - c * cfg.chunk) / 16;
@@ -410,13 +413,14 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
       __syncwarp();
       finish_row_sums(s_acc, w, kTokWarps, n, [&](int r, double s) { im.nrm[r0 + r] = sqrt(s); });
     }
+norms_end:
     pdl_wait();
   } else {
     const int team = threadIdx.x >= kTokGroup + kTokTeam, t = threadIdx.x & (kTokTeam - 1), w = t >> 5;   // within the team
     const int P = rpp <= 8 ? 4 : rpp <= 16 ? 2 : 1;     // lanes per token
     uint8_t *s_mine = s_key + (size_t)team * rpp * ks;
     auto issue_keys = [&](int u) {                      // lane 0 of every warp: its share of the scoring keys of unit u
-      if (u >= u1) return;
+      if (u >= u1 || *const_cast<volatile int *>(&s_abort)) return;
       const int b = image_of(u, 0);
       const ImgDesc &im = bt.img[b];
       const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
@@ -455,7 +459,7 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
       const uint8_t *keys = cfg.keys ? s_mine : reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.Ke) + (size_t)r0 * im.ldKe);
       const size_t kstride = cfg.keys ? (size_t)ks : (size_t)im.ldKe * sizeof(T);
       if (mine) {
-        if (cfg.keys && !mbar_wait_warp(&s_kbar[team], par)) s_abort = 1;
+        if (cfg.keys && !mbar_wait_warp(&s_kbar[team], par)) s_abort = 1;   // (on through the teams' barriers, but without copies)
         par ^= 1u;
         if (im.Kc) {                                     // inverse norms: eight lanes per row, four rows at a time
           const bool same = cfg.keys && im.Kc == im.Ke;
@@ -511,8 +515,12 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && s_abort)
-    for (int i = 0; i < bt.B; ++i) atomicMin(&bt.img[i].cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+  if (threadIdx.x < 32 && s_abort) {
+    land_copies(&s_rbar[0][0], kTokWarps * kTokMaxBuf);
+    land_copies(s_kbar, 2);
+    if (threadIdx.x == 0)
+      for (int i = 0; i < bt.B; ++i) atomicMin(&bt.img[i].cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+  }
 }
 
 __device__ __forceinline__ void ld_cg_f64x2(const double *p, double &a, double &b) {

@@ -690,6 +690,12 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
         }
       }
       if (!ok) atomicExch(&sh.abort, 1);
+      // drain: the copies of both CTAs into every armed stage complete before either may exit
+      const uint32_t armed = leader ? min(it, (uint32_t)PSTAGES) : 0u;
+      for (uint32_t k = 0; k < armed; ++k) {
+        const uint32_t j = it - 1 - k;
+        mbar_wait(&sh.full[j % PSTAGES], (j / PSTAGES) & 1);
+      }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (CTA 0 for both) ----------------

@@ -534,9 +534,9 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
     auto issue = [&](int j, int hh) {
       const int n = min(half, tn - j);
       if (n <= 0) return;
+      if ((t & 31) != 0 || *const_cast<volatile int *>(&s_abort)) return;   // (nothing is asked for after a wait that ran out)
       if (t == 0) mbar_arrive_expect_tx(&s_bar[hh], (uint32_t)n * rowb);
-      if ((t & 31) == 0)
-        for (int k = t >> 5; k < n; k += kMrgThreads / 32)
+      for (int k = t >> 5; k < n; k += kMrgThreads / 32)
           bulk_load(reinterpret_cast<uint8_t *>(ring) + (size_t)(hh * half + k) * rowb, H + (size_t)s_row[j + k] * im.ldH, rowb, &s_bar[hh]);
     };
     const int j0 = max(start - t0, 0);                // (a first tile may begin with items of the range before)
@@ -576,7 +576,9 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
   if (first_cut) cut(cut_head, cut_head_n, cur_inv, cur_dst, 0);
   else if (cut_tail >= 0) cut(cut_tail, cut_tail_n, cur_inv, cur_dst, 1);
   else store_row(cur_inv, cur_dst);
-  if (t == 0 && s_abort) atomicMin(&im.counters_user[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+  if (t >= 32 || !s_abort) return;
+  land_copies(s_bar, 2);
+  if (t == 0) atomicMin(&im.counters_user[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
 }
 
 // ---- launchers -----------------------------------------------------------------------------------

@@ -55,6 +55,16 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
+// For a CTA that gives up after a wait that ran out: the copies it has under way still write to its shared memory, which the
+// next CTA may have by then.  Threads 0 .. n - 1 wait for a barrier each, whichever its phase: the wait for the phase that is
+// over returns at once, and one for which nothing was asked runs out.  (A call, out of the way of the code that runs.)
+static __device__ __noinline__ void land_copies(uint64_t *bars, int n) {
+  if ((int)threadIdx.x < n) {
+    mbar_wait_slow(bars + threadIdx.x, 0);
+    mbar_wait_slow(bars + threadIdx.x, 1);
+  }
+}
+
 // Wait of a whole warp: one lane polls (32 lanes spinning on one barrier word get in the way of the
 // copy engine that has to update it), the result is shared.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
