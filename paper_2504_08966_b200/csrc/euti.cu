@@ -758,6 +758,7 @@ __device__ __forceinline__ uint32_t euti_threshold(const ImgDesc &im, const uint
     __syncthreads();
     if (lo > 0 && sh.s_cnt == 1) {                      // one key left under the prefix: it is the threshold
       const uint32_t fixed = ~((1u << lo) - 1u), pre2 = sh.s_prefix;
+      __syncthreads();                                  // (its owner overwrites the prefix that the others read)
       if (KPT > 0) {
 #pragma unroll
         for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u)
