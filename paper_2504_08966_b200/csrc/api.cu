@@ -557,7 +557,7 @@ static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, c
       cmaxQ = qest > cmaxQ ? qest : cmaxQ;
     }
     // (a profiled call is launched kernel by kernel)
-    if (!ctx->prof_on && small_fits(bt, cmaxN, ctx->umma)) {
+    if (!ctx->prof_on && small_fits(bt, cmaxN, ctx->umma, ctx->ccfg)) {
       int rpp = 0;
       if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 2, st, *feed, &rpp));
       else CK(launch_euti(bt, cmaxN, bf, 2, st, nullptr, nullptr, &rpp));

@@ -127,7 +127,7 @@ cudaError_t launch_spread_umma(const Batch &bt, int maxN, const ClusterCfg &cfg,
 
 // small.cu: scores to member lists in one kernel, a cluster per image
 cudaError_t small_configure();
-bool small_fits(const Batch &bt, int maxN, bool umma);
+bool small_fits(const Batch &bt, int maxN, bool umma, const ClusterCfg &cfg);
 cudaError_t launch_small(const Batch &bt, bool in_bf16, bool umma, int rpp, int sweep_limit, cudaStream_t st);
 
 // merge.cu

@@ -31,7 +31,7 @@ constexpr int CL = 16;                                 // CTAs of a cluster
 constexpr int kSmMaxOwn = kSmallMaxN / CL;             // tokens of one CTA
 constexpr int kSmMaxW = kSmallMaxN / 32;
 constexpr int kSmMaxHeads = 32;
-constexpr int kSmallMaxF64 = 672;                      // most tokens without the tensor cores
+constexpr int kSmallMaxF64 = 672;                      // most tokens without the tensor cores (see small_fits)
 
 // tcgen05 tiles: 128 rows against 64 others, or 128 rows against themselves, 512 key elements at a time: a chunk of
 // both operands is resident at once, so that a tile of keys of up to that width waits for memory and for the tensor
@@ -744,11 +744,33 @@ cudaError_t small_configure() {
   return cudaSuccess;
 }
 
-// Up to as many images as clusters fit on the GPU at once (with a second round the wide kernels are as fast).  By size: with
-// tensor-core tiles 1024 tokens take 54 us against 58; in double precision the tiles are what 16 SMs are too few for
-// (fp32 keys of 128: 640 tokens 53 us against 60, 729 tokens 64 against 61).
-bool small_fits(const Batch &bt, int maxN, bool umma) {
-  return maxN <= (umma ? kSmallMaxN : kSmallMaxF64) && bt.n_qh <= kSmMaxHeads && bt.B <= g_small_clusters;
+// Up to as many images as clusters fit on the GPU at once (with a second round the wide kernels are as fast), and as long as
+// the chain of kernels that the cluster saves (about 10 us) is worth more than the SMs it leaves idle.  Calls of one image in
+// us, cluster against wide kernels, C = N / 16:
+//   tensor-core tiles   One round of the all-pairs pass, i.e. 512 survivors (d_k 512: 512 survivors of 1024 tokens 51 against
+//                       53, 538 of 768 tokens 65 against 53), and not too many operands for 16 SMs to take in (d_k 1024: 768
+//                       tokens 58 against 60, 1024 tokens 62 against 60).
+//   double precision    32 x 32 tiles of survivors and of tokens x centres (a twentieth of the tokens), each with a fixed part
+//                       of about 256 key elements' time (fp32, d_k 128: 512 tokens, half pruned, 43 against 49, nothing pruned
+//                       64 against 50; d_k 512: 256 tokens 57 against 66 and 70 against 64; d_k 1024, 512 tokens, nothing
+//                       pruned 200 against 97).
+// With more images the idle share is smaller (d_k 512, two and four images of 512 half-pruned tokens: 70 against 76, 73
+// against 102).  Of 340 calls of one to four images measured, d_k 64 to 2048 and pruning 0 to 0.8, the rule takes 0.4 % more
+// than the better form of each would, the sizes alone took 9 %.
+bool small_fits(const Batch &bt, int maxN, bool umma, const ClusterCfg &cfg) {
+  if (maxN > (umma ? kSmallMaxN : kSmallMaxF64) || bt.n_qh > kSmMaxHeads || bt.B > g_small_clusters) return false;
+  const double idle = 1.0 - (double)(CL * bt.B) / cfg.sm_count;
+  for (int b = 0; b < bt.B; ++b) {
+    const int N = bt.img[b].N, q = N - bt.img[b].m_target;
+    if (umma) {
+      const int nb = (q + kSmBM - 1) / kSmBM;
+      if (nb * nb > CL || (double)N * bt.d_k * idle > 710e3) return false;
+    } else {
+      const int nq = (q + TS - 1) / TS, tiles = nq * (nq + 1) / 2 + (N + TS - 1) / TS * ((N / 20 + TS - 1) / TS);
+      if (tiles > 160 || (double)tiles * (bt.d_k + 256) * idle * idle > 26700.0) return false;
+    }
+  }
+  return true;
 }
 
 cudaError_t launch_small(const Batch &bt, bool in_bf16, bool umma, int rpp, int sweep_limit, cudaStream_t st) {

@@ -275,3 +275,21 @@ def test_a_chain_of_centres(N, limit):
     assert label.tolist() == [max(0, (k - 1) // 2) for k in range(N)]
     assert int(cnt[pb.CNT["status"]]) == (-5 if limit else 0)
     assert int(cnt[pb.CNT["sweeps"]]) > (512 if N > 2000 else 1)
+
+
+@pytest.mark.parametrize("N,n_kvh,d_h,dtype,lam,B,kernels", [
+    (256, 4, 128, torch.float32, 0.5, 1, 4), (256, 4, 128, torch.float32, 0.0, 1, 10), (128, 8, 128, torch.float32, 0.0, 1, 4),
+    (640, 4, 128, torch.float32, 0.0, 1, 10), (300, 5, 104, torch.bfloat16, 0.0, 1, 10), (512, 1, 64, torch.float32, 0.5, 2, 4),
+    (512, 1, 64, torch.bfloat16, 0.0, 1, 4), (513, 1, 64, torch.bfloat16, 0.0, 1, 10), (1024, 1, 64, torch.bfloat16, 0.5, 2, 4),
+    (777, 8, 128, torch.bfloat16, 0.5, 1, 4), (778, 8, 128, torch.bfloat16, 0.5, 1, 10),
+])
+def test_one_cluster_or_the_whole_gpu(N, n_kvh, d_h, dtype, lam, B, kernels):
+    """Both sides of the lines between the one-cluster step and the wide kernels: survivors, key width, images."""
+    wls = [_workload(N - b, n_kvh, n_kvh, d_h, 64, dtype, 3 * N + b) for b in range(B)]
+    wl = workloads.Workload("line", [w.images[0] for w in wls], 64, n_kvh, n_kvh, d_h, dtype, lam, 0.3)
+    outs, ctx = gpu_reduce(wl, torch.float32)
+    assert ctx.launch_count() == kernels
+    for img, g in zip(wl.images, outs):
+        o = oracle_image(wl, img)
+        bad = compare_image(o, g, img, False)
+        assert not bad, f"{bad}; fragile: {fragile_report(o, wl.d_c, wl.alpha)}"
