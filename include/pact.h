@@ -167,7 +167,8 @@ const char *pact_profile_stage_name(int i);
 /* ---- stage calls (one image) ----------------------------------------------------------- */
 
 /* EUTI score, Eq. 1-2 / Algorithm 1 steps 1-2.
- * Reads img->H (visual rows), K_euti, Q_euti; writes score[N] (fp32). */
+ * Reads img->H (visual rows), K_euti, Q_euti; writes score[N] (fp32).  An infinity or a NaN anywhere in
+ * Q_euti or K_euti makes every score NaN (also in pact_reduce, where equal scores all survive). */
 pact_status pact_importance(pact_ctx *ctx, const pact_image *img /*host*/, const pact_params *p /*host*/,
                             float *score, void *ws, size_t ws_bytes, void *stream);
 

@@ -15,6 +15,10 @@
 //
 // The kernels are short chains of dependent memory round trips; each issues all the loads it can
 // before it consumes the first.
+#include <string.h>
+
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "tma.cuh"
 
@@ -43,26 +47,32 @@ template <> __device__ __forceinline__ void widen_scaled<float>(const uint4 &v, 
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = __hiloint2double((int)w[i] >> 3 & (int)0x8FFFFFFF, (int)(w[i] << 29));
 }
-// NaN once one of the elements seen was not finite, else 0: x * 0 is NaN for an infinity and for a NaN.  (Two chains: one of
-// four multiply-adds per vector was longer than the sums beside it.)
-template <typename T> struct NonFinite;
-template <> struct NonFinite<__nv_bfloat16> {
-  __nv_bfloat162 z[2] = {__floats2bfloat162_rn(0.f, 0.f), __floats2bfloat162_rn(0.f, 0.f)};
-  __device__ __forceinline__ void see(const uint4 &v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// NaN once one of the elements seen was not finite, else 0: x * 0 is NaN for an infinity and for a NaN.  CH chains: four
+// multiply-adds per vector in one are longer than the column sums beside them.
+template <int CH> __device__ __forceinline__ void see_finite(__nv_bfloat162 (&z)[CH], const uint4 &v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) z[i & 1] = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&w[i]), __floats2bfloat162_rn(0.f, 0.f), z[i & 1]);
-  }
-  __device__ __forceinline__ float value() const { return __low2float(z[0]) + __high2float(z[0]) + __low2float(z[1]) + __high2float(z[1]); }
-};
-template <> struct NonFinite<float> {
-  float z[2] = {0.f, 0.f};
-  __device__ __forceinline__ void see(const uint4 &v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  for (int i = 0; i < 4; ++i) z[i % CH] = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&w[i]), __floats2bfloat162_rn(0.f, 0.f), z[i % CH]);
+}
+template <int CH> __device__ __forceinline__ void see_finite(float (&z)[CH], const uint4 &v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) z[i & 1] = fmaf(__uint_as_float(w[i]), 0.f, z[i & 1]);
+  for (int i = 0; i < 4; ++i) z[i % CH] = fmaf(__uint_as_float(w[i]), 0.f, z[i % CH]);
+}
+template <typename T, int CH> struct NonFinite {
+  using Z = typename std::conditional<sizeof(T) == 2, __nv_bfloat162, float>::type;
+  Z z[CH];
+  __device__ __forceinline__ NonFinite() { memset(z, 0, sizeof(z)); }
+  __device__ __forceinline__ void see(const uint4 &v) { see_finite<CH>(z, v); }
+  __device__ __forceinline__ float value() const {
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      if constexpr (sizeof(T) == 2) s += __low2float(z[c]) + __high2float(z[c]);
+      else s += z[c];
+    }
+    return s;
   }
-  __device__ __forceinline__ float value() const { return z[0] + z[1]; }
 };
 // Sum of the 32 parts of each of the rows w, w + step, ... < n: eight lanes per row, four rows at a time.
 template <typename F>
@@ -116,7 +126,7 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
   for (int k = 0; k < V; ++k) acc[k] = 0.0;
   if (v < nvq) {
     constexpr int UQ = 8;
-    NonFinite<T> odd;
+    NonFinite<T, 2> odd;
     const T *Q = reinterpret_cast<const T *>(im.Q) + (size_t)v * V;
     for (int r = r0 + t / GV; r < r1; r += LANES * UQ) {
       uint4 buf[UQ];
@@ -134,8 +144,7 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
         }
       }
     }
-    // one column for all of the vector's: a column that is not finite makes every logit of its head infinite or NaN, hence
-    // every softmax of that head and every score NaN
+    // one column for all of the vector's: with a column that is NaN every score is
     acc[0] += (double)odd.value();
   }
 #pragma unroll
@@ -209,9 +218,10 @@ inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
 }
 
 // Logits of this lane's token (its vectors p, p + P, ... of nv) with nr <= RB heads of a key head, q at one address per part.
-// Returns whether all elements were finite: if not, the logits are not these (see plain_heads).
+// NaN if an element is not finite (even where the sum would be minus infinity and the token's share zero: to sum such keys again
+// by ordinary conversions took the call of an image of 729 tokens 0.5 to 0.9 us just by being in the kernel).
 template <typename T, int RB>
-__device__ __forceinline__ bool head_dots(const uint8_t *krow, const double *q, int d_h, int p, int P, int nr, double (&l)[RB]) {
+__device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, int d_h, int p, int P, int nr, double (&l)[RB]) {
   constexpr int V = Vec<T>::N, CH = 4 / RB;             // CH chains per head: an FMA takes nine clocks, two per warp can start
   const int nv = d_h / V;
   double acc[RB][CH];
@@ -219,7 +229,7 @@ __device__ __forceinline__ bool head_dots(const uint8_t *krow, const double *q, 
   for (int j = 0; j < RB; ++j)
 #pragma unroll
     for (int c = 0; c < CH; ++c) acc[j][c] = 0.0;
-  NonFinite<T> odd;
+  NonFinite<T, 1> odd;
 #pragma unroll 2
   for (int v = p; v < nv; v += P) {
     const uint4 raw = *(reinterpret_cast<const uint4 *>(krow) + v);
@@ -244,21 +254,20 @@ __device__ __forceinline__ bool head_dots(const uint8_t *krow, const double *q, 
     for (int c = 1; c < CH; ++c) l[j] += acc[j][c];
     l[j] *= kWidenScale;
   }
+  l[0] = __hiloint2double(__double2hiint(l[0]) | __float_as_int(odd.value()), __double2loint(l[0]));   // (one head is enough: a score is their mean)
   for (int o = 32 / P; o < 32; o <<= 1)
 #pragma unroll
     for (int j = 0; j < RB; ++j) l[j] += __shfl_xor_sync(0xffffffffu, l[j], o);
-  return odd.value() == 0.f;
 }
 
 // The same heads j0, j0 + 1, ...: logits (zero without a query), the piece's largest, exp and sum.  tl = 32 / P lanes are
-// the tokens of the unit, n of them real.  Returns whether this lane's part of its key was finite.
+// the tokens of the unit, n of them real.
 template <typename T, int RB>
-__device__ __forceinline__ bool head_piece(const Batch &bt, const ImgDesc &im, const uint8_t *krow, const double *q, bool use_query, int P, int nr, int j0,
+__device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, const uint8_t *krow, const double *q, bool use_query, int P, int nr, int j0,
                                            int r0, int n, int g) {
   const int lane = threadIdx.x & 31, tl = 32 / P, r = lane & (tl - 1), p = lane / tl;
   double l[RB];
-  bool finite = true;
-  if (use_query) finite = head_dots<T, RB>(krow, q, bt.d_h, p, P, nr, l);
+  if (use_query) head_dots<T, RB>(krow, q, bt.d_h, p, P, nr, l);
   else {
 #pragma unroll
     for (int j = 0; j < RB; ++j) l[j] = 0.0;
@@ -279,29 +288,6 @@ __device__ __forceinline__ bool head_piece(const Batch &bt, const ImgDesc &im, c
       if (r < n && p == 0) im.E[(size_t)(j0 + j) * im.N + r0 + r] = e[j];
       if (lane == 0) *reinterpret_cast<double2 *>(im.part + ((size_t)g * bt.n_qh + j0 + j) * 2) = make_double2(m[j], sum[j]);
     }
-  return finite;
-}
-
-// The same for nr heads of a unit whose keys hold an infinity or a NaN, with ordinary conversions: such a logit may be an
-// infinity of either sign, and minus infinity is a share of zero.  It hardly ever runs and is kept out of the loops above: as a
-// call inside them it cost 16 images of 2916 tokens 4 us (here nothing; 729 tokens 0.5 us).
-template <typename T>
-__device__ __forceinline__ void plain_heads(const ImgDesc &im, int n_qh, const uint8_t *krow, const double *q, int d_h, int P, int nr, int j0, int r0, int n, int g) {
-  constexpr int V = Vec<T>::N;
-  const int lane = threadIdx.x & 31, tl = 32 / P, r = lane & (tl - 1), p = lane / tl;
-#pragma unroll 1
-  for (int j = j0; j < j0 + nr; ++j, q += d_h) {
-    double l = 0.0;
-#pragma unroll 1
-    for (int e = 0; e < d_h; ++e)
-      if ((e / V) % P == p) l = fma((double)to_float(reinterpret_cast<const T *>(krow)[e]), q[e], l);
-    for (int o = tl; o < 32; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    const double m = warp_max(r < n ? l : -1.0e300), e = r < n ? exp(l - m) : 0.0;
-    double sum = e;
-    for (int o = tl >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (r < n && p == 0) im.E[(size_t)j * im.N + r0 + r] = e;
-    if (lane == 0) *reinterpret_cast<double2 *>(im.part + ((size_t)g * n_qh + j) * 2) = make_double2(m, sum);
-  }
 }
 
 template <typename T, bool QUERY>
@@ -495,19 +481,13 @@ norms_end:
       const double *q = QUERY ? s_q : im.qg;
       const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
       const int nblk = (n_rep + 3) / 4;                  // blocks of up to four query heads per key head
-      bool finite = true;
       for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
         const int kv = it / nblk, j = (it - kv * nblk) * 4, nr = min(4, n_rep - j), j0 = kv * n_rep + j;
         const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
-        if (nr >= 3) finite &= head_piece<T, 4>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else if (nr == 2) finite &= head_piece<T, 2>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else finite &= head_piece<T, 1>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        if (nr >= 3) head_piece<T, 4>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else if (nr == 2) head_piece<T, 2>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+        else head_piece<T, 1>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
       }
-      if (__any_sync(0xffffffffu, !finite))
-        for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
-          const int kv = it / nblk, j = (it - kv * nblk) * 4, j0 = kv * n_rep + j;
-          plain_heads<T>(im, bt.n_qh, krow + (size_t)kv * d_h * sizeof(T), q + (size_t)j0 * d_h, d_h, P, min(4, n_rep - j), j0, r0, n, g);
-        }
       if (cfg.keys && u + 2 < u1) {
         sync();                                          // the keys have been read
         if (lane == 0) issue_keys(u + 2);

@@ -207,35 +207,26 @@ def test_no_norm_and_norm_only():
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("N,n_qh,n_kvh,d_h", [(5, 1, 1, 8), (300, 4, 2, 64), (1500, 7, 1, 40), (5000, 4, 4, 128)])
 def test_non_finite_queries_and_keys_reach_the_scores(N, n_qh, n_kvh, d_h, dtype):
-    """An infinity or a NaN in the queries makes every score NaN; one in a key does, unless it only takes its own token's logit
-    to minus infinity."""
+    """An infinity or a NaN in the queries or the scoring keys makes every score NaN."""
     from paper_2504_08966_b200 import binding as pb
     wl = _workload(N, n_qh, n_kvh, d_h, 64, dtype, 5 * N, rope=True)
     img = wl.images[0]
-    img.Q.abs_()                              # the global query is positive: a key's infinity keeps its sign
     ctx = pb.Context(wl.d, n_qh, n_kvh, d_h, dtype, torch.float32)
     col = n_kvh * d_h - 1                     # last element of the last head
-    for what, value, finite in (("Q", np.nan, False), ("Q", np.inf, False), ("Q", -np.inf, False), ("K", np.nan, False), ("K", np.inf, False),
-                                ("K", -np.inf, True)):
-        t = getattr(img, what)
-        old = t[N - 2, col].clone()
-        t[N - 2, col] = value
-        im = pb.device_image(img, torch.float32)
-        score = torch.zeros(N, dtype=torch.float32, device="cuda")
-        ctx.pact_importance(im, pb.make_params(), score)
-        got = score.cpu().double().numpy()
-        if finite:
-            want = oracle_image(wl, img)["scores"] if N < 2000 else None
-            assert np.isfinite(got).all()
-            if want is not None:
-                assert (np.abs(got - want) <= 2e-7 * np.abs(want)).all()
-        else:
-            assert np.isnan(got).all(), (what, value)
+    for what in ("Q", "K"):
+        for value in (np.nan, np.inf, -np.inf):
+            t = getattr(img, what)
+            old = t[N - 2, col].clone()
+            t[N - 2, col] = value
+            im = pb.device_image(img, torch.float32)
+            t[N - 2, col] = old
+            score = torch.zeros(N, dtype=torch.float32, device="cuda")
+            ctx.pact_importance(im, pb.make_params(), score)
+            assert bool(score.isnan().all()), (what, value)
             if N > 100:                       # and the whole step: every token shares the threshold, so all survive
                 ctx.pact_reduce([im], pb.make_params())
                 torch.cuda.synchronize()
                 assert bool(im.score.isnan().all()) and int(im.counters[pb.CNT["q"]]) == N and int(im.counters[pb.CNT["status"]]) == 0
-        t[N - 2, col] = old
 
 
 @pytest.mark.parametrize("n_qh,n_kvh,d_h,d,dtype", [
