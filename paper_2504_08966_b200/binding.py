@@ -110,9 +110,17 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
-def _stream():
-    """Handle of the current stream of the current device, without a Stream object around it (3 us of a call)."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+def _stream_getter():
+    """Handle of the current stream of the current device, without a Stream object around it (3 us of a call) where this
+    version of torch has the two functions for that."""
+    private = getattr(torch, "_C", None)
+    raw, device = getattr(private, "_cuda_getCurrentRawStream", None), getattr(private, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
+_stream = _stream_getter()
 
 
 def _dt(dtype) -> int:

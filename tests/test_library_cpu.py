@@ -73,6 +73,21 @@ def test_host_side_checks_without_a_gpu(lib):
     assert lib.pact_reduce(None, None, 0, None, 0, None, 0, None) == -1
 
 
+def test_current_stream_without_the_private_functions(monkeypatch):
+    import torch
+    from paper_2504_08966_b200 import binding
+
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 100 + device, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 7, raising=False)
+    assert binding._stream_getter()() == 107
+    monkeypatch.delattr(torch._C, "_cuda_getDevice")
+    assert binding._stream_getter()() == 1234
+
+
 def test_product_does_not_import_the_oracle():
     pkg = os.path.join(ROOT, "paper_2504_08966_b200")
     for dirpath, _, files in os.walk(pkg):
