@@ -28,6 +28,7 @@ struct pact_ctx {
   cudaEvent_t ev[kProfStages + 1];
   // pact_reduce_host: a stream for the copies in, used by one call at a time (another thread's call does without)
   std::atomic_flag feed_busy = ATOMIC_FLAG_INIT;
+  bool fed_before = false;                             // there has been a call large enough for it
   cudaStream_t feed_stream = nullptr;
   cudaEvent_t feed_start = nullptr, feed_keys = nullptr, feed_part[kFeedParts] = {};
 };
@@ -273,7 +274,7 @@ static void release_feed(pact_ctx *ctx) {
   if (ctx->feed_stream) cudaStreamDestroy(ctx->feed_stream);
   ctx->feed_stream = nullptr;
 }
-static bool prepare_feed(pact_ctx *ctx) {            // on the first call that uses it
+static bool prepare_feed(pact_ctx *ctx) {            // on the second call that could use it
   if (ctx->feed_stream) return true;
   bool ok = cudaStreamCreateWithFlags(&ctx->feed_stream, cudaStreamNonBlocking) == cudaSuccess;
   for (cudaEvent_t *e : {&ctx->feed_start, &ctx->feed_keys, &ctx->feed_part[0], &ctx->feed_part[1]})
@@ -757,10 +758,13 @@ pact_status pact_reduce_host(pact_ctx *ctx, const pact_image *img, const pact_pa
   // The hidden states are most of what comes in: they come last, on a stream of their own, while the global query and the
   // logits are formed, and their norms are formed part by part; what is left after the last byte is the split, the
   // clustering and the merge.  (7290 tokens: 20 us of kernels hidden, 1474 -> 1465; 2916: 659 -> 657; with less to copy the
-  // events cost what that gives.)
+  // events cost what that gives.)  The stream and its events take 65 us to create and as long to destroy: the first such call of a
+  // context does without, since a program may make only one.
   const bool fed = bH >= kFeedBytes && !ctx->prof_on && !ctx->feed_busy.test_and_set(std::memory_order_acquire);
   pact_status s = PACT_OK;
-  if (fed && prepare_feed(ctx)) {
+  const bool parts = fed && ctx->fed_before && prepare_feed(ctx);
+  if (fed) ctx->fed_before = true;
+  if (parts) {
     s = feed_and_reduce(ctx, img, &dv, p, bH, bK, bQ, alias, ws, ws_bytes, st);
   } else {
     cudaError_t e = copy_small_inputs(img, dv, bK, bQ, alias, st);

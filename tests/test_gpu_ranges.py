@@ -284,3 +284,16 @@ def test_one_cluster_or_the_whole_gpu(N, n_kvh, d_h, dtype, lam, B, kernels):
         o = oracle_image(wl, img)
         bad = compare_image(o, g, img, False)
         assert not bad, f"{bad}; fragile: {fragile_report(o, wl.d_c, wl.alpha)}"
+
+
+def test_first_host_call_of_a_context_needs_no_stream_of_its_own():
+    """Hidden states arrive in parts from the second call on (a kernel more for each part)."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = _workload(900, 2, 2, 64, 8192, torch.bfloat16, 17)
+    ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
+    want = gpu_reduce(wl, torch.float32)[0][0]
+    counts = [0]
+    for _ in range(3):
+        _same_as_device(_host_call(wl, ctx), want)
+        counts.append(ctx.launch_count())
+    assert np.diff(counts).tolist() == [4, 6, 6]
