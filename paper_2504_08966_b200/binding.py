@@ -206,9 +206,8 @@ PRUNE_STATIC_MAX_N = 65536
 
 
 def pact_prune_static(score, params: Params, keep, kept_idx, pruned_idx, counts):
-    """pact_prune without context or workspace, for callers that may not allocate device memory:
-    the scratch is a fixed array inside the library.  score.numel() <= PRUNE_STATIC_MAX_N.
-    Calls on one stream are ordered; calls that could overlap on the GPU share the array and race."""
+    """pact_prune without context or workspace, for callers that may not allocate device memory.
+    score.numel() <= PRUNE_STATIC_MAX_N."""
     _check(None, lib().pact_prune_static(_ptr(score), score.numel(), C.byref(params), _ptr(keep), _ptr(kept_idx),
                                          _ptr(pruned_idx), _ptr(counts), _stream()))
 

@@ -82,7 +82,6 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   cv.take(m.rnk, (size_t)Np * sizeof(float));
   cv.take(m.rnk64, (size_t)Np * sizeof(double));
   cv.take(m.rho_fix, (size_t)Np * sizeof(unsigned long long));
-  cv.take(m.rho, (size_t)Np * sizeof(float));
   cv.take(m.adj, (size_t)Np * Wp * sizeof(uint32_t));
   cv.take(m.cmask, (size_t)Wp * sizeof(uint32_t));
   cv.take(m.rmask, (size_t)Wp * sizeof(uint32_t));

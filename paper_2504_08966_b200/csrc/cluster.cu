@@ -439,11 +439,7 @@ __global__ void __launch_bounds__(kCenKeyThreads) k_center_keys(const __grid_con
     if (im.C_user) *im.C_user = s_carry;
   }
   for (int r = gw; r < q; r += nwarps) {
-    if (lane == 0) {
-      const float rf = (float)((double)__ldcg(&im.rho_fix[r]) * (1.0 / (double)(1u << kRhoShift)));
-      im.rho[r] = rf;
-      if (im.rho_user) im.rho_user[r] = rf;
-    }
+    if (lane == 0 && im.rho_user) im.rho_user[r] = (float)((double)__ldcg(&im.rho_fix[r]) * (1.0 / (double)(1u << kRhoShift)));
     const uint32_t m = cm[r >> 5];
     if (!((m >> (r & 31)) & 1u)) continue;
     const int c = pref[r >> 5] + __popc(m & ((1u << (r & 31)) - 1u));

@@ -54,7 +54,6 @@ struct ImgDesc {
   float *rnk;            // [Np] 1/|k| in survivor order
   double *rnk64;         // [Np]
   unsigned long long *rho_fix;  // [Np] integer density
-  float *rho;            // [Np]
   uint32_t *adj;         // [Np][Wp] adjacency bits (d <= d_c), later masked to earlier neighbours
   uint32_t *cmask;       // [Wp] centres
   uint32_t *rmask;       // [Wp] removed (within d_c of an earlier centre)
@@ -137,26 +136,6 @@ struct TlScope {
 template <typename T> struct Vec;      // 16-byte vector of T
 template <> struct Vec<__nv_bfloat16> { static constexpr int N = 8; };
 template <> struct Vec<float> { static constexpr int N = 4; };
-
-// Loads 16 bytes and widens to float.
-template <typename T> __device__ __forceinline__ void load_vec(const T *p, float (&out)[Vec<T>::N]);
-
-template <> __device__ __forceinline__ void load_vec<__nv_bfloat16>(const __nv_bfloat16 *p, float (&out)[8]) {
-  uint4 v = *reinterpret_cast<const uint4 *>(p);
-  uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    out[2 * i] = __uint_as_float(w[i] << 16);
-    out[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-  }
-}
-template <> __device__ __forceinline__ void load_vec<float>(const float *p, float (&out)[4]) {
-  float4 v = *reinterpret_cast<const float4 *>(p);
-  out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-}
-
-__device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float to_float(float v) { return v; }
 
 // Largest value over the warp: the order of doubles is that of their bits as integers (negative numbers flipped), upper
 // word first.  (Five rounds of shuffle and fmax take 700 clocks, the two reductions about 100.)

@@ -17,6 +17,7 @@
 // before it consumes the first.
 #include <string.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -1057,8 +1058,8 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
 // ---- launchers -----------------------------------------------------------------------------
 
 namespace {
-int g_sm_count = 148;
-size_t g_smem_optin = 48 * 1024;
+std::atomic<int> g_sm_count{148};            // (any thread may configure a device)
+std::atomic<size_t> g_smem_optin{48 * 1024};
 constexpr size_t kSplitReserve = 12288;      // static shared memory of k_split, rounded up
 constexpr size_t kTokReserve = 2048;         // of k_tokens
 }  // namespace
@@ -1109,7 +1110,8 @@ template <typename T> static TokCfg tokens_config(const Batch &bt) {
 static int tokens_grid(const Batch &bt, int rpp) {
   long long units = 0;
   for (int b = 0; b < bt.B; ++b) units += (bt.img[b].N + rpp - 1) / rpp;
-  return (int)(units < g_sm_count ? units : g_sm_count);
+  const int most = g_sm_count;
+  return units < most ? (int)units : most;
 }
 
 template <typename T>

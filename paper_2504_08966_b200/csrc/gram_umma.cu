@@ -30,10 +30,7 @@ constexpr int BK = 64;            // bf16 elements per K-slab = one 128-byte swi
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int TMEM_COLS = 512;    // all of an SM's tensor memory
 constexpr int MAX_STAGES = 6;
-#ifndef PACT_EPI_WARPS
-#define PACT_EPI_WARPS 16
-#endif
-constexpr int EPI_WARPS = PACT_EPI_WARPS;      // per tensor-memory lane quadrant EPI_WARPS / 4 warps share the columns
+constexpr int EPI_WARPS = 16;      // per tensor-memory lane quadrant EPI_WARPS / 4 warps share the columns
                                   // (16 measured 0.35 us per step faster than 8 once a stage held two K-slabs)
 constexpr int THREADS = 64 + EPI_WARPS * 32;
 constexpr int MAX_ACC = 4;

@@ -91,7 +91,7 @@ int euti_kernels(int mode);
 // threshold + ordered compaction of given scores (pact_prune, one image)
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st);
 cudaError_t euti_configure(int n_qcols, int n_qh);
-cudaError_t select_configure();            // what launch_split needs, once per device
+cudaError_t select_configure();            // what launch_split needs, for the current device
 
 // cluster.cu
 struct ClusterCfg {

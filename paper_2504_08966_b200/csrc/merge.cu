@@ -11,8 +11,6 @@
 //            the running cluster in registers and writes a row out whenever the cluster id changes.
 //            Large clusters cut by a range boundary leave partial sums; the last CTA to arrive adds them in
 //            range order, so the result does not depend on timing.
-#include <cooperative_groups.h>
-
 #include "kernels.cuh"
 #include "tma.cuh"
 

@@ -28,7 +28,6 @@ namespace {
 constexpr int kSmThreads = 512;
 constexpr int kSmWarps = kSmThreads / 32;
 constexpr int CL = 16;                                 // CTAs of a cluster
-constexpr int kSmMaxOwn = kSmallMaxN / CL;             // tokens of one CTA
 constexpr int kSmMaxW = kSmallMaxN / 32;
 constexpr int kSmMaxHeads = 32;
 constexpr int kSmallMaxF64 = 672;                      // most tokens without the tensor cores (see small_fits)

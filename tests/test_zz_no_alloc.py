@@ -2,10 +2,9 @@
 
 Some hosts of the library have no way to obtain a workspace: they run inside another framework's
 callback, or are handed tensors but no allocator, or live in a process whose device memory is
-already fully parcelled out.  For them the scratch of the split is a fixed array inside the
-library.  This test calls that entry point through the C ABI twice in a row (the second call finds
-the array as the first one left it, with a different N and pruning fraction) and requires bit-equal
-outputs to pact_prune, which uses a caller workspace, and to the CPU oracle's split.  Larger inputs go
+already fully parcelled out.  For them there is a split without a workspace.  This test calls that entry
+point through the C ABI twice in a row (with a different N and pruning fraction) and requires bit-equal
+outputs to pact_prune, which takes a caller workspace, and to the CPU oracle's split.  Larger inputs go
 through the other variants of the kernel (keys in registers, in shared memory, re-read), and one case
 runs in a process of its own in which nothing else has touched the library, so that the entry point's
 own first-call set-up is what makes the large launch possible.  The file sorts last so that a failure
@@ -59,7 +58,7 @@ def test_static_scratch_split_matches_workspace_split_twice_in_a_row():
     a[3] = -0.25
     b = torch.rand(1237, generator=g).cuda()
     q1, m1 = _run_both(pb, ctx, a, 0.5)
-    q2, m2 = _run_both(pb, ctx, b, 0.3)            # second call: smaller N, stale scratch from the first
+    q2, m2 = _run_both(pb, ctx, b, 0.3)            # second call: smaller N
     assert m1 == 2500 and m2 == 371
     q3, _ = _run_both(pb, ctx, a, 0.0)             # nothing pruned
     assert q3 == 5000
@@ -68,7 +67,7 @@ def test_static_scratch_split_matches_workspace_split_twice_in_a_row():
 @pytest.mark.parametrize("N", [12000, 40000, 65536])
 def test_static_scratch_split_at_the_sizes_of_the_other_kernel_variants(N):
     """Up to 8192 scores a thread keeps 8 keys in registers, up to 16384 it keeps 16, beyond that the keys
-    live in shared memory; 65536 is the largest input the array admits."""
+    live in shared memory or are read again; 65536 is the largest input the entry point admits."""
     from paper_2504_08966_b200 import binding as pb
     ctx = pb.Context(256, 2, 2, 32, torch.bfloat16, torch.bfloat16)
     g = torch.Generator().manual_seed(N)
@@ -76,7 +75,7 @@ def test_static_scratch_split_at_the_sizes_of_the_other_kernel_variants(N):
     a[N // 3] = a[N // 2]                          # a tie
     q, m = _run_both(pb, ctx, a, 0.37)
     assert m <= int(0.37 * N + 1e-6)
-    _run_both(pb, ctx, a[: N // 2].contiguous(), 0.8)   # second call in a row, stale scratch from the first
+    _run_both(pb, ctx, a[: N // 2].contiguous(), 0.8)   # second call in a row
 
 
 _FRESH = r"""
@@ -105,11 +104,45 @@ print("fresh ok")
 
 
 def test_static_scratch_split_as_the_first_call_of_a_fresh_process():
-    """No context is ever created in the child: the entry point's own first call on the device must look up
-    the array's address and enable the large shared-memory launch that 40000 scores need."""
+    """No context is ever created in the child: the entry point's own first call on the device must enable the
+    large shared-memory launch that 40000 scores need."""
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", _FRESH, root], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "fresh ok" in r.stdout, r.stdout + r.stderr
+
+
+def test_splits_on_two_streams_at_once_and_in_a_graph():
+    """Calls without an order between them share nothing, and a call may be captured."""
+    from paper_2504_08966_b200 import binding as pb
+    g = torch.Generator().manual_seed(3)
+    scores = [torch.rand(n, generator=g).cuda() for n in (65536, 40000, 9000, 700)]
+    outs = [[torch.full((s.numel(),), 7, dtype=dt, device="cuda") for dt in (torch.uint8, torch.int32, torch.int32)] + [torch.zeros(2, dtype=torch.int32, device="cuda")]
+            for s in scores]
+    streams = [torch.cuda.Stream() for _ in scores]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for s, o, st in zip(scores, outs, streams):
+            with torch.cuda.stream(st):
+                pb.pact_prune_static(s, pb.make_params(lam=0.4), *o)
+    torch.cuda.synchronize()
+
+    def check():
+        for s, o in zip(scores, outs):
+            _, keep, kept, pruned = orc.split(s.cpu().numpy(), 0.4)
+            assert o[3].cpu().tolist() == [kept.size, pruned.size] and np.array_equal(o[0].cpu().numpy().astype(bool), keep)
+            assert np.array_equal(o[1][:kept.size].cpu().numpy(), kept) and np.array_equal(o[2][:pruned.size].cpu().numpy(), pruned)
+
+    check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for s, o in zip(scores, outs):
+            pb.pact_prune_static(s, pb.make_params(lam=0.4), *o)
+    for o in outs:
+        for x in o:
+            x.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    check()
 
 
 def test_static_scratch_split_rejects_sizes_beyond_its_array():
