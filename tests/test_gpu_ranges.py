@@ -297,3 +297,17 @@ def test_first_host_call_of_a_context_needs_no_stream_of_its_own():
         _same_as_device(_host_call(wl, ctx), want)
         counts.append(ctx.launch_count())
     assert np.diff(counts).tolist() == [4, 6, 6]
+
+
+@pytest.mark.parametrize("N,T,d", [(2309, 40, 3584), (900, 3, 8192)])
+def test_host_buffers_with_the_flags_of_the_ablations(N, T, d):
+    """Hidden states in parts, with the score's factors left out and with centres in place of means: the wide kernels and the
+    one-cluster step."""
+    from paper_2504_08966_b200 import binding as pb
+    wl = _workload(N, 4, 2, 64, d, torch.bfloat16, N + 1, T=T)
+    for flags in (pb.FLAG_NO_NORM, pb.FLAG_NORM_ONLY, pb.FLAG_CENTER_ONLY, pb.FLAG_CENTER_ONLY | pb.FLAG_NO_NORM):
+        params = pb.make_params(lam=wl.lam, d_c=wl.d_c, flags=flags)
+        want = gpu_reduce(wl, torch.float32, params=params)[0][0]
+        ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
+        for _ in range(3):
+            _same_as_device(_host_call(wl, ctx, params), want)
