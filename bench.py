@@ -32,14 +32,14 @@ N_COPIES = 4          # input copies rotated between steps so that no step finds
 # (workload, kernel) -> bytes; absent = not captured for the kernel as it stands
 NCU_TRAFFIC: dict = {
     ("single_image", "qsum"): 7.48e6,
-    ("single_image", "tokens"): 59.80e6 + 0.23e6,
+    ("single_image", "tokens"): 59.80e6 + 0.13e6,
     ("single_image", "scores"): 0.35e6,
     ("single_image", "select"): 3.83e6,
     ("single_image", "gram_density"): 3.91e6,
-    ("single_image", "centers"): 2.15e6 + 0.63e6,
+    ("single_image", "centers"): 2.16e6 + 0.60e6,
     ("single_image", "assign"): 9.25e6,
     ("single_image", "label_lists"): 0.15e6,
-    ("single_image", "merge"): 52.35e6 + 0.81e6,
+    ("single_image", "merge"): 52.35e6 + 0.65e6,
 }
 
 

@@ -128,7 +128,8 @@ typedef struct {
 
 /* Creates a context for hidden size d, n_qh query heads, n_kvh key heads of width d_h, on the
  * current CUDA device.  Requirements: d_h * n_kvh and d_h * n_qh and d multiples of 8 (bf16) or
- * 4 (fp32); n_qh a multiple of n_kvh; `out` is the element type of H_out. */
+ * 4 (fp32); n_qh a multiple of n_kvh, at most 256; d <= 8192; n_qh * (d_h + 32) <= 28928 (the global query in
+ * double has to fit an SM's shared memory); `out` is the element type of H_out. */
 pact_status pact_create(pact_ctx **ctx, int d, int n_qh, int n_kvh, int d_h, pact_dtype in,
                         pact_dtype out);
 pact_status pact_destroy(pact_ctx *ctx);
@@ -148,7 +149,8 @@ const char *pact_last_cuda_error(const pact_ctx *ctx);
  * within bounds; the call itself still returns PACT_OK and the outputs of that image are not valid.
  * barrier_polls: polls of the member-list barrier; center_sweeps: sweeps of the centre selection (rows that are
  * still open are then decided without waiting, in at most one pass per surviving token; the same happens, with no
- * status, when no row has been removed for 512 sweeps); 0 restores the default (about a million).  Graphs recorded earlier keep the limits they were recorded with. */
+ * status, when no row has been removed for 512 sweeps); 0 restores the default (about a million).  Graphs recorded
+ * earlier keep the limits they were recorded with. */
 pact_status pact_set_wait_limits(pact_ctx *ctx, int barrier_polls, int center_sweeps);
 
 /* ---- instrumentation ---------------------------------------------------------------------- */

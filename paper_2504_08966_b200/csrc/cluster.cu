@@ -219,8 +219,8 @@ __global__ void k_spread_finish(const __grid_constant__ Batch bt, float *max_dis
 // remainder).  A CTA has a block of rows, their adjacency words and all densities of its image in shared memory (what does
 // not fit stays in the L2); lane k of warp w keeps the state of row w + 32 k.  In a sweep the CTA copies the mask of removed
 // rows to shared memory once (thousands of warps polling the same few L2 lines queue up there), and its warps decide what
-// they can from the copy.  Bound by latency, a trip to the L2 per sweep: 7 us for one image of 3645 survivors, 10 us for 16
-// of 1458, 15 us for 4 of 4916.
+// they can from the copy.  Bound by latency, a trip to the L2 per sweep: 8 us for one image of 3645 survivors, 11 us for 16
+// of 1458, 14 us for 4 of 4916.
 // CTAs wait for one another's decisions but need not be resident together: after kCenIdle sweeps in which no row of the image
 // was removed a CTA leaves its open rows to k_center_keys, where every CTA resolves what is open by itself.  (Progress is
 // what counts, not the number of sweeps: 2600 rows whose decisions hang on one another in a chain of 1300 take 1300 sweeps

@@ -54,7 +54,7 @@ struct ImgDesc {
   float *rnk;            // [Np] 1/|k| in survivor order
   double *rnk64;         // [Np]
   unsigned long long *rho_fix;  // [Np] integer density
-  uint32_t *adj;         // [Np][Wp] adjacency bits (d <= d_c), later masked to earlier neighbours
+  uint32_t *adj;         // [Np][Wp] adjacency bits (d <= d_c)
   uint32_t *cmask;       // [Wp] centres
   uint32_t *rmask;       // [Wp] removed (within d_c of an earlier centre)
   void *Kcen;            // [Np][d_k] centre keys in cluster-id order

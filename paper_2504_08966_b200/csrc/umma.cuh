@@ -66,8 +66,10 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {   // clamp
 // through a shared-memory buffer `tr` (row stride 36 words: conflict-free stores, 16-byte loads), lane k
 // adds the 32 terms of column k, and a 32 x 32 bit transpose gives it the column's adjacency word.
 //
-// Instructions are what this pass is bound by (2.2 issued per clock and SM, half of the tensor pipe idle), so the arithmetic
-// of DistF (common.cuh) is written for few of them, with the same results: all of it on half the distance, whose clamp to
+// This pass is bound by its epilogue: 7290 keys on pairs of CTAs take 46 us by themselves with 20 instructions per pair, the
+// issue slots 45 % busy, the special functions and the tensor pipe 36 %; four epilogue warps per scheduler wait for shuffles,
+// conversions and shared memory as often as they issue.  Fewer instructions shorten those chains, so the arithmetic of DistF
+// (common.cuh) is written for few of them, with the same results: all of it on half the distance, whose clamp to
 // [0, 1] is part of the multiply-add and whose scaling by two is exact (rn_col holds -1/2 of the columns' inverse norms);
 // the adjacency bit is the sign of h minus the number after d_c / 2; `nearest`, the smallest magnitude of that, tells whether
 // a pair may be within the band (see gram_band); three terms are summed in 32 bits.  DBDPC of 7290 tokens as a call:

@@ -172,7 +172,7 @@ def test_no_text_tokens_and_gqa_and_distinct_clustering_keys():
     _check_workload(_small(seed=42, n_qh=4), torch.bfloat16)
     _check_workload(_small(seed=43, distinct_k_clu=True), torch.bfloat16)
     _check_workload(_small(seed=44, dtype=torch.float32, d_h=16, n_h=3, d=136), torch.float32)
-    # bf16 keys whose width is not a multiple of 64 take the SIMT tile kernels
+    # bf16 keys whose width is not a multiple of 64 take the tile kernels on the double-precision tensor instruction
     _check_workload(_small(seed=45, d_h=48, n_h=2, d=264), torch.bfloat16)
 
 
