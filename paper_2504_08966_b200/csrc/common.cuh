@@ -40,7 +40,7 @@ struct ImgDesc {
   // workspace
   double *qg;            // [n_qcols] global query
   double *E;             // [n_qh][N] exp(logit - largest of its piece)
-  double *part;          // [G][n_qh][2] (max, sum) of the pieces of k_tokens, G <= ceil(N / kMinPiece)
+  double *part;          // [n_qh][ceil(N / kMinPiece)][2] (max, sum) of the pieces of k_tokens, see piece_at
   int32_t *ghist;        // [2^kHistBits] scores per bin of their top key bits
   double *nrm;           // [N] hidden-state norms
   float *score;          // [N]
@@ -89,6 +89,11 @@ struct Batch {
   int B;
   int d, n_qh, n_kvh, d_h, d_k, n_qcols;
 };
+
+// (max, sum) of head j in softmax piece g
+__device__ __forceinline__ double *piece_at(const ImgDesc &im, int j, int g) {
+  return im.part + ((size_t)j * ((im.N + kMinPiece - 1) / kMinPiece) + g) * 2;
+}
 
 // ---- optional per-CTA timeline (instrumented build only; compiles to nothing otherwise) ----------
 #ifdef PACT_TIMELINE

@@ -30,6 +30,9 @@ __device__ __forceinline__ double ld_cg_f64(const double *p) {
   asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p));
   return v;
 }
+__device__ __forceinline__ void ld_cg_f64x2(const double *p, double &a, double &b) {
+  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "l"(p));
+}
 
 // Widening to double by moving bits: the exponent field of the element becomes the low bits of the double's, i.e. the
 // double is the element times 2^-896, exactly, zeros and subnormal numbers included (the sum is multiplied by 2^896 at
@@ -43,10 +46,11 @@ template <> __device__ __forceinline__ void widen_scaled<__nv_bfloat16>(const ui
 #pragma unroll
   for (int i = 0; i < 4; ++i) { x[2 * i] = scaled_hi(w[i] << 16); x[2 * i + 1] = scaled_hi(w[i]); }
 }
+__device__ __forceinline__ double scaled_f32(uint32_t w) { return __hiloint2double((int)w >> 3 & (int)0x8FFFFFFF, (int)(w << 29)); }
 template <> __device__ __forceinline__ void widen_scaled<float>(const uint4 &v, double (&x)[4]) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int i = 0; i < 4; ++i) x[i] = __hiloint2double((int)w[i] >> 3 & (int)0x8FFFFFFF, (int)(w[i] << 29));
+  for (int i = 0; i < 4; ++i) x[i] = scaled_f32(w[i]);
 }
 // NaN once one of the elements seen was not finite, else 0: x * 0 is NaN for an infinity and for a NaN.  CH chains: four
 // multiply-adds per vector in one are longer than the column sums beside them.
@@ -204,6 +208,7 @@ constexpr int kTokWarps = kTokGroup / 32;
 constexpr int kTeamWarps = kTokTeam / 32;
 constexpr int kTokMaxBuf = 2;                           // row buffers per warp
 constexpr int kTokSmem = 200 * 1024;
+constexpr int kGroupHeads = 3;                          // query heads per key head from which they go through group_piece
 
 struct TokCfg {
   int rpp;                                              // tokens per unit (piece)
@@ -218,11 +223,11 @@ inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
   return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)c.query * n_qcols * 8 + (size_t)c.rpp * 32 * 8;
 }
 
-// Logits of this lane's token (its vectors p, p + P, ... of nv) with nr <= RB heads of a key head, q at one address per part.
+// Logits of this lane's token (its vectors p, p + P, ... of nv) with RB heads of a key head, q at one address per part.
 // NaN if an element is not finite (even where the sum would be minus infinity and the token's share zero: to sum such keys again
 // by ordinary conversions took the call of an image of 729 tokens 0.5 to 0.9 us just by being in the kernel).
 template <typename T, int RB>
-__device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, int d_h, int p, int P, int nr, double (&l)[RB]) {
+__device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, int d_h, int p, int P, double (&l)[RB]) {
   constexpr int V = Vec<T>::N, CH = 4 / RB;             // CH chains per head: an FMA takes nine clocks, two per warp can start
   const int nv = d_h / V;
   double acc[RB][CH];
@@ -239,7 +244,7 @@ __device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, 
     odd.see(raw);
 #pragma unroll
     for (int j = 0; j < RB; ++j) {
-      const double2 *qj = reinterpret_cast<const double2 *>(q + (size_t)min(j, nr - 1) * d_h + v * V);
+      const double2 *qj = reinterpret_cast<const double2 *>(q + (size_t)j * d_h + v * V);
 #pragma unroll
       for (int e = 0; e < V; e += 2) {
         const double2 x = qj[e / 2];
@@ -264,11 +269,11 @@ __device__ __forceinline__ void head_dots(const uint8_t *krow, const double *q, 
 // The same heads j0, j0 + 1, ...: logits (zero without a query), the piece's largest, exp and sum.  tl = 32 / P lanes are
 // the tokens of the unit, n of them real.
 template <typename T, int RB>
-__device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, const uint8_t *krow, const double *q, bool use_query, int P, int nr, int j0,
+__device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, const uint8_t *krow, const double *q, bool use_query, int P, int j0,
                                            int r0, int n, int g) {
   const int lane = threadIdx.x & 31, tl = 32 / P, r = lane & (tl - 1), p = lane / tl;
   double l[RB];
-  if (use_query) head_dots<T, RB>(krow, q, bt.d_h, p, P, nr, l);
+  if (use_query) head_dots<T, RB>(krow, q, bt.d_h, p, P, l);
   else {
 #pragma unroll
     for (int j = 0; j < RB; ++j) l[j] = 0.0;
@@ -284,14 +289,135 @@ __device__ __forceinline__ void head_piece(const Batch &bt, const ImgDesc &im, c
 #pragma unroll
     for (int j = 0; j < RB; ++j) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
 #pragma unroll
-  for (int j = 0; j < RB; ++j)
-    if (j < nr) {
-      if (r < n && p == 0) im.E[(size_t)(j0 + j) * im.N + r0 + r] = e[j];
-      if (lane == 0) *reinterpret_cast<double2 *>(im.part + ((size_t)g * bt.n_qh + j0 + j) * 2) = make_double2(m[j], sum[j]);
-    }
+  for (int j = 0; j < RB; ++j) {
+    if (r < n && p == 0) im.E[(size_t)(j0 + j) * im.N + r0 + r] = e[j];
+    if (lane == 0) *reinterpret_cast<double2 *>(piece_at(im, j0 + j, g)) = make_double2(m[j], sum[j]);
+  }
 }
 
-template <typename T, bool QUERY>
+// Two at a time, as a call: one chain of dependent steps takes 180 clocks, and every copy of the code is fetched from a cold
+// instruction cache.
+__device__ __noinline__ double2 exp_two(double a, double b) { return make_double2(exp(a), exp(b)); }
+// Two elements of a key row, widened as widen_scaled does.
+template <typename T> struct Pair;
+template <> struct Pair<__nv_bfloat16> {
+  uint32_t w;
+  __device__ __forceinline__ void load(const uint8_t *p) { w = *reinterpret_cast<const uint32_t *>(p); }
+  __device__ __forceinline__ void widen(double &a, double &b) const { a = scaled_hi(w << 16); b = scaled_hi(w); }
+  __device__ __forceinline__ void see(float &z) const {     // (an infinity or a NaN times zero is a NaN)
+    z = fmaf(__uint_as_float(w << 16), 0.f, z);
+    z = fmaf(__uint_as_float(w & 0xFFFF0000u), 0.f, z);
+  }
+};
+template <> struct Pair<float> {
+  uint2 w;
+  __device__ __forceinline__ void load(const uint8_t *p) { w = *reinterpret_cast<const uint2 *>(p); }
+  __device__ __forceinline__ void widen(double &a, double &b) const { a = scaled_f32(w.x); b = scaled_f32(w.y); }
+  __device__ __forceinline__ void see(float &z) const {
+    z = fmaf(__uint_as_float(w.x), 0.f, z);
+    z = fmaf(__uint_as_float(w.y), 0.f, z);
+  }
+};
+// The larger of two doubles by their bits as integers, as warp_max orders them.
+__device__ __forceinline__ double max_by_bits(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  const long long kx = x ^ ((x >> 63) & 0x7fffffffffffffffll), ky = y ^ ((y >> 63) & 0x7fffffffffffffffll);
+  return kx > ky ? a : b;
+}
+
+// The same for nr <= 8 heads of a key head at once, on the double-precision tensor instruction (m8n8k4: 8 tokens x 4 elements
+// by 4 elements x 8 heads).  Lane 4 m + c holds of the keys the elements 2 c, 2 c + 1 of each eight of token m of a block,
+// of the query the same elements of head m, and of the product the heads 2 c, 2 c + 1 of token m; the order in which the
+// elements of a sum meet is free.  The query is read once for up to four blocks of eight tokens.
+// With a token per lane every multiply-add takes eight bytes of the query per lane from shared memory, which hands out 128
+// bytes a clock: 32 tokens of one head of 128 cost 256 clocks of it, against 512 clocks of the double-precision unit for up
+// to eight heads here.  So heads come here from three per key head on: three images, 5190 tokens, 28 heads on 4 key heads:
+// 13 us from the query to the pieces with a token per lane, 5 here; one of 7426 tokens 14 and 9.
+// NB: blocks of eight tokens.  SMEM: keys and query are in shared memory.
+template <typename T, int NB, bool SMEM>
+__device__ __forceinline__ void group_piece(const Batch &bt, const ImgDesc &im, const uint8_t *kh, size_t kstride, const double *q,
+                                            bool use_query, int nr, int j0, int r0, int n, int g) {
+  constexpr int CH = NB <= 2 ? 2 : 1;                    // chains per block: a multiply takes 27 clocks, one can start every 16
+  if constexpr (SMEM) {
+    __builtin_assume(__isShared(kh));
+    __builtin_assume(__isShared(q));
+  }
+  const int lane = threadIdx.x & 31, m = lane >> 2, c = lane & 3;
+  double l[NB][2];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) l[b][0] = l[b][1] = 0.0;
+  if (use_query) {
+    float odd[NB];
+    double acc[NB][CH][2];
+    const uint8_t *kr[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      odd[b] = 0.f;
+#pragma unroll
+      for (int h = 0; h < CH; ++h) acc[b][h][0] = acc[b][h][1] = 0.0;
+      kr[b] = kh + (size_t)min(b * 8 + m, n - 1) * kstride + 2 * c * sizeof(T);
+    }
+    const double *qr = q + (size_t)min(m, nr - 1) * bt.d_h + 2 * c;
+#pragma unroll 2
+    for (int k0 = 0; k0 < bt.d_h; k0 += 8) {
+      const bool in = sizeof(T) == 2 || k0 + 2 * c < bt.d_h;       // (fp32 head widths are multiples of four)
+      const double2 x = in ? *reinterpret_cast<const double2 *>(qr + k0) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        Pair<T> k = {};
+        if (in) k.load(kr[b] + (size_t)k0 * sizeof(T));
+        double a0, a1;
+        k.widen(a0, a1);
+        k.see(odd[b]);
+        asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(acc[b][0][0]), "+d"(acc[b][0][1]) : "d"(a0), "d"(x.x));
+        asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(acc[b][CH - 1][0]), "+d"(acc[b][CH - 1][1]) : "d"(a1), "d"(x.y));
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      odd[b] += __shfl_xor_sync(0xffffffffu, odd[b], 1);
+      odd[b] += __shfl_xor_sync(0xffffffffu, odd[b], 2);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const double v = (CH == 2 ? acc[b][0][e] + acc[b][CH - 1][e] : acc[b][0][e]) * kWidenScale;
+        l[b][e] = __hiloint2double(__double2hiint(v) | __float_as_int(odd[b]), __double2loint(v));
+      }
+    }
+  }
+  double mx[2] = {-1.0e300, -1.0e300}, sum[2] = {0.0, 0.0};
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+    if (b * 8 + m < n) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) mx[e] = max_by_bits(mx[e], l[b][e]);
+    }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) mx[e] = max_by_bits(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const double2 x = exp_two(l[b][0] - mx[0], l[b][1] - mx[1]);
+    if (b * 8 + m < n) {
+      double *E = im.E + (size_t)(j0 + 2 * c) * im.N + r0 + b * 8 + m;
+      sum[0] += x.x;
+      sum[1] += x.y;
+      if (2 * c < nr) E[0] = x.x;
+      if (2 * c + 1 < nr) E[im.N] = x.y;
+    }
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (m == 0 && 2 * c + e < nr) *reinterpret_cast<double2 *>(piece_at(im, j0 + 2 * c + e, g)) = make_double2(mx[e], sum[e]);
+}
+
+// QUERY: the global query in shared memory; GROUP: heads through group_piece (a kernel of its own: in one, either path has
+// fewer registers).
+template <typename T, bool QUERY, bool GROUP>
 __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int what) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
@@ -474,20 +600,36 @@ norms_end:
       const bool use_query = !(im.flags & PACT_FLAG_NORM_ONLY) && im.Q != nullptr;
       if (QUERY && use_query && loaded != b) {                  // both teams come by here for every image of the CTA's units
         if (loaded >= 0) sync_both();
-        for (int c = threadIdx.x - kTokGroup; c < bt.n_qcols; c += kTokGroup) s_q[c] = ld_cg_f64(&im.qg[c]);
+#pragma unroll 4
+        for (int c = 2 * (threadIdx.x - kTokGroup); c < bt.n_qcols; c += 2 * kTokGroup) {
+          double2 x;
+          ld_cg_f64x2(&im.qg[c], x.x, x.y);
+          *reinterpret_cast<double2 *>(s_q + c) = x;
+        }
         loaded = b;
         sync_both();
       }
       if (!mine) continue;
       const double *q = QUERY ? s_q : im.qg;
-      const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
-      const int nblk = (n_rep + 3) / 4;                  // blocks of up to four query heads per key head
-      for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
-        const int kv = it / nblk, j = (it - kv * nblk) * 4, nr = min(4, n_rep - j), j0 = kv * n_rep + j;
-        const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
-        if (nr >= 3) head_piece<T, 4>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else if (nr == 2) head_piece<T, 2>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
-        else head_piece<T, 1>(bt, im, kh, q + (size_t)j0 * d_h, use_query, P, nr, j0, r0, n, g);
+      if constexpr (GROUP) {
+        const int nblk = (n_rep + 7) / 8;                // blocks of up to eight query heads per key head
+        const bool in_smem = QUERY && cfg.keys;
+        for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
+          const int kv = it / nblk, j = (it - kv * nblk) * 8, j0 = kv * n_rep + j, nr = min(8, n_rep - j);
+          const uint8_t *kh = keys + (size_t)kv * d_h * sizeof(T);
+          if (!in_smem) group_piece<T, 4, false>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          else if (n <= 8) group_piece<T, 1, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          else if (n <= 16) group_piece<T, 2, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          else if (n <= 24) group_piece<T, 3, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          else group_piece<T, 4, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+        }
+      } else {
+        const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
+        for (int kv = w; kv < n_kvh; kv += kTeamWarps) {
+          const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
+          if (n_rep == 2) head_piece<T, 2>(bt, im, kh, q + (size_t)2 * kv * d_h, use_query, P, 2 * kv, r0, n, g);
+          else head_piece<T, 1>(bt, im, kh, q + (size_t)kv * d_h, use_query, P, kv, r0, n, g);
+        }
       }
       if (cfg.keys && u + 2 < u1) {
         sync();                                          // the keys have been read
@@ -504,62 +646,77 @@ norms_end:
   }
 }
 
-__device__ __forceinline__ void ld_cg_f64x2(const double *p, double &a, double &b) {
-  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "l"(p));
-}
-
 // ---- Eq. 2, second half: merge the pieces (M = max, Z = sum S_g exp(M_g - M), fixed order), scores --------
-// grid (ceil(maxN / 256), B), 256 threads.  Every CTA merges all G pieces itself: the warps share out the
-// heads (and, with fewer heads than warps, the pieces of a head), eight loads per lane in flight; what turns a term into
-// a share, exp(M_g - M) / (Z n_qh), is formed once per piece and head of the CTA's tokens.  with_hist:
+// grid (ceil(maxN / 256) rounded up to CL, B) in clusters of CL CTAs, 512 threads: two per token, each with half of the heads.
+// A cluster merges all G pieces for itself: its CTAs share out the heads (four or fewer per CTA up to 32 heads), the warps of a
+// CTA the heads and the pieces of a head, four loads per lane in flight; the results go to every CTA of the cluster.  What
+// turns a term into a share, exp(M_g - M) / (Z n_qh), is formed once per piece and head of the CTA's tokens.  with_hist:
 // every score also counts in the histogram of its top key bits, the first level of the threshold selection.
-constexpr int kScoreWarps = 8;
+// EP: terms of a token that a thread asks for before the merge (all of its half up to four heads, else eight).
+// Bound by latency and by the instructions it takes: what does not depend on k_tokens comes before the wait for it (a microsecond of
+// divisions), a value that has to be spilled while it is loaded costs its whole latency, and two exponentials at a time come
+// from one copy of the code.  With every CTA merging all heads, 286 pieces of 28 heads took 22 us, 10 now; three images with
+// 28 heads (5190 tokens) 13 us, 10 now; four heads 4.9 us, 4.1 now.  (Going through the code once before the wait, to have the
+// instructions in the cache, halved the time behind the wait and cost as much before it.)
+constexpr int kScoreTok = 256;                          // tokens per CTA
+constexpr int kScoreThreads = 2 * kScoreTok;
+constexpr int kScoreWarps = kScoreThreads / 32;
 constexpr int kScoreHeads = 32;                         // heads whose factors are in shared memory at a time
-constexpr int kScorePieces = 256 / kMinPiece + 1;       // most pieces that 256 tokens belong to
+constexpr int kScorePieces = kScoreTok / kMinPiece + 1; // most pieces that a CTA's tokens belong to
+constexpr int kScoreMaxCl = 8;
 
-// (Three CTAs per SM: at 112 registers a call of three images with 28 heads took 1 us more.)
-__global__ void __launch_bounds__(256, 3) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist) {
+template <int EP>
+__global__ void __launch_bounds__(kScoreThreads, 2) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist, int CL) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 2);
-  pdl_wait();
-  pdl_trigger();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int N = im.N, n_qh = bt.n_qh, i0 = blockIdx.x * 256;
-  if (i0 >= N) return;
-  const int G = (N + rpp - 1) / rpp, g0 = i0 / rpp, np = (min(N, i0 + 256) - 1) / rpp - g0 + 1;   // pieces of the CTA's tokens
+  const int N = im.N, n_qh = bt.n_qh, i0 = blockIdx.x * kScoreTok, rank = blockIdx.x % CL;
+  if (i0 - rank * kScoreTok >= N) {                     // no CTA of the cluster has tokens
+    pdl_wait();
+    return;
+  }
   __shared__ double sM[256], sInv[256];
   __shared__ double pmx[kScoreWarps], pz[kScoreWarps];
-  __shared__ double s_fac[kScorePieces * kScoreHeads];
-  const int i = i0 + t;
-  // this token's terms and the first of the CTA's pieces, requested before the merge so that they arrive meanwhile
-  constexpr int EP = 4;
-  double e_pre[EP], nrm_i = 0.0, m_pre = 0.0;
-  if (i < N) {
-#pragma unroll
-    for (int j = 0; j < EP; ++j) e_pre[j] = j < n_qh ? im.E[(size_t)j * N + i] : 0.0;
-    nrm_i = im.nrm[i];
-  }
-  const int nf0 = np * min(n_qh, kScoreHeads);
-  if (t < nf0) m_pre = im.part[((size_t)(g0 + t % np) * n_qh + t / np) * 2];
-  const int wph = n_qh >= kScoreWarps ? 1 : kScoreWarps / n_qh;   // warps per head
-  const int hpp = kScoreWarps / wph;                    // heads per pass
-  constexpr int U = 8;
-  const int step = 32 * wph;
+  __shared__ double s_fac[kScorePieces * kScoreHeads], s_half[kScoreTok];
+  // pieces of the CTA's tokens: np from g0 on; this thread's token, its half of the heads and its factor of the first 32 heads
+  const int G = (N + rpp - 1) / rpp, g0 = i0 / rpp, np = i0 < N ? (min(N, i0 + kScoreTok) - 1) / rpp - g0 + 1 : 0;
+  const int tok = t & (kScoreTok - 1), half = t / kScoreTok, i = i0 + tok, tok_piece = i / rpp - g0;
+  const int nh0 = min(n_qh, kScoreHeads), per0 = (nh0 + 1) >> 1, jb = half * per0, je = i < N ? min(nh0, jb + per0) : jb;
+  const double *e_src = im.E + (size_t)jb * N + i;
+  const int f_head = t / max(np, 1), f_piece = t - f_head * np;
+  const double *m_src = t < np * nh0 ? piece_at(im, f_head, g0 + f_piece) : im.part;
+  const double *nrm_src = i < N ? im.nrm + i : im.nrm;
+  // heads of this CTA, warps per head, pieces of this warp: 32 sub + lane, + step, ...
+  const int hpc = (n_qh + CL - 1) / CL, j_lo = rank * hpc, nh = max(0, min(hpc, n_qh - j_lo));
+  int wph = 1;
+  while (wph < kScoreWarps && hpc * wph * 2 <= kScoreWarps) wph *= 2;
+  const int hpp = kScoreWarps / wph, wh = w / wph, sub = w - wh * wph, step = 32 * wph;   // heads per pass
+  constexpr int U = 4;
   const int nbatch = (G + U * step - 1) / (U * step);
-  for (int j0 = 0; j0 < n_qh; j0 += hpp) {
-    const int j = j0 + w / wph, sub = w % wph;
-    const bool mine = j < n_qh && w / wph < hpp;
+  if (CL > 1) cluster_sync();                           // every CTA of the cluster runs before one stores to another
+  double e_pre[EP], nrm_i = 0.0, m_pre = 0.0, s = 0.0;
+  pdl_wait();
+  pdl_trigger();
+  for (int p = 0; p < hpc; p += hpp) {
+    const bool mine = p + wh < nh;
+    const int j = j_lo + p + wh;
     auto load = [&](int b, double (&pm)[U], double (&ps)[U]) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int h = sub * 32 + lane + step * (U * b + u);
         pm[u] = -1.0e300;
         ps[u] = 0.0;
-        if (mine && h < G) ld_cg_f64x2(im.part + ((size_t)h * n_qh + j) * 2, pm[u], ps[u]);
+        if (mine && h < G) ld_cg_f64x2(piece_at(im, j, h), pm[u], ps[u]);
       }
     };
     double pm0[U], ps0[U], m = -1.0e300;
     load(0, pm0, ps0);
+    if (p == 0) {                                       // the token's terms and the first factor's piece arrive during the merge
+#pragma unroll
+      for (int u = 0; u < EP; ++u) e_pre[u] = ld_cg_f64(jb + u < je ? e_src + (size_t)u * N : im.E);
+      nrm_i = ld_cg_f64(nrm_src);
+      m_pre = ld_cg_f64(m_src);
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) m = pm0[u] > m ? pm0[u] : m;
     for (int b = 1; b < nbatch; ++b) {
@@ -570,58 +727,85 @@ __global__ void __launch_bounds__(256, 3) k_scores(const __grid_constant__ Batch
     }
     m = warp_max(m);
     if (wph > 1) {
-      __syncthreads();
-      if (lane == 0) pmx[w] = m;
+      if (lane == 0) pmx[w] = m;                        // (then all heads of the CTA are in one pass)
       __syncthreads();
       if (mine)
         for (int k = 0; k < wph; ++k) { const double o = pmx[w - sub + k]; m = o > m ? o : m; }
     }
     double z = 0.0;
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (step * u < G) z += ps0[u] * exp(pm0[u] - m);  // (an empty slot adds 0 * exp(-huge) = 0)
+    for (int u = 0; u < U; u += 2)
+      if (step * u < G) {                               // (an empty slot adds 0 * exp(-huge) = 0)
+        const double2 x = exp_two(pm0[u] - m, pm0[u + 1] - m);
+        z += ps0[u] * x.x;
+        z += ps0[u + 1] * x.y;
+      }
     for (int b = 1; b < nbatch; ++b) {
       double pm[U], ps[U];
       load(b, pm, ps);
 #pragma unroll
-      for (int u = 0; u < U; ++u) z += ps[u] * exp(pm[u] - m);
+      for (int u = 0; u < U; u += 2) {
+        const double2 x = exp_two(pm[u] - m, pm[u + 1] - m);
+        z += ps[u] * x.x;
+        z += ps[u + 1] * x.y;
+      }
     }
     z = warp_sum(z);
     if (wph > 1) {
       if (lane == 0) pz[w] = z;
       __syncthreads();
+      z = 0.0;
+      for (int k = 0; k < wph; ++k) z += pz[w - sub + k];
     }
-    if (mine && sub == 0 && lane == 0) {
-      if (wph > 1) {
-        z = 0.0;
-        for (int k = 0; k < wph; ++k) z += pz[w + k];
+    if (mine && sub == 0 && lane < CL) {                // to every CTA of the cluster
+      const double inv = 1.0 / (z * (double)n_qh);
+      if (CL > 1) {
+        st_cluster_f64(&sM[j], lane, m);
+        st_cluster_f64(&sInv[j], lane, inv);
+      } else {
+        sM[j] = m;
+        sInv[j] = inv;
       }
-      sM[j] = m;
-      sInv[j] = 1.0 / (z * (double)n_qh);
     }
   }
-  double s = 0.0;
+  if (CL > 1) cluster_sync();
+  // (heads EP .. of the half; the registers are not free earlier)
+  double e_more[EP];
+  if (EP > 2) {
+#pragma unroll
+    for (int u = 0; u < EP; ++u) e_more[u] = jb + EP + u < je ? ld_cg_f64(e_src + (size_t)(EP + u) * N) : 0.0;
+  }
+  s = 0.0;
   for (int h0 = 0; h0 < n_qh; h0 += kScoreHeads) {
-    const int nh = min(kScoreHeads, n_qh - h0);
+    const int nhh = min(kScoreHeads, n_qh - h0);
     __syncthreads();
-    for (int f = t; f < np * nh; f += 256) {            // factor f: head h0 + f / np, piece f % np
-      const int j = h0 + f / np;
-      const double mg = h0 == 0 && f == t ? m_pre : im.part[((size_t)(g0 + f % np) * n_qh + j) * 2];
-      s_fac[f] = exp(mg - sM[j]) * sInv[j];
+    for (int f = t; f < np * nhh; f += kScoreThreads) { // factor f: head h0 + f / np, piece f % np
+      const int jf = h0 + f / np;
+      const double mg = h0 == 0 && f == t ? m_pre : ld_cg_f64(piece_at(im, jf, g0 + f % np));
+      s_fac[f] = exp(mg - sM[jf]) * sInv[jf];
     }
     __syncthreads();
     if (i < N) {
-      const double *fac = s_fac + (i / rpp - g0);
-      int j = 0;
+      const double *fac = s_fac + tok_piece;
       if (h0 == 0) {
 #pragma unroll
-        for (; j < EP; ++j) if (j < nh) s = fma(e_pre[j], fac[j * np], s);
+        for (int j = 0; j < EP; ++j)
+          if (jb + j < je) s = fma(e_pre[j], fac[(jb + j) * np], s);
+        if (EP > 2) {
+#pragma unroll
+          for (int j = 0; j < EP; ++j)
+            if (jb + EP + j < je) s = fma(e_more[j], fac[(jb + EP + j) * np], s);
+        }
+      } else {
+        const int per = (nhh + 1) >> 1, hi = min(nhh, half * per + per);
+        for (int j = half * per; j < hi; ++j) s = fma(ld_cg_f64(im.E + (size_t)(h0 + j) * N + i), fac[j * np], s);
       }
-      for (; j < nh; ++j) s = fma(im.E[(size_t)(h0 + j) * N + i], fac[j * np], s);
     }
   }
-  if (i >= N) return;
-  const float sf = (float)(s * nrm_i);
+  if (half == 1) s_half[tok] = s;
+  __syncthreads();
+  if (half == 1 || i >= N) return;
+  const float sf = (float)((s + s_half[tok]) * nrm_i);
   im.score[i] = sf;
   if (im.score_user) im.score_user[i] = sf;
   if (with_hist) atomicAdd(&im.ghist[score_key(sf) >> kHistShift], 1);
@@ -1094,7 +1278,9 @@ template <typename T> static TokCfg tokens_config(const Batch &bt) {
   c.query = 1;
   const auto fits = [&]() { return tok_smem(c, keyb, bt.n_qcols) <= (size_t)kTokSmem; };
   for (int most = 32; most >= kMinPiece; most /= 2) {
-    const long long rounds = (total + (long long)most * g_sm_count - 1) / ((long long)most * g_sm_count);
+    long long rounds = (total + (long long)most * g_sm_count - 1) / ((long long)most * g_sm_count);
+    // (a unit for each of the two teams, where the logits are what takes the time)
+    if (rounds < 2 && bt.n_qh / bt.n_kvh >= kGroupHeads) rounds = 2;
     const long long rpp = (total + rounds * g_sm_count - 1) / (rounds * g_sm_count);
     c.rpp = (int)(rpp < kMinPiece ? kMinPiece : rpp);
     if (fits()) return c;
@@ -1118,7 +1304,9 @@ template <typename T>
 static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, cudaStream_t st, int *rpp) {
   const TokCfg tc = tokens_config<T>(bt);
   if (rpp) *rpp = tc.rpp;
-  return launch_k(tc.query ? k_tokens<T, true> : k_tokens<T, false>, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
+  const bool group = bt.n_qh / bt.n_kvh >= kGroupHeads;
+  const auto kernel = tc.query ? (group ? k_tokens<T, true, true> : k_tokens<T, true, false>) : (group ? k_tokens<T, false, true> : k_tokens<T, false, false>);
+  return launch_k(kernel, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
 }
 
 template <typename T>
@@ -1144,7 +1332,12 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
-  e = launch_k(k_scores, dim3((maxN + 255) / 256, bt.B), dim3(256), 0, st, true, bt, rpp, mode == 0 ? 1 : 0);
+  LaunchOpt opt;
+  int CL = 1;
+  while (CL < kScoreMaxCl && bt.n_qh > 4 * CL) CL *= 2;
+  if (CL > 1) opt.cluster = CL;
+  const int nb = (maxN + kScoreTok - 1) / kScoreTok;
+  e = launch_opt(opt, bt.n_qh <= 4 ? k_scores<2> : k_scores<8>, dim3((nb + CL - 1) / CL * CL, bt.B), dim3(kScoreThreads), 0, st, bt, rpp, mode == 0 ? 1 : 0, CL);
   if (e != cudaSuccess) return e;
   if (mode == 0) {
     if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
@@ -1204,15 +1397,15 @@ cudaError_t euti_configure(int n_qcols, int n_qh) {
   if (e != cudaSuccess) return e;
   if ((size_t)(n_qcols + 32 * n_qh) * 8 > g_smem_optin - 1024) return cudaErrorInvalidConfiguration;   // the widest query
   const int tok = (int)(g_smem_optin - kTokReserve);
-  if ((e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_tokens<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_tokens<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_tokens<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
+  for (const auto f : {k_tokens<__nv_bfloat16, true, true>, k_tokens<__nv_bfloat16, true, false>, k_tokens<__nv_bfloat16, false, true>, k_tokens<__nv_bfloat16, false, false>,
+                       k_tokens<float, true, true>, k_tokens<float, true, false>, k_tokens<float, false, true>, k_tokens<float, false, false>})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
   for (const auto f : {k_select<__nv_bfloat16, 0, true>, k_select<float, 0, true>})   // (the others need less than the default)
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelKeyBytes)) != cudaSuccess) return e;
   // k_tokens can only begin beside k_qsum if both run under the same split of the SM's memory (with the default it waited
   // for k_qsum to drain, 9 us at 6272 tokens); for the other kernels the default is as good or better (16384-token images: 10 us)
-  return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16, true>, k_tokens<float, true>);
+  return prefer_shared(k_qsum<__nv_bfloat16, 4>, k_qsum<__nv_bfloat16, 8>, k_qsum<float, 4>, k_qsum<float, 8>, k_tokens<__nv_bfloat16, true, true>,
+                       k_tokens<__nv_bfloat16, true, false>, k_tokens<float, true, true>, k_tokens<float, true, false>, k_scores<2>, k_scores<8>);
 }
 
 }  // namespace pact

@@ -269,8 +269,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
 #pragma unroll
     for (int k = 0; k < PL; ++k) {
       const int g = lane + 32 * k;
-      m[k] = g < G ? im.part[((size_t)g * n_qh + j) * 2] : -1.0e300;
-      z[k] = g < G ? im.part[((size_t)g * n_qh + j) * 2 + 1] : 0.0;
+      m[k] = g < G ? *piece_at(im, j, g) : -1.0e300;
+      z[k] = g < G ? piece_at(im, j, g)[1] : 0.0;
     }
 #pragma unroll
     for (int k = 0; k < PL; ++k) M = m[k] > M ? m[k] : M;

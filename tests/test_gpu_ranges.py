@@ -83,6 +83,18 @@ def test_token_units(N, n_qh, n_kvh, d_h, d, dtype, scale, rope):
     _check(_workload(N, n_qh, n_kvh, d_h, d, dtype, N, scale, rope), torch.float32)
 
 
+@pytest.mark.parametrize("N,n_qh,n_kvh,d_h,dtype", [
+    (2368, 8, 1, 64, torch.bfloat16), (2369, 3, 1, 64, torch.bfloat16),       # units of eight and nine tokens: one block of eight, two
+    (4736, 18, 2, 40, torch.bfloat16), (4737, 6, 2, 64, torch.float32),       # sixteen, seventeen; nine heads: eight and one
+    (7104, 8, 2, 16, torch.float32), (7105, 28, 4, 32, torch.bfloat16),       # twenty-four, twenty-five
+    (1700, 9, 3, 20, torch.float32),                                          # heads of five fours: the last step has half of its elements
+    (777, 256, 2, 8, torch.bfloat16), (2600, 33, 11, 8, torch.bfloat16),      # more heads per CTA of the merge than warps, more than 32 in all
+])
+def test_heads_of_a_key_head_together(N, n_qh, n_kvh, d_h, dtype):
+    """Three and more query heads per key head go through the double-precision tensor instruction, eight tokens at a time."""
+    _check(_workload(N, n_qh, n_kvh, d_h, 64, dtype, 3 * N + 1), torch.float32)
+
+
 @pytest.mark.parametrize("dtype,n_qh,n_kvh,d_h", [(torch.bfloat16, 4, 2, 64), (torch.bfloat16, 3, 3, 24), (torch.float32, 2, 2, 20)])
 @pytest.mark.parametrize("N", [1, 2, 15, 17, 127, 129, 511, 513, 1023, 1024, 1025])
 def test_small_images(N, dtype, n_qh, n_kvh, d_h):
