@@ -69,7 +69,7 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   cv.take(m.qg, (size_t)c->n_qcols * sizeof(double));
   cv.take(m.E, (size_t)N * c->n_qh * sizeof(double));
   cv.take(m.part, (size_t)((N + kMinPiece - 1) / kMinPiece) * c->n_qh * 2 * sizeof(double));
-  cv.take(m.ghist, ((size_t)1 << kHistBits) * sizeof(int32_t));
+  cv.take(m.ghist, (size_t)kHistBins * sizeof(int32_t));
   cv.take(m.nrm, (size_t)N * sizeof(double));
   cv.take(m.score, (size_t)N * sizeof(float));
   cv.take(m.keep, (size_t)N);

@@ -41,7 +41,7 @@ struct ImgDesc {
   double *qg;            // [n_qcols] global query
   double *E;             // [n_qh][N] exp(logit - largest of its piece)
   double *part;          // [n_qh][ceil(N / kMinPiece)][2] (max, sum) of the pieces of k_tokens, see piece_at
-  int32_t *ghist;        // [2^kHistBits] scores per bin of their top key bits
+  int32_t *ghist;        // [kHistBins] scores per bin of their top key bits
   double *nrm;           // [N] hidden-state norms
   float *score;          // [N]
   unsigned char *keep;   // [N]

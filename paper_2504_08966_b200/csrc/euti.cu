@@ -553,7 +553,7 @@ norms_end:
         for (int r = gt; r < im.N; r += gs) im.best[r] = kBestInit;
         uint4 *tab = reinterpret_cast<uint4 *>(im.cnt_cb);
         for (int r = gt; r < im.Np * (im.nbp / 8); r += gs) tab[r] = make_uint4(0u, 0u, 0u, 0u);
-        for (int r = gt; r < (1 << kHistBits); r += gs) im.ghist[r] = 0;
+        for (int r = gt; r < kHistBins; r += gs) im.ghist[r] = 0;
         if (gt < kCntInts) im.cnt[gt] = 0;
       }
     }
@@ -808,265 +808,287 @@ __global__ void __launch_bounds__(kScoreThreads, 2) k_scores(const __grid_consta
   const float sf = (float)((s + s_half[tok]) * nrm_i);
   im.score[i] = sf;
   if (im.score_user) im.score_user[i] = sf;
-  if (with_hist) atomicAdd(&im.ghist[score_key(sf) >> kHistShift], 1);
+  if (with_hist) atomicAdd(&im.ghist[key_bin(score_key(sf))], 1);
 }
 
 // ---- Eq. 3-4 in the whole step: threshold, ordered compaction, survivor keys (Eq. 7) ------------------------
-// grid (X, B), 512 threads, one or two CTAs per SM; dynamic smem: N sort keys when they fit.  CTA x owns the tokens
-// [x tpc, (x + 1) tpc).  Every CTA selects the threshold itself (identical in all of them), counts the
-// survivors before its tokens, writes keep flags, lists and slots of its tokens and copies the clustering keys
+// grid (X, B), 512 threads, one CTA per SM; dynamic smem: N sort keys where a thread's share does not fit its registers.
+// CTA x owns the tokens [x tpc, (x + 1) tpc).  Every CTA selects the threshold itself (identical in all of them),
+// counts the survivors before its tokens, writes keep flags, lists and slots of its tokens and copies the clustering keys
 // of its survivors to their rows of K'.
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
-constexpr int kHistPerThread = (1 << kHistBits) / kSelThreads;
-constexpr size_t kSelKeyBytes = 96 * 1024;     // most sort keys kept in shared memory
+constexpr int kHistPerThread = kHistBins / kSelThreads;
+constexpr size_t kSelKeyBytes = 96 * 1024;     // most shared memory for sort keys or rows
 constexpr int kSelBits = 10;                  // key bits per pass of the selection below the first-level histogram
-constexpr int kSelPerThread = (1 << kSelBits) / kSelThreads;
-static_assert(kHistPerThread % 4 == 0 && kHistPerThread * kSelThreads == (1 << kHistBits), "histogram split");
+constexpr int kSelFew = 64;                   // candidates that are ranked one against another
+static_assert((1 << kSelBits) == 2 * kSelThreads && kHistPerThread == 8 && kSelWarps <= 32, "bins per thread, a warp total per lane");
 
 struct SelShared {
-  int hist[1 << kSelBits];
+  int hist[1 << kSelBits];                     // keys of the threshold's bin by the bits below, and one key of each
+  uint32_t one[1 << kSelBits];
   int wtot[kSelWarps], wtot2[kSelWarps];
+  uint32_t few[kSelFew];
   uint32_t s_prefix;
-  int s_k, s_bin, s_cnt;
+  int s_k, s_bin, s_cnt, s_less, s_few;
   int own_tok[kSelThreads], own_slot[kSelThreads];
 };
 
-// The key of the (m_target + 1)-th smallest score.  The histogram of the top kHistBits key
-// bits, filled by k_scores, gives the bin of the threshold and its rank inside that bin; radix passes
-// over the bits below, kSelBits at a time, finish the selection (only the keys of that bin take part, so the
-// shared-memory counters see little contention; the bins of a pass are scanned by all threads).  KPT > 0: thread t holds the keys t, t + 512, ... in
-// registers (N <= 512 KPT); KPT == 0: keys from shared memory (IN_SMEM) or re-read from the scores.
-template <int KPT, bool IN_SMEM>
-__device__ __forceinline__ uint32_t euti_threshold(const ImgDesc &im, const uint32_t *skey, const uint32_t (&kreg)[KPT > 0 ? KPT : 1],
-                                                   const int (&hv)[kHistPerThread], SelShared &sh) {
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, N = im.N;
-  auto key_at = [&](int i) -> uint32_t { return IN_SMEM ? skey[i] : score_key(__ldcg(im.score + i)); };
-  {
-    int sum = 0;
+// Warp-inclusive sum.
+__device__ __forceinline__ int warp_scan(int v, int lane) {
 #pragma unroll
-    for (int u = 0; u < kHistPerThread; ++u) sum += hv[u];
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) sh.wtot[w] = incl;
-    if (t == 0) { sh.s_bin = -1; sh.s_k = 0; }
-#pragma unroll
-    for (int u = 0; u < kSelPerThread; ++u) sh.hist[t * kSelPerThread + u] = 0;
-    __syncthreads();
-    int below = incl - sum;                             // keys in the bins before this thread's
-#pragma unroll
-    for (int k = 0; k < kSelWarps; ++k) if (k < w) below += sh.wtot[k];
-    const int m_t = im.m_target;
-    if (below <= m_t && m_t < below + sum) {            // exactly one thread, unless a wait ran out
-      int k = m_t - below;
-#pragma unroll
-      for (int u = 0; u < kHistPerThread; ++u) {
-        if (k >= 0 && k < hv[u]) { sh.s_k = k; sh.s_bin = t * kHistPerThread + u; k = -1; }
-        else if (k >= 0) k -= hv[u];
-      }
-    }
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
   }
-  if (sh.s_bin < 0) return 0xffffffffu;                 // inconsistent histogram: keep nothing
-  if (t == 0) sh.s_prefix = (uint32_t)sh.s_bin << kHistShift;
-  __syncthreads();
-  for (int hi = kHistShift; hi > 0; hi -= kSelBits) {
-    const int lo = hi > kSelBits ? hi - kSelBits : 0;
-    const uint32_t dmask = (1u << (hi - lo)) - 1u;
-    const uint32_t above = ~((1u << hi) - 1u);          // bits already fixed
-    const uint32_t prefix = sh.s_prefix;
-    const int k = sh.s_k;
-    if (KPT > 0) {
-#pragma unroll
-      for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u) {
-        const uint32_t kk = kreg[u];
-        if (t + kSelThreads * u < N && (kk & above) == (prefix & above)) atomicAdd(&sh.hist[(kk >> lo) & dmask], 1);
-      }
-    } else {
-      for (int i = t; i < N; i += kSelThreads) {
-        const uint32_t kk = key_at(i);
-        if ((kk & above) == (prefix & above)) atomicAdd(&sh.hist[(kk >> lo) & dmask], 1);
-      }
-    }
-    __syncthreads();
-    // every thread takes kSelPerThread bins: the one whose bins hold rank k names the digit
-    int c[kSelPerThread], sum = 0;
-#pragma unroll
-    for (int u = 0; u < kSelPerThread; ++u) { c[u] = sh.hist[t * kSelPerThread + u]; sum += c[u]; sh.hist[t * kSelPerThread + u] = 0; }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) sh.wtot[w] = incl;
-    __syncthreads();
-    int below = incl - sum;
-#pragma unroll
-    for (int q = 0; q < kSelWarps; ++q) if (q < w) below += sh.wtot[q];
-    if (below <= k && k < below + sum) {                // exactly one thread: the candidates number more than k
-      int kk = k - below;
-#pragma unroll
-      for (int u = 0; u < kSelPerThread; ++u) {
-        if (kk >= 0 && kk < c[u]) {
-          sh.s_k = kk;
-          sh.s_cnt = c[u];
-          sh.s_prefix = prefix | ((uint32_t)(t * kSelPerThread + u) << lo);
-          kk = -1;
-        } else if (kk >= 0) kk -= c[u];
-      }
-    }
-    __syncthreads();
-    if (lo > 0 && sh.s_cnt == 1) {                      // one key left under the prefix: it is the threshold
-      const uint32_t fixed = ~((1u << lo) - 1u), pre2 = sh.s_prefix;
-      __syncthreads();                                  // (its owner overwrites the prefix that the others read)
-      if (KPT > 0) {
-#pragma unroll
-        for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u)
-          if (t + kSelThreads * u < N && (kreg[u] & fixed) == pre2) sh.s_prefix = kreg[u];
-      } else {
-        for (int i = t; i < N; i += kSelThreads) {
-          const uint32_t kk = key_at(i);
-          if ((kk & fixed) == pre2) sh.s_prefix = kk;
-        }
-      }
-      __syncthreads();
-      break;
-    }
-  }
-  return sh.s_prefix;
+  return v;
 }
 
-// Survivors before the own tokens (every CTA counts them itself), then keep flags, lists and
-// slots of the own tokens, and the clustering keys of the own survivors copied to their rows of K'.
-template <typename T, int KPT, bool IN_SMEM>
-__device__ __forceinline__ void euti_compact(const Batch &bt, const ImgDesc &im, const uint32_t *skey,
-                                             const uint32_t (&kreg)[KPT > 0 ? KPT : 1], uint32_t tau_key, int g, int tok0,
-                                             int ntok, SelShared &sh) {
-  using D = typename DistOf<T>::type;
-  constexpr int V = Vec<T>::N;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, N = im.N;
-  auto key_at = [&](int i) -> uint32_t { return IN_SMEM ? skey[i] : score_key(__ldcg(im.score + i)); };
-  int nb = 0, nall = 0;
-  if (KPT > 0) {
-#pragma unroll
-    for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u) {
-      const int i = t + kSelThreads * u;
-      const int kp = i < N && kreg[u] >= tau_key;
-      nall += kp;
-      nb += kp && i < tok0;
-    }
-  } else {
+// The bins of a pass are in sh.hist: the one with rank k among them, by all threads: its digit to sh.s_bin, the keys in it to
+// sh.s_cnt, the rank in it to sh.s_k.  The bins are zero again afterwards.
+__device__ __forceinline__ void find_digit(int k, SelShared &sh) {
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  int2 *mine = reinterpret_cast<int2 *>(sh.hist) + t;
+  const int2 c = *mine;
+  *mine = make_int2(0, 0);
+  const int incl = warp_scan(c.x + c.y, lane);
+  if (lane == 31) sh.wtot[w] = incl;
+  __syncthreads();
+  const int below = incl - c.x - c.y + (int)__reduce_add_sync(0xffffffffu, lane < w ? sh.wtot[lane] : 0);
+  if (below <= k && k < below + c.x + c.y) {            // exactly one thread: the candidates number more than k
+    const bool second = k >= below + c.x;
+    sh.s_bin = 2 * t + second;
+    sh.s_cnt = second ? c.y : c.x;
+    sh.s_k = k - below - (second ? c.x : 0);
+  }
+  __syncthreads();
+}
+
+// The threshold by radix passes over the bits below `hi`, kSelBits at a time: rank k among the keys with these upper bits, `less`
+// keys of the first-level bin before them.  (skey: the keys in shared memory, or null.  A call: it hardly ever runs.)
+__device__ __noinline__ void radix_threshold(const float *score, const uint32_t *skey, int N, int hi, uint32_t prefix, int k, int less, SelShared &sh) {
+  const int t = threadIdx.x;
+  for (; hi > 0; hi -= kSelBits) {
+    const int lo = hi > kSelBits ? hi - kSelBits : 0;
+    const uint32_t dmask = (1u << (hi - lo)) - 1u;
+    const uint32_t above = hi >= 32 ? 0u : ~((1u << hi) - 1u);          // bits already fixed
+    __syncthreads();
     for (int i = t; i < N; i += kSelThreads) {
-      const int kp = key_at(i) >= tau_key;
-      nall += kp;
-      nb += kp && i < tok0;
+      const uint32_t kk = skey ? skey[i] : score_key(__ldcg(score + i));
+      if ((kk & above) == (prefix & above)) atomicAdd(&sh.hist[(kk >> lo) & dmask], 1);
+    }
+    __syncthreads();
+    find_digit(k, sh);
+    less += k - sh.s_k;                                 // keys under the prefix that come before the digit
+    k = sh.s_k;
+    prefix |= (uint32_t)sh.s_bin << lo;
+  }
+  if (t == 0) {
+    sh.s_less = less;
+    sh.s_prefix = prefix;
+  }
+  __syncthreads();
+}
+
+// KPT > 0: thread t holds the keys t, t + 512, ... in registers (N <= 512 KPT); KPT == 0: keys from shared memory (IN_SMEM)
+// or re-read from the scores.  (A kernel for each case: the code runs once, from a cold instruction cache.)
+// The histogram of the keys' top bits, filled by k_scores, gives the bin of the threshold, the (m_target + 1)-th smallest
+// key, and its rank in the bin (sixteen bins per factor of two: some hundred keys of 7290); a pass over the next ten bits
+// of those mostly leaves one key, which has been put down beside the count, else a few, which are ranked one against another.
+// Bound by latency and by the instructions of 16 warps, four clocks each, most of them run once: 1024 threads were 0.5 us slower
+// (eight clocks), ranking all keys of the bin by counting 3 us, and a pass through the code before the wait, for the
+// instruction cache, cost what it gave.  The rows of the own tokens wait in shared memory when it is known which survive; scores,
+// histogram and norms come in one trip.  From the end of k_scores: one image of 7290 8.0 us -> 6.7, four of 16384 (16 keys per
+// thread from shared memory, three passes over them) 22 -> 15.
+template <typename T, int KPT, bool IN_SMEM>
+__global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant__ Batch bt, int pre) {
+  using D = typename DistOf<T>::type;
+  constexpr int V = Vec<T>::N, KR = KPT > 0 ? KPT : 1;
+  const ImgDesc &im = bt.img[blockIdx.y];
+  TL_SCOPE(im, 3);
+  extern __shared__ __align__(16) uint8_t sel_smem[];
+  uint32_t *skey = reinterpret_cast<uint32_t *>(sel_smem);     // KPT == 0: the keys; else (pre) the rows of the own tokens
+  __shared__ SelShared sh;
+  __shared__ uint64_t s_bar;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int N = im.N, X = gridDim.x, x = blockIdx.x, m_t = im.m_target;
+  const int tpc = (N + X - 1) / X, tok0 = min(N, x * tpc), ntok = min(N, tok0 + tpc) - tok0;
+  const int nv = bt.d_k / V, rowb = nv * 16, npre = KPT > 0 && pre ? ntok : 0;
+  const T *Kc = reinterpret_cast<const T *>(im.Kc);
+  T *Kp = reinterpret_cast<T *>(im.Kp);
+  const float *score = im.score;
+  const int4 *hist = reinterpret_cast<const int4 *>(im.ghist) + 2 * t;
+  const auto key_at = [&](int i) -> uint32_t { return IN_SMEM ? skey[i] : score_key(__ldcg(score + i)); };
+  reinterpret_cast<int2 *>(sh.hist)[t] = make_int2(0, 0);
+  // the keys of the own tokens, before it is known which of them survive (they are an input)
+  if (w == 1 && npre > 0) {
+    if (lane == 0) {
+      mbar_init(&s_bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_arrive_expect_tx(&s_bar, npre * rowb);
+    }
+    __syncwarp();
+    for (int r = lane; r < npre; r += 32) bulk_load(sel_smem + (size_t)r * rowb, Kc + (size_t)(tok0 + r) * im.ldKc, rowb, &s_bar);
+  }
+  uint32_t kreg[KR], own, tau;
+  typename D::rn_t rn_own;
+  int bin, rank, less;
+  if (t == 0) { sh.s_bin = -1; sh.s_k = 0; sh.s_few = 0; }
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  {
+    const int4 ha = __ldcg(hist), hb = __ldcg(hist + 1);   // bins [8 t, 8 t + 8)
+    float sc[KR];
+    if (KPT > 0) {
+#pragma unroll
+      for (int u = 0; u < KR; ++u) sc[u] = __ldcg(score + min(t + kSelThreads * u, N - 1));
+    }
+    const float so = __ldcg(score + min(tok0 + t, N - 1));
+    rn_own = __ldcg(rn_tok<D>(im) + min(tok0 + t, N - 1));
+    const int suma = ha.x + ha.y + ha.z + ha.w, sum = suma + (hb.x + hb.y + hb.z + hb.w), incl = warp_scan(sum, lane);
+    if (lane == 31) sh.wtot[w] = incl;
+    own = score_key(so);
+    if (KPT > 0) {
+#pragma unroll
+      for (int u = 0; u < KR; ++u) kreg[u] = t + kSelThreads * u < N ? score_key(sc[u]) : 0u;   // (never in a bin but 0, never kept)
+    } else if (IN_SMEM) {
+#pragma unroll 8
+      for (int i = t; i < N; i += kSelThreads) skey[i] = score_key(__ldcg(score + i));
+    }
+    __syncthreads();
+    const int below = incl - sum + (int)__reduce_add_sync(0xffffffffu, lane < w ? sh.wtot[lane] : 0);   // keys in the bins before this thread's
+    if (below <= m_t && m_t < below + sum) {            // exactly one thread, unless a wait ran out
+      const bool upper = m_t - below >= suma;
+      const int4 h = upper ? hb : ha;
+      const int k = m_t - below - (upper ? suma : 0), u = (k >= h.x) + (k >= h.x + h.y) + (k >= h.x + h.y + h.z);
+      sh.s_bin = 8 * t + (upper ? 4 : 0) + u;
+      sh.s_k = k - (u > 0 ? h.x : 0) - (u > 1 ? h.y : 0) - (u > 2 ? h.z : 0);
+    }
+    __syncthreads();
+    bin = sh.s_bin;
+    rank = sh.s_k;
+    tau = 0xffffffffu;                                  // (an inconsistent histogram: nothing is kept)
+    less = 0;                                           // keys of the bin before the threshold
+    if (bin > 0) {
+      constexpr int lo = kHistShift - kSelBits;
+      const uint32_t top = bin_first(bin) >> kHistShift;
+      const auto count = [&](uint32_t key) {
+        if (key >> kHistShift == top) {
+          const int d = (key >> lo) & ((1 << kSelBits) - 1);
+          atomicAdd(&sh.hist[d], 1);
+          sh.one[d] = key;
+        }
+      };
+      if (KPT > 0) {
+#pragma unroll
+        for (int u = 0; u < KR; ++u) count(kreg[u]);
+      } else {
+        for (int i = t; i < N; i += kSelThreads) count(key_at(i));
+      }
+      __syncthreads();
+      find_digit(rank, sh);
+      const int digit = sh.s_bin;
+      less = rank - sh.s_k;
+      tau = sh.one[digit];
+      if (sh.s_cnt > 1) {
+        const uint32_t prefix = bin_first(bin) | (uint32_t)digit << lo;
+        const int k2 = sh.s_k;
+        if (sh.s_cnt <= kSelFew) {
+          const auto put = [&](uint32_t key) { if ((key ^ prefix) >> lo == 0u) sh.few[atomicAdd(&sh.s_few, 1)] = key; };
+          if (KPT > 0) {
+#pragma unroll
+            for (int u = 0; u < KR; ++u) put(kreg[u]);
+          } else {
+            for (int i = t; i < N; i += kSelThreads) put(key_at(i));
+          }
+          __syncthreads();
+          if (t < sh.s_cnt) {
+            int l = 0, same = 0;
+            for (int j = 0; j < sh.s_cnt; ++j) { l += sh.few[j] < sh.few[t]; same += sh.few[j] == sh.few[t]; }
+            if (l <= k2 && k2 < l + same) { sh.s_prefix = sh.few[t]; sh.s_less = less + l; }   // (equal keys write the same)
+          }
+          __syncthreads();
+        } else radix_threshold(score, IN_SMEM ? skey : nullptr, N, lo, prefix, k2, less, sh);
+        less = sh.s_less;
+        tau = sh.s_prefix;
+      }
+    } else if (bin == 0) {                              // the bin of all of the smallest keys, whatever their bits
+      radix_threshold(score, IN_SMEM ? skey : nullptr, N, 32, 0u, rank, 0, sh);
+      less = sh.s_less;
+      tau = sh.s_prefix;
     }
   }
-  nb = __reduce_add_sync(0xffffffffu, nb);
-  nall = __reduce_add_sync(0xffffffffu, nall);
-  __syncthreads();
-  if (lane == 0) { sh.wtot[w] = nb; sh.wtot2[w] = nall; }
-  __syncthreads();
-  int before0 = 0, q = 0;
+  TL_POINT(im, 7);
+
+  // ---- survivors before the own tokens, then keep flags, lists, slots and keys of the own ones ----
+  int nb = 0;
+  if (KPT > 0) {
 #pragma unroll
-  for (int k = 0; k < kSelWarps; ++k) { before0 += sh.wtot[k]; q += sh.wtot2[k]; }
-  if (g == 0 && t == 0) {
+    for (int u = 0; u < KR; ++u) nb += t + kSelThreads * u < tok0 && kreg[u] >= tau;
+  } else {
+    for (int i = t; i < tok0; i += kSelThreads) nb += key_at(i) >= tau;
+  }
+  nb = __reduce_add_sync(0xffffffffu, nb);
+  if (x == 0 && t == 0) {
+    const int q = bin >= 0 ? N - (m_t - rank) - less : 0;   // all but the keys of lower bins and the smaller ones of its own
     im.cnt[PACT_CNT_Q] = q;
     im.cnt[PACT_CNT_M] = N - q;
   }
-  const int nv = bt.d_k / V;
-  const T *Kc = reinterpret_cast<const T *>(im.Kc);
-  T *Kp = reinterpret_cast<T *>(im.Kp);
-  for (int c0 = 0; c0 < ntok; c0 += kSelThreads) {     // the own tokens, 512 at a time
+  int before0 = 0;                                      // survivors with a lower index than the round's tokens
+  for (int c0 = 0; c0 < ntok; c0 += kSelThreads) {      // the own tokens, 512 at a time
     const int i = tok0 + c0 + t;
     const bool ok = c0 + t < ntok;
-    const bool kp = ok && key_at(i) >= tau_key;
+    const bool kp = ok && (c0 == 0 ? own : score_key(__ldcg(score + i))) >= tau;
     const unsigned bal = __ballot_sync(0xffffffffu, kp);
+    if (lane == 0) {
+      sh.wtot[w] = __popc(bal);
+      if (c0 == 0) sh.wtot2[w] = nb;
+    }
     __syncthreads();
-    if (lane == 0) sh.wtot[w] = __popc(bal);
-    __syncthreads();
-    int excl = __popc(bal & ((1u << lane) - 1u)), tot = 0;
-#pragma unroll
-    for (int k = 0; k < kSelWarps; ++k) { if (k < w) excl += sh.wtot[k]; tot += sh.wtot[k]; }
+    const int wt = lane < kSelWarps ? sh.wtot[lane] : 0, tot = __reduce_add_sync(0xffffffffu, wt);
+    const int excl = __popc(bal & ((1u << lane) - 1u)) + (int)__reduce_add_sync(0xffffffffu, lane < w ? wt : 0);
+    if (c0 == 0) before0 = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? sh.wtot2[lane] : 0);
     if (ok) {
       const int pos = before0 + excl;                   // survivors with a lower index
+      if (kp) { sh.own_tok[excl] = i; sh.own_slot[excl] = pos; }
       im.keep[i] = kp ? 1 : 0;
       if (im.keep_user) im.keep_user[i] = kp ? 1 : 0;
-      if (kp) { im.kept_idx[pos] = i; im.slot[i] = pos; sh.own_tok[excl] = i; sh.own_slot[excl] = pos; }
+      if (kp) { im.kept_idx[pos] = i; im.slot[i] = pos; rn_kept<D>(im)[pos] = c0 == 0 ? rn_own : rn_tok<D>(im)[i]; }
       else { im.pruned_idx[i - pos] = i; im.slot[i] = -1 - (i - pos); }
     }
     __syncthreads();
-    for (int e = w; e < tot; e += kSelWarps) {         // one warp per surviving row
-      const int tok = sh.own_tok[e], rr = sh.own_slot[e];
-      const uint4 *src = reinterpret_cast<const uint4 *>(Kc + (size_t)tok * im.ldKc);
-      uint4 *dst = reinterpret_cast<uint4 *>(Kp + (size_t)rr * bt.d_k);
-      for (int v0 = lane; v0 < nv; v0 += 128) {
-        uint4 buf[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (v0 + 32 * u < nv) buf[u] = __ldg(src + v0 + 32 * u);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (v0 + 32 * u < nv) dst[v0 + 32 * u] = buf[u];
+    // the rows: those in shared memory by bulk copies, the others by sixteen lanes each with eight 16-byte loads in flight
+    if (npre > 0) {
+      const bool landed = mbar_wait_warp(&s_bar, 0);
+      if (!landed) {
+        land_copies(&s_bar, 1);
+        if (t == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
       }
-      if (lane == 0) rn_kept<D>(im)[rr] = rn_tok<D>(im)[tok];
+      if (landed && lane == 0) {
+        for (int r = w; r < tot; r += kSelWarps)
+          bulk_store(Kp + (size_t)sh.own_slot[r] * bt.d_k, sel_smem + (size_t)(sh.own_tok[r] - tok0) * rowb, rowb);
+        bulk_store_wait();
+      }
+      break;                                            // (all of the own tokens are in this round)
+    }
+    for (int r = t >> 4; r < tot; r += kSelThreads / 8) {
+      const int r2 = r + kSelThreads / 16 < tot ? r + kSelThreads / 16 : r;
+      const uint4 *s0 = reinterpret_cast<const uint4 *>(Kc + (size_t)sh.own_tok[r] * im.ldKc), *s1 = reinterpret_cast<const uint4 *>(Kc + (size_t)sh.own_tok[r2] * im.ldKc);
+      uint4 *d0 = reinterpret_cast<uint4 *>(Kp + (size_t)sh.own_slot[r] * bt.d_k), *d1 = reinterpret_cast<uint4 *>(Kp + (size_t)sh.own_slot[r2] * bt.d_k);
+      for (int v = t & 15; v < nv; v += 64) {
+        uint4 b0[4], b1[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v + 16 * u < nv) { b0[u] = __ldg(s0 + v + 16 * u); b1[u] = __ldg(s1 + v + 16 * u); }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v + 16 * u < nv) { d0[v + 16 * u] = b0[u]; d1[v + 16 * u] = b1[u]; }
+      }
     }
     before0 += tot;
     __syncthreads();                                    // own_tok / own_slot are rewritten by the next round
   }
-}
-
-template <typename T, int KPT, bool IN_SMEM>
-__device__ __forceinline__ void euti_select(const Batch &bt, const ImgDesc &im, uint32_t *skey, int g, int tok0, int ntok,
-                                            SelShared &sh) {
-  const int t = threadIdx.x, N = im.N;
-  uint32_t kreg[KPT > 0 ? KPT : 1];
-  int hv[kHistPerThread];                               // bins [t kHistPerThread, (t + 1) kHistPerThread) of the histogram
-  {
-    const int4 *hp = reinterpret_cast<const int4 *>(im.ghist + t * kHistPerThread);
-#pragma unroll
-    for (int u = 0; u < kHistPerThread / 4; ++u) {
-      const int4 x = __ldcg(hp + u);
-      hv[4 * u] = x.x; hv[4 * u + 1] = x.y; hv[4 * u + 2] = x.z; hv[4 * u + 3] = x.w;
-    }
-  }
-  if (KPT > 0) {
-    float sc[KPT > 0 ? KPT : 1];
-#pragma unroll
-    for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u) sc[u] = t + kSelThreads * u < N ? __ldcg(im.score + t + kSelThreads * u) : 0.f;
-#pragma unroll
-    for (int u = 0; u < (KPT > 0 ? KPT : 1); ++u) {
-      kreg[u] = score_key(sc[u]);
-      if (t + kSelThreads * u < N) skey[t + kSelThreads * u] = kreg[u];
-    }
-  } else if (IN_SMEM) {
-    for (int i = t; i < N; i += kSelThreads) skey[i] = score_key(__ldcg(im.score + i));
-  }
-  // (the first barrier inside euti_threshold orders these stores before the first read)
-  const uint32_t tau_key = euti_threshold<KPT, IN_SMEM>(im, skey, kreg, hv, sh);
-  TL_POINT(im, 7);
-  euti_compact<T, KPT, IN_SMEM>(bt, im, skey, kreg, tau_key, g, tok0, ntok, sh);
-}
-
-// KPT > 0: N <= 512 KPT for every image.  (A kernel for each case: the code runs once, from a cold instruction cache, and
-// for images of up to 3072 tokens six keys per thread in place of sixteen take 2 us off the call.)
-template <typename T, int KPT, bool IN_SMEM>
-__global__ void __launch_bounds__(kSelThreads, 2) k_select(const __grid_constant__ Batch bt) {
-  const ImgDesc &im = bt.img[blockIdx.y];
-  TL_SCOPE(im, 3);
-  pdl_wait();
-  pdl_trigger();
-  extern __shared__ uint32_t skey_dyn[];
-  __shared__ SelShared sh;
-  const int N = im.N, X = gridDim.x, x = blockIdx.x;
-  const int tpc = (N + X - 1) / X;
-  const int tok0 = min(N, x * tpc), ntok = min(N, tok0 + tpc) - tok0;
-  euti_select<T, KPT, IN_SMEM>(bt, im, skey_dyn, x, tok0, ntok, sh);
 }
 
 // ---- Eq. 3-4 as a stage of its own (pact_prune): order statistic, ordered compaction ------------------
@@ -1344,15 +1366,21 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
     size_t keys = (size_t)maxN * sizeof(uint32_t);
     const bool in_smem = keys <= kSelKeyBytes;
     if (!in_smem) keys = 0;
-    // One CTA per SM while it has few tokens: all of them begin beside k_scores (with two a tenth waited for its end; one
-    // image of 7290 tokens: 1.9 us).  With more than 128 tokens the lists and rows of K' are what counts, and two share them.
     int X = g_sm_count / bt.B;
-    if (X < 1 || (maxN + X - 1) / X > 128) X = 2 * g_sm_count / bt.B;
     const int want = (maxN + 15) / 16;         // at least sixteen tokens per CTA
     if (X > want) X = want;
     if (X < 1) X = 1;
-    const auto kernel = maxN <= 6 * kSelThreads ? k_select<T, 6, true> : maxN <= 16 * kSelThreads ? k_select<T, 16, true> : in_smem ? k_select<T, 0, true> : k_select<T, 0, false>;
-    e = launch_k(kernel, dim3(X, bt.B), dim3(kSelThreads), keys, st, true, bt);
+    const auto kernel = maxN <= 6 * kSelThreads ? k_select<T, 6, false> : maxN <= 16 * kSelThreads ? k_select<T, 16, false>
+                        : maxN <= 32 * kSelThreads ? k_select<T, 32, false> : in_smem ? k_select<T, 0, true> : k_select<T, 0, false>;
+    // The rows of the own tokens wait in shared memory where all of them fit; with more per CTA (batches, long images) what
+    // counts is their bytes, and the pruned ones would be read for nothing.
+    int pre = 0;
+    if (maxN <= 32 * kSelThreads) {
+      const int rowb = bt.d_k * (int)sizeof(T), tpc = (maxN + X - 1) / X;
+      pre = (size_t)tpc * rowb <= kSelKeyBytes && tpc <= kSelThreads ? tpc : 0;
+      keys = (size_t)pre * rowb;
+    }
+    e = launch_k(kernel, dim3(X, bt.B), dim3(kSelThreads), keys, st, true, bt, pre);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
@@ -1400,7 +1428,8 @@ cudaError_t euti_configure(int n_qcols, int n_qh) {
   for (const auto f : {k_tokens<__nv_bfloat16, true, true>, k_tokens<__nv_bfloat16, true, false>, k_tokens<__nv_bfloat16, false, true>, k_tokens<__nv_bfloat16, false, false>,
                        k_tokens<float, true, true>, k_tokens<float, true, false>, k_tokens<float, false, true>, k_tokens<float, false, false>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;
-  for (const auto f : {k_select<__nv_bfloat16, 0, true>, k_select<float, 0, true>})   // (the others need less than the default)
+  for (const auto f : {k_select<__nv_bfloat16, 0, true>, k_select<__nv_bfloat16, 6, false>, k_select<__nv_bfloat16, 16, false>, k_select<__nv_bfloat16, 32, false>,
+                       k_select<float, 0, true>, k_select<float, 6, false>, k_select<float, 16, false>, k_select<float, 32, false>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelKeyBytes)) != cudaSuccess) return e;
   // k_tokens can only begin beside k_qsum if both run under the same split of the SM's memory (with the default it waited
   // for k_qsum to drain, 9 us at 6272 tokens); for the other kernels the default is as good or better (16384-token images: 10 us)

@@ -70,8 +70,11 @@ enum RowMode { ROWS_ALL = 0, ROWS_KEPT_LIST = 1, ROWS_PRUNED_LIST = 2 };
 
 // euti.cu
 constexpr int kQPartRows = 8;             // most row blocks the column sums of Q are split into: the CTAs of a cluster
-constexpr int kHistBits = 12;             // key bits of the first-level histogram of the threshold selection
-constexpr int kHistShift = 32 - kHistBits; // a key's bin in that histogram is key >> kHistShift
+// First-level histogram of the threshold selection: scores are not negative, so a key's top bit is set (but of a NaN with its
+// sign bit set); the bins are the thirteen top bits of the others, eight of exponent and four of mantissa.
+constexpr int kHistShift = 19, kHistBins = 1 << (31 - kHistShift);
+__device__ __forceinline__ int key_bin(uint32_t key) { return max(0, (int)(key >> kHistShift) - kHistBins); }
+__device__ __forceinline__ uint32_t bin_first(int bin) { return (uint32_t)(bin + kHistBins) << kHistShift; }   // (bin 0 also holds what is below)
 // Algorithm 1.  mode 0: scores, threshold, lists, survivor keys (four kernels; the first also clears what later
 // kernels accumulate into); mode 1: scores only (three kernels); mode 2: mode 0 up to the token pass (two kernels).
 // mark (optional) is called between the kernels of the group (the per-kernel timing of a profiled call)

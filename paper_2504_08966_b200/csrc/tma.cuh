@@ -55,6 +55,16 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
+// The same way back, 16-byte aligned, a multiple of 16 bytes; after bulk_store_wait the shared memory of the thread's copies
+// so far has been read, and the kernels after this one find the data.
+__device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() {
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+
 // For a CTA that gives up after a wait that ran out: the copies it has under way still write to its shared memory, which the
 // next CTA may have by then.  Threads 0 .. n - 1 wait for a barrier each, whichever its phase: the wait for the phase that is
 // over returns at once, and one for which nothing was asked runs out.  (A call, out of the way of the code that runs.)

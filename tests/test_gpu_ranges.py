@@ -116,6 +116,33 @@ def test_select_key_registers(N):
     _check(_workload(N, 2, 1, 16, 32, torch.bfloat16, N), torch.float32)
 
 
+@pytest.mark.parametrize("N,d_h", [(1500, 64), (3100, 512), (9000, 64), (16384, 64), (16385, 64), (24577, 64)])
+@pytest.mark.parametrize("same", [1, 2, 40, 300, 10 ** 6])
+def test_split_with_equal_scores(N, d_h, same):
+    """`same` tokens with each score: one key, a few or many under the threshold's prefix, and all; a tenth are zero, then most."""
+    from paper_2504_08966_b200 import binding as pb
+    g = torch.Generator().manual_seed(N + same)
+    ctx = pb.Context(64, 1, 1, d_h, torch.bfloat16, torch.float32)
+    for zeros, lam in ((0.1, 0.95), (0.1, 0.05), (0.7, 0.8)):
+        # norms: one element per row, of more values than bf16 has between two powers of two
+        a = torch.exp(1.5 * torch.randn(N // same + 1, generator=g))[torch.arange(N) // same % (N // same + 1)][torch.randperm(N, generator=g)]
+        a[torch.rand(N, generator=g) < zeros] = 0.0
+        H = torch.zeros(N, 64)
+        for k in range(3):                        # a row's norm in three pieces of eight bits
+            H[:, k] = (a - H[:, :k].sum(1)).to(torch.bfloat16).float()
+        img = workloads.Image(H=H.to(torch.bfloat16), K=torch.randn(N, d_h, generator=g).to(torch.bfloat16), Q=torch.zeros(N, d_h, dtype=torch.bfloat16),
+                              P=torch.arange(N, dtype=torch.int32), n_total=N, vis_start=0, N=N)
+        im = pb.device_image(img, torch.float32)
+        ctx.pact_reduce([im], pb.make_params(lam=lam, d_c=1.9, flags=pb.FLAG_NORM_ONLY))
+        torch.cuda.synchronize()
+        score = im.score.cpu().numpy()
+        want = np.linalg.norm(H.numpy().astype(np.float64), axis=1) / N
+        assert (np.abs(score - want) <= 2e-7 * want).all()
+        keep = score >= np.sort(score)[int(np.floor(lam * N + 1e-6))]
+        assert np.array_equal(im.keep.cpu().numpy(), keep)
+        assert int(im.counters[pb.CNT["q"]]) == keep.sum() and int(im.counters[pb.CNT["status"]]) == 0
+
+
 @pytest.mark.parametrize("case", ["many rows", "more survivors than estimated"])
 def test_centres_outside_shared_memory(case):
     """Blocks of more than 1024 rows, adjacency words and densities that stay in global memory."""
