@@ -11,7 +11,7 @@
 //   k_select         every CTA selects the threshold (histogram bin, then radix passes inside the bin) and
 //                    counts the survivors before its tokens, then writes its share of the lists and gathers
 //                    its share of the survivor keys
-//   k_split          the split for the stage call pact_prune (scores given, no histogram): radix select
+//   k_split_regs, k_split   the split for the stage call pact_prune (scores given, no histogram): radix select
 //
 // The kernels are short chains of dependent memory round trips; each issues all the loads it can
 // before it consumes the first.
@@ -1093,60 +1093,149 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant
 
 // ---- Eq. 3-4 as a stage of its own (pact_prune): order statistic, ordered compaction ------------------
 
-// grid (1), 1024 threads; dynamic smem: N keys when KPT == 0 and keys_in_smem.
-// KPT > 0: thread t keeps the keys of tokens [t KPT, t KPT + KPT) in registers (N <= 1024 KPT);
-// KPT == 0: any N, keys in shared memory when they fit, else re-read from the scores.
+// N <= 512 KPT: grid (1), 512 threads, thread t holds the keys t, t + 512, ... in registers.  As k_select, but without a
+// histogram to begin with: keys are taken relative to the smallest one, which spreads them evenly over the digits of the first
+// pass (raw float bits of scores that span a few binades share most of their top bits), and the bits above the highest one in which
+// two keys differ need no pass.  One CTA, bound by its instructions (four
+// clocks each with 16 warps, eight with 32) and barriers: with the tokens of a thread next to one another in 1024 threads, radix passes
+// until one key was left and flags and lists written thread by thread, 7290 tokens took 8.5 us from the scores, 5 now.
+template <int KPT>
+__global__ void __launch_bounds__(kSelThreads, 1) k_split_regs(const __grid_constant__ Batch bt) {
+  const ImgDesc &im = bt.img[0];
+  TL_SCOPE(im, 3);
+  __shared__ SelShared sh;
+  __shared__ int s_base[kSelThreads];
+  static_assert(KPT * kSelWarps <= kSelThreads, "a count for each warp and key");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, N = im.N;
+  const float *score = im.score;
+  reinterpret_cast<int2 *>(sh.hist)[t] = make_int2(0, 0);
+  if (t == 0) sh.s_few = 0;
+  pdl_wait();
+  pdl_trigger();
+  uint32_t kreg[KPT], kmin = 0xffffffffu, kmax = 0u;
+  {
+    float sc[KPT];
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) sc[u] = __ldcg(score + min(t + kSelThreads * u, N - 1));   // (the last one again past the end)
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      kreg[u] = score_key(sc[u]);
+      kmin = min(kmin, kreg[u]);
+      kmax = max(kmax, kreg[u]);
+    }
+  }
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) { sh.wtot[w] = (int)kmin; sh.wtot2[w] = (int)kmax; }
+  __syncthreads();
+  const uint32_t kbase = __reduce_min_sync(0xffffffffu, (uint32_t)sh.wtot[lane & (kSelWarps - 1)]);
+  kmax = __reduce_max_sync(0xffffffffu, (uint32_t)sh.wtot2[lane & (kSelWarps - 1)]);
+  uint32_t prefix = 0u;                                 // of the threshold, relative to kbase
+  int k = im.m_target;
+  for (int hi = 32 - __clz(kmax - kbase); hi > 0;) {
+    const int lo = hi > kSelBits ? hi - kSelBits : 0;
+    const uint32_t dmask = (1u << (hi - lo)) - 1u;
+    const uint32_t above = hi >= 32 ? 0u : ~((1u << hi) - 1u);
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      const uint32_t kk = kreg[u] - kbase;
+      if (t + kSelThreads * u < N && (kk & above) == prefix) {
+        const int d = (kk >> lo) & dmask;
+        atomicAdd(&sh.hist[d], 1);
+        sh.one[d] = kk;
+      }
+    }
+    __syncthreads();
+    find_digit(k, sh);
+    const int cnt = sh.s_cnt;
+    prefix |= (uint32_t)sh.s_bin << lo;
+    k = sh.s_k;
+    if (lo == 0) break;
+    if (cnt == 1) {                                     // one key left under the prefix: it is the threshold
+      prefix = sh.one[sh.s_bin];
+      break;
+    }
+    if (cnt <= kSelFew) {
+#pragma unroll
+      for (int u = 0; u < KPT; ++u) {
+        const uint32_t kk = kreg[u] - kbase;
+        if (t + kSelThreads * u < N && (kk ^ prefix) >> lo == 0u) sh.few[atomicAdd(&sh.s_few, 1)] = kk;
+      }
+      __syncthreads();
+      if (t < cnt) {
+        const uint32_t mine = sh.few[t];
+        int less = 0, same = 0;
+        for (int j = 0; j < cnt; ++j) { less += sh.few[j] < mine; same += sh.few[j] == mine; }
+        if (less <= k && k < less + same) sh.s_prefix = mine;   // (equal keys write the same)
+      }
+      __syncthreads();
+      prefix = sh.s_prefix;
+      break;
+    }
+    hi = lo;
+  }
+  const uint32_t tau = prefix + kbase;
+
+  // ordered compaction: survivors of every 32 tokens, then before them
+  unsigned bal[KPT];
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) {
+    bal[u] = __ballot_sync(0xffffffffu, t + kSelThreads * u < N && kreg[u] >= tau);
+    if (lane == 0) s_base[u * kSelWarps + w] = __popc(bal[u]);
+  }
+  __syncthreads();
+  const int mine = t < KPT * kSelWarps ? s_base[t] : 0, incl = warp_scan(mine, lane);
+  if (lane == 31) sh.wtot[w] = incl;
+  __syncthreads();
+  const int wt = lane < kSelWarps ? sh.wtot[lane] : 0, q = __reduce_add_sync(0xffffffffu, wt);
+  s_base[t] = incl - mine + (int)__reduce_add_sync(0xffffffffu, lane < w ? wt : 0);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) {
+    const int i = t + kSelThreads * u;
+    if (i >= N) break;
+    const bool kp = (bal[u] >> lane) & 1u;
+    const int pos = s_base[u * kSelWarps + w] + __popc(bal[u] & ((1u << lane) - 1u));   // survivors with a lower index
+    im.keep[i] = kp ? 1 : 0;
+    if (kp) im.kept_idx[pos] = i;
+    else im.pruned_idx[i - pos] = i;
+  }
+  if (t == 0) {
+    im.counts_user[0] = q;
+    im.counts_user[1] = N - q;
+  }
+}
+
+// More tokens: grid (1), 1024 threads, thread t has the tokens [t CH, (t + 1) CH); dynamic smem: N keys when keys_in_smem, else
+// they are read again from the scores.
 constexpr int kSplitBits = 11;
 
-template <int KPT>
 __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt, int keys_in_smem) {
-  const ImgDesc &im = bt.img[blockIdx.y];
+  const ImgDesc &im = bt.img[0];
   TL_SCOPE(im, 3);
   pdl_wait();
   pdl_trigger();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int N = im.N;
-  extern __shared__ uint32_t skey[];                        // [N] when KPT == 0 and keys_in_smem
+  extern __shared__ uint32_t skey[];                        // [N] when keys_in_smem
   __shared__ __align__(8) int hist[1 << kSplitBits];
   __shared__ int warp_tot[32];
   __shared__ uint32_t wmin[32], wmax[32];
   __shared__ uint32_t s_prefix;
   __shared__ int s_k, s_cnt;
-  constexpr int KR = KPT > 0 ? KPT : 1;
-  const int CH = KPT > 0 ? KPT : (N + 1023) / 1024;         // tokens per thread, contiguous
-  const int i0 = min(N, t * CH), i1 = min(N, i0 + CH);
-  const int cnt_mine = i1 - i0;
-
-  // keys of this thread's tokens
-  uint32_t kreg[KR];
-  if (KPT > 0) {
-    float sc[KR];
-#pragma unroll
-    for (int j = 0; j < KR; ++j) sc[j] = j < cnt_mine ? __ldg(im.score + i0 + j) : 0.f;
-#pragma unroll
-    for (int j = 0; j < KR; ++j) kreg[j] = score_key(sc[j]);
-  } else if (keys_in_smem) {
+  const int CH = (N + 1023) / 1024;                         // tokens per thread, contiguous
+  const int i0 = min(N, t * CH), cnt_mine = min(N, i0 + CH) - i0;
+  if (keys_in_smem)
     for (int i = t; i < N; i += 1024) skey[i] = score_key(im.score[i]);
-  }
   if (t == 0) s_k = im.m_target;
   reinterpret_cast<int2 *>(hist)[t] = make_int2(0, 0);
   __syncthreads();
   // j-th key of this thread (j < cnt_mine)
-  auto key = [&](int j) -> uint32_t {
-    if (KPT > 0) return kreg[j < KR ? j : 0];
-    return keys_in_smem ? skey[i0 + j] : score_key(im.score[i0 + j]);
-  };
+  auto key = [&](int j) -> uint32_t { return keys_in_smem ? skey[i0 + j] : score_key(im.score[i0 + j]); };
 
-  // Keys are taken relative to the smallest one: that spreads them evenly over the digits of the first
-  // pass (raw float bits of scores that span a few binades share most of their top bits), and the bits
-  // above the highest one in which two keys differ need no pass.
+  // keys relative to the smallest one, as in k_split_regs
   uint32_t kmin = 0xffffffffu, kmax = 0u;
-  if (KPT > 0) {
-#pragma unroll
-    for (int j = 0; j < KR; ++j) if (j < cnt_mine) { kmin = min(kmin, kreg[j]); kmax = max(kmax, kreg[j]); }
-  } else {
-    for (int j = 0; j < cnt_mine; ++j) { const uint32_t kk = key(j); kmin = min(kmin, kk); kmax = max(kmax, kk); }
-  }
+  for (int j = 0; j < cnt_mine; ++j) { const uint32_t kk = key(j); kmin = min(kmin, kk); kmax = max(kmax, kk); }
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   kmax = __reduce_max_sync(0xffffffffu, kmax);
   if (lane == 0) { wmin[w] = kmin; wmax[w] = kmax; }
@@ -1166,17 +1255,9 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
     const uint32_t above = hi >= 32 ? 0u : ~((1u << hi) - 1u);   // bits already fixed
     const uint32_t prefix = s_prefix;
     const int k = s_k;
-    if (KPT > 0) {
-#pragma unroll
-      for (int j = 0; j < KR; ++j) {
-        const uint32_t kk = kreg[j] - kbase;
-        if (j < cnt_mine && (kk & above) == prefix) atomicAdd(&hist[(kk >> lo) & dmask], 1);
-      }
-    } else {
-      for (int j = 0; j < cnt_mine; ++j) {
-        const uint32_t kk = key(j) - kbase;
-        if ((kk & above) == prefix) atomicAdd(&hist[(kk >> lo) & dmask], 1);
-      }
+    for (int j = 0; j < cnt_mine; ++j) {
+      const uint32_t kk = key(j) - kbase;
+      if ((kk & above) == prefix) atomicAdd(&hist[(kk >> lo) & dmask], 1);
     }
     __syncthreads();
     const int2 c = reinterpret_cast<const int2 *>(hist)[t];      // every thread takes two bins
@@ -1200,14 +1281,8 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
     if (lo > 0 && s_cnt == 1) {                                  // one key left under the prefix: it is the threshold
       const uint32_t fixed = ~((1u << lo) - 1u), pre = s_prefix;
       __syncthreads();
-      if (KPT > 0) {
-#pragma unroll
-        for (int j = 0; j < KR; ++j)
-          if (j < cnt_mine && ((kreg[j] - kbase) & fixed) == pre) s_prefix = kreg[j] - kbase;
-      } else {
-        for (int j = 0; j < cnt_mine; ++j)
-          if (((key(j) - kbase) & fixed) == pre) s_prefix = key(j) - kbase;
-      }
+      for (int j = 0; j < cnt_mine; ++j)
+        if (((key(j) - kbase) & fixed) == pre) s_prefix = key(j) - kbase;
       __syncthreads();
       break;
     }
@@ -1215,16 +1290,11 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
   const uint32_t tau_key = s_prefix + kbase;
 
   // ordered compaction over the contiguous blocks of tokens
+  // more than 32 tokens per thread only beyond 32768 tokens: the bits are recomputed below then
   uint32_t keptbits = 0u;
-  if (KPT > 0) {
-#pragma unroll
-    for (int j = 0; j < KR; ++j) if (j < cnt_mine && kreg[j] >= tau_key) keptbits |= 1u << j;
-  } else {
-    // more than 32 tokens per thread only beyond 32768 tokens: the bits are recomputed below then
-    for (int j = 0; j < cnt_mine && j < 32; ++j) if (key(j) >= tau_key) keptbits |= 1u << j;
-  }
+  for (int j = 0; j < cnt_mine && j < 32; ++j) if (key(j) >= tau_key) keptbits |= 1u << j;
   int mine = 0;
-  if (KPT > 0 || CH <= 32) mine = __popc(keptbits);
+  if (CH <= 32) mine = __popc(keptbits);
   else for (int j = 0; j < cnt_mine; ++j) mine += key(j) >= tau_key;
   int incl = mine;
 #pragma unroll
@@ -1250,7 +1320,7 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
   int before = warp_tot[w] + incl - mine;                   // survivors with a lower index
   for (int j = 0; j < cnt_mine; ++j) {
     const int i = i0 + j;
-    const bool kp = (KPT > 0 || CH <= 32) ? ((keptbits >> j) & 1u) != 0u : key(j) >= tau_key;
+    const bool kp = CH <= 32 ? ((keptbits >> j) & 1u) != 0u : key(j) >= tau_key;
     im.keep[i] = kp ? 1 : 0;
     if (kp) { im.kept_idx[before] = i; ++before; }
     else im.pruned_idx[i - before] = i;
@@ -1398,11 +1468,12 @@ cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cuda
 int euti_kernels(int mode) { return mode == 0 ? 4 : mode == 1 ? 3 : 2; }
 
 cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st) {
-  if (N <= 8 * 1024) return launch_k(k_split<8>, dim3(1), dim3(1024), 0, st, true, bt, 0);
-  if (N <= 16 * 1024) return launch_k(k_split<16>, dim3(1), dim3(1024), 0, st, true, bt, 0);
+  if (N <= 6 * kSelThreads) return launch_k(k_split_regs<6>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
+  if (N <= 16 * kSelThreads) return launch_k(k_split_regs<16>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
+  if (N <= 32 * kSelThreads) return launch_k(k_split_regs<32>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
   const size_t sm = (size_t)N * sizeof(uint32_t);
   const bool in_smem = sm + kSplitReserve <= g_smem_optin;
-  return launch_k(k_split<0>, dim3(1), dim3(1024), in_smem ? sm : 0, st, true, bt, in_smem ? 1 : 0);
+  return launch_k(k_split, dim3(1), dim3(1024), in_smem ? sm : 0, st, true, bt, in_smem ? 1 : 0);
 }
 
 cudaError_t select_configure() {
@@ -1415,7 +1486,7 @@ cudaError_t select_configure() {
   e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   g_smem_optin = (size_t)v;
-  e = cudaFuncSetAttribute(k_split<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
+  e = cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
   if (e != cudaSuccess) return e;
   return e;
 }

@@ -143,6 +143,28 @@ def test_split_with_equal_scores(N, d_h, same):
         assert int(im.counters[pb.CNT["q"]]) == keep.sum() and int(im.counters[pb.CNT["status"]]) == 0
 
 
+@pytest.mark.parametrize("N", [1, 2, 31, 33, 511, 513, 3072, 3073, 8192, 8193, 16384, 16385])
+@pytest.mark.parametrize("kind", ["spread", "signs", "tenths", "pairs", "hundreds", "one value", "infinities"])
+def test_split_of_given_scores(N, kind):
+    """pact_prune around the sizes of its kernels: one, a few and many candidates under a prefix, keys that differ in every bit."""
+    from oracle import pact_oracle as orc
+    from paper_2504_08966_b200 import binding as pb
+    rng = np.random.default_rng(N)
+    x = {"spread": lambda: np.exp(3 * rng.standard_normal(N)), "signs": lambda: rng.standard_normal(N) * 10.0 ** rng.integers(-30, 30, N),
+         "tenths": lambda: rng.integers(0, 10, N) / 10, "pairs": lambda: rng.permutation(np.arange(N) // 2).astype(float),
+         "hundreds": lambda: np.exp(rng.integers(0, 1 + N // 100, N) / 7.0 % 40), "one value": lambda: np.full(N, 0.25),
+         "infinities": lambda: np.where(rng.random(N) < 0.3, np.inf, rng.standard_normal(N)) * np.where(rng.random(N) < 0.3, -1, 1)}[kind]().astype(np.float32)
+    score = torch.from_numpy(x).cuda()
+    ctx = pb.Context(64, 1, 1, 64, torch.bfloat16, torch.float32)
+    out = [torch.full((N,), 7, dtype=dt, device="cuda") for dt in (torch.uint8, torch.int32, torch.int32)] + [torch.zeros(2, dtype=torch.int32, device="cuda")]
+    for lam in (0.0, 0.3, 0.5, 0.97, 1.0):
+        ctx.pact_prune(score, pb.make_params(lam=lam), *out)
+        _, keep, kept, pruned = orc.split(x, lam)
+        assert out[3].cpu().tolist() == [kept.size, pruned.size]
+        assert np.array_equal(out[0].cpu().numpy().astype(bool), keep)
+        assert np.array_equal(out[1][:kept.size].cpu().numpy(), kept) and np.array_equal(out[2][:pruned.size].cpu().numpy(), pruned)
+
+
 @pytest.mark.parametrize("case", ["many rows", "more survivors than estimated"])
 def test_centres_outside_shared_memory(case):
     """Blocks of more than 1024 rows, adjacency words and densities that stay in global memory."""
