@@ -203,6 +203,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
   int bi = 0;
   const float d_c = im.d_c, neg_k = -im.inv_dn_log2e;
   const int r0 = tmi * BM + qd * 32;
+  uint32_t first_bits = 0u;
   const bool above = MODE == MODE_GRAM && cbase / BM > tmi;   // block above the diagonal: rows and columns
 #pragma unroll 1
   for (int ch = 0; ch < HALF / 32; ++ch) {
@@ -237,7 +238,16 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
         tmem_ld_wait();
         band += gram_band(v, rn_col + ch * 32, rni, row, c0, ncols, d_c);
       }
-      if (row_ok) im.adj[(size_t)row * im.Wp + (c0 >> 5)] = bits;
+      // Two words of a row in one store, where a warp has them: a sector of the L2 is written once instead of twice.  (Adjacency
+      // words are four bytes in a sector each and were 5 us of the 43 over 7290 keys; DBDPC of those 115.1 -> 113.3 us.)
+      if constexpr (HALF == 64) {
+        if (ch == 0) first_bits = bits;
+        if (row_ok) {
+          uint32_t *at = im.adj + (size_t)row * im.Wp + (cbase >> 5);
+          if (ch == 1) *reinterpret_cast<uint2 *>(at) = make_uint2(first_bits, bits);
+          else if (cbase + 32 >= ncols) *at = bits;
+        }
+      } else if (row_ok) im.adj[(size_t)row * im.Wp + (c0 >> 5)] = bits;
     } else if (MODE == MODE_SPREAD) {
       // The largest distance of the chunk belongs to its smallest cosine: d = clamp(1 - c) does not increase
       // with c, in floating point either, so the products dot * rn_j are compared and one cosine and distance is

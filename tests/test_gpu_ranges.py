@@ -110,6 +110,13 @@ def test_small_batches(B):
     _check(wl, torch.bfloat16)
 
 
+def test_pairs_of_ctas_with_ragged_ends():
+    """The all-pairs pass on pairs of CTAs (sixteen images of eleven blocks): last columns at every place in a word and a pair of words."""
+    wls = [_workload(1281 + 13 * b, 2, 1, 64, 64, torch.bfloat16, 60 + b) for b in range(16)]
+    wl = workloads.Workload("edge", [w.images[0] for w in wls], 64, 2, 1, 64, torch.bfloat16, 0.0, 0.3)
+    _check(wl, torch.float32)
+
+
 @pytest.mark.parametrize("N", [3072, 3073, 8192, 8193])
 def test_select_key_registers(N):
     """The last size with the keys of the split in six, in sixteen registers per thread, and the first without."""
