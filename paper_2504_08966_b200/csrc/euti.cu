@@ -190,11 +190,12 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
 //            Sums of squares in float over a 16-byte vector and in double across.  Nothing here needs the global query.
 //   logits   Two teams of four warps take the units in turn; a team's scoring keys come through a buffer of its own, in
 //            flight before the global query is known: inverse key norms; k_i . Qglobal per head in double; per head the
-//            largest logit of the unit, exp(l - that) per token and their sum.  A lane is a token (with few tokens a
-//            part of its elements), a warp has up to four query heads of a key head at a time, and their global query
+//            largest logit of the unit, exp(l - that) per token and their sum.  Up to two
+//            query heads per key head a lane is a token (with few tokens a part of its elements), and the global query
 //            comes from shared memory at one address per warp: with the lanes spread over the row the loads of the
 //            query were what took the time, and with the double-precision tensor instruction (m8n8k4, whose rate is
 //            that of the ordinary one) the seven idle heads of eight: 16 tokens of four heads took 4100 clocks a team.
+//            With more heads per key head that instruction is the better form, see group_piece.
 // `what` names the parts of the work (kTok...): hidden states that arrive from the host piece by piece have their norms
 // formed by launches of their own.
 // As 16-byte loads of four tokens per warp, one token's row at a time and the logits between them, the pass took 4.2 TB/s
@@ -652,11 +653,12 @@ norms_end:
 // CTA the heads and the pieces of a head, four loads per lane in flight; the results go to every CTA of the cluster.  What
 // turns a term into a share, exp(M_g - M) / (Z n_qh), is formed once per piece and head of the CTA's tokens.  with_hist:
 // every score also counts in the histogram of its top key bits, the first level of the threshold selection.
-// EP: terms of a token that a thread asks for before the merge (all of its half up to four heads, else eight).
+// EP: terms of a token that a thread asks for before the merge (all of its half up to four heads, else eight, with 128 registers:
+// at 64 some are spilled, 1 us of a call with 28 heads, although the CTA could then begin beside k_tokens).
 // Bound by latency and by the instructions it takes: what does not depend on k_tokens comes before the wait for it (a microsecond of
 // divisions), a value that has to be spilled while it is loaded costs its whole latency, and two exponentials at a time come
-// from one copy of the code.  With every CTA merging all heads, 286 pieces of 28 heads took 22 us, 10 now; three images with
-// 28 heads (5190 tokens) 13 us, 10 now; four heads 4.9 us, 4.1 now.  (Going through the code once before the wait, to have the
+// from one copy of the code.  With every CTA merging all heads, 286 pieces of 28 heads took 22 us, 9 now; three images with
+// 28 heads (5190 tokens) 13 us, 9 now; four heads 4.9 us, 4.1 now.  (Going through the code once before the wait, to have the
 // instructions in the cache, halved the time behind the wait and cost as much before it.)
 constexpr int kScoreTok = 256;                          // tokens per CTA
 constexpr int kScoreThreads = 2 * kScoreTok;
@@ -666,7 +668,7 @@ constexpr int kScorePieces = kScoreTok / kMinPiece + 1; // most pieces that a CT
 constexpr int kScoreMaxCl = 8;
 
 template <int EP>
-__global__ void __launch_bounds__(kScoreThreads, 2) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist, int CL) {
+__global__ void __launch_bounds__(kScoreThreads, EP > 2 ? 1 : 2) k_scores(const __grid_constant__ Batch bt, int rpp, int with_hist, int CL) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 2);
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
