@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
       for (int u = 0; u < 4; ++u)
         if (l + u * kCenWarps < nsm) sadj[(size_t)(l + u * kCenWarps) * nv + v] = x[u];
     }
-  if (in_smem && !mbar_wait_warp(&s_bar, 0) && lane == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+  if (in_smem) mbar_wait_warp_or_report(&s_bar, 0, &im.cnt[PACT_CNT_STATUS]);
   __syncthreads();
   TL_POINT(bt.img[0], 10);
 

@@ -1062,11 +1062,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant
     __syncthreads();
     // the rows: those in shared memory by bulk copies, the others by sixteen lanes each with eight 16-byte loads in flight
     if (npre > 0) {
-      const bool landed = mbar_wait_warp(&s_bar, 0);
-      if (!landed) {
-        land_copies(&s_bar, 1);
-        if (t == 0) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
-      }
+      const bool landed = mbar_wait_warp_or_report(&s_bar, 0, &im.cnt[PACT_CNT_STATUS]);
+      if (!landed) land_copies(&s_bar, 1);              // (thread 0 waits for them, if its own wait ran out)
       if (landed && lane == 0) {
         for (int r = w; r < tot; r += kSelWarps)
           bulk_store(Kp + (size_t)sh.own_slot[r] * bt.d_k, sel_smem + (size_t)(sh.own_tok[r] - tok0) * rowb, rowb);

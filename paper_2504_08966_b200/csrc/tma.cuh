@@ -3,6 +3,8 @@
 #pragma once
 #include <stdint.h>
 
+#include "../../include/pact.h"
+
 namespace pact {
 
 constexpr unsigned long long kWaitNs = 1000000000ull;   // one second per wait, then give up
@@ -81,6 +83,14 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// The same for warps that go on by themselves: whichever of them gives up raises the status word (one warp's wait may run out
+// and another's not, a moment later).
+__device__ __forceinline__ bool mbar_wait_warp_or_report(uint64_t *bar, uint32_t parity, int32_t *status) {
+  const bool ok = mbar_wait_warp(bar, parity);
+  if (!ok && (threadIdx.x & 31) == 0) atomicMin(status, (int32_t)PACT_ERR_TIMEOUT);
+  return ok;
 }
 
 }  // namespace pact
