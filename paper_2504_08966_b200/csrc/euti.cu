@@ -573,7 +573,7 @@ norms_end:
       const uint8_t *keys = cfg.keys ? s_mine : reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.Ke) + (size_t)r0 * im.ldKe);
       const size_t kstride = cfg.keys ? (size_t)ks : (size_t)im.ldKe * sizeof(T);
       if (mine) {
-        if (cfg.keys && !mbar_wait_warp(&s_kbar[team], par)) s_abort = 1;   // (on through the teams' barriers, but without copies)
+        if (cfg.keys && !mbar_wait_warp_unless(&s_abort, &s_kbar[team], par)) s_abort = 1;   // (on through the teams' barriers, but without copies)
         par ^= 1u;
         if (im.Kc) {                                     // inverse norms: eight lanes per row, four rows at a time
           const bool same = cfg.keys && im.Kc == im.Ke;

@@ -32,3 +32,15 @@ def test_any_warp_reports_a_wait_that_ran_out(waits, late):
     torch.cuda.synchronize()
     assert ok.tolist() == [int(w != late) for w in range(WARPS)]
     assert status.tolist() == [-5 if late >= 0 else 0]
+
+
+def test_a_cta_that_has_given_up_does_not_wait_again(waits):
+    """Twenty waits after one another take the second of the first one, not twenty."""
+    failed = torch.zeros(WARPS, dtype=torch.int32, device="cuda")
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    begin.record()
+    assert waits.many_waits(20, WARPS, C.c_void_p(failed.data_ptr()), _stream()) == 0
+    end.record()
+    torch.cuda.synchronize()
+    assert failed.tolist() == [20] * WARPS
+    assert begin.elapsed_time(end) < 3000
