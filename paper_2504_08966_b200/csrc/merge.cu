@@ -536,14 +536,15 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
       if ((t & 31) != 0 || *const_cast<volatile int *>(&s_abort)) return;   // (nothing is asked for after a wait that ran out)
       if (t == 0) mbar_arrive_expect_tx(&s_bar[hh], (uint32_t)n * rowb);
       for (int k = t >> 5; k < n; k += kMrgThreads / 32)
-          bulk_load(reinterpret_cast<uint8_t *>(ring) + (size_t)(hh * half + k) * rowb, H + (size_t)s_row[j + k] * im.ldH, rowb, &s_bar[hh]);
+        bulk_load(reinterpret_cast<uint8_t *>(ring) + (size_t)(hh * half + k) * rowb, H + (size_t)s_row[j + k] * im.ldH, rowb, &s_bar[hh]);
     };
     const int j0 = max(start - t0, 0);                // (a first tile may begin with items of the range before)
     issue(j0, h);
     issue(j0 + half, h ^ 1);
 #pragma unroll 1
     for (int jh = j0; jh < tn; jh += half) {
-      if (!mbar_wait_warp(&s_bar[h], (par >> h) & 1)) s_abort = 1;
+      // (after a wait that ran out the CTA goes on through its barriers and tickets, but without copies and without waiting)
+      if (!mbar_wait_warp_unless(&s_abort, &s_bar[h], (par >> h) & 1)) s_abort = 1;
       par ^= 1u << h;
       const uint8_t *buf = reinterpret_cast<const uint8_t *>(ring) + (size_t)(h * half) * rowb + (size_t)t * 8 * sizeof(T);
       const int je = min(jh + half, tn);
