@@ -5,11 +5,11 @@
 #include <stdint.h>
 
 #include "../../include/pact.h"
+#include "tok_units.h"
 
 namespace pact {
 
 constexpr int kMaxBatchPerLaunch = 16;   // images described by one kernel parameter block
-constexpr int kMinPiece = 8;             // fewest visual tokens in a softmax piece of k_tokens (at most 32)
 constexpr uint32_t kRhoShift = 30;       // density terms are summed as integers scaled by 2^30
 constexpr unsigned long long kBestInit = 0xFFFFFFFFFFFFFFFFull;
 constexpr int kCntSpread = 24;           // slot of cnt[]: largest key distance of a layer, as float bits

@@ -205,24 +205,8 @@ constexpr int kTokInit = 1, kTokNorms = 2, kTokLogits = 4;
 constexpr int kTokThreads = 512;
 constexpr int kTokGroup = 256;                          // threads of the norms group and of the logits group
 constexpr int kTokTeam = kTokGroup / 2;                 // threads of a logits team
-constexpr int kTokWarps = kTokGroup / 32;
+static_assert(kTokWarps == kTokGroup / 32, "a row buffer for each warp of the norms");
 constexpr int kTeamWarps = kTokTeam / 32;
-constexpr int kTokMaxBuf = 2;                           // row buffers per warp
-constexpr int kTokSmem = 200 * 1024;
-constexpr int kGroupHeads = 3;                          // query heads per key head from which they go through group_piece
-
-struct TokCfg {
-  int rpp;                                              // tokens per unit (piece)
-  int chunk, nchunk;                                    // bytes of a hidden-state row per copy, copies per row
-  int nbuf;                                             // row buffers per warp
-  int keys;                                             // a key buffer per team (else the keys are read from global memory)
-  int query;                                            // the global query in shared memory (else read from global memory)
-};
-// stride of a key row in shared memory: an odd number of 16-byte vectors, so that a vector of 8 rows is in 8 different banks
-__host__ __device__ inline int tok_key_stride(int row_bytes) { return row_bytes | 16; }
-inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
-  return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)c.query * n_qcols * 8 + (size_t)c.rpp * 32 * 8;
-}
 
 // Logits of this lane's token (its vectors p, p + P, ... of nv) with RB heads of a key head, q at one address per part.
 // NaN if an element is not finite (even where the sum would be minus infinity and the token's share zero: to sum such keys again
@@ -334,7 +318,7 @@ __device__ __forceinline__ double max_by_bits(double a, double b) {
 // bytes a clock: 32 tokens of one head of 128 cost 256 clocks of it, against 512 clocks of the double-precision unit for up
 // to eight heads here.  So heads come here from three per key head on: three images, 5190 tokens, 28 heads on 4 key heads:
 // 13 us from the query to the pieces with a token per lane, 5 here; one of 7426 tokens 14 and 9.
-// NB: blocks of eight tokens.  SMEM: keys and query are in shared memory.
+// NB: blocks of eight tokens.  SMEM: keys and query are in shared memory (else a unit is one block).
 template <typename T, int NB, bool SMEM>
 __device__ __forceinline__ void group_piece(const Batch &bt, const ImgDesc &im, const uint8_t *kh, size_t kstride, const double *q,
                                             bool use_query, int nr, int j0, int r0, int n, int g) {
@@ -618,7 +602,7 @@ norms_end:
         for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
           const int kv = it / nblk, j = (it - kv * nblk) * 8, j0 = kv * n_rep + j, nr = min(8, n_rep - j);
           const uint8_t *kh = keys + (size_t)kv * d_h * sizeof(T);
-          if (!in_smem) group_piece<T, 4, false>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          if (!in_smem) group_piece<T, 1, false>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);   // (n <= kMinPiece)
           else if (n <= 8) group_piece<T, 1, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
           else if (n <= 16) group_piece<T, 2, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
           else if (n <= 24) group_piece<T, 3, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
@@ -1354,35 +1338,10 @@ static cudaError_t launch_qsum(const Batch &bt, cudaStream_t st) {
   return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster);
 }
 
-// Tokens per unit: the fewest rounds of units of `most` tokens over the SMs, then as few tokens as that many rounds allow
-// (but eight), so that the rounds are full.  Keys, then a part of the row buffers, then the global query (more than 26496
-// columns with the largest rows) go without shared memory where it is too small.
 template <typename T> static TokCfg tokens_config(const Batch &bt) {
-  TokCfg c;
   long long total = 0;
   for (int b = 0; b < bt.B; ++b) total += bt.img[b].N;
-  const int rowb = bt.d * (int)sizeof(T), keyb = bt.d_k * (int)sizeof(T);
-  c.nchunk = (rowb + 8191) / 8192;
-  c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
-  c.nbuf = kTokMaxBuf;
-  c.keys = 1;
-  c.query = 1;
-  const auto fits = [&]() { return tok_smem(c, keyb, bt.n_qcols) <= (size_t)kTokSmem; };
-  for (int most = 32; most >= kMinPiece; most /= 2) {
-    long long rounds = (total + (long long)most * g_sm_count - 1) / ((long long)most * g_sm_count);
-    // (a unit for each of the two teams, where the logits are what takes the time)
-    if (rounds < 2 && bt.n_qh / bt.n_kvh >= kGroupHeads) rounds = 2;
-    const long long rpp = (total + rounds * g_sm_count - 1) / (rounds * g_sm_count);
-    c.rpp = (int)(rpp < kMinPiece ? kMinPiece : rpp);
-    if (fits()) return c;
-  }
-  c.keys = 0;                                                             // very wide keys or queries
-  while (!fits() && c.chunk > 1024) {
-    c.nchunk *= 2;
-    c.chunk = ((rowb + c.nchunk - 1) / c.nchunk + 15) / 16 * 16;
-  }
-  c.query = tok_smem(c, keyb, bt.n_qcols) <= g_smem_optin - kTokReserve;
-  return c;
+  return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, g_sm_count, g_smem_optin - kTokReserve);
 }
 static int tokens_grid(const Batch &bt, int rpp) {
   long long units = 0;

@@ -83,6 +83,17 @@ def test_token_units(N, n_qh, n_kvh, d_h, d, dtype, scale, rope):
     _check(_workload(N, n_qh, n_kvh, d_h, d, dtype, N, scale, rope), torch.float32)
 
 
+@pytest.mark.parametrize("N,n_qh,n_kvh,d_h,d,dtype", [
+    (43, 64, 8, 128, 8192, torch.bfloat16), (2369, 64, 8, 128, 8192, torch.bfloat16),    # rows in halves beside the keys: units of eight and nine
+    (301, 32, 8, 128, 4096, torch.float32), (1185, 16, 16, 128, 8192, torch.bfloat16),
+    (301, 128, 8, 128, 8192, torch.bfloat16), (9, 96, 32, 96, 8192, torch.float32),       # no room for the keys: grouped heads, eight tokens
+    (301, 40, 40, 128, 8192, torch.bfloat16),                                            # ... one head per key head
+])
+def test_wide_keys_and_queries(N, n_qh, n_kvh, d_h, d, dtype):
+    """Models whose keys, global query and hidden states do not fit an SM's shared memory together."""
+    _check(_workload(N, n_qh, n_kvh, d_h, d, dtype, N + d), torch.float32)
+
+
 @pytest.mark.parametrize("N,n_qh,n_kvh,d_h,dtype", [
     (2368, 8, 1, 64, torch.bfloat16), (2369, 3, 1, 64, torch.bfloat16),       # units of eight and nine tokens: one block of eight, two
     (4736, 18, 2, 40, torch.bfloat16), (4737, 6, 2, 64, torch.float32),       # sixteen, seventeen; nine heads: eight and one
