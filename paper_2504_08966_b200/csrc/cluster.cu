@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(kCenThreads, 1) k_centers(const __grid_constan
     mbar_init(&s_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // the number of survivors was final before the all-pairs pass began, and this kernel cannot start before every CTA of that
-  // pass has begun: it may be read ahead of the wait (DBDPC and merge of 7290 tokens 113.9 -> 112.9 us with that here and in k_center_keys)
+  // the number of survivors comes from a kernel before the all-pairs pass, and this kernel begins when every CTA of that pass is
+  // past its wait (pdl_trigger() never comes first): it may be read ahead of the wait (DBDPC and merge of 7290 tokens 113.9 -> 112.9 us with that here and in k_center_keys)
   const int q = (int)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(im.q_ptr)), nw = (q + 31) >> 5, nv = (nw + 3) >> 2;
   const int rows = (q + ncta - 1) / ncta, r0 = min(q, rank * rows), n = min(q, r0 + rows) - r0;
   for (int wd = t; wd < nw; wd += kCenThreads) rm[wd] = 0u;

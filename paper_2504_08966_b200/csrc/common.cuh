@@ -242,6 +242,10 @@ __device__ __forceinline__ uint32_t score_key(float s) {
 // over the hidden states) runs before.  pdl_trigger() in the predecessor lets the successor's CTAs be
 // scheduled from then on.  Every CTA of every kernel calls pdl_wait() before it returns, so completion of a
 // kernel implies completion of all kernels before it.
+// No CTA calls pdl_trigger() before pdl_wait().  So when a kernel begins, every CTA of its predecessor is past its wait (or has
+// ended), and everything before the predecessor is complete and visible: what a kernel reads ahead of its own wait may come
+// from there (k_tokens: the call's inputs; k_centers and k_center_keys: the number of survivors), though never from the predecessor itself.
+// A trigger ahead of the wait in any kernel would make such a read stale without a sign.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

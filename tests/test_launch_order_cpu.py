@@ -1,0 +1,70 @@
+"""Kernels read ahead of pdl_wait() what comes from before their predecessor (csrc/common.cuh).  That rests on every kernel of
+the chain: no trigger and no return before the wait.  Read from the source, block by block."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2504_08966_b200", "csrc")
+FILES = sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def _read(name):
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    return re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+
+
+def _kernels(text):
+    """(name, body) of every __global__ function."""
+    for m in re.finditer(r"__global__[^;{]*?\b(k_\w+)\s*\(", text):
+        start = text.index("{", m.end())
+        depth, i = 1, start + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        yield m.group(1), text[start:i]
+
+
+def _too_early(body):
+    """Triggers and returns that no wait precedes in their block or one around it (returns of lambdas aside)."""
+    waited, in_lambda, bad, begin = [False], [False], [], 0
+    for m in re.finditer(r"[{};]|\bpdl_wait\(\)|\bpdl_trigger\(\)|\breturn\b", body):
+        tok = m.group(0)
+        if tok == "{":
+            waited.append(waited[-1])
+            in_lambda.append(in_lambda[-1] or bool(re.search(r"\[&?\]\s*\(", body[begin:m.start()])))
+        elif tok == "}":
+            waited.pop()
+            in_lambda.pop()
+        elif tok == "pdl_wait()":
+            waited[-1] = True
+        elif tok == "pdl_trigger()" and not waited[-1]:
+            bad.append("trigger")
+        elif tok == "return" and not waited[-1] and not in_lambda[-1]:
+            bad.append("return")
+        if tok in "{};":
+            begin = m.end()
+    return bad
+
+
+KERNELS = [(f, name, body) for f in FILES for name, body in _kernels(_read(f))]
+
+
+def test_all_kernels_are_found():
+    names = {name for _, name, _ in KERNELS}
+    assert {"k_qsum", "k_tokens", "k_scores", "k_select", "k_split", "k_split_regs", "k_tiles_umma", "k_tiles_pair", "k_centers", "k_center_keys", "k_members",
+            "k_lists", "k_merge", "k_small"} <= names
+
+
+@pytest.mark.parametrize("f,name,body", [pytest.param(*k, id=k[1]) for k in KERNELS])
+def test_nothing_is_triggered_before_the_wait(f, name, body):
+    assert "pdl_wait()" in body and not _too_early(body), f
+
+
+def test_a_planted_trigger_is_found():
+    for name, want in (("k_select", ["trigger"]), ("k_qsum", ["trigger"]), ("k_centers", ["trigger"])):
+        body = next(b for _, n, b in KERNELS if n == name)
+        early = re.sub(r"pdl_wait\(\);\s*pdl_trigger\(\);", "pdl_trigger(); pdl_wait();", body, count=1)
+        assert early != body and _too_early(early) == want
+    body = next(b for _, n, b in KERNELS if n == "k_scores")
+    assert _too_early(body.replace("pdl_wait();", ";", 1)) == ["return"]
