@@ -16,7 +16,7 @@ struct pact_ctx {
   int d, n_qh, n_kvh, d_h, d_k, n_qcols;
   pact_dtype in, out;
   int elt;                 // bytes per input element
-  ClusterCfg ccfg;
+  DeviceCfg dev;           // of the device the context was created on
   bool umma;               // bf16 keys of a width the tcgen05 tile kernels take
   int device;
   char err[256];
@@ -247,11 +247,12 @@ pact_status pact_create(pact_ctx **out, int d, int n_qh, int n_kvh, int d_h, pac
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
     if (e == cudaSuccess && major != 10) { delete c; return PACT_ERR_UNSUPPORTED; }
   }
-  if (e == cudaSuccess) e = euti_configure(c->n_qcols, n_qh);
-  if (e == cudaSuccess) e = cluster_configure(&c->ccfg);
-  if (e == cudaSuccess) e = merge_configure();
-  if (e == cudaSuccess) e = small_configure();
-  if (e == cudaSuccess && in == PACT_BF16) e = umma_configure();
+  if (e == cudaSuccess) e = select_configure(&c->dev);
+  if (e == cudaSuccess) e = euti_configure(c->dev, c->n_qcols, n_qh);
+  if (e == cudaSuccess) e = cluster_configure(&c->dev);
+  if (e == cudaSuccess) e = merge_configure(&c->dev);
+  if (e == cudaSuccess) e = small_configure(&c->dev);
+  if (e == cudaSuccess && in == PACT_BF16) e = umma_configure(&c->dev);
   if (e != cudaSuccess) {
     pact_status s = fail_cuda(ctx, e, "pact_create");
     (void)s;
@@ -351,7 +352,7 @@ pact_status pact_importance(pact_ctx *ctx, const pact_image *img, const pact_par
   m.score_user = score;
   set_params(m, p, img->N);
   point_counts_at_workspace(m);
-  CK(launch_euti(bt, img->N, ctx->in == PACT_BF16, 1, st));
+  CK(launch_euti(bt, img->N, ctx->in == PACT_BF16, 1, ctx->dev, st));
   ctx->launches += euti_kernels(1);
   CK(cudaGetLastError());
   return PACT_OK;
@@ -377,7 +378,7 @@ pact_status pact_prune(pact_ctx *ctx, const float *score, int N, const pact_para
   m.score = const_cast<float *>(score);
   m.keep = keep; m.kept_idx = kept_idx; m.pruned_idx = pruned_idx;
   m.counts_user = counts;
-  CK(launch_split(bt, N, st));
+  CK(launch_split(bt, N, ctx->dev, st));
   ctx->launches += 1;
   CK(cudaGetLastError());
   return PACT_OK;
@@ -408,11 +409,11 @@ pact_status pact_dbdpc(pact_ctx *ctx, const void *K, int64_t ldK, int N, const i
   m.q_ptr = q_dev;
   m.rho_user = rho; m.center_idx_user = center_idx; m.C_user = C_dev; m.label_user = label;
   CK(launch_keynorm_gather(bt, N, bf, st));
-  if (ctx->umma) CK(launch_gram_umma(bt, N, ctx->ccfg, st));
-  else CK(launch_gram(bt, N, bf, ctx->ccfg, st));
-  CK(launch_centers(bt, N, bf, ctx->ccfg, ctx->sweep_limit, st));
-  if (ctx->umma) CK(launch_assign_umma(bt, N, true, ctx->ccfg, st));
-  else CK(launch_assign(bt, N, bf, ROWS_KEPT_LIST, ctx->ccfg, st));
+  if (ctx->umma) CK(launch_gram_umma(bt, N, ctx->dev, st));
+  else CK(launch_gram(bt, N, bf, ctx->dev, st));
+  CK(launch_centers(bt, N, bf, ctx->dev, ctx->sweep_limit, st));
+  if (ctx->umma) CK(launch_assign_umma(bt, N, true, ctx->dev, st));
+  else CK(launch_assign(bt, N, bf, ROWS_KEPT_LIST, ctx->dev, st));
   CK(launch_label(bt, N, bf, ROWS_KEPT_LIST, st));
   ctx->launches += 6;
   CK(cudaGetLastError());
@@ -447,8 +448,8 @@ pact_status pact_key_spread(pact_ctx *ctx, const void *const *K_layers, int n_la
       point_counts_at_workspace(m);
     }
     CK(launch_key_rnorm(bt, N, bf, st));
-    if (ctx->umma) CK(launch_spread_umma(bt, N, ctx->ccfg, st));
-    else CK(launch_spread(bt, N, bf, ctx->ccfg, st));
+    if (ctx->umma) CK(launch_spread_umma(bt, N, ctx->dev, st));
+    else CK(launch_spread(bt, N, bf, ctx->dev, st));
     CK(launch_spread_finish(bt, max_dist, layer_out, base, threshold, st));
     ctx->launches += 3;
     CK(cudaGetLastError());
@@ -484,8 +485,8 @@ pact_status pact_reincorporate(pact_ctx *ctx, const void *K, int64_t ldK, int N,
   // the rows x centres pass on the tensor cores covers every token (the survivors' distances are computed
   // and not used), so every token needs its inverse key norm
   CK(launch_center_key_gather(bt, N, bf, ctx->umma, st));
-  if (ctx->umma) CK(launch_assign_umma(bt, N, false, ctx->ccfg, st));
-  else CK(launch_assign(bt, N, bf, ROWS_PRUNED_LIST, ctx->ccfg, st));
+  if (ctx->umma) CK(launch_assign_umma(bt, N, false, ctx->dev, st));
+  else CK(launch_assign(bt, N, bf, ROWS_PRUNED_LIST, ctx->dev, st));
   CK(launch_label(bt, N, bf, ROWS_PRUNED_LIST, st));
   ctx->launches += 3;
   CK(cudaGetLastError());
@@ -515,9 +516,9 @@ pact_status pact_merge(pact_ctx *ctx, const pact_image *img, const int32_t *labe
   m.label = const_cast<int32_t *>(label);
   m.C_ptr = C_dev; m.cidx_ptr = center_idx;
   CK(launch_list_clear(bt, st));
-  CK(launch_lists(bt, img->N, ctx->in == PACT_BF16, false, ctx->spin_limit, st));
-  CK(launch_merge(bt, ctx->in == PACT_BF16, ctx->out == PACT_BF16, ctx->ccfg, st));
-  ctx->launches += lists_kernels(img->N, 1) + 2;
+  CK(launch_lists(bt, img->N, ctx->in == PACT_BF16, false, ctx->spin_limit, ctx->dev, st));
+  CK(launch_merge(bt, ctx->in == PACT_BF16, ctx->out == PACT_BF16, ctx->dev, st));
+  ctx->launches += lists_kernels(img->N, 1, ctx->dev) + 2;
   CK(cudaGetLastError());
   return PACT_OK;
 }
@@ -557,12 +558,12 @@ static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, c
       cmaxQ = qest > cmaxQ ? qest : cmaxQ;
     }
     // (a profiled call is launched kernel by kernel)
-    if (!ctx->prof_on && small_fits(bt, cmaxN, ctx->umma, ctx->ccfg)) {
+    if (!ctx->prof_on && small_fits(bt, cmaxN, ctx->umma, ctx->dev)) {
       int rpp = 0;
-      if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 2, st, *feed, &rpp));
-      else CK(launch_euti(bt, cmaxN, bf, 2, st, nullptr, nullptr, &rpp));
+      if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 2, ctx->dev, st, *feed, &rpp));
+      else CK(launch_euti(bt, cmaxN, bf, 2, ctx->dev, st, nullptr, nullptr, &rpp));
       CK(launch_small(bt, bf, ctx->umma, rpp, ctx->sweep_limit, st));
-      CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->ccfg, st));
+      CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->dev, st));
       ctx->launches += euti_kernels(2) + 2;
       continue;
     }
@@ -577,26 +578,26 @@ static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, c
     struct MarkFn {
       static cudaError_t call(void *p) { return (*static_cast<decltype(mark) *>(p))(); }
     };
-    if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 0, st, *feed, nullptr));
-    else CK(launch_euti(bt, cmaxN, bf, 0, st, ctx->prof_on ? &MarkFn::call : nullptr, &mark));
+    if (feed) CK(launch_euti_fed(bt, cmaxN, bf, 0, ctx->dev, st, *feed, nullptr));
+    else CK(launch_euti(bt, cmaxN, bf, 0, ctx->dev, st, ctx->prof_on ? &MarkFn::call : nullptr, &mark));
     CK(mark());
-    if (ctx->umma) CK(launch_gram_umma(bt, cmaxN, ctx->ccfg, st, cmaxQ));
-    else CK(launch_gram(bt, cmaxN, bf, ctx->ccfg, st));
+    if (ctx->umma) CK(launch_gram_umma(bt, cmaxN, ctx->dev, st, cmaxQ));
+    else CK(launch_gram(bt, cmaxN, bf, ctx->dev, st));
     CK(mark());
-    CK(launch_centers(bt, cmaxQ, bf, ctx->ccfg, ctx->sweep_limit, st));  CK(mark());
+    CK(launch_centers(bt, cmaxQ, bf, ctx->dev, ctx->sweep_limit, st));  CK(mark());
     // On the tensor-core path with little work per SM (one image) the labels and member counts are formed as
     // the rows x centres pass finishes groups of rows, and one kernel places the members.  With much work per SM
     // the pass runs on pairs of CTAs, and k_lists forms labels and lists as it does on the fp32 path.
-    const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, nb, ctx->ccfg);
+    const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, nb, ctx->dev);
     const bool fused_labels = ctx->umma && !pairs;
-    if (ctx->umma) CK(launch_assign_umma(bt, cmaxN, false, ctx->ccfg, st, fused_labels, pairs));
-    else CK(launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->ccfg, st));
+    if (ctx->umma) CK(launch_assign_umma(bt, cmaxN, false, ctx->dev, st, fused_labels, pairs));
+    else CK(launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->dev, st));
     CK(mark());
     if (fused_labels) CK(launch_members(bt, cmaxN, st));
-    else CK(launch_lists(bt, cmaxN, bf, true, ctx->spin_limit, st));
+    else CK(launch_lists(bt, cmaxN, bf, true, ctx->spin_limit, ctx->dev, st));
     CK(mark());
-    CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->ccfg, st));  CK(mark());
-    ctx->launches += euti_kernels(0) + 5 + (fused_labels ? 1 : lists_kernels(cmaxN, nb));
+    CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->dev, st));  CK(mark());
+    ctx->launches += euti_kernels(0) + 5 + (fused_labels ? 1 : lists_kernels(cmaxN, nb, ctx->dev));
     CK(cudaGetLastError());
   }
   return PACT_OK;

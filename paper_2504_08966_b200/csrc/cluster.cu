@@ -558,17 +558,9 @@ __global__ void __launch_bounds__(256) k_label(const __grid_constant__ Batch bt,
 
 // ---- launchers ---------------------------------------------------------------------------------
 
-cudaError_t cluster_configure(ClusterCfg *cfg) {
-  int dev = 0, sms = 0, optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
-  cfg->sm_count = sms;
-  cfg->centers_smem_max = optin - 1024;
-  e = cudaFuncSetAttribute(k_centers, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
+cudaError_t cluster_configure(DeviceCfg *cfg) {
+  cfg->centers_smem_max = (int)cfg->smem_optin - 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_centers, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg->centers_smem_max);
   constexpr int masks = (kMaxTokens / 32 + 4) * 12;
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_center_keys<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, masks);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_center_keys<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, masks);
@@ -589,13 +581,13 @@ cudaError_t launch_center_key_gather(const Batch &bt, int maxN, bool bf16, bool 
 
 static int tile_grid(long long tiles, int cap) { return (int)(tiles < 1 ? 1 : (tiles > cap ? cap : tiles)); }
 
-cudaError_t launch_gram(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_gram(const Batch &bt, int maxN, bool bf16, const DeviceCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
   dim3 grid(tile_grid(nt * (nt + 1) / 2, cfg.sm_count * 5), bt.B);
   return PACT_DISPATCH(bf16, k_gram_f64, grid, kTileThreads, st, bt);
 }
 
-cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCfg &cfg, int sweep_limit, cudaStream_t st) {
+cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const DeviceCfg &cfg, int sweep_limit, cudaStream_t st) {
   // maxQ is an estimate of the largest survivor count (ties can exceed it): the masks are sized for every token, densities
   // and adjacency by the estimate, and what does not fit is read from global memory.
   int maxN = 1;
@@ -616,7 +608,7 @@ cudaError_t launch_centers(const Batch &bt, int maxQ, bool bf16, const ClusterCf
               : launch_k(k_center_keys<float>, grid, block, (size_t)mask_cap * 12, st, true, bt, mask_cap);
 }
 
-cudaError_t launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_assign(const Batch &bt, int maxN, bool bf16, RowMode mode, const DeviceCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
   dim3 grid(tile_grid(nt * nt, cfg.sm_count * 5), bt.B);
   return PACT_DISPATCH(bf16, k_assign_f64, grid, kTileThreads, st, bt, (int)mode);
@@ -627,7 +619,7 @@ cudaError_t launch_key_rnorm(const Batch &bt, int maxN, bool bf16, cudaStream_t 
   return PACT_DISPATCH(bf16, k_key_rnorm, grid, 256, st, bt);
 }
 
-cudaError_t launch_spread(const Batch &bt, int maxN, bool bf16, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_spread(const Batch &bt, int maxN, bool bf16, const DeviceCfg &cfg, cudaStream_t st) {
   const long long nt = (maxN + TS - 1) / TS;
   dim3 grid(tile_grid(nt * (nt + 1) / 2, cfg.sm_count * 5), bt.B);
   return PACT_DISPATCH(bf16, k_spread_f64, grid, kTileThreads, st, bt);

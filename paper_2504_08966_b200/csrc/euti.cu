@@ -17,7 +17,6 @@
 // before it consumes the first.
 #include <string.h>
 
-#include <atomic>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -1317,57 +1316,55 @@ __global__ void __launch_bounds__(1024) k_split(const __grid_constant__ Batch bt
 // ---- launchers -----------------------------------------------------------------------------
 
 namespace {
-std::atomic<int> g_sm_count{148};            // (any thread may configure a device)
-std::atomic<size_t> g_smem_optin{48 * 1024};
 constexpr size_t kSplitReserve = 12288;      // static shared memory of k_split, rounded up
 constexpr size_t kTokReserve = 2048;         // of k_tokens
 }  // namespace
 
 template <typename T>
-static cudaError_t launch_qsum(const Batch &bt, cudaStream_t st) {
+static cudaError_t launch_qsum(const Batch &bt, const DeviceCfg &cfg, cudaStream_t st) {
   // column groups of four vectors where that does not take more CTAs than two per SM, else of eight; then as many row
   // blocks (CTAs of a cluster) as keep the grid within three CTAs per SM (three images with 28 query heads: 168 CTAs of
   // very different length took 26 us, twice as many take 20; with five per SM k_tokens has no room beside them)
   const int nvq = bt.n_qcols / Vec<T>::N;
-  const bool narrow = (nvq + 3) / 4 * bt.B * kQPartRows <= 2 * g_sm_count;
+  const bool narrow = (nvq + 3) / 4 * bt.B * kQPartRows <= 2 * cfg.sm_count;
   const int ncg = narrow ? (nvq + 3) / 4 : (nvq + 7) / 8;
   LaunchOpt opt;
   opt.cluster = 1;
-  while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 3 * g_sm_count) opt.cluster *= 2;
+  while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 3 * cfg.sm_count) opt.cluster *= 2;
   const dim3 grid(ncg * opt.cluster, bt.B), block(kQsumThreads);
   return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster);
 }
 
-template <typename T> static TokCfg tokens_config(const Batch &bt) {
+template <typename T> static TokCfg tokens_config(const Batch &bt, const DeviceCfg &cfg) {
   long long total = 0;
   for (int b = 0; b < bt.B; ++b) total += bt.img[b].N;
-  return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, g_sm_count, g_smem_optin - kTokReserve);
+  return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, cfg.sm_count, cfg.smem_optin - kTokReserve);
 }
-static int tokens_grid(const Batch &bt, int rpp) {
+static int tokens_grid(const Batch &bt, int rpp, const DeviceCfg &cfg) {
   long long units = 0;
   for (int b = 0; b < bt.B; ++b) units += (bt.img[b].N + rpp - 1) / rpp;
-  const int most = g_sm_count;
-  return units < most ? (int)units : most;
+  return units < cfg.sm_count ? (int)units : cfg.sm_count;
 }
 
 template <typename T>
-static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, cudaStream_t st, int *rpp) {
-  const TokCfg tc = tokens_config<T>(bt);
+static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
+  const TokCfg tc = tokens_config<T>(bt, cfg);
   if (rpp) *rpp = tc.rpp;
   const bool group = bt.n_qh / bt.n_kvh >= kGroupHeads;
   const auto kernel = tc.query ? (group ? k_tokens<T, true, true> : k_tokens<T, true, false>) : (group ? k_tokens<T, false, true> : k_tokens<T, false, false>);
-  return launch_k(kernel, dim3(tokens_grid(bt, tc.rpp)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
+  return launch_k(kernel, dim3(tokens_grid(bt, tc.rpp, cfg)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
 }
 
 template <typename T>
-static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp_out, const HostFeed *feed) {
+static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const DeviceCfg &cfg, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp_out,
+                                 const HostFeed *feed) {
   cudaError_t e = cudaSuccess;
   if (feed && (e = cudaStreamWaitEvent(st, feed->keys, 0)) != cudaSuccess) return e;
-  e = launch_qsum<T>(bt, st);
+  e = launch_qsum<T>(bt, cfg, st);
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
   int rpp = 0;
-  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, st, &rpp);
+  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
   if (e != cudaSuccess) return e;
   for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
     // (a part without visual tokens may still bring text rows, which k_merge copies)
@@ -1377,7 +1374,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
     part.img[0].N = feed->end[k] - first;
     part.img[0].vis_start += first;
     part.img[0].nrm += first;
-    if ((e = launch_tokens<T>(part, kTokNorms, false, st, nullptr)) != cudaSuccess) return e;
+    if ((e = launch_tokens<T>(part, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
   }
   if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;
@@ -1394,7 +1391,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
     size_t keys = (size_t)maxN * sizeof(uint32_t);
     const bool in_smem = keys <= kSelKeyBytes;
     if (!in_smem) keys = 0;
-    int X = g_sm_count / bt.B;
+    int X = cfg.sm_count / bt.B;
     const int want = (maxN + 15) / 16;         // at least sixteen tokens per CTA
     if (X > want) X = want;
     if (X < 1) X = 1;
@@ -1414,46 +1411,43 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
-  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, mark, mark_arg, rpp, nullptr)
-              : launch_euti_t<float>(bt, maxN, mode, st, mark, mark_arg, rpp, nullptr);
+cudaError_t launch_euti(const Batch &bt, int maxN, bool bf16, int mode, const DeviceCfg &cfg, cudaStream_t st, StageMark mark, void *mark_arg, int *rpp) {
+  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, cfg, st, mark, mark_arg, rpp, nullptr)
+              : launch_euti_t<float>(bt, maxN, mode, cfg, st, mark, mark_arg, rpp, nullptr);
 }
-cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, cudaStream_t st, const HostFeed &feed, int *rpp) {
-  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, st, nullptr, nullptr, rpp, &feed)
-              : launch_euti_t<float>(bt, maxN, mode, st, nullptr, nullptr, rpp, &feed);
+cudaError_t launch_euti_fed(const Batch &bt, int maxN, bool bf16, int mode, const DeviceCfg &cfg, cudaStream_t st, const HostFeed &feed, int *rpp) {
+  return bf16 ? launch_euti_t<__nv_bfloat16>(bt, maxN, mode, cfg, st, nullptr, nullptr, rpp, &feed)
+              : launch_euti_t<float>(bt, maxN, mode, cfg, st, nullptr, nullptr, rpp, &feed);
 }
 
 int euti_kernels(int mode) { return mode == 0 ? 4 : mode == 1 ? 3 : 2; }
 
-cudaError_t launch_split(const Batch &bt, int N, cudaStream_t st) {
+cudaError_t launch_split(const Batch &bt, int N, const DeviceCfg &cfg, cudaStream_t st) {
   if (N <= 6 * kSelThreads) return launch_k(k_split_regs<6>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
   if (N <= 16 * kSelThreads) return launch_k(k_split_regs<16>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
   if (N <= 32 * kSelThreads) return launch_k(k_split_regs<32>, dim3(1), dim3(kSelThreads), 0, st, true, bt);
   const size_t sm = (size_t)N * sizeof(uint32_t);
-  const bool in_smem = sm + kSplitReserve <= g_smem_optin;
+  const bool in_smem = sm + kSplitReserve <= cfg.smem_optin;
   return launch_k(k_split, dim3(1), dim3(1024), in_smem ? sm : 0, st, true, bt, in_smem ? 1 : 0);
 }
 
-cudaError_t select_configure() {
+cudaError_t select_configure(DeviceCfg *cfg) {
   int dev = 0, v = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  g_sm_count = v;
+  cfg->sm_count = v;
   e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  g_smem_optin = (size_t)v;
-  e = cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g_smem_optin - kSplitReserve));
-  if (e != cudaSuccess) return e;
-  return e;
+  cfg->smem_optin = (size_t)v;
+  return cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(cfg->smem_optin - kSplitReserve));
 }
 
-cudaError_t euti_configure(int n_qcols, int n_qh) {
-  cudaError_t e = select_configure();
-  if (e != cudaSuccess) return e;
-  if ((size_t)(n_qcols + 32 * n_qh) * 8 > g_smem_optin - 1024) return cudaErrorInvalidConfiguration;   // the widest query
-  const int tok = (int)(g_smem_optin - kTokReserve);
+cudaError_t euti_configure(const DeviceCfg &cfg, int n_qcols, int n_qh) {
+  cudaError_t e = cudaSuccess;
+  if ((size_t)(n_qcols + 32 * n_qh) * 8 > cfg.smem_optin - 1024) return cudaErrorInvalidConfiguration;   // the widest query
+  const int tok = (int)(cfg.smem_optin - kTokReserve);
   for (const auto f : {k_tokens<__nv_bfloat16, true, true>, k_tokens<__nv_bfloat16, true, false>, k_tokens<__nv_bfloat16, false, true>, k_tokens<__nv_bfloat16, false, false>,
                        k_tokens<float, true, true>, k_tokens<float, true, false>, k_tokens<float, false, true>, k_tokens<float, false, false>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tok)) != cudaSuccess) return e;

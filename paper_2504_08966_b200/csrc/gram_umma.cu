@@ -799,14 +799,13 @@ namespace {
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
 
-bool encode_rows(CUtensorMap *map, const void *base, long long rows, long long ld_elems, int d_k) {
+bool encode_rows(const DeviceCfg &cfg, CUtensorMap *map, const void *base, long long rows, long long ld_elems, int d_k) {
   const cuuint64_t dims[2] = {(cuuint64_t)d_k, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld_elems * 2};
   const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)BM};
   const cuuint32_t estr[2] = {1, 1};
-  return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+  return reinterpret_cast<EncodeTiledFn>(cfg.encode_tiled)(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -815,15 +814,11 @@ constexpr int kGramBN = 128, kWideBN = 256;
 
 }  // namespace
 
-bool umma_supported(int d_k) { return g_encode != nullptr && d_k % BK == 0; }
+bool umma_supported(int d_k) { return d_k % BK == 0; }
 
 namespace {
-bool g_pair_ok = false;                               // clusters of two CTAs of the pair kernel can be launched
-bool g_pair_gram_ok = false;                          // ... of its all-pairs form with 16 epilogue warps
-bool g_pair_assign_ok = false;                        // ... of its rows x centres form
-
 template <int MODE, int EW>
-cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, int kept_rows, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, int kept_rows, const DeviceCfg &cfg, cudaStream_t st) {
   using PC = PairCfg<MODE, EW>;
   long long P = cfg.sm_count / 2;                     // one pair per two SMs
   if (P > tiles * bt.B) P = tiles * bt.B;
@@ -858,13 +853,13 @@ template <int MODE, int EW> cudaError_t pair_configure(bool &ok) {
 }
 }  // namespace
 
-cudaError_t umma_configure() {
+cudaError_t umma_configure(DeviceCfg *cfg) {
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
   cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
   if (e != cudaSuccess) return e;
   if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-  g_encode = reinterpret_cast<EncodeTiledFn>(fn);
+  cfg->encode_tiled = fn;
   e = cudaFuncSetAttribute(k_tiles_umma<MODE_GRAM, kGramBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)TileCfg<kGramBN>::SMEM);
   if (e != cudaSuccess) return e;
@@ -874,11 +869,11 @@ cudaError_t umma_configure() {
   e = cudaFuncSetAttribute(k_tiles_umma<MODE_ASSIGN, kWideBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)TileCfg<kWideBN>::SMEM);
   if (e != cudaSuccess) return e;
-  e = pair_configure<MODE_ASSIGN, 8>(g_pair_assign_ok);
+  e = pair_configure<MODE_ASSIGN, 8>(cfg->pair_assign);
   if (e != cudaSuccess) return e;
-  e = pair_configure<MODE_GRAM, 16>(g_pair_gram_ok);
+  e = pair_configure<MODE_GRAM, 16>(cfg->pair_gram);
   if (e != cudaSuccess) return e;
-  return pair_configure<MODE_SPREAD, 8>(g_pair_ok);
+  return pair_configure<MODE_SPREAD, 8>(cfg->pair_spread);
 }
 
 static int umma_grid_x(long long tiles, int B, int sms) {
@@ -888,11 +883,11 @@ static int umma_grid_x(long long tiles, int B, int sms) {
   return (int)(x < 1 ? 1 : x);
 }
 
-cudaError_t launch_gram_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, cudaStream_t st, int est_rows) {
+cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cudaStream_t st, int est_rows) {
   TmapSet tm;
   for (int b = 0; b < bt.B; ++b) {
     const ImgDesc &im = bt.img[b];
-    if (!encode_rows(&tm.a[b], im.Kp, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
+    if (!encode_rows(cfg, &tm.a[b], im.Kp, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
     tm.b[b] = tm.a[b];
   }
   // With many blocks per SM (batches, long images) pairs of CTAs on 256 x 256 tiles with 16 epilogue warps each are
@@ -900,7 +895,7 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, c
   // 7290-token image) the coarser tiles cost a round, and single CTAs on 128 x 128 blocks are.
   if (est_rows < 1 || est_rows > maxN) est_rows = maxN;
   const long long nq = (est_rows + BM - 1) / BM;
-  if (g_pair_gram_ok && nq * (nq + 1) / 2 * bt.B >= 6LL * cfg.sm_count) {
+  if (cfg.pair_gram && nq * (nq + 1) / 2 * bt.B >= 6LL * cfg.sm_count) {
     const long long n2 = (maxN + 2 * BM - 1) / (2 * BM);
     return launch_pair<MODE_GRAM, 16>(bt, tm, n2 * (n2 + 1) / 2, 0, cfg, st);
   }
@@ -909,25 +904,25 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, c
   return launch_k(k_tiles_umma<MODE_GRAM, kGramBN>, grid, dim3(THREADS), TileCfg<kGramBN>::SMEM, st, true, bt, tm, 0);
 }
 
-bool umma_pairs_for_assign(int maxN, int B, const ClusterCfg &cfg) {
+bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
   // with two or more 128-row blocks per SM (batches, long images) pairs of CTAs on 256 x 256 tiles are faster:
   // the pass is bound by operand bytes from the L2, and a pair fetches two thirds of them
-  return g_pair_assign_ok && (long long)((maxN + BM - 1) / BM) * B >= 2LL * cfg.sm_count;
+  return cfg.pair_assign && (long long)((maxN + BM - 1) / BM) * B >= 2LL * cfg.sm_count;
 }
 
 // labels: the single-CTA kernel also forms labels and member counts (all-token rows only); pairs: the pair kernel
 // (all-token rows, no labels)
-cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const ClusterCfg &cfg, cudaStream_t st, bool labels,
+cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const DeviceCfg &cfg, cudaStream_t st, bool labels,
                                bool pairs) {
   TmapSet tm;
   for (int b = 0; b < bt.B; ++b) {
     const ImgDesc &im = bt.img[b];
     if (kept_rows) {
-      if (!encode_rows(&tm.a[b], im.Kp, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
-    } else if (!encode_rows(&tm.a[b], im.Kc, im.N, im.ldKc, bt.d_k)) return cudaErrorInvalidValue;
-    if (!encode_rows(&tm.b[b], im.Kcen, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
+      if (!encode_rows(cfg, &tm.a[b], im.Kp, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
+    } else if (!encode_rows(cfg, &tm.a[b], im.Kc, im.N, im.ldKc, bt.d_k)) return cudaErrorInvalidValue;
+    if (!encode_rows(cfg, &tm.b[b], im.Kcen, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
   }
-  if (pairs && !kept_rows && g_pair_assign_ok) {
+  if (pairs && !kept_rows && cfg.pair_assign) {
     const long long pt = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
     return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, 0, cfg, st);
   }
@@ -937,14 +932,14 @@ cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const 
 }
 
 // every layer of the batch is one "image": rows and columns are all N keys of K_clu
-cudaError_t launch_spread_umma(const Batch &bt, int maxN, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_spread_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cudaStream_t st) {
   TmapSet tm;
   for (int b = 0; b < bt.B; ++b) {
     const ImgDesc &im = bt.img[b];
-    if (!encode_rows(&tm.a[b], im.Kc, im.N, im.ldKc, bt.d_k)) return cudaErrorInvalidValue;
+    if (!encode_rows(cfg, &tm.a[b], im.Kc, im.N, im.ldKc, bt.d_k)) return cudaErrorInvalidValue;
     tm.b[b] = tm.a[b];
   }
-  if (g_pair_ok) {
+  if (cfg.pair_spread) {
     const long long ptiles = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
     return launch_pair<MODE_SPREAD, 8>(bt, tm, ptiles, 0, cfg, st);
   }

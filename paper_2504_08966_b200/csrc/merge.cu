@@ -583,14 +583,10 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
 
 // ---- launchers -----------------------------------------------------------------------------------
 
-namespace {
-int g_lists_resident = 0;                            // CTAs of k_lists that fit on the device at once
-}
-
 template <typename T, bool FB>
-static cudaError_t launch_lists_t(const Batch &bt, int maxN, int spin_limit, cudaStream_t st) {
+static cudaError_t launch_lists_t(const Batch &bt, int maxN, int spin_limit, const DeviceCfg &cfg, cudaStream_t st) {
   const dim3 grid((maxN + kListBlock - 1) / kListBlock, bt.B);
-  if ((long long)grid.x * grid.y <= g_lists_resident) {
+  if ((long long)grid.x * grid.y <= cfg.lists_resident) {
     return launch_coop(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 0, spin_limit);
   }
   cudaError_t e = launch_k(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 1, spin_limit);
@@ -598,12 +594,12 @@ static cudaError_t launch_lists_t(const Batch &bt, int maxN, int spin_limit, cud
   return launch_k(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 2, spin_limit);
 }
 
-cudaError_t launch_lists(const Batch &bt, int maxN, bool bf16, bool from_best, int spin_limit, cudaStream_t st) {
+cudaError_t launch_lists(const Batch &bt, int maxN, bool bf16, bool from_best, int spin_limit, const DeviceCfg &cfg, cudaStream_t st) {
   if (from_best) {
-    if (bf16) return launch_lists_t<__nv_bfloat16, true>(bt, maxN, spin_limit, st);
-    return launch_lists_t<float, true>(bt, maxN, spin_limit, st);
+    if (bf16) return launch_lists_t<__nv_bfloat16, true>(bt, maxN, spin_limit, cfg, st);
+    return launch_lists_t<float, true>(bt, maxN, spin_limit, cfg, st);
   }
-  return launch_lists_t<float, false>(bt, maxN, spin_limit, st);
+  return launch_lists_t<float, false>(bt, maxN, spin_limit, cfg, st);
 }
 
 cudaError_t launch_members(const Batch &bt, int maxN, cudaStream_t st) {
@@ -611,8 +607,8 @@ cudaError_t launch_members(const Batch &bt, int maxN, cudaStream_t st) {
   return launch_k(k_members, grid, dim3(kListBlock), 0, st, true, bt);
 }
 
-int lists_kernels(int maxN, int B) {
-  return (long long)((maxN + kListBlock - 1) / kListBlock) * B <= g_lists_resident ? 1 : 2;
+int lists_kernels(int maxN, int B, const DeviceCfg &cfg) {
+  return (long long)((maxN + kListBlock - 1) / kListBlock) * B <= cfg.lists_resident ? 1 : 2;
 }
 
 // items per range: 24 (with 16: 2.5 us more of 16 images of 2916 tokens, 2 us of three of 2309; with 48 as much), 16 where
@@ -630,7 +626,7 @@ static int merge_per(int n_items, int slices, int B, int sm_count) {
 size_t merge_scratch_rows() { return 2 * kMrgRanges; }
 
 template <typename T, typename O, int VPL>
-static cudaError_t launch_merge_v(const Batch &bt, int n_items, int slices, const ClusterCfg &cfg, cudaStream_t st) {
+static cudaError_t launch_merge_v(const Batch &bt, int n_items, int slices, const DeviceCfg &cfg, cudaStream_t st) {
   const int per = merge_per(n_items, slices, bt.B, cfg.sm_count), ranges = (n_items + per - 1) / per;
   const long long per_sm = ((long long)ranges * slices * bt.B + cfg.sm_count - 1) / cfg.sm_count;
   int ring = per_sm >= kMrgCtasPerSm ? kMrgRingBytes : (int)(kMrgCtasPerSm * kMrgRingBytes / per_sm);
@@ -643,7 +639,7 @@ static cudaError_t launch_merge_v(const Batch &bt, int n_items, int slices, cons
 }
 
 template <typename T, typename O>
-static cudaError_t launch_merge_t(const Batch &bt, const ClusterCfg &cfg, cudaStream_t st) {
+static cudaError_t launch_merge_t(const Batch &bt, const DeviceCfg &cfg, cudaStream_t st) {
   int n_items = 1;
   for (int b = 0; b < bt.B; ++b) n_items = bt.img[b].n_total > n_items ? bt.img[b].n_total : n_items;
   const int s1 = (bt.d / 8 + kMrgThreads - 1) / kMrgThreads, s2 = (bt.d / 8 + 2 * kMrgThreads - 1) / (2 * kMrgThreads);
@@ -662,13 +658,9 @@ template <typename T, typename O> static cudaError_t merge_attr() {
   return e;
 }
 
-cudaError_t merge_configure() {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<__nv_bfloat16, true>, kListBlock, 0);
+cudaError_t merge_configure(DeviceCfg *cfg) {
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<__nv_bfloat16, true>, kListBlock, 0);
   if (e != cudaSuccess) return e;
   int m = per_sm;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<float, true>, kListBlock, 0);
@@ -677,7 +669,7 @@ cudaError_t merge_configure() {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<float, false>, kListBlock, 0);
   if (e != cudaSuccess) return e;
   m = per_sm < m ? per_sm : m;
-  g_lists_resident = m * sms;
+  cfg->lists_resident = m * cfg->sm_count;
   e = merge_attr<__nv_bfloat16, __nv_bfloat16>();
   if (e == cudaSuccess) e = merge_attr<__nv_bfloat16, float>();
   if (e == cudaSuccess) e = merge_attr<float, __nv_bfloat16>();
@@ -691,7 +683,7 @@ cudaError_t launch_list_clear(const Batch &bt, cudaStream_t st) {
   return launch_k(k_list_clear, dim3((unsigned)(X < 1 ? 1 : (X > 1184 ? 1184 : X)), bt.B), dim3(256), 0, st, true, bt);
 }
 
-cudaError_t launch_merge(const Batch &bt, bool in_bf16, bool out_bf16, const ClusterCfg &cfg, cudaStream_t st) {
+cudaError_t launch_merge(const Batch &bt, bool in_bf16, bool out_bf16, const DeviceCfg &cfg, cudaStream_t st) {
   if (in_bf16) return out_bf16 ? launch_merge_t<__nv_bfloat16, __nv_bfloat16>(bt, cfg, st)
                                : launch_merge_t<__nv_bfloat16, float>(bt, cfg, st);
   return out_bf16 ? launch_merge_t<float, __nv_bfloat16>(bt, cfg, st) : launch_merge_t<float, float>(bt, cfg, st);

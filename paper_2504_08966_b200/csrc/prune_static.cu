@@ -18,7 +18,8 @@ extern "C" pact_status pact_prune_static(const float *score, int N, const pact_p
   if (!score || !keep || !kept_idx || !pruned_idx || !counts || !p || N < 1) return PACT_ERR_INVALID_ARG;
   if (N > PACT_PRUNE_STATIC_MAX_N) return PACT_ERR_UNSUPPORTED;
   if (!(p->lambda >= 0.0 && p->lambda <= 1.0)) return PACT_ERR_INVALID_ARG;
-  if (select_configure() != cudaSuccess) return PACT_ERR_CUDA;   // (of the current device; no context has done it)
+  DeviceCfg cfg;
+  if (select_configure(&cfg) != cudaSuccess) return PACT_ERR_CUDA;   // (of the current device; no context has done it)
   cudaStream_t st = (cudaStream_t)stream;
   Batch bt;
   memset(&bt, 0, sizeof(bt));
@@ -34,5 +35,5 @@ extern "C" pact_status pact_prune_static(const float *score, int N, const pact_p
   m.kept_idx = kept_idx;
   m.pruned_idx = pruned_idx;
   m.counts_user = counts;
-  return launch_split(bt, N, st) == cudaSuccess ? PACT_OK : PACT_ERR_CUDA;
+  return launch_split(bt, N, cfg, st) == cudaSuccess ? PACT_OK : PACT_ERR_CUDA;
 }

@@ -701,8 +701,6 @@ static_assert(4 * sizeof(F64Group) <= kSmDynF64 - 1024, "double-precision tiles"
 static_assert((size_t)kSmallMaxN * (kSmMaxW / 4 + 1) * 16 + kSmallMaxN * 8 <= kSmDynF64 - 1024, "adjacency of the survivors");
 static_assert(kSmMaxHeads * (kSmallMaxN / kMinPiece) * 8 <= kSmDynF64 - 1024 && kSmMaxW * kSmallMaxN <= kSmDynF64 - 1024, "softmax pieces, member table");
 
-int g_small_clusters = 0;                              // clusters that fit on the device at once
-
 template <typename T, bool UMMA> cudaError_t small_attr() {
   constexpr int dyn = (int)(UMMA ? kSmDynUmma : kSmDynF64);
   cudaError_t e = cudaFuncSetAttribute(k_small<T, UMMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
@@ -719,7 +717,7 @@ cudaError_t launch_small_t(const Batch &bt, int rpp, int sweep_limit, cudaStream
 
 }  // namespace
 
-cudaError_t small_configure() {
+cudaError_t small_configure(DeviceCfg *cfg) {
   cudaError_t e = small_attr<__nv_bfloat16, true>();
   if (e == cudaSuccess) e = small_attr<__nv_bfloat16, false>();
   if (e == cudaSuccess) e = small_attr<float, false>();
@@ -739,7 +737,7 @@ cudaError_t small_configure() {
     (void)cudaGetLastError();
     n = 0;
   }
-  g_small_clusters = n;
+  cfg->small_clusters = n;
   return cudaSuccess;
 }
 
@@ -756,8 +754,8 @@ cudaError_t small_configure() {
 // With more images the idle share is smaller (d_k 512, two and four images of 512 half-pruned tokens: 70 against 76, 73
 // against 102).  Of 340 calls of one to four images measured, d_k 64 to 2048 and pruning 0 to 0.8, the rule takes 0.4 % more
 // than the better form of each would, the sizes alone took 9 %.
-bool small_fits(const Batch &bt, int maxN, bool umma, const ClusterCfg &cfg) {
-  if (maxN > (umma ? kSmallMaxN : kSmallMaxF64) || bt.n_qh > kSmMaxHeads || bt.B > g_small_clusters) return false;
+bool small_fits(const Batch &bt, int maxN, bool umma, const DeviceCfg &cfg) {
+  if (maxN > (umma ? kSmallMaxN : kSmallMaxF64) || bt.n_qh > kSmMaxHeads || bt.B > cfg.small_clusters) return false;
   const double idle = 1.0 - (double)(CL * bt.B) / cfg.sm_count;
   for (int b = 0; b < bt.B; ++b) {
     const int N = bt.img[b].N, q = N - bt.img[b].m_target;

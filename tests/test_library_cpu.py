@@ -88,6 +88,14 @@ def test_current_stream_without_the_private_functions(monkeypatch):
     assert binding._stream_getter()() == 1234
 
 
+def test_no_state_outside_the_contexts(lib):
+    """Contexts are created and used by several threads: what one learns about its device is written where no other reads it."""
+    from paper_2504_08966_b200 import binding
+    out = subprocess.check_output(["nm", "-C", binding.LIB_PATH], text=True)
+    own = [ln.split(None, 2)[2] for ln in out.splitlines() if re.search(r" [bBdDC] ", ln) and ("pact" in ln or re.search(r" g_\w+$", ln))]
+    assert own == []
+
+
 def test_product_does_not_import_the_oracle():
     pkg = os.path.join(ROOT, "paper_2504_08966_b200")
     for dirpath, _, files in os.walk(pkg):
