@@ -130,7 +130,7 @@ def test_pairs_of_ctas_with_ragged_ends():
 
 @pytest.mark.parametrize("N", [3072, 3073, 8192, 8193])
 def test_select_key_registers(N):
-    """The last size with the keys of the split in six, in sixteen registers per thread, and the first without."""
+    """The last sizes with the keys of the split in six and in sixteen registers per thread, and the ones after them."""
     _check(_workload(N, 2, 1, 16, 32, torch.bfloat16, N), torch.float32)
 
 
@@ -225,20 +225,21 @@ def test_host_buffers(N, T, vis, d, rope, pinned):
     ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
     z = lambda m, dt: torch.full(m, 7, dtype=dt).pin_memory() if pinned else torch.full(m, 7, dtype=dt)   # noqa: E731
     n = N + T
-    host = dict(H=img.H.pin_memory(), K_euti=img.K.pin_memory(), Q_euti=img.Q.pin_memory(), P=img.P.pin_memory(), vis_start=vis, N=N,
-                H_out=z((n, d), torch.float32), P_out=z((n,), torch.int32), size_out=z((n,), torch.int32), logw_out=z((n,), torch.float32),
-                label=z((N,), torch.int32), counters=z((16,), torch.int32))
+    host = dict(H=img.H.pin_memory(), K_euti=img.K.pin_memory(), Q_euti=img.Q.pin_memory(), P=img.P.pin_memory(), vis_start=vis, N=N)
+    results = dict(H_out=z((n, d), torch.float32), P_out=z((n,), torch.int32), size_out=z((n,), torch.int32), logw_out=z((n,), torch.float32),
+                   label=z((N,), torch.int32), counters=z((16,), torch.int32))
+    host.update(results)
     host["K_clu"] = img.K_clu.pin_memory() if rope else host["K_euti"]
     staging = torch.empty(ctx.host_staging_bytes(n, N), dtype=torch.uint8, device="cuda")
-    for _ in range(2):
-        ctx.pact_reduce_host(host, pb.make_params(lam=wl.lam, d_c=wl.d_c), staging)
     want = gpu_reduce(wl, torch.float32)[0][0]
-    n_out = int(host["counters"][0])
-    assert n_out == want["n_out"] and np.array_equal(host["label"].numpy(), want["label"])
-    for key in ("P_out", "size_out", "logw_out"):
-        assert np.array_equal(host[key][:n_out].numpy(), want[key])
-    assert torch.equal(host["H_out"][:n_out], want["H_out_raw"])
-    assert bool((host["H_out"][n_out:] == 7).all()) and bool((host["P_out"][n_out:] == 7).all())
+    for _ in range(3):                        # (large hidden states come in parts from the second call on)
+        for t in results.values():
+            t.fill_(7)
+        staging.fill_(255)                    # nothing of the call before is left to be found
+        ctx.pact_reduce_host(host, pb.make_params(lam=wl.lam, d_c=wl.d_c), staging)
+        _same_as_device(host, want)
+        n_out = want["n_out"]
+        assert bool((host["H_out"][n_out:] == 7).all()) and bool((host["P_out"][n_out:] == 7).all())
 
 
 def _host_call(wl, ctx, params=None):
