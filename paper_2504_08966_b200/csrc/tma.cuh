@@ -94,10 +94,11 @@ __device__ __forceinline__ bool mbar_wait_warp_or_report(uint64_t *bar, uint32_t
 }
 
 // The same for a warp with more waits to come in a CTA that may have given up: once *abort is set nothing is asked for any more,
-// and it does not wait a second for each of them.  (One lane looks: the answer has to be the warp's.)
+// and it does not wait a second for each of them.  (One lane looks: the answer has to be the warp's.  It looks when the first
+// attempt has failed: 0.4 us of k_merge's 75 for 16 images of 2916 tokens, 0.5 with the look first.)
 __device__ __forceinline__ bool mbar_wait_warp_unless(const int *abort, uint64_t *bar, uint32_t parity) {
   int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = !*const_cast<const volatile int *>(abort) && mbar_wait(bar, parity) ? 1 : 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_try_wait(bar, parity) || (!*const_cast<const volatile int *>(abort) && mbar_wait(bar, parity)) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
