@@ -170,7 +170,8 @@ const char *pact_profile_stage_name(int i);
 
 /* EUTI score, Eq. 1-2 / Algorithm 1 steps 1-2.
  * Reads img->H (visual rows), K_euti, Q_euti; writes score[N] (fp32).  An infinity or a NaN anywhere in
- * Q_euti or K_euti makes every score NaN (also in pact_reduce, where equal scores all survive). */
+ * Q_euti or K_euti makes every score NaN (also in pact_reduce, where equal scores all survive); with PACT_FLAG_NORM_ONLY
+ * neither is read. */
 pact_status pact_importance(pact_ctx *ctx, const pact_image *img /*host*/, const pact_params *p /*host*/,
                             float *score, void *ws, size_t ws_bytes, void *stream);
 
@@ -270,6 +271,8 @@ pact_status pact_graph_destroy(pact_graph *graph);
 /* Same computation with HOST buffers for one image: copies the inputs to the device, runs
  * pact_reduce, brings H_out/P_out/size_out/logw_out/label/counters back (results in mapped host memory are
  * written there by the kernels) and synchronises.
+ * From the second call of a context with hidden states of 12 MB or more on, they arrive while the queries are scored, on a
+ * stream of the context's own: that call creates it (about 65 us, once) and pact_destroy gives it back.
  * dev_staging is a device buffer the caller provides (size from
  * pact_host_staging_bytes); every pointer inside `img` is a host pointer here. */
 pact_status pact_reduce_host(pact_ctx *ctx, const pact_image *img /*host, host pointers*/,

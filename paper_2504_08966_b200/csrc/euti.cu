@@ -8,9 +8,9 @@
 //                    softmax pieces of up to 32 tokens (HBM-bound, the first of two reads of H); also clears what later
 //                    kernels accumulate into
 //   k_scores         merges the pieces, writes the float32 scores and the histogram of their top key bits
-//   k_select         every CTA selects the threshold (histogram bin, then radix passes inside the bin) and
-//                    counts the survivors before its tokens, then writes its share of the lists and gathers
-//                    its share of the survivor keys
+//   k_select         every CTA selects the threshold (histogram bin, then one pass inside it that mostly leaves the key
+//                    itself, else a few that are ranked; radix passes for many equal scores) and counts the survivors
+//                    before its tokens, then writes its share of the lists and gathers its share of the survivor keys
 //   k_split_regs, k_split   the split for the stage call pact_prune (scores given, no histogram): radix select
 //
 // The kernels are short chains of dependent memory round trips; each issues all the loads it can
@@ -884,7 +884,8 @@ __device__ __noinline__ void radix_threshold(const float *score, const uint32_t 
 // (eight clocks), ranking all keys of the bin by counting 3 us, and a pass through the code before the wait, for the
 // instruction cache, cost what it gave.  The rows of the own tokens wait in shared memory when it is known which survive; scores,
 // histogram and norms come in one trip.  From the end of k_scores: one image of 7290 8.0 us -> 6.7, four of 16384 (16 keys per
-// thread from shared memory, three passes over them) 22 -> 15.
+// thread from shared memory, three passes over them) 22 -> 15.  Above 16384 tokens, with one CTA per SM where there were two (events
+// around the kernel): 24577 29 us -> 18, 65536 60 -> 41, 131072 107 -> 72; the own tokens then go in rounds of 512.
 template <typename T, int KPT, bool IN_SMEM>
 __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant__ Batch bt, int pre) {
   using D = typename DistOf<T>::type;

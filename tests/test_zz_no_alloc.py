@@ -111,6 +111,35 @@ def test_static_scratch_split_as_the_first_call_of_a_fresh_process():
     assert r.returncode == 0 and "fresh ok" in r.stdout, r.stdout + r.stderr
 
 
+_FRESH_CAPTURE = r"""
+import sys
+import numpy as np, torch
+sys.path.insert(0, sys.argv[1])
+from paper_2504_08966_b200 import binding as pb
+from oracle import pact_oracle as orc
+N, lam = int(sys.argv[2]), 0.61
+score = torch.rand(N, generator=torch.Generator().manual_seed(7)).cuda()
+out = [torch.full((N,), 7, dtype=torch.uint8, device="cuda")] + [torch.full((n,), -5, dtype=torch.int32, device="cuda") for n in (N, N, 2)]
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):                      # nothing of the library has run before
+    pb.pact_prune_static(score, pb.make_params(lam=lam), *out)
+graph.replay()
+torch.cuda.synchronize()
+q, m = out[3].cpu().tolist()
+_, keep, kept, pruned = orc.split(score.cpu().numpy(), lam)
+assert [q, m] == [kept.size, pruned.size] and np.array_equal(out[0].cpu().numpy().astype(bool), keep)
+assert np.array_equal(out[1][:q].cpu().numpy(), kept) and np.array_equal(out[2][:m].cpu().numpy(), pruned)
+print("fresh ok")
+"""
+
+
+@pytest.mark.parametrize("N", [700, 40000])
+def test_the_first_call_of_a_process_may_be_captured(N):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FRESH_CAPTURE, root, str(N)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "fresh ok" in r.stdout, r.stdout + r.stderr
+
+
 def test_splits_on_two_streams_at_once_and_in_a_graph():
     """Calls without an order between them share nothing, and a call may be captured."""
     from paper_2504_08966_b200 import binding as pb
