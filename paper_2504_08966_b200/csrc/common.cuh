@@ -9,7 +9,6 @@
 
 namespace pact {
 
-constexpr int kMaxBatchPerLaunch = 16;   // images described by one kernel parameter block
 constexpr uint32_t kRhoShift = 30;       // density terms are summed as integers scaled by 2^30
 constexpr unsigned long long kBestInit = 0xFFFFFFFFFFFFFFFFull;
 constexpr int kCntSpread = 24;           // slot of cnt[]: largest key distance of a layer, as float bits

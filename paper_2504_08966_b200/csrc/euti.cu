@@ -78,21 +78,18 @@ template <typename T, int CH> struct NonFinite {
     return s;
   }
 };
-// Sum of the 32 parts of each of the rows w, w + step, ... < n: eight lanes per row, four rows at a time.
+// Sum of the 32 parts of each of n <= 4 rows of this warp: eight lanes per row.
 template <typename F>
-__device__ __forceinline__ void finish_row_sums(const double (*acc)[32], int w, int step, int n, F put_sum) {
-  const int lane = threadIdx.x & 31;
-  for (int i = 0; w + i * step < n; i += 4) {
-    const int r = w + (i + lane / 8) * step;
-    double s = 0.0;
-    if (r < n) {
+__device__ __forceinline__ void finish_row_sums(const double (*acc)[32], int n, F put_sum) {
+  const int lane = threadIdx.x & 31, j = lane >> 3;
+  double s = 0.0;
+  if (j < n) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s += acc[r][(lane & 7) * 4 + k];
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (r < n && (lane & 7) == 0) put_sum(r, s);
+    for (int k = 0; k < 4; ++k) s += acc[j][(lane & 7) * 4 + k];
   }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (j < n && (lane & 7) == 0) put_sum(j, s);
   __syncwarp();
 }
 
@@ -109,7 +106,7 @@ constexpr int kQsumThreads = 256;
 constexpr int kQsumWarps = kQsumThreads / 32;
 
 template <typename T, int GV>
-__global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant__ Batch bt, int RP) {
+__global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant__ Batch bt, int RP, uint64_t policy) {
   constexpr int V = Vec<T>::N, LANES = kQsumThreads / GV;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 0);
@@ -136,7 +133,7 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
       uint4 buf[UQ];
 #pragma unroll
       for (int u = 0; u < UQ; ++u)
-        if (r + u * LANES < r1) buf[u] = __ldg(reinterpret_cast<const uint4 *>(Q + (size_t)(r + u * LANES) * im.ldQ));
+        if (r + u * LANES < r1) buf[u] = ld_hint(Q + (size_t)(r + u * LANES) * im.ldQ, policy);
 #pragma unroll
       for (int u = 0; u < UQ; ++u) {
         if (r + u * LANES < r1) {
@@ -183,12 +180,14 @@ __global__ void __launch_bounds__(kQsumThreads, 4) k_qsum(const __grid_constant_
 
 // ---- Eq. 2, token pass: hidden-state norm, inverse key norm, logits, softmax pieces --------------------------------
 // Persistent: one CTA of 512 threads and at most 64 registers per SM (beside it a CTA of k_qsum still fits), units of
-// at most 32 tokens dealt out in turn over all images of the call.  Two groups of warps work side by side:
-//   norms    Every warp takes each eighth token of a unit.  The hidden-state rows run through two buffers of the warp's
+// at most 32 tokens shared out over all images of the call (cut on the host: divisions from a cold instruction cache, before
+// the first row was asked for, took 0.4 us).  Two groups of warps work side by side:
+//   norms    Every warp takes each eighth token of the CTA's units (of each unit by itself, units of 25 tokens cost a round of
+//            rows: one image of 7290 0.7 us).  The hidden-state rows run through two buffers of the warp's
 //            own in shared memory, one bulk copy per row (or per 8 KB of it), so that copies never wait for arithmetic.
 //            Sums of squares in float over a 16-byte vector and in double across.  Nothing here needs the global query.
 //   logits   Two teams of four warps take the units in turn; a team's scoring keys come through a buffer of its own, in
-//            flight before the global query is known: inverse key norms; k_i . Qglobal per head in double; per head the
+//            flight before the global query is known: inverse key norms (of the first unit of either team before the wait for it); k_i . Qglobal per head in double; per head the
 //            largest logit of the unit, exp(l - that) per token and their sum.  Up to two
 //            query heads per key head a lane is a token (with few tokens a part of its elements), and the global query
 //            comes from shared memory at one address per warp: with the lanes spread over the row the loads of the
@@ -402,7 +401,7 @@ __device__ __forceinline__ void group_piece(const Batch &bt, const ImgDesc &im, 
 // QUERY: the global query in shared memory; GROUP: heads through group_piece (a kernel of its own: in one, either path has
 // fewer registers).
 template <typename T, bool QUERY, bool GROUP>
-__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, int what) {
+__global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant__ Batch bt, const TokCfg cfg, const __grid_constant__ TokUnits un, uint64_t row_policy, int what) {
   using D = typename DistOf<T>::type;
   using rn_t = typename D::rn_t;
   constexpr int V = Vec<T>::N;
@@ -414,33 +413,28 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
   const int ks = tok_key_stride(bt.d_k * (int)sizeof(T));
   uint8_t *s_key = smem + (size_t)kTokWarps * cfg.nbuf * cfg.chunk;   // [2][rpp][ks], behind the row buffers
   double *s_q = reinterpret_cast<double *>(s_key + (size_t)2 * cfg.keys * rpp * ks);     // [n_qh][d_h] global query
-  double(*s_acc)[32] = reinterpret_cast<double(*)[32]>(s_q + (QUERY ? bt.n_qcols : 0));  // [rpp][32] parts of the sums of squares
-  __shared__ int s_first[kMaxBatchPerLaunch + 1];                     // first unit of each image
+  double(*s_acc)[32] = reinterpret_cast<double(*)[32]>(s_q + (QUERY ? bt.n_qcols : 0));  // [kTokWarps tok_warp_rows(rpp)][32] parts of the sums of squares
   __shared__ uint64_t s_rbar[kTokWarps][kTokMaxBuf], s_kbar[2];
   __shared__ int s_abort, s_query;                                    // s_query: the global queries are complete
-  if (threadIdx.x == 0) {
-    s_query = 0;
-    int first = 0;
-    for (int b = 0; b < bt.B; ++b) { s_first[b] = first; first += (bt.img[b].N + rpp - 1) / rpp; }
-    s_first[bt.B] = first;
-    for (int k = 0; k < kTokWarps; ++k)
-      for (int i = 0; i < kTokMaxBuf; ++i) mbar_init(&s_rbar[k][i], 1);
-    mbar_init(&s_kbar[0], 1);
-    mbar_init(&s_kbar[1], 1);
-    s_abort = 0;
+  if (lane == 0) {
+    const int w = threadIdx.x >> 5;
+    if (w < kTokWarps) {
+      for (int i = 0; i < kTokMaxBuf; ++i) mbar_init(&s_rbar[w][i], 1);
+    } else if (w < kTokWarps + 2) mbar_init(&s_kbar[w - kTokWarps], 1);
+    else if (w == kTokWarps + 2) { s_query = 0; s_abort = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const int units = s_first[bt.B];
   // units of this CTA: neighbours, so that it meets few images (each brings another query)
-  const int u0 = (int)((long long)blockIdx.x * units / gridDim.x), u1 = (int)((long long)(blockIdx.x + 1) * units / gridDim.x);
-  auto image_of = [&](int u, int b) { while (u >= s_first[b + 1]) ++b; return b; };
+  const int cta = blockIdx.x, u0 = cta * un.per + min(cta, un.extra), u1 = u0 + un.per + (cta < un.extra);
+  auto image_of = [&](int u, int b) { while (u >= un.first[b + 1]) ++b; return b; };
 
   if (norms) {
     const int w = threadIdx.x >> 5, t = threadIdx.x;
     uint8_t *s_rows = smem + (size_t)w * cfg.nbuf * cfg.chunk;        // this warp's row buffers
+    double(*s_part)[32] = s_acc + tok_warp_rows(rpp) * w;   // parts of the sums of squares of its rows of a unit
     // the stream of this warp's row chunks, ahead of their use: unit, next row, rows left of the unit, chunk of the row
-    int lu = u0 - 1, lb = 0, lrows = 0, lc = 0, islot = 0;
+    int lu = u0 - 1, lb = 0, lrows = 0, lc = 0, islot = 0, ldealt = 0;
     const uint8_t *lsrc = nullptr;
     size_t lstep = 0;
     const int last = bt.d * (int)sizeof(T) - (cfg.nchunk - 1) * cfg.chunk;   // bytes of a row's last chunk
@@ -449,15 +443,18 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
         if (++lu >= u1) { lu = u1; return; }
         lb = image_of(lu, lb);
         const ImgDesc &im = bt.img[lb];
-        const int r0 = (lu - s_first[lb]) * rpp, n = min(rpp, im.N - r0);
-        if ((im.flags & PACT_FLAG_NO_NORM) || !(what & kTokNorms) || n <= w) continue;
-        lrows = (n - w + kTokWarps - 1) / kTokWarps;
-        lsrc = reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + r0 + w) * im.ldH);
+        const int r0 = (lu - un.first[lb]) * rpp, n = min(rpp, im.N - r0);
+        if (im.flags & PACT_FLAG_NO_NORM) continue;
+        const int first = (w - ldealt) & (kTokWarps - 1);   // this warp's first row of the unit
+        ldealt += n;
+        if (n <= first) continue;
+        lrows = (n - first + kTokWarps - 1) / kTokWarps;
+        lsrc = reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.H) + (size_t)(im.vis_start + r0 + first) * im.ldH);
         lstep = (size_t)im.ldH * kTokWarps * sizeof(T);
       }
       const int bytes = lc == cfg.nchunk - 1 ? last : cfg.chunk;
       mbar_arrive_expect_tx(&s_rbar[w][islot], bytes);
-      bulk_load(s_rows + (size_t)islot * cfg.chunk, lsrc + (size_t)lc * cfg.chunk, bytes, &s_rbar[w][islot]);
+      bulk_load_hint(s_rows + (size_t)islot * cfg.chunk, lsrc + (size_t)lc * cfg.chunk, bytes, &s_rbar[w][islot], row_policy);
       if (++islot == cfg.nbuf) islot = 0;
       if (++lc == cfg.nchunk) { lc = 0; lsrc += lstep; --lrows; }
     };
@@ -466,17 +463,20 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
     // idles towards the end of k_qsum.
     if (lane == 0) issue_row();
     bool all = false;
-    int slot = 0, b = 0;                                // buffer that is next
+    int slot = 0, b = 0, dealt = 0;                     // buffer that is next; rows of the units before
     uint32_t par = 0;                                   // parity of each buffer's barrier
     for (int u = u0; u < u1 && (what & kTokNorms); ++u) {
       b = image_of(u, b);
       const ImgDesc &im = bt.img[b];
-      const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
+      const int r0 = (u - un.first[b]) * rpp, n = min(rpp, im.N - r0);
       if (im.flags & PACT_FLAG_NO_NORM) {
         for (int r = t; r < n; r += kTokGroup) im.nrm[r0 + r] = 1.0;
         continue;
       }
-      for (int r = w; r < n; r += kTokWarps) {
+      const int first = (w - dealt) & (kTokWarps - 1);
+      dealt += n;
+      int mine = 0;
+      for (int r = first; r < n; r += kTokWarps, ++mine) {
         double a0 = 0.0, a1 = 0.0;
         for (int c = 0; c < cfg.nchunk; ++c) {
           if (!mbar_wait_warp(&s_rbar[w][slot], (par >> slot) & 1)) {
@@ -505,10 +505,10 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
           }
           if (++slot == cfg.nbuf) slot = 0;
         }
-        s_acc[r][lane] = a0 + a1;
+        s_part[mine][lane] = a0 + a1;
       }
       __syncwarp();
-      finish_row_sums(s_acc, w, kTokWarps, n, [&](int r, double s) { im.nrm[r0 + r] = sqrt(s); });
+      finish_row_sums(s_part, mine, [&](int j, double s) { im.nrm[r0 + first + j * kTokWarps] = sqrt(s); });
     }
 norms_end:
     pdl_wait();
@@ -520,7 +520,7 @@ norms_end:
       if (u >= u1 || *const_cast<volatile int *>(&s_abort)) return;
       const int b = image_of(u, 0);
       const ImgDesc &im = bt.img[b];
-      const int r0 = (u - s_first[b]) * rpp, n = min(rpp, im.N - r0);
+      const int r0 = (u - un.first[b]) * rpp, n = min(rpp, im.N - r0);
       if (w == 0) mbar_arrive_expect_tx(&s_kbar[team], n * bt.d_k * (int)sizeof(T));
       for (int r = w; r < n; r += kTeamWarps)
         bulk_load(s_mine + (size_t)r * ks, reinterpret_cast<const T *>(im.Ke) + (size_t)(r0 + r) * im.ldKe, bt.d_k * (int)sizeof(T), &s_kbar[team]);
@@ -548,14 +548,17 @@ norms_end:
       s_query = 1;
       pdl_trigger();
     }
-    for (int u = u0; u < u1 && (what & kTokLogits); ++u) {
-      b = image_of(u, b);
-      const ImgDesc &im = bt.img[b];
-      const bool mine = ((u - u0) & 1) == team;
-      const int g = u - s_first[b], r0 = g * rpp, n = min(rpp, im.N - r0);
+    const auto has_query = [&](int i) { return !(bt.img[i].flags & PACT_FLAG_NORM_ONLY) && bt.img[i].Q != nullptr; };
+    for (int p0 = u0; p0 < u1 && (what & kTokLogits); p0 += 2) {   // a unit for each team, of the images b and b2
+      b = image_of(p0, b);
+      const int b2 = p0 + 1 < u1 ? image_of(p0 + 1, b) : b, mu = p0 + team, mb = team ? b2 : b;
+      const ImgDesc &im = bt.img[mb];
+      const int g = mu - un.first[mb], r0 = g * rpp, n = mu < u1 ? min(rpp, im.N - r0) : 0;
+      const bool use_query = has_query(mb), need_b = QUERY && has_query(b), need_b2 = QUERY && has_query(b2);
+      const double *qg_b = bt.img[b].qg, *qg_b2 = bt.img[b2].qg;
       const uint8_t *keys = cfg.keys ? s_mine : reinterpret_cast<const uint8_t *>(reinterpret_cast<const T *>(im.Ke) + (size_t)r0 * im.ldKe);
       const size_t kstride = cfg.keys ? (size_t)ks : (size_t)im.ldKe * sizeof(T);
-      if (mine) {
+      if (n > 0) {
         if (cfg.keys && !mbar_wait_warp_unless(&s_abort, &s_kbar[team], par)) s_abort = 1;   // (on through the teams' barriers, but without copies)
         par ^= 1u;
         if (im.Kc) {                                     // inverse norms: eight lanes per row, four rows at a time
@@ -576,48 +579,51 @@ norms_end:
           }
         }
       }
-      if (u == u0) {
+      if (p0 == u0) {
         pdl_wait();                                      // the global queries are complete
         s_query = 1;
         pdl_trigger();
       }
-      const bool use_query = !(im.flags & PACT_FLAG_NORM_ONLY) && im.Q != nullptr;
-      if (QUERY && use_query && loaded != b) {                  // both teams come by here for every image of the CTA's units
-        if (loaded >= 0) sync_both();
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (h ? need_b2 && loaded != b2 : need_b && loaded != b) {   // (the same for both teams)
+          if (loaded >= 0) sync_both();
+          loaded = h ? b2 : b;
+          const double *qg = h ? qg_b2 : qg_b;
 #pragma unroll 4
-        for (int c = 2 * (threadIdx.x - kTokGroup); c < bt.n_qcols; c += 2 * kTokGroup) {
-          double2 x;
-          ld_cg_f64x2(&im.qg[c], x.x, x.y);
-          *reinterpret_cast<double2 *>(s_q + c) = x;
+          for (int c = 2 * (threadIdx.x - kTokGroup); c < bt.n_qcols; c += 2 * kTokGroup) {
+            double2 x;
+            ld_cg_f64x2(qg + c, x.x, x.y);
+            *reinterpret_cast<double2 *>(s_q + c) = x;
+          }
+          sync_both();
         }
-        loaded = b;
-        sync_both();
+        if (h != team || n == 0) continue;
+        const double *q = QUERY ? s_q : im.qg;
+        if constexpr (GROUP) {
+          const int nblk = (n_rep + 7) / 8;              // blocks of up to eight query heads per key head
+          const bool in_smem = QUERY && cfg.keys;
+          for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
+            const int kv = it / nblk, j = (it - kv * nblk) * 8, j0 = kv * n_rep + j, nr = min(8, n_rep - j);
+            const uint8_t *kh = keys + (size_t)kv * d_h * sizeof(T);
+            if (!in_smem) group_piece<T, 1, false>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);   // (n <= kMinPiece)
+            else if (n <= 8) group_piece<T, 1, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+            else if (n <= 16) group_piece<T, 2, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+            else if (n <= 24) group_piece<T, 3, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+            else group_piece<T, 4, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
+          }
+        } else {
+          const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
+          for (int kv = w; kv < n_kvh; kv += kTeamWarps) {
+            const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
+            if (n_rep == 2) head_piece<T, 2>(bt, im, kh, q + (size_t)2 * kv * d_h, use_query, P, 2 * kv, r0, n, g);
+            else head_piece<T, 1>(bt, im, kh, q + (size_t)kv * d_h, use_query, P, kv, r0, n, g);
+          }
+        }
       }
-      if (!mine) continue;
-      const double *q = QUERY ? s_q : im.qg;
-      if constexpr (GROUP) {
-        const int nblk = (n_rep + 7) / 8;                // blocks of up to eight query heads per key head
-        const bool in_smem = QUERY && cfg.keys;
-        for (int it = w; it < n_kvh * nblk; it += kTeamWarps) {
-          const int kv = it / nblk, j = (it - kv * nblk) * 8, j0 = kv * n_rep + j, nr = min(8, n_rep - j);
-          const uint8_t *kh = keys + (size_t)kv * d_h * sizeof(T);
-          if (!in_smem) group_piece<T, 1, false>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);   // (n <= kMinPiece)
-          else if (n <= 8) group_piece<T, 1, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
-          else if (n <= 16) group_piece<T, 2, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
-          else if (n <= 24) group_piece<T, 3, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
-          else group_piece<T, 4, true>(bt, im, kh, kstride, q + (size_t)j0 * d_h, use_query, nr, j0, r0, n, g);
-        }
-      } else {
-        const uint8_t *krow = keys + (size_t)min(lane & (32 / P - 1), n - 1) * kstride;
-        for (int kv = w; kv < n_kvh; kv += kTeamWarps) {
-          const uint8_t *kh = krow + (size_t)kv * d_h * sizeof(T);
-          if (n_rep == 2) head_piece<T, 2>(bt, im, kh, q + (size_t)2 * kv * d_h, use_query, P, 2 * kv, r0, n, g);
-          else head_piece<T, 1>(bt, im, kh, q + (size_t)kv * d_h, use_query, P, kv, r0, n, g);
-        }
-      }
-      if (cfg.keys && u + 2 < u1) {
+      if (cfg.keys && mu + 2 < u1) {
         sync();                                          // the keys have been read
-        if (lane == 0) issue_keys(u + 2);
+        if (lane == 0) issue_keys(mu + 2);
       }
     }
   }
@@ -1333,7 +1339,12 @@ static cudaError_t launch_qsum(const Batch &bt, const DeviceCfg &cfg, cudaStream
   opt.cluster = 1;
   while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 3 * cfg.sm_count) opt.cluster *= 2;
   const dim3 grid(ncg * opt.cluster, bt.B), block(kQsumThreads);
-  return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster);
+  // nothing reads the queries again: where they are many they leave the L2 first (three images with 28 heads, 37 MB: 93.7 -> 92.2
+  // us; 16 images of four heads, 48 MB: 251.5 -> 249.8; 7.5 MB of one image: no difference)
+  long long rows = 0;
+  for (int b = 0; b < bt.B; ++b) rows += bt.img[b].N;
+  const uint64_t policy = rows * bt.n_qcols * (long long)sizeof(T) > (16ll << 20) ? kEvictFirst : kEvictNormal;
+  return narrow ? launch_opt(opt, k_qsum<T, 4>, grid, block, 0, st, bt, opt.cluster, policy) : launch_opt(opt, k_qsum<T, 8>, grid, block, 0, st, bt, opt.cluster, policy);
 }
 
 template <typename T> static TokCfg tokens_config(const Batch &bt, const DeviceCfg &cfg) {
@@ -1341,19 +1352,23 @@ template <typename T> static TokCfg tokens_config(const Batch &bt, const DeviceC
   for (int b = 0; b < bt.B; ++b) total += bt.img[b].N;
   return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, cfg.sm_count, cfg.smem_optin - kTokReserve);
 }
-static int tokens_grid(const Batch &bt, int rpp, const DeviceCfg &cfg) {
-  long long units = 0;
-  for (int b = 0; b < bt.B; ++b) units += (bt.img[b].N + rpp - 1) / rpp;
-  return units < cfg.sm_count ? (int)units : cfg.sm_count;
-}
-
 template <typename T>
-static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
+static cudaError_t launch_tokens(const Batch &bt, bool scores_only, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
   const TokCfg tc = tokens_config<T>(bt, cfg);
   if (rpp) *rpp = tc.rpp;
   const bool group = bt.n_qh / bt.n_kvh >= kGroupHeads;
   const auto kernel = tc.query ? (group ? k_tokens<T, true, true> : k_tokens<T, true, false>) : (group ? k_tokens<T, false, true> : k_tokens<T, false, false>);
-  return launch_k(kernel, dim3(tokens_grid(bt, tc.rpp, cfg)), dim3(kTokThreads), tok_smem(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, what);
+  int N[kMaxBatchPerLaunch];
+  long long tokens = 0;
+  for (int b = 0; b < bt.B; ++b) tokens += N[b] = bt.img[b].N;
+  TokUnits un;
+  const int grid = tokens_units(N, bt.B, tc.rpp, cfg.sm_count, un);
+  // Hidden states that the merge will not find in the L2 in any case (a call with more than 72 MB of them, scores as a stage of
+  // their own) leave it first, so that queries, keys and what the kernels hand to one another stay: 16 images of 2916 tokens (334
+  // MB) 254.6 -> 249.4 us with all of them marked, 253.1 with the first 72 MB kept; scores and split of 7290 tokens 27.9 ->
+  // 27.3; one image of 7290 (52 MB) the other way, 94.3 -> 96.5.
+  const uint64_t policy = scores_only || tokens * bt.d * (long long)sizeof(T) > (72ll << 20) ? kEvictFirst : kEvictNormal;
+  return launch_k(kernel, dim3(grid), dim3(kTokThreads), tok_smem_launch(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, un, policy, what);
 }
 
 template <typename T>
@@ -1365,7 +1380,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
   int rpp = 0;
-  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
+  e = launch_tokens<T>(bt, mode == 1, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
   if (e != cudaSuccess) return e;
   for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
     // (a part without visual tokens may still bring text rows, which k_merge copies)
@@ -1375,7 +1390,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
     part.img[0].N = feed->end[k] - first;
     part.img[0].vis_start += first;
     part.img[0].nrm += first;
-    if ((e = launch_tokens<T>(part, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
+    if ((e = launch_tokens<T>(part, false, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
   }
   if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;

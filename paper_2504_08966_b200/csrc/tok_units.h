@@ -2,6 +2,7 @@
 // Arithmetic on sizes alone, without CUDA, so that every size a context accepts can be gone through on the host.
 #pragma once
 #include <stddef.h>
+#include <stdint.h>
 
 #ifdef __CUDACC__
 #define PACT_HD __host__ __device__
@@ -11,6 +12,7 @@
 
 namespace pact {
 
+constexpr int kMaxBatchPerLaunch = 16;   // images described by one kernel parameter block
 constexpr int kMinPiece = 8;             // fewest visual tokens in a softmax piece of k_tokens (at most 32)
 constexpr int kTokWarps = 8;             // warps that stream hidden-state rows
 constexpr int kTokMaxBuf = 2;            // row buffers per warp
@@ -30,6 +32,13 @@ PACT_HD inline int tok_key_stride(int row_bytes) { return row_bytes | 16; }
 
 inline size_t tok_smem(const TokCfg &c, int key_bytes, int n_qcols) {
   return (size_t)kTokWarps * c.nbuf * c.chunk + (size_t)2 * c.keys * c.rpp * tok_key_stride(key_bytes) + (size_t)c.query * n_qcols * 8 + (size_t)c.rpp * 32 * 8;
+}
+
+// What a launch asks for: the parts of the sums of squares have a row for each of a warp's tokens of a unit, so that no other warp
+// writes there, up to seven rows more than the unit has tokens.  (kTokSmem leaves room for them.)
+PACT_HD inline int tok_warp_rows(int rpp) { return (rpp + kTokWarps - 1) / kTokWarps; }
+inline size_t tok_smem_launch(const TokCfg &c, int key_bytes, int n_qcols) {
+  return tok_smem(c, key_bytes, n_qcols) + (size_t)(tok_warp_rows(c.rpp) * kTokWarps - c.rpp) * 32 * 8;
 }
 
 // total tokens of the call, rows of row_bytes, keys of key_bytes, n_rep query heads per key head, and the GPU's SMs and shared memory.
@@ -68,6 +77,25 @@ inline TokCfg tokens_config(long long total, int row_bytes, int key_bytes, int n
   while (!fits() && c.chunk > 1024) cut_rows(2 * c.nchunk);
   c.query = tok_smem(c, key_bytes, n_qcols) <= smem_optin;
   return c;
+}
+
+// The units of a call: those of image b begin at first[b]; CTA c takes `per` of them and one more if c < extra, in a row.
+struct TokUnits {
+  int first[kMaxBatchPerLaunch + 1];
+  int per, extra;
+};
+
+// Units of rpp tokens of B images of N[b] tokens each, shared out; returns the number of CTAs.  (At most 16 x 2^18 / 8 units.)
+inline int tokens_units(const int *N, int B, int rpp, int sm_count, TokUnits &un) {
+  int units = 0;
+  for (int b = 0; b <= kMaxBatchPerLaunch; ++b) {
+    un.first[b] = units;
+    if (b < B) units += (N[b] + rpp - 1) / rpp;
+  }
+  const int grid = units < sm_count ? units : sm_count;
+  un.per = units / grid;
+  un.extra = units - un.per * grid;
+  return grid;
 }
 
 }  // namespace pact

@@ -74,3 +74,31 @@ def test_what_fits_beside_whole_copies_stays_as_it_was(configs):
         want = plain(*case)
         if want is not None:
             assert got[:3] == want and got[4], case
+
+
+def test_every_unit_has_one_cta(tmp_path):
+    """Images of any sizes: the CTAs' shares follow one another, differ by one unit at most and end with the last one."""
+    (tmp_path / "share.cpp").write_text(r"""
+#include <stdio.h>
+#include "tok_units.h"
+int main() {
+  int B, rpp, N[pact::kMaxBatchPerLaunch];
+  while (scanf("%d %d", &B, &rpp) == 2) {
+    for (int b = 0; b < B; ++b) if (scanf("%d", N + b) != 1) return 1;
+    pact::TokUnits un;
+    printf("%d", pact::tokens_units(N, B, rpp, 148, un));
+    for (int b = 0; b <= pact::kMaxBatchPerLaunch; ++b) printf(" %d", un.first[b]);
+    printf(" %d %d\n", un.per, un.extra);
+  }
+}
+""")
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Werror", "-I", os.path.join(ROOT, "paper_2504_08966_b200", "csrc"), str(tmp_path / "share.cpp"), "-o", str(tmp_path / "share")])
+    cases = [(rpp, N) for rpp in (8, 25, 32) for N in ([1], [8], [9], [1184], [1185], [7290], [1 << 18], [1, 262144], [2309, 1731, 1153], [33] * 16, [1 << 18] * 16)]
+    out = subprocess.run([str(tmp_path / "share")], input="\n".join(f"{len(N)} {rpp} {' '.join(map(str, N))}" for rpp, N in cases), capture_output=True, text=True, check=True).stdout
+    for (rpp, N), line in zip(cases, out.splitlines()):
+        grid, *first, per, extra = (int(x) for x in line.split())
+        want = [0]
+        for n in N:
+            want.append(want[-1] + -(-n // rpp))
+        assert first == want + [want[-1]] * (17 - len(want))
+        assert grid == min(148, want[-1]) and per >= 1 and 0 <= extra < grid and per * grid + extra == want[-1]
