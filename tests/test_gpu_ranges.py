@@ -391,3 +391,23 @@ def test_host_buffers_with_the_flags_of_the_ablations(N, T, d):
         ctx = pb.Context(wl.d, wl.n_qh, wl.n_kvh, wl.d_h, wl.dtype, torch.float32)
         for _ in range(3):
             _same_as_device(_host_call(wl, ctx, params), want)
+
+
+def test_merged_rows_of_any_bf16_value():
+    """Rows with every bf16 value (subnormal numbers, infinities, NaN): text rows and clusters of one row, and sums of two in fp32."""
+    from paper_2504_08966_b200 import binding as pb
+    d, N, T = 4096, 18, 14
+    bits = torch.arange(65536, dtype=torch.int32).reshape(16, d).to(torch.int16).view(torch.bfloat16)
+    H = torch.cat([bits, bits]).cuda()                # token i of the second half of the rows is row i + T
+    z = lambda m, dt: torch.zeros(m, dtype=dt, device="cuda")   # noqa: E731
+    K = z((N, 64), torch.bfloat16)
+    label = torch.arange(N, dtype=torch.int32, device="cuda") % 17           # tokens 0 and 17 share a cluster
+    im = pb.DeviceImage(H, K, K, K, torch.arange(N + T, dtype=torch.int32, device="cuda"), T, N, z((N + T, d), torch.float32), z(N + T, torch.int32),
+                        z(N + T, torch.int32), z(N, torch.int32), z(N, torch.float32), z(N, torch.uint8), z(pb.N_COUNTERS, torch.int32))
+    pb.Context(d, 1, 1, 64, torch.bfloat16, torch.float32).pact_merge(im, label, torch.arange(17, dtype=torch.int32, device="cuda"),
+                                                                      torch.tensor([17], dtype=torch.int32, device="cuda"), pb.make_params())
+    want = 0.0 + H[:T + 17].float()                   # (a sum begins at +0)
+    want[T] = (want[T] + H[T + 17].float()) * 0.5
+    got = im.H_out[:T + 17]
+    assert torch.equal(torch.isnan(got), torch.isnan(want))
+    assert torch.equal(torch.nan_to_num(got, nan=0.0).view(torch.int32), torch.nan_to_num(want, nan=0.0).view(torch.int32))
