@@ -58,6 +58,10 @@ struct TmapSet {
   CUtensorMap a[kMaxBatchPerLaunch];
   CUtensorMap b[kMaxBatchPerLaunch];
 };
+struct AssignMaps {
+  CUtensorMap a[kMaxBatchPerLaunch], b[kMaxBatchPerLaunch];
+  CUtensorMap b32[kMaxBatchPerLaunch];             // the centres in boxes of 32 rows
+};
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {
   asm volatile(
@@ -107,14 +111,6 @@ template <int MODE> __device__ __forceinline__ void tile_at(int t, int ntm, int 
     tni = t % ntn;
   }
 }
-// Columns of tile column tni that the MMA has to produce: the rows x centres pass stops at the last
-// centre, rounded up to the instruction's granularity of 16.
-template <int MODE, int BN> __device__ __forceinline__ int tile_width(int tni, int ncols) {
-  if (MODE != MODE_ASSIGN) return BN;
-  const int left = ncols - tni * BN;
-  return left >= BN ? BN : ((left + 15) & ~15);
-}
-
 // Labels of a group of 32 tokens (lane = token) whose nearest centres are final, formed by the last epilogue
 // warp of the rows x centres pass to finish the group: a survivor takes its nearest centre's cluster (a centre
 // its own), a pruned token that cluster iff the distance is strictly below alpha * d_c (Eq. 8-9), else -1.
@@ -163,11 +159,10 @@ __device__ __forceinline__ void label_group(const ImgDesc &im, int i, int lane, 
 // block tmi against HALF columns from cbase on.  Waits for the accumulator, reads it 32 columns at a time and
 // applies the mode's arithmetic; arrive() is called once the accumulator has been read.  skip: the warp only
 // waits and releases (a block below the diagonal of the all-pairs pass).  Returns false when the wait ran out.
-template <int MODE, int HALF, bool WAIT_MIN = false, typename Arrive>
+template <int MODE, int HALF, typename Arrive>
 __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int tmi, int cbase, bool skip, int nrows,
                                          int ncols, uint32_t taddr, uint64_t *acc_full, uint32_t parity, float *rn_col,
-                                         uint32_t *tr, int lane, int qd, int &band, float &mx, Arrive arrive,
-                                         unsigned long long &seen) {
+                                         uint32_t *tr, int lane, int qd, int &band, float &mx, Arrive arrive) {
   // inverse norms of this warp's columns and of this lane's row (in flight while the MMAs run)
   const float *rn_src = MODE == MODE_GRAM ? im.rnk : (MODE == MODE_SPREAD ? im.rn : im.rnc);
   float4 r4;
@@ -306,8 +301,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
     if (MODE == MODE_GRAM) atomicAdd(&im.rho_fix[row], rowsum);
     else if (MODE == MODE_ASSIGN && bd <= 2.0f) {
       const unsigned long long pk = ((unsigned long long)__float_as_uint(bd) << 32) | (unsigned)bi;
-      const unsigned long long old = atomicMin(&im.best[kept_rows ? im.kept_idx[row] : row], pk);
-      if (WAIT_MIN) seen |= old;                   // the caller waits for the value: the minimum is then in place
+      atomicMin(&im.best[kept_rows ? im.kept_idx[row] : row], pk);
     }
   }
   return true;
@@ -316,17 +310,14 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
 }  // namespace
 
 // grid (X, B), 64 + 32 EPI_WARPS threads, dynamic smem = TileCfg<BN>::SMEM.
-// kept_rows (assignment only), bit 0: rows are the gathered survivors (Kp, rnk) instead of all tokens;
-// bit 1: the labels, cluster sizes and per-block member counts are formed here as groups of rows finish.
 template <int MODE, int BN>
 __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant__ Batch bt,
-                                                           const __grid_constant__ TmapSet tm, int kept_rows) {
+                                                           const __grid_constant__ TmapSet tm) {
   using Cfg = TileCfg<BN>;
   constexpr int STAGES = Cfg::STAGES, NACC = Cfg::NACC, HALF = Cfg::HALF, SLABS = Cfg::SLABS;
   constexpr int STAGE_BYTES = Cfg::STAGE_BYTES, B_BYTES = Cfg::B_BYTES;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, MODE == MODE_GRAM ? 4 : 6);
-  (void)kept_rows;
   extern __shared__ uint8_t smem_raw[];
   __shared__ Shared sh;
   uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -350,8 +341,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
 
   int nrows, ncols;
   if (MODE == MODE_GRAM) { nrows = *im.q_ptr; ncols = nrows; }
-  else if (MODE == MODE_SPREAD) { nrows = im.N; ncols = im.N; }
-  else { nrows = (kept_rows & 1) ? *im.q_ptr : im.N; ncols = *im.C_ptr; }
+  else { nrows = im.N; ncols = im.N; }
   const int ntm = (nrows + BM - 1) / BM, ntn = (ncols + BN - 1) / BN;
   const int ntiles = tile_count<MODE>(ntm, ntn);
   const bool active = (int)blockIdx.x < ntiles;       // CTAs without a tile only give their tensor memory back
@@ -368,19 +358,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
         int tmi, tni;
         tile_at<MODE>(tile, ntm, ntn, tmi, tni);
         if (!tile_wanted<MODE, BN>(tmi, tni)) continue;
-        const int bw = tile_width<MODE, BN>(tni, ncols);
         for (int ks = 0; ks < nslab; ks += SLABS, ++it) {
           const int s = it % STAGES;
           const int n = min(SLABS, nslab - ks);
           if (!mbar_wait(&sh.empty[s], ((it / STAGES) & 1) ^ 1)) { ok = false; break; }
           uint8_t *a_dst = ring + (size_t)s * STAGE_BYTES, *b_dst = a_dst + SLABS * A_BYTES;
-          const bool second = BN == 256 && bw > BN / 2;   // the second 128 rows of B are needed
-          const uint32_t per = second || BN != 256 ? (A_BYTES + B_BYTES) : (A_BYTES + B_BYTES / 2);
-          mbar_arrive_expect_tx(&sh.full[s], (uint32_t)n * per);
+          mbar_arrive_expect_tx(&sh.full[s], (uint32_t)n * (A_BYTES + B_BYTES));
           for (int h = 0; h < n; ++h) {
             tma_load_2d(a_dst + h * A_BYTES, ma, &sh.full[s], (ks + h) * BK, tmi * BM);
             tma_load_2d(b_dst + h * B_BYTES, mb, &sh.full[s], (ks + h) * BK, tni * BN);
-            if (second) tma_load_2d(b_dst + h * B_BYTES + B_BYTES / 2, mb, &sh.full[s], (ks + h) * BK, tni * BN + BN / 2);
+            if (BN == 256) tma_load_2d(b_dst + h * B_BYTES + B_BYTES / 2, mb, &sh.full[s], (ks + h) * BK, tni * BN + BN / 2);
           }
         }
       }
@@ -405,20 +392,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
         if (!mbar_wait(&sh.acc_empty[a], ((tcount / NACC) & 1) ^ 1)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * BN;
-        // instruction descriptor with this tile's width in its N field
-        const uint32_t idesc = (Cfg::IDESC & ~(0x3Fu << 17)) | ((uint32_t)(tile_width<MODE, BN>(tni, ncols) >> 3) << 17);
         for (int ks = 0; ks < nslab; ks += SLABS, ++it) {
           const int s = it % STAGES;
           const int n = min(SLABS, nslab - ks);
           if (!mbar_wait(&sh.full[s], (it / STAGES) & 1)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(ring + (size_t)s * STAGE_BYTES), b_addr = a_addr + SLABS * A_BYTES;
+          const uint32_t a_addr = smem_u32(ring + (size_t)s * STAGE_BYTES);
+          const uint64_t da = smem_desc(a_addr), db = smem_desc(a_addr + SLABS * A_BYTES);
 #pragma unroll
           for (int h = 0; h < SLABS; ++h) {
             if (h < n) {
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k)
-                umma_bf16(d_tmem, smem_desc(a_addr + h * A_BYTES + k * 32), smem_desc(b_addr + h * B_BYTES + k * 32), idesc, (ks | h | k) != 0);
+                umma_bf16(d_tmem, desc_at(da, h * A_BYTES + k * 32), desc_at(db, h * B_BYTES + k * 32), Cfg::IDESC, (ks | h | k) != 0);
             }
           }
           umma_commit(&sh.empty[s]);               // frees the slab once these MMAs have read it
@@ -442,14 +428,198 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
     int band = 0;
     bool ok = true;
     float mx = 0.f;                                 // largest distance seen by this lane (MODE_SPREAD)
-    // Labels (rows x centres pass with bit 1 of kept_rows): a group of 32 tokens is final once `need` warps
-    // (every column tile, every column half) have put their nearest centres in place; each warp draws a
-    // ticket per group and the one that draws the last labels the group.  The tickets of up to kPend tiles
-    // are drawn together, so that a warp waits for its atomics to land once, not once per tile.
+    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+      int tmi, tni;
+      tile_at<MODE>(tile, ntm, ntn, tmi, tni);
+      if (!tile_wanted<MODE, BN>(tmi, tni)) continue;
+      const uint32_t a = tcount % NACC;
+      const int cbase = tni * BN + half * HALF;     // first column of this warp
+      const uint32_t taddr = tmem_base + a * BN + half * HALF + ((uint32_t)(qd * 32) << 16);
+      ok = epi_tile<MODE, HALF>(im, 0, tmi, cbase, false, nrows, ncols, taddr, &sh.acc_full[a], (tcount / NACC) & 1,
+                                rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive(&sh.acc_empty[a]); });
+      if (!ok) break;
+      ++tcount;
+    }
+    if (!ok) atomicExch(&sh.abort, 1);
+    if (MODE == MODE_GRAM && band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
+    if (MODE == MODE_SPREAD) {
+      // distances are clamped to [0, 2]: their bit patterns order like unsigned integers
+      const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+      if (lane == 0 && w) atomicMax(reinterpret_cast<unsigned *>(&im.cnt[kCntSpread]), w);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+  if (threadIdx.x == 0 && sh.abort) atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
+}
+
+// ---- rows x centres on single CTAs ---------------------------------------------------------------------------------
+// grid (X, B), 64 + 32 EPI_WARPS threads, one CTA per SM with the roles of k_tiles_umma.  Tiles are 128 rows x W centres.
+// kept_rows, bit 0: rows are the gathered survivors (Kp, rnk) instead of all tokens; bit 1: the labels, cluster sizes and
+// per-block member counts are formed here as groups of rows finish.
+//
+// Where the row blocks are few enough that every CTA needs one tile only, the centres are shared out among as many columns of tiles
+// as give every CTA one, all of the same width: up to 512 columns, i.e. the whole tensor memory, in two instructions per
+// step.  With columns of 256 whatever C is, one image of 7290 tokens and 535 centres had 171 tiles for 148 CTAs, and the pass
+// ended with the 23 second ones: 14.0 us from the centres to the labels, 12.3 now (call 93.2 -> 91.6).  More row blocks: tiles of 256 in
+// rounds, two accumulators, the (usually narrow) last column last.  Bound by latency: of the 12 us 2.0 pass until the first operands are
+// there, 3.7 until the last, 1.1 until the accumulator is complete, 2.0 in the epilogue, 1.1 for the tickets.
+constexpr int kAsnRing = 192 * 1024;                 // (with more of it the next kernels' CTAs find no room beside this one and crowd on a few SMs)
+constexpr int kAsnSmem = 1024 + kAsnRing;
+constexpr int kAsnMostCols = TMEM_COLS, kAsnLeastCols = 64;
+
+// a / b for a below 2^22 and b > 0 (the compiler's division is three times as long, from a cold instruction cache)
+__device__ __forceinline__ int div_small(int a, int b) {
+  int q = (int)__fdividef((float)a, (float)b);
+  q -= q * b > a;
+  return q + ((q + 1) * b <= a);
+}
+struct AsnTiles {
+  int ntm, ntn, W, slabs, stages, nacc, stage_bytes;
+  __device__ __forceinline__ AsnTiles(int nrows, int C, int ctas) {
+    ntm = (nrows + BM - 1) / BM;
+    W = 256;
+    if (ntm * ((C + kAsnMostCols - 1) / kAsnMostCols) <= ctas && ntm > 0) {
+      const int n = min(div_small(ctas, ntm), (C + kAsnLeastCols - 1) / kAsnLeastCols);
+      W = n > 0 ? (div_small(C + n - 1, n) + 31) & ~31 : kAsnLeastCols;
+    }
+    ntn = div_small(C + W - 1, W);
+    nacc = W <= 256 ? 2 : 1;
+    const int slab = A_BYTES + W * BK * 2;
+    slabs = 4 * slab <= kAsnRing ? 2 : 1;              // two K-slabs per stage where two stages fit
+    stage_bytes = slabs * slab;
+    stages = 4 * stage_bytes <= kAsnRing ? 4 : 3 * stage_bytes <= kAsnRing ? 3 : 2;
+  }
+  // columns of tile column tni that the MMA has to produce, in steps of 32
+  __device__ __forceinline__ int width(int tni, int C) const { return min(W, (C - tni * W + 31) & ~31); }
+};
+
+// (80 registers: with 94 no CTA of k_merge finds room beside one of this kernel before it ends, and the calls took 3 to 4 us more)
+__global__ void __maxnreg__(80) k_assign(const __grid_constant__ Batch bt, const __grid_constant__ AssignMaps tm, int kept_rows) {
+  const ImgDesc &im = bt.img[blockIdx.y];
+  TL_SCOPE(im, 6);
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ Shared sh;
+  uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], EPI_WARPS); }
+    mbar_init(&sh.done, 1);
+    sh.abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tmem_alloc(&sh.tmem_base, TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = sh.tmem_base;
+  pdl_wait();
+  pdl_trigger();
+
+  const int nrows = (kept_rows & 1) ? *im.q_ptr : im.N, C = *im.C_ptr;
+  const AsnTiles tl(nrows, C, gridDim.x);
+  const int ntiles = tl.ntm * tl.ntn, nslab = bt.d_k / BK;
+  const bool active = (int)blockIdx.x < ntiles;       // CTAs without a tile only give their tensor memory back
+
+  if (!active) {
+  } else if (warp == 0) {
+    // ---------------- TMA producer ----------------
+    if (lane == 0) {
+      const CUtensorMap *ma = &tm.a[blockIdx.y], *mb = &tm.b[blockIdx.y], *mc = &tm.b32[blockIdx.y];
+      uint32_t it = 0;
+      int s = 0;
+      uint32_t par = 1;
+      bool ok = true;
+      for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+        int tmi, tni;
+        tile_at<MODE_ASSIGN>(tile, tl.ntm, tl.ntn, tmi, tni);
+        const int wd = tl.width(tni, C);
+        for (int ks = 0; ks < nslab; ks += tl.slabs, ++it) {
+          const int n = min(tl.slabs, nslab - ks);
+          if (!mbar_wait(&sh.empty[s], par)) { ok = false; break; }
+          uint8_t *a_dst = ring + (size_t)s * tl.stage_bytes, *b_dst = a_dst + tl.slabs * A_BYTES;
+          mbar_arrive_expect_tx(&sh.full[s], (uint32_t)n * (A_BYTES + wd * BK * 2));
+          for (int h = 0; h < n; ++h, b_dst += tl.W * BK * 2) {
+            tma_load_2d(a_dst + h * A_BYTES, ma, &sh.full[s], (ks + h) * BK, tmi * BM);
+            int r = 0;
+            for (; r + BM <= wd; r += BM) tma_load_2d(b_dst + r * BK * 2, mb, &sh.full[s], (ks + h) * BK, tni * tl.W + r);
+            for (; r < wd; r += 32) tma_load_2d(b_dst + r * BK * 2, mc, &sh.full[s], (ks + h) * BK, tni * tl.W + r);
+          }
+          if (++s == tl.stages) { s = 0; par ^= 1; }
+        }
+      }
+      if (!ok) atomicExch(&sh.abort, 1);
+      // drain: every armed stage completes before the CTA may exit (its copies target this smem)
+      const uint32_t armed = min(it, (uint32_t)tl.stages);
+      for (uint32_t k = 0; k < armed; ++k) {
+        const uint32_t j = it - 1 - k;
+        mbar_wait(&sh.full[j % tl.stages], (j / tl.stages) & 1);
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    if (lane == 0) {
+      uint32_t tcount = 0;
+      int s = 0;
+      uint32_t par = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++tcount) {
+        int tmi, tni;
+        tile_at<MODE_ASSIGN>(tile, tl.ntm, tl.ntn, tmi, tni);
+        const int wd = tl.width(tni, C);
+        const uint32_t a = tl.nacc == 2 ? tcount & 1 : 0, ph = tl.nacc == 2 ? tcount >> 1 : tcount;
+        if (!mbar_wait(&sh.acc_empty[a], (ph & 1) ^ 1)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + a * 256;
+        // kind::f16, fp32 accumulate, bf16 x bf16, both operands K-major, M = 128, N = the first 256 columns and the others
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
+        const uint32_t first = idesc | ((uint32_t)(min(wd, 256) >> 3) << 17), second = idesc | ((uint32_t)(max(wd - 256, 0) >> 3) << 17);
+        for (int ks = 0; ks < nslab; ks += tl.slabs) {
+          const int n = min(tl.slabs, nslab - ks);
+          if (!mbar_wait(&sh.full[s], par)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t a_addr = smem_u32(ring + (size_t)s * tl.stage_bytes);
+          const uint64_t da = smem_desc(a_addr), db = smem_desc(a_addr + tl.slabs * A_BYTES);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (h < n) {
+              const uint64_t ah = desc_at(da, h * A_BYTES), bh = desc_at(db, h * tl.W * BK * 2);
+#pragma unroll
+              for (int k = 0; k < BK / 16; ++k) umma_bf16(d_tmem, desc_at(ah, k * 32), desc_at(bh, k * 32), first, (ks | h | k) != 0);
+              if (wd > 256) {
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k) umma_bf16(d_tmem + 256, desc_at(ah, k * 32), desc_at(bh, 256 * BK * 2 + k * 32), second, (ks | h | k) != 0);
+              }
+            }
+          umma_commit(&sh.empty[s]);                 // frees the stage once these MMAs have read it
+          if (++s == tl.stages) { s = 0; par ^= 1; }
+        }
+        if (ok) umma_commit(&sh.acc_full[a]);        // accumulator complete
+      }
+      // whatever way the loop ended, no MMA may still be running when the tensor memory is given back
+      umma_commit(&sh.done);
+      if (!mbar_wait(&sh.done, 0)) ok = false;
+      if (!ok) atomicExch(&sh.abort, 1);
+    }
+  } else {
+    // ---------------- epilogue ----------------
+    const int ew = warp - 2;
+    const int qd = warp & 3;                          // tensor-memory lane quadrant this warp may read
+    const int part = ew >> 2;                         // which quarter of the tile's columns
+    float *rn_col = sh.rn_col[ew];
+    uint32_t tcount = 0;
+    bool ok = true;
+    // Labels: a group of 32 tokens is final once `need` warps (every column tile, every quarter of the columns) have put their
+    // nearest centres in place; each warp draws a ticket per group and the one that draws the last labels the group.  The
+    // tickets of up to kPend tiles are drawn together, so that a warp waits for its atomics to land once, not once per tile.
     constexpr int kPend = 4;
-    const int need = (MODE == MODE_ASSIGN && (kept_rows & 2)) ? ntn * (EPI_WARPS / 4) : 0;
-    int pend_tmi[kPend], pend_r[kPend], pend_cid[kPend], npend = 0;
-    unsigned long long seen = 0ull;                 // previous values of the minima this lane has updated
+    const int need = (kept_rows & 2) ? tl.ntn * (EPI_WARPS / 4) : 0;
+    int pend_tmi[kPend] = {}, pend_r[kPend] = {}, pend_cid[kPend] = {}, npend = 0;
+    unsigned long long seen = 0ull;                   // previous values of the minima this lane has updated
     auto flush_labels = [&]() {
       // Every lane's atomic minima have returned, i.e. are in place, once their return values have been used:
       // the fence then has nothing left to wait for.  (No stored value has distance bits above 2.0f.)
@@ -468,44 +638,78 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
 #pragma unroll
       for (int k = 0; k < kPend; ++k)
         if (k < npend && ((lastmask >> k) & 1u))
-          label_group(im, pend_tmi[k] * BM + qd * 32 + lane, lane, ncols, pend_r[k], pend_cid[k]);
+          label_group(im, pend_tmi[k] * BM + qd * 32 + lane, lane, C, pend_r[k], pend_cid[k]);
       npend = 0;
     };
-    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
       int tmi, tni;
-      tile_at<MODE>(tile, ntm, ntn, tmi, tni);
-      if (!tile_wanted<MODE, BN>(tmi, tni)) continue;
-      const uint32_t a = tcount % NACC;
-      const int cbase = tni * BN + half * HALF;     // first column of this warp
-      const uint32_t taddr = tmem_base + a * BN + half * HALF + ((uint32_t)(qd * 32) << 16);
-      if (MODE == MODE_ASSIGN && need > 0) {
-        // what the labels of this warp's 32 tokens need besides the nearest centre (known before the pass)
-        const int row = tmi * BM + qd * 32 + lane;
+      tile_at<MODE_ASSIGN>(tile, tl.ntm, tl.ntn, tmi, tni);
+      const int wd = tl.width(tni, C);
+      const uint32_t a = tl.nacc == 2 ? tcount & 1 : 0, ph = tl.nacc == 2 ? tcount >> 1 : tcount;
+      // this warp's columns of the tile
+      const int cw = ((wd >> 2) + 15) & ~15, c_lo = tni * tl.W + part * cw, c_hi = min(min(c_lo + cw, tni * tl.W + wd), C);
+      const int row = tmi * BM + qd * 32 + lane;
+      const bool row_ok = row < nrows;
+      // inverse norms of the warp's columns and of the lane's row, and what the labels need besides the nearest centre (known before the pass)
+      float4 r4;
+      {
+        const int gj = c_lo + lane * 4;
+        r4.x = gj + 0 < c_hi ? im.rnc[gj + 0] : 0.f;
+        r4.y = gj + 1 < c_hi ? im.rnc[gj + 1] : 0.f;
+        r4.z = gj + 2 < c_hi ? im.rnc[gj + 2] : 0.f;
+        r4.w = gj + 3 < c_hi ? im.rnc[gj + 3] : 0.f;
+      }
+      const float rni = row_ok ? ((kept_rows & 1) ? im.rnk[row] : im.rn[row]) : 0.f;
+      if (need > 0) {
         int r = -1, own = -1;
-        if (row < nrows) {
+        if (row_ok) {
           r = im.slot[row];
           if (r >= 0 && ((im.cmask[r >> 5] >> (r & 31)) & 1u)) own = im.cid[r];
         }
         pend_tmi[npend] = tmi; pend_r[npend] = r; pend_cid[npend] = own;
       }
-      if (need > 0)
-        ok = epi_tile<MODE, HALF, true>(im, kept_rows & 1, tmi, cbase, false, nrows, ncols, taddr, &sh.acc_full[a], (tcount / NACC) & 1,
-                                        rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive(&sh.acc_empty[a]); }, seen);
-      else
-        ok = epi_tile<MODE, HALF>(im, kept_rows & 1, tmi, cbase, false, nrows, ncols, taddr, &sh.acc_full[a], (tcount / NACC) & 1,
-                                  rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive(&sh.acc_empty[a]); }, seen);
-      if (!ok) break;
+      __syncwarp();
+      reinterpret_cast<float4 *>(rn_col)[lane] = r4;
+      __syncwarp();
+      if (!mbar_wait_warp(&sh.acc_full[a], ph & 1)) { ok = false; break; }
+      tc_fence_after();
+      // the nearest centre is the one with the largest cosine (dot * rn_i) * rn_j; the first of equal cosines wins, i.e. the
+      // centre with the lowest index; the distance is formed once per tile
+      float bc = -4.0f;
+      int bi = 0;
+#pragma unroll 1
+      for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + a * 256 + (uint32_t)(c0 - tni * tl.W) + ((uint32_t)(qd * 32) << 16), v);
+        tmem_ld_wait();
+        const int lim = c_hi - c0;
+#pragma unroll
+        for (int k4 = 0; k4 < 32; k4 += 4) {
+          const float4 rn4 = *reinterpret_cast<const float4 *>(rn_col + (c0 - c_lo) + k4);
+          const float rnj[4] = {rn4.x, rn4.y, rn4.z, rn4.w};
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const float c = (__uint_as_float(v[k4 + kk]) * rni) * rnj[kk];
+            if (k4 + kk < lim && c > bc) { bc = c; bi = c0 + k4 + kk; }
+          }
+        }
+      }
+      // the accumulator may be overwritten once all epilogue warps have read it
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.acc_empty[a]);
+      if (row_ok && bc > -3.0f) {
+        const float bd = fminf(fmaxf(1.0f - bc, 0.0f), 2.0f);
+        const unsigned long long pk = ((unsigned long long)__float_as_uint(bd) << 32) | (unsigned)bi;
+        unsigned long long *best = &im.best[(kept_rows & 1) ? im.kept_idx[row] : row];
+        if (need > 0) seen |= atomicMin(best, pk);   // the labels wait for the value: the minimum is then in place
+        else atomicMin(best, pk);
+      }
       ++tcount;
-      if (MODE == MODE_ASSIGN && need > 0 && ++npend == kPend) flush_labels();
+      if (need > 0 && ++npend == kPend) flush_labels();
     }
-    if (MODE == MODE_ASSIGN && need > 0 && ok && npend > 0) flush_labels();
+    if (need > 0 && ok && npend > 0) flush_labels();
     if (!ok) atomicExch(&sh.abort, 1);
-    if (MODE == MODE_GRAM && band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
-    if (MODE == MODE_SPREAD) {
-      // distances are clamped to [0, 2]: their bit patterns order like unsigned integers
-      const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
-      if (lane == 0 && w) atomicMax(reinterpret_cast<unsigned *>(&im.cnt[kCntSpread]), w);
-    }
   }
 
   tc_fence_before();
@@ -724,14 +928,14 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
           const int n = min(SLABS, nslab - ks);
           if (!mbar_wait(&sh.full[s], (it / PSTAGES) & 1)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(ring + (size_t)s * PSTAGE_BYTES), b_addr = a_addr + SLABS * A_BYTES;
+          const uint32_t a_addr = smem_u32(ring + (size_t)s * PSTAGE_BYTES);
+          const uint64_t da = smem_desc(a_addr), db = smem_desc(a_addr + SLABS * A_BYTES);
 #pragma unroll
           for (int h = 0; h < SLABS; ++h) {
             if (h < n) {
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k)
-                umma_bf16_pair(d_tmem, smem_desc(a_addr + h * A_BYTES + k * 32), smem_desc(b_addr + h * A_BYTES + k * 32), idesc,
-                               (ks | h | k) != 0);
+                umma_bf16_pair(d_tmem, desc_at(da, h * A_BYTES + k * 32), desc_at(db, h * A_BYTES + k * 32), idesc, (ks | h | k) != 0);
             }
           }
           umma_commit_pair(&sh.empty[s]);          // frees the stage in both CTAs once these MMAs have read it
@@ -755,7 +959,6 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
     bool ok = true;
     float mx = 0.f;                                 // largest distance of the current image (layer)
     int b = 0, b_mx = 0;
-    unsigned long long unused_seen = 0ull;
     auto flush_mx = [&](int bb) {
       const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
       if (lane == 0 && w) atomicMax(reinterpret_cast<unsigned *>(&bt.img[bb].cnt[kCntSpread]), w);
@@ -774,7 +977,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
       const uint32_t rel = map_to_rank(smem_u32(&sh.acc_empty[a]), 0);
       int band = 0;
       ok = epi_tile<MODE, PC::COLS>(im, kept_rows, R, cbase, skip, nrows, ncols, taddr, &sh.acc_full[a], (tcount / PNACC) & 1,
-                                    rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive_remote(rel); }, unused_seen);
+                                    rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive_remote(rel); });
       if (MODE == MODE_GRAM && band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
       if (!ok) break;
       ++tcount;
@@ -800,10 +1003,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-bool encode_rows(const DeviceCfg &cfg, CUtensorMap *map, const void *base, long long rows, long long ld_elems, int d_k) {
+bool encode_rows(const DeviceCfg &cfg, CUtensorMap *map, const void *base, long long rows, long long ld_elems, int d_k, int box_rows = BM) {
   const cuuint64_t dims[2] = {(cuuint64_t)d_k, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld_elems * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)BM};
+  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return reinterpret_cast<EncodeTiledFn>(cfg.encode_tiled)(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -866,8 +1069,7 @@ cudaError_t umma_configure(DeviceCfg *cfg) {
   e = cudaFuncSetAttribute(k_tiles_umma<MODE_SPREAD, kWideBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)TileCfg<kWideBN>::SMEM);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_tiles_umma<MODE_ASSIGN, kWideBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)TileCfg<kWideBN>::SMEM);
+  e = cudaFuncSetAttribute(k_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, kAsnSmem);
   if (e != cudaSuccess) return e;
   e = pair_configure<MODE_ASSIGN, 8>(cfg->pair_assign);
   if (e != cudaSuccess) return e;
@@ -901,7 +1103,7 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
   }
   const long long nb = (maxN + BM - 1) / BM;
   dim3 grid(umma_grid_x(nb * (nb + 1) / 2, bt.B, cfg.sm_count), bt.B);
-  return launch_k(k_tiles_umma<MODE_GRAM, kGramBN>, grid, dim3(THREADS), TileCfg<kGramBN>::SMEM, st, true, bt, tm, 0);
+  return launch_k(k_tiles_umma<MODE_GRAM, kGramBN>, grid, dim3(THREADS), TileCfg<kGramBN>::SMEM, st, true, bt, tm);
 }
 
 bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
@@ -914,21 +1116,26 @@ bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
 // (all-token rows, no labels)
 cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const DeviceCfg &cfg, cudaStream_t st, bool labels,
                                bool pairs) {
-  TmapSet tm;
-  for (int b = 0; b < bt.B; ++b) {
-    const ImgDesc &im = bt.img[b];
-    if (kept_rows) {
-      if (!encode_rows(cfg, &tm.a[b], im.Kp, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
-    } else if (!encode_rows(cfg, &tm.a[b], im.Kc, im.N, im.ldKc, bt.d_k)) return cudaErrorInvalidValue;
-    if (!encode_rows(cfg, &tm.b[b], im.Kcen, im.Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
-  }
+  const auto rows_map = [&](const ImgDesc &im, CUtensorMap *m) {
+    return kept_rows ? encode_rows(cfg, m, im.Kp, im.Np, bt.d_k, bt.d_k) : encode_rows(cfg, m, im.Kc, im.N, im.ldKc, bt.d_k);
+  };
   if (pairs && !kept_rows && cfg.pair_assign) {
+    TmapSet tm;
+    for (int b = 0; b < bt.B; ++b)
+      if (!rows_map(bt.img[b], &tm.a[b]) || !encode_rows(cfg, &tm.b[b], bt.img[b].Kcen, bt.img[b].Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
     const long long pt = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
     return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, 0, cfg, st);
   }
-  const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kWideBN - 1) / kWideBN);
+  AssignMaps tm;
+  for (int b = 0; b < bt.B; ++b) {
+    const ImgDesc &im = bt.img[b];
+    if (!rows_map(im, &tm.a[b]) || !encode_rows(cfg, &tm.b[b], im.Kcen, im.Np, bt.d_k, bt.d_k) ||
+        !encode_rows(cfg, &tm.b32[b], im.Kcen, im.Np, bt.d_k, bt.d_k, 32))
+      return cudaErrorInvalidValue;
+  }
+  const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kAsnLeastCols - 1) / kAsnLeastCols);
   dim3 grid(umma_grid_x(tiles, bt.B, cfg.sm_count), bt.B);
-  return launch_k(k_tiles_umma<MODE_ASSIGN, kWideBN>, grid, dim3(THREADS), TileCfg<kWideBN>::SMEM, st, true, bt, tm, (kept_rows ? 1 : 0) | (labels && !kept_rows ? 2 : 0));
+  return launch_k(k_assign, grid, dim3(THREADS), kAsnSmem, st, true, bt, tm, (kept_rows ? 1 : 0) | (labels && !kept_rows ? 2 : 0));
 }
 
 // every layer of the batch is one "image": rows and columns are all N keys of K_clu
@@ -945,7 +1152,7 @@ cudaError_t launch_spread_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, 
   }
   const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kWideBN - 1) / kWideBN);
   dim3 grid(umma_grid_x(tiles, bt.B, cfg.sm_count), bt.B);
-  return launch_k(k_tiles_umma<MODE_SPREAD, kWideBN>, grid, dim3(THREADS), TileCfg<kWideBN>::SMEM, st, true, bt, tm, 0);
+  return launch_k(k_tiles_umma<MODE_SPREAD, kWideBN>, grid, dim3(THREADS), TileCfg<kWideBN>::SMEM, st, true, bt, tm);
 }
 
 }  // namespace pact

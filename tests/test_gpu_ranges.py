@@ -411,3 +411,27 @@ def test_merged_rows_of_any_bf16_value():
     got = im.H_out[:T + 17]
     assert torch.equal(torch.isnan(got), torch.isnan(want))
     assert torch.equal(torch.nan_to_num(got, nan=0.0).view(torch.int32), torch.nan_to_num(want, nan=0.0).view(torch.int32))
+
+
+@pytest.mark.parametrize("C", [1, 31, 33, 257, 500, 513, 1030])
+@pytest.mark.parametrize("N,n_kvh,d_h", [(1100, 1, 64), (3000, 3, 64), (7290, 4, 128), (19100, 2, 64)])
+def test_nearest_centres_in_tiles(N, n_kvh, d_h, C):
+    """Rows x centres at the edges of its tiles: one round of equal tiles (up to 512 centres wide) and rounds of 256, one K-slab per stage and two."""
+    from paper_2504_08966_b200 import binding as pb
+    g = torch.Generator(device="cuda").manual_seed(N + C)
+    K = torch.randn(N, n_kvh * d_h, device="cuda", generator=g).to(torch.bfloat16)
+    i32 = lambda x: torch.as_tensor(x, dtype=torch.int32, device="cuda")   # noqa: E731
+    cen = torch.randperm(N, device="cuda", generator=g)[:C].sort().values
+    rows = torch.ones(N, dtype=torch.bool, device="cuda")
+    rows[cen] = False
+    pruned = rows.nonzero().flatten()
+    label, r = torch.full((N,), -7, dtype=torch.int32, device="cuda"), i32([0])
+    ctx = pb.Context(256, n_kvh, n_kvh, d_h)
+    ctx.pact_reincorporate(K, i32(pruned), i32([pruned.numel()]), i32(cen), i32([C]), pb.make_params(d_c=2.0, alpha=1.5), label, r)
+    assert int(r) == pruned.numel() and bool((label[cen] == -7).all())
+    Kd = torch.nn.functional.normalize(K.double(), dim=1)
+    dist = 1.0 - Kd[pruned] @ Kd[cen].T
+    got = label[pruned].long()
+    assert int(got.min()) >= 0 and int(got.max()) < C
+    # a dot product of d_k terms in fp32 is good to about 1e-6 of the norms
+    assert float((dist.gather(1, got[:, None])[:, 0] - dist.min(1).values).max()) < 2e-6
