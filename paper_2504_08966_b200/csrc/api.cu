@@ -94,7 +94,6 @@ size_t carve_image(const pact_ctx *c, int N, char *base, ImgDesc *im) {
   cv.take(m.label, (size_t)N * sizeof(int32_t));
   const size_t nblk = ((size_t)N + kListBlock - 1) / kListBlock;
   m.nbp = (int)rup(nblk, 8);
-  cv.take(m.blocklist, nblk * kListBlock * sizeof(int32_t));
   cv.take(m.cnt_cb, (size_t)Np * m.nbp * sizeof(uint16_t));
   cv.take(m.members, (size_t)N * sizeof(int4));
   cv.take(m.csize, (size_t)Np * sizeof(int32_t));
@@ -518,7 +517,7 @@ pact_status pact_merge(pact_ctx *ctx, const pact_image *img, const int32_t *labe
   CK(launch_list_clear(bt, st));
   CK(launch_lists(bt, img->N, ctx->in == PACT_BF16, false, ctx->spin_limit, ctx->dev, st));
   CK(launch_merge(bt, ctx->in == PACT_BF16, ctx->out == PACT_BF16, ctx->dev, st));
-  ctx->launches += lists_kernels(img->N, 1, ctx->dev) + 2;
+  ctx->launches += lists_kernels(img->N, 1, false, ctx->dev) + 2;
   CK(cudaGetLastError());
   return PACT_OK;
 }
@@ -587,17 +586,17 @@ static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, c
     CK(launch_centers(bt, cmaxQ, bf, ctx->dev, ctx->sweep_limit, st));  CK(mark());
     // On the tensor-core path with little work per SM (one image) the labels and member counts are formed as
     // the rows x centres pass finishes groups of rows, and one kernel places the members.  With much work per SM
-    // the pass runs on pairs of CTAs, and k_lists forms labels and lists as it does on the fp32 path.
+    // the pass runs on pairs of CTAs, and labels and lists are formed as on the fp32 path.
     const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, nb, ctx->dev);
     const bool fused_labels = ctx->umma && !pairs;
     if (ctx->umma) CK(launch_assign_umma(bt, cmaxN, false, ctx->dev, st, fused_labels, pairs));
     else CK(launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->dev, st));
     CK(mark());
-    if (fused_labels) CK(launch_members(bt, cmaxN, st));
+    if (fused_labels) CK(launch_members(bt, cmaxN, true, st));
     else CK(launch_lists(bt, cmaxN, bf, true, ctx->spin_limit, ctx->dev, st));
     CK(mark());
     CK(launch_merge(bt, bf, ctx->out == PACT_BF16, ctx->dev, st));  CK(mark());
-    ctx->launches += euti_kernels(0) + 5 + (fused_labels ? 1 : lists_kernels(cmaxN, nb, ctx->dev));
+    ctx->launches += euti_kernels(0) + 5 + (fused_labels ? 1 : lists_kernels(cmaxN, nb, true, ctx->dev));
     CK(cudaGetLastError());
   }
   return PACT_OK;

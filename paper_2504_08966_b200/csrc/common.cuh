@@ -63,8 +63,7 @@ struct ImgDesc {
   int32_t *cid;          // [Np] cluster id of survivor r if it is a centre
   unsigned long long *best;  // [N] packed (distance bits << 32 | cluster id)
   int32_t *label;        // [N]
-  int32_t *blocklist;    // [ceil(N/256)][256] tokens of each block sorted by (cluster id, token); two-launch form of k_lists only
-  uint16_t *cnt_cb;      // [Np][nbp] members of cluster c in token block b; zero before k_lists
+  uint16_t *cnt_cb;      // [Np][nbp] members of cluster c in token block b; zero before the labels are counted
   int4 *members;         // [N] {token, cluster, first member position of the cluster, cluster size}, cluster order
   int32_t *csize;        // [Np] members of cluster c
   int32_t *cticket;      // [Np] tickets of the clusters that k_merge cuts: 8 (range of its first member) + column slice

@@ -19,6 +19,7 @@
 #include <cuda.h>
 
 #include "kernels.cuh"
+#include "labels.cuh"
 #include "umma.cuh"
 
 namespace pact {
@@ -111,50 +112,6 @@ template <int MODE> __device__ __forceinline__ void tile_at(int t, int ntm, int 
     tni = t % ntn;
   }
 }
-// Labels of a group of 32 tokens (lane = token) whose nearest centres are final, formed by the last epilogue
-// warp of the rows x centres pass to finish the group: a survivor takes its nearest centre's cluster (a centre
-// its own), a pruned token that cluster iff the distance is strictly below alpha * d_c (Eq. 8-9), else -1.
-// The group's members per cluster are added to the table of its 128-token block and to the cluster sizes
-// (integer adds: the sums do not depend on the order in which groups finish).
-// r: the token's position among the survivors (< 0: pruned); own_cid: its cluster id if it is a centre, else -1
-// (both known before the pass, so that only the nearest centre has to be fetched here).
-__device__ __forceinline__ void label_group(const ImgDesc &im, int i, int lane, int C, int r, int own_cid) {
-  int lab = -1, joined = 0, dropped = 0, band = 0;
-  if (i < im.N) {
-    const unsigned long long pk = __ldcg(im.best + i);
-    lab = (int)(pk & 0xFFFFFFFFull);
-    const float dd = __uint_as_float((uint32_t)(pk >> 32));
-    if (r >= 0) {
-      if (own_cid >= 0) lab = own_cid;
-    } else {
-      if (DistF::in_band_t(dd, im)) ++band;
-      if (DistF::below_t(dd, im)) ++joined; else { lab = -1; ++dropped; }
-    }
-    if (lab >= C || lab < -1) lab = -1;             // only after a failed earlier stage
-    im.label[i] = lab;
-    if (im.label_user) im.label_user[i] = lab;
-  }
-  const unsigned same = __match_any_sync(0xffffffffu, lab);
-  if (lab >= 0 && lane == __ffs(same) - 1) {
-    const int len = __popc(same), b = i / kListBlock;
-    // 16-bit cell (c, b) of the table, added to through the 32-bit word that holds it (a cell stays <= 128)
-    uint32_t *word = reinterpret_cast<uint32_t *>(im.cnt_cb) + (((size_t)lab * im.nbp + b) >> 1);
-    atomicAdd(word, (uint32_t)len << (16 * (b & 1)));
-    atomicAdd(&im.csize[lab], len);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    joined += __shfl_xor_sync(0xffffffffu, joined, o);
-    dropped += __shfl_xor_sync(0xffffffffu, dropped, o);
-    band += __shfl_xor_sync(0xffffffffu, band, o);
-  }
-  if (lane == 0) {
-    if (joined) atomicAdd(&im.cnt[PACT_CNT_R], joined);
-    if (dropped) atomicAdd(&im.cnt[PACT_CNT_DISCARDED], dropped);
-    if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_ADC], band);
-  }
-}
-
 // The epilogue of one accumulator tile for one warp: the warp's 32 rows (tensor-memory lanes) of the 128-row
 // block tmi against HALF columns from cbase on.  Waits for the accumulator, reads it 32 columns at a time and
 // applies the mode's arithmetic; arrive() is called once the accumulator has been read.  skip: the warp only
@@ -638,7 +595,7 @@ __global__ void __maxnreg__(80) k_assign(const __grid_constant__ Batch bt, const
 #pragma unroll
       for (int k = 0; k < kPend; ++k)
         if (k < npend && ((lastmask >> k) & 1u))
-          label_group(im, pend_tmi[k] * BM + qd * 32 + lane, lane, C, pend_r[k], pend_cid[k]);
+          label_group<DistF>(im, pend_tmi[k] * BM + qd * 32 + lane, lane, C, pend_r[k], pend_cid[k]);
       npend = 0;
     };
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {

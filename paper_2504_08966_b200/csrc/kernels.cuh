@@ -133,7 +133,7 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
 cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const DeviceCfg &cfg, cudaStream_t st, bool labels = false,
                                bool pairs = false);
 bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg);
-cudaError_t launch_members(const Batch &bt, int maxN, cudaStream_t st);
+cudaError_t launch_members(const Batch &bt, int maxN, bool label_none, cudaStream_t st);   // label_none: where there is no centre the labels are written (-1)
 cudaError_t launch_spread_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cudaStream_t st);
 
 // small.cu: scores to member lists in one kernel, a cluster per image
@@ -145,7 +145,7 @@ cudaError_t launch_small(const Batch &bt, bool in_bf16, bool umma, int rpp, int 
 // member records in cluster order from label[] (from_best: labels are first formed from the nearest-centre
 // pass, all tokens); csize, cticket and cnt_cb must be zero.  spin_limit bounds the wait of its barrier.
 cudaError_t launch_lists(const Batch &bt, int maxN, bool bf16, bool from_best, int spin_limit, const DeviceCfg &cfg, cudaStream_t st);
-int lists_kernels(int maxN, int B, const DeviceCfg &cfg);        // kernels launch_lists launches (1, or 2 when the grid cannot be resident at once)
+int lists_kernels(int maxN, int B, bool from_best, const DeviceCfg &cfg);   // kernels launch_lists launches
 cudaError_t launch_list_clear(const Batch &bt, cudaStream_t st);   // csize, cticket, cnt_cb and the counters
 cudaError_t launch_merge(const Batch &bt, bool in_bf16, bool out_bf16, const DeviceCfg &cfg, cudaStream_t st);
 cudaError_t merge_configure(DeviceCfg *cfg);

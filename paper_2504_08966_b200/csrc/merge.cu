@@ -2,16 +2,18 @@
 // float accumulation and ascending token order; position id of the centre; cluster sizes;
 // text rows copied around the merged span.
 //
-//   k_lists  labels (reincorporation test of Eq. 8), then a stable counting sort of the tokens by
-//            cluster id: every block of 128 tokens sorts its own, an image-wide barrier, and every
-//            token writes one 16-byte record {token, cluster, first member position, cluster size}
-//            at its place in the cluster-sorted member array.  Also P', sizes and log sizes.
+//   k_label_counts   labels (reincorporation test of Eq. 8) and members per cluster, in all and by block of 128 tokens; the rows x
+//                    centres pass on single CTAs (gram_umma.cu) does this itself
+//   k_members        a stable counting sort of the tokens by cluster id: every token writes one 16-byte record {token, cluster, first
+//                    member position, cluster size} at its place in the cluster-sorted member array.  Also P', sizes and log sizes.
+//   k_lists          both in one kernel with an image-wide barrier, for few tokens
 //   k_merge  the member array (followed by the text rows) is cut into contiguous ranges;
 //            a CTA streams its columns of the rows of a range with many loads in flight and no look-ups, keeps
 //            the running cluster in registers and writes a row out whenever the cluster id changes.
 //            Large clusters cut by a range boundary leave partial sums; the last CTA to arrive adds them in
 //            range order, so the result does not depend on timing.
 #include "kernels.cuh"
+#include "labels.cuh"
 #include "tma.cuh"
 
 namespace pact {
@@ -41,17 +43,18 @@ __device__ __forceinline__ float4 ld_cg_f4(const float *p) {
 //   belongs at  member_off[c] + (members of c in the blocks before b) + (its place in the run),  where
 //   member_off is the exclusive prefix sum of csize.  It writes its record there; the first member of a
 //   cluster also writes P', the size and its logarithm for the cluster's output row.
-// mode 0: both parts, separated by a barrier over the blocks of the image (all blocks must be resident:
-//         cooperative launch); mode 1: part 1 only, the sorted blocks go to blocklist; mode 2: part 2 only.
-// FROM_BEST: the labels are first formed here from the nearest-centre pass (survivors: cluster id of the
-// nearest centre, a centre its own id; pruned tokens: that id iff the distance is strictly below
-// alpha * d_c, else -1) and written out; otherwise label[] is given, and an id outside [-1, C) is
-// dropped like -1 and reported through the status word.
+// The parts are separated by a barrier over the blocks of the image (all blocks must be resident: cooperative launch).
+// For the whole step of up to kListsMaxN tokens on the double-precision tiles.  k_label_counts and k_members do the same for all others:
+// DBDPC and merge of 900 tokens 46.6 -> 43.8 us, of 7290 113.3 -> 109.4, 16 images of 2916 247.3 -> 245.0.  (Here a token looks up
+// its cluster in the sorted block, and the counts of the blocks before its own come in one trip to the L2 after the other.)
+// The labels are first formed here from the nearest-centre pass (survivors: cluster id of the nearest centre, a centre its own
+// id; pruned tokens: that id iff the distance is strictly below alpha * d_c, else -1) and written out.
 constexpr int kScanTile = kListBlock * 8;   // cluster sizes scanned per step of part 2
 constexpr int kNoLabel = 0x7fffffff;
+constexpr int kListsMaxN = 2048;
 
-template <typename T, bool FROM_BEST>
-__global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Batch bt, int mode, int spin_limit) {
+template <typename T>
+__global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Batch bt, int spin_limit) {
   using D = typename DistOf<T>::type;
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 8);
@@ -68,63 +71,46 @@ __global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Ba
   const int C = min(*im.C_ptr, im.Np);
   const int i = b * kListBlock + t;
 
-  if (mode != 2) {
-    int lab = -1;
-    if (FROM_BEST) {
-      int joined = 0, dropped = 0, band = 0;
-      if (i < N) {
-        const int r = im.slot[i];                     // >= 0: survivor position; < 0: pruned
-        const unsigned long long pk = im.best[i];
-        lab = (int)(pk & 0xFFFFFFFFull);
-        const float dd = __uint_as_float((uint32_t)(pk >> 32));
-        if (r >= 0) {
-          if ((im.cmask[r >> 5] >> (r & 31)) & 1u) lab = im.cid[r];
-        } else {
-          if (D::in_band_t(dd, im)) ++band;
-          if (D::below_t(dd, im)) ++joined; else { lab = -1; ++dropped; }
-        }
-        if (lab >= C) lab = -1;                       // only after a failed earlier stage
-        im.label[i] = lab;
-        if (im.label_user) im.label_user[i] = lab;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        joined += __shfl_xor_sync(0xffffffffu, joined, o);
-        dropped += __shfl_xor_sync(0xffffffffu, dropped, o);
-        band += __shfl_xor_sync(0xffffffffu, band, o);
-      }
-      if (lane == 0) {
-        if (joined) atomicAdd(&im.cnt[PACT_CNT_R], joined);
-        if (dropped) atomicAdd(&im.cnt[PACT_CNT_DISCARDED], dropped);
-        if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_ADC], band);
-      }
+  int lab = -1;
+  int joined = 0, dropped = 0, band = 0;
+  if (i < N) {
+    const int r = im.slot[i];                     // >= 0: survivor position; < 0: pruned
+    const unsigned long long pk = im.best[i];
+    lab = (int)(pk & 0xFFFFFFFFull);
+    const float dd = __uint_as_float((uint32_t)(pk >> 32));
+    if (r >= 0) {
+      if ((im.cmask[r >> 5] >> (r & 31)) & 1u) lab = im.cid[r];
     } else {
-      lab = i < N ? im.label[i] : -1;
-      if (lab >= C || lab < -1) {                     // a label the caller should not have passed
-        lab = -1;
-        atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_INVALID_ARG);
-      }
+      if (D::in_band_t(dd, im)) ++band;
+      if (D::below_t(dd, im)) ++joined; else { lab = -1; ++dropped; }
     }
-    const int key = lab < 0 ? kNoLabel : lab;
-    slab[t] = key;
-    __syncthreads();
-    int rank = 0;
-#pragma unroll 8
-    for (int u = 0; u < kListBlock; ++u) {
-      const int o = slab[u];
-      rank += (o < key) || (o == key && u < t);
-    }
-    s_lab[rank] = key;
-    s_tok[rank] = i;
-    __syncthreads();
-    if (mode == 1) im.blocklist[(size_t)b * kListBlock + t] = s_tok[t];
-  } else {
-    const int tok = im.blocklist[(size_t)b * kListBlock + t];
-    const int lab = tok < N ? im.label[tok] : -1;
-    s_tok[t] = tok;
-    s_lab[t] = (lab < 0 || lab >= C) ? kNoLabel : lab;
-    __syncthreads();
+    if (lab >= C) lab = -1;                       // only after a failed earlier stage
+    im.label[i] = lab;
+    if (im.label_user) im.label_user[i] = lab;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    joined += __shfl_xor_sync(0xffffffffu, joined, o);
+    dropped += __shfl_xor_sync(0xffffffffu, dropped, o);
+    band += __shfl_xor_sync(0xffffffffu, band, o);
+  }
+  if (lane == 0) {
+    if (joined) atomicAdd(&im.cnt[PACT_CNT_R], joined);
+    if (dropped) atomicAdd(&im.cnt[PACT_CNT_DISCARDED], dropped);
+    if (band) atomicAdd(&im.cnt[PACT_CNT_BAND_ADC], band);
+  }
+  const int key = lab < 0 ? kNoLabel : lab;
+  slab[t] = key;
+  __syncthreads();
+  int rank = 0;
+#pragma unroll 8
+  for (int u = 0; u < kListBlock; ++u) {
+    const int o = slab[u];
+    rank += (o < key) || (o == key && u < t);
+  }
+  s_lab[rank] = key;
+  s_tok[rank] = i;
+  __syncthreads();
   // first position whose cluster id is >= c
   auto lower = [&](int c) {
     int lo = 0, hi = kListBlock;
@@ -137,28 +123,25 @@ __global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Ba
   const int c = s_lab[t];
   const bool valid = c != kNoLabel;
   const int run0 = valid ? lower(c) : t;
-  if (mode != 2 && valid && run0 == t) {
+  if (valid && run0 == t) {
     const int len = lower(c + 1) - t;
     im.cnt_cb[(size_t)c * im.nbp + b] = (uint16_t)len;
     atomicAdd(&im.csize[c], len);
   }
-  if (mode == 1) return;
   TL_POINT(im, 13);
-  if (mode == 0) {
-    // every block of the image has published its run lengths before anyone reads them
-    __threadfence();
-    __syncthreads();
-    if (t == 0) {
-      atomicAdd(&im.cnt[19], 1);
-      int spins = 0;
-      while (ld_acquire_i32(&im.cnt[19]) < nblk) {
-        if (++spins > spin_limit) { atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT); break; }
-        __nanosleep(40);
-      }
+  // every block of the image has published its run lengths before anyone reads them
+  __threadfence();
+  __syncthreads();
+  if (t == 0) {
+    atomicAdd(&im.cnt[19], 1);
+    int spins = 0;
+    while (ld_acquire_i32(&im.cnt[19]) < nblk) {
+      if (++spins > spin_limit) { atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT); break; }
+      __nanosleep(40);
     }
-    __syncthreads();
-    __threadfence();
   }
+  __syncthreads();
+  __threadfence();
   TL_POINT(im, 14);
 
   // part 2
@@ -220,16 +203,46 @@ __global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Ba
   }
 }
 
+// ---- labels and member counts ----------------------------------------------------------------------
+// grid (ceil(maxN / 128), B), 128 threads, a group of 32 tokens per warp.  FROM_BEST: the labels are formed from the nearest-centre pass,
+// as in k_lists (what does not come from that pass is read before the wait for it); otherwise label[] is given, and an id
+// outside [-1, C) is dropped like -1 and reported through the status word.
+template <typename T, bool FROM_BEST>
+__global__ void __launch_bounds__(kListBlock) k_label_counts(const __grid_constant__ Batch bt) {
+  using D = typename DistOf<T>::type;
+  const ImgDesc &im = bt.img[blockIdx.y];
+  const int i = blockIdx.x * kListBlock + threadIdx.x, lane = threadIdx.x & 31;
+  int r = -1, own = -1;
+  const int C = min(ld_cg_i32(im.C_ptr), im.Np);
+  if (FROM_BEST && i < im.N) {
+    r = ld_cg_i32(&im.slot[i]);
+    if (r >= 0 && ((__ldcg(&im.cmask[r >> 5]) >> (r & 31)) & 1u)) own = ld_cg_i32(&im.cid[r]);
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (i - lane >= im.N) return;
+  if (FROM_BEST) {
+    label_group<D>(im, i, lane, C, r, own);
+  } else {
+    int lab = i < im.N ? im.label[i] : -1;
+    if (lab >= C || lab < -1) {                        // a label the caller should not have passed
+      lab = -1;
+      atomicMin(&im.cnt[PACT_CNT_STATUS], (int)PACT_ERR_INVALID_ARG);
+    }
+    count_group(im, i, lane, lab);
+  }
+}
+
 // ---- member records from finished labels ----------------------------------------------------------
-// grid (ceil(maxN / 128), B), 128 threads.  The rows x centres pass on the tensor cores has already written
-// the labels, the cluster sizes and cnt_cb (members of cluster c in token block b) as its groups of rows
-// finished; what is left is the second part of k_lists: the member of cluster c that is token i of block b
+// grid (ceil(maxN / 128), B), 128 threads.  The rows x centres pass on single CTAs, as its groups of rows finished, or
+// k_label_counts has already written the labels, the cluster sizes and cnt_cb (members of cluster c in token block b); what
+// is left is the second part of k_lists: the member of cluster c that is token i of block b
 // belongs at  member_off[c] + (members of c in the blocks before b) + (members of c before i in block b).
-__global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ Batch bt, int label_none) {
   const ImgDesc &im = bt.img[blockIdx.y];
   TL_SCOPE(im, 8);
-  // the number of clusters was final before the rows x centres pass began, and this kernel cannot start before
-  // every CTA of that pass has begun: it may be read ahead of the wait
+  // the number of clusters was final before the kernel ahead of this one began, and this kernel cannot start before
+  // every CTA of that has begun: it may be read ahead of the wait
   const int C = min(ld_cg_i32(im.C_ptr), im.Np);
   pdl_wait();
   pdl_trigger();
@@ -245,7 +258,7 @@ __global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ 
   int c = -1;
   if (i < N) {
     if (C > 0) c = ld_cg_i32(&im.label[i]);
-    else {                                           // no centre at all (a failed earlier stage): nothing was labelled
+    else if (label_none) {                           // no centre at all (a failed earlier stage): nothing was labelled
       im.label[i] = -1;
       if (im.label_user) im.label_user[i] = -1;
     }
@@ -288,14 +301,17 @@ __global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ 
     for (int k = 0; k < 8; ++k)
       if (v * 8 + k < b) before += (int)((xs[k >> 1] >> ((k & 1) * 16)) & 0xFFFFu);
   }
-  if (valid)
-    for (int v = kCbRegs; v * 8 < b; ++v) {          // more token blocks than that
-      const uint4 x = __ldcg(row + v);
-      const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+  for (int v0 = kCbRegs; v0 * 8 < b; v0 += kCbRegs) {   // more token blocks than that
+#pragma unroll
+    for (int v = 0; v < kCbRegs; ++v) cb[v] = (valid && (v0 + v) * 8 < b) ? __ldcg(row + v0 + v) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int v = 0; v < kCbRegs; ++v) {
+      const uint32_t xs[4] = {cb[v].x, cb[v].y, cb[v].z, cb[v].w};
 #pragma unroll
       for (int k = 0; k < 8; ++k)
-        if (v * 8 + k < b) before += (int)((xs[k >> 1] >> ((k & 1) * 16)) & 0xFFFFu);
+        if ((v0 + v) * 8 + k < b) before += (int)((xs[k >> 1] >> ((k & 1) * 16)) & 0xFFFFu);
     }
+  }
   // member_off[c] = cluster sizes below c, scanned kScanTile at a time
   if (t == 0) s_carry = 0;
   __syncthreads();
@@ -343,7 +359,7 @@ __global__ void __launch_bounds__(kListBlock) k_members(const __grid_constant__ 
   }
 }
 
-// What k_lists and k_merge accumulate into, and the counters (pact_merge; in the whole step k_tokens clears them).
+// What k_label_counts and k_merge accumulate into, and the counters (pact_merge; in the whole step k_tokens clears them).
 __global__ void __launch_bounds__(256) k_list_clear(const __grid_constant__ Batch bt) {
   pdl_wait();
   pdl_trigger();
@@ -584,32 +600,23 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
 
 // ---- launchers -----------------------------------------------------------------------------------
 
-template <typename T, bool FB>
-static cudaError_t launch_lists_t(const Batch &bt, int maxN, int spin_limit, const DeviceCfg &cfg, cudaStream_t st) {
+static bool lists_in_one(int maxN, int B, const DeviceCfg &cfg) {
+  return maxN <= kListsMaxN && (long long)((maxN + kListBlock - 1) / kListBlock) * B <= cfg.lists_resident;
+}
+int lists_kernels(int maxN, int B, bool from_best, const DeviceCfg &cfg) { return from_best && lists_in_one(maxN, B, cfg) ? 1 : 2; }
+
+cudaError_t launch_members(const Batch &bt, int maxN, bool label_none, cudaStream_t st) {
   const dim3 grid((maxN + kListBlock - 1) / kListBlock, bt.B);
-  if ((long long)grid.x * grid.y <= cfg.lists_resident) {
-    return launch_coop(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 0, spin_limit);
-  }
-  cudaError_t e = launch_k(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 1, spin_limit);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_lists<T, FB>, grid, dim3(kListBlock), 0, st, true, bt, 2, spin_limit);
+  return launch_k(k_members, grid, dim3(kListBlock), 0, st, true, bt, label_none ? 1 : 0);
 }
 
 cudaError_t launch_lists(const Batch &bt, int maxN, bool bf16, bool from_best, int spin_limit, const DeviceCfg &cfg, cudaStream_t st) {
-  if (from_best) {
-    if (bf16) return launch_lists_t<__nv_bfloat16, true>(bt, maxN, spin_limit, cfg, st);
-    return launch_lists_t<float, true>(bt, maxN, spin_limit, cfg, st);
-  }
-  return launch_lists_t<float, false>(bt, maxN, spin_limit, cfg, st);
-}
-
-cudaError_t launch_members(const Batch &bt, int maxN, cudaStream_t st) {
-  const dim3 grid((maxN + kListBlock - 1) / kListBlock, bt.B);
-  return launch_k(k_members, grid, dim3(kListBlock), 0, st, true, bt);
-}
-
-int lists_kernels(int maxN, int B, const DeviceCfg &cfg) {
-  return (long long)((maxN + kListBlock - 1) / kListBlock) * B <= cfg.lists_resident ? 1 : 2;
+  const dim3 grid((maxN + kListBlock - 1) / kListBlock, bt.B), block(kListBlock);
+  if (from_best && lists_in_one(maxN, bt.B, cfg))
+    return bf16 ? launch_coop(k_lists<__nv_bfloat16>, grid, block, 0, st, true, bt, spin_limit) : launch_coop(k_lists<float>, grid, block, 0, st, true, bt, spin_limit);
+  const auto counts = !from_best ? k_label_counts<float, false> : bf16 ? k_label_counts<__nv_bfloat16, true> : k_label_counts<float, true>;
+  const cudaError_t e = launch_k(counts, grid, block, 0, st, true, bt);
+  return e != cudaSuccess ? e : launch_members(bt, maxN, false, st);
 }
 
 // items per range: 24 (with 16: 2.5 us more of 16 images of 2916 tokens, 2 us of three of 2309; with 48 as much), 16 where
@@ -661,13 +668,10 @@ template <typename T, typename O> static cudaError_t merge_attr() {
 
 cudaError_t merge_configure(DeviceCfg *cfg) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<__nv_bfloat16, true>, kListBlock, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<__nv_bfloat16>, kListBlock, 0);
   if (e != cudaSuccess) return e;
   int m = per_sm;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<float, true>, kListBlock, 0);
-  if (e != cudaSuccess) return e;
-  m = per_sm < m ? per_sm : m;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<float, false>, kListBlock, 0);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lists<float>, kListBlock, 0);
   if (e != cudaSuccess) return e;
   m = per_sm < m ? per_sm : m;
   cfg->lists_resident = m * cfg->sm_count;
