@@ -49,7 +49,7 @@ struct F64Group {
 
 template <typename T> struct SmallShared {
   using rn_t = typename DistOf<T>::type::rn_t;
-  uint32_t key[kSmallMaxN];                            // sort keys of all tokens
+  __align__(16) uint32_t key[kSmallMaxN];              // sort keys of all tokens
   rn_t rn[kSmallMaxN];                                 // inverse norms of all clustering keys
   float rn_col[kSmWarps][32];
   short lab[kSmallMaxN];                               // labels of all tokens
@@ -314,7 +314,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
     const int li = t / tpt, part = t % tpt;
     const uint32_t mine = li < nown ? sh.key[own0 + li] : 0u;
     int cnt = 0;
-    for (int j = part; j < N; j += tpt) cnt += sh.key[j] <= mine;
+    const uint4 *k4 = reinterpret_cast<const uint4 *>(sh.key);
+#pragma unroll 2
+    for (int j = part; j < N >> 2; j += tpt) {
+      const uint4 k = k4[j];
+      cnt += (k.x <= mine) + (k.y <= mine) + (k.z <= mine) + (k.w <= mine);
+    }
+    if (part < (N & 3)) cnt += sh.key[(N & ~3) + part] <= mine;   // (at least eight threads per token)
     for (int o = tpt >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     if (li < nown) {
       const unsigned char kp = cnt > im.m_target;
