@@ -435,3 +435,9 @@ def test_nearest_centres_in_tiles(N, n_kvh, d_h, C):
     assert int(got.min()) >= 0 and int(got.max()) < C
     # a dot product of d_k terms in fp32 is good to about 1e-6 of the norms
     assert float((dist.gather(1, got[:, None])[:, 0] - dist.min(1).values).max()) < 2e-6
+
+
+@pytest.mark.parametrize("N,C,d", [(9, 2, 3584), (41, 3, 3584), (57, 2, 896), (95, 1, 1024), (97, 30, 896), (600, 11, 3584), (881, 25, 896), (1200, 36, 3584)])
+def test_merge_ranges_of_few_rows(N, C, d):
+    """Ranges of eight and twelve items, clusters that end up to 24 items past theirs and clusters cut at every boundary."""
+    test_merge_ranges(N, C, 5, d, torch.bfloat16)
