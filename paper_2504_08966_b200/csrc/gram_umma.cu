@@ -418,12 +418,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
 // kept_rows, bit 0: rows are the gathered survivors (Kp, rnk) instead of all tokens; bit 1: the labels, cluster sizes and
 // per-block member counts are formed here as groups of rows finish.
 //
+// For the stage calls and the whole step of images of up to 1024 tokens; the whole step of larger ones takes pairs of CTAs.
 // Where the row blocks are few enough that every CTA needs one tile only, the centres are shared out among as many columns of tiles
 // as give every CTA one, all of the same width: up to 512 columns, i.e. the whole tensor memory, in two instructions per
-// step.  With columns of 256 whatever C is, one image of 7290 tokens and 535 centres had 171 tiles for 148 CTAs, and the pass
-// ended with the 23 second ones: 14.0 us from the centres to the labels, 12.3 now (call 93.2 -> 91.6).  More row blocks: tiles of 256 in
-// rounds, two accumulators, the (usually narrow) last column last.  Bound by latency: of the 12 us 2.0 pass until the first operands are
-// there, 3.7 until the last, 1.1 until the accumulator is complete, 2.0 in the epilogue, 1.1 for the tickets.
+// step (DBDPC and merge of 2977 keys 61.5 -> 60.0 us against columns of 256 whatever C is; where some CTAs had a second, narrow tile,
+// 7290 rows and 535 centres, the pass ended 1.7 us earlier).  More row blocks: tiles of 256 in rounds, two accumulators, the (usually
+// narrow) last column last.  Bound by latency: of 12 us with 7290 rows 2.0 pass until the first operands are there, 3.7 until the last,
+// 1.1 until the accumulator is complete, 2.0 in the epilogue, 1.1 for the tickets.
 constexpr int kAsnRing = 192 * 1024;                 // (with more of it the next kernels' CTAs find no room beside this one and crowd on a few SMs)
 constexpr int kAsnSmem = 1024 + kAsnRing;
 constexpr int kAsnMostCols = TMEM_COLS, kAsnLeastCols = 64;
@@ -681,8 +682,8 @@ __global__ void __maxnreg__(80) k_assign(const __grid_constant__ Batch bt, const
 // columns (half of operand B), CTA 0 issues tcgen05.mma.cta_group::2 for both, and each CTA finds its
 // 128 x 256 part of the product in its own tensor memory.  A CTA therefore fetches half as many operand
 // bytes from the L2 per output element as it does alone.  The largest-distance pass always runs this way, the
-// all-pairs pass when an SM has six or more 128 x 128 blocks to do and the rows x centres pass when it has two or
-// more 128-row blocks (with fewer, the coarser tiles cost a round).
+// all-pairs pass when an SM has six or more 128 x 128 blocks to do (with fewer, the coarser tiles cost a round) and the rows x
+// centres pass of the whole step from 1025 tokens on.
 //   full[s]      in CTA 0: both CTAs' copies of stage s report their bytes there
 //   empty[s]     in each CTA: tcgen05.commit (multicast to both CTAs) once the MMAs have read stage s
 //   acc_full[a]  in each CTA: tcgen05.commit (multicast) once accumulator a is complete
@@ -1063,10 +1064,12 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
   return launch_k(k_tiles_umma<MODE_GRAM, kGramBN>, grid, dim3(THREADS), TileCfg<kGramBN>::SMEM, st, true, bt, tm);
 }
 
-bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
-  // with two or more 128-row blocks per SM (batches, long images) pairs of CTAs on 256 x 256 tiles are faster:
-  // the pass is bound by operand bytes from the L2, and a pair fetches two thirds of them
-  return cfg.pair_assign && (long long)((maxN + BM - 1) / BM) * B >= 2LL * cfg.sm_count;
+bool umma_pairs_for_assign(int maxN, const DeviceCfg &cfg) {
+  // In the whole step, from 1025 tokens on, pairs of CTAs on 256 x 256 tiles: a pair fetches two thirds of the operand bytes, and
+  // the labels, formed by a kernel of their own, cost less than the tickets of single CTAs that form them as they go.  One
+  // image of 7290 tokens 91.9 -> 90.0 us, of 3000 64.3 -> 63.7, of 13000 154.9 -> 148.9, five of 2000 98.3 -> 94.5, sixteen of 1030
+  // 118.1 -> 119.8.
+  return cfg.pair_assign && maxN > 1024;
 }
 
 // labels: the single-CTA kernel also forms labels and member counts (all-token rows only); pairs: the pair kernel

@@ -45,13 +45,13 @@ __device__ __forceinline__ float4 ld_cg_f4(const float *p) {
 //   cluster also writes P', the size and its logarithm for the cluster's output row.
 // The parts are separated by a barrier over the blocks of the image (all blocks must be resident: cooperative launch).
 // For the whole step of up to kListsMaxN tokens on the double-precision tiles.  k_label_counts and k_members do the same for all others:
-// DBDPC and merge of 900 tokens 46.6 -> 43.8 us, of 7290 113.3 -> 109.4, 16 images of 2916 247.3 -> 245.0.  (Here a token looks up
+// DBDPC and merge of 900 tokens 46.6 -> 43.8 us, of 7290 113.3 -> 109.4, one fp32 image of 1100 57.7 -> 53.7.  (Here a token looks up
 // its cluster in the sorted block, and the counts of the blocks before its own come in one trip to the L2 after the other.)
 // The labels are first formed here from the nearest-centre pass (survivors: cluster id of the nearest centre, a centre its own
 // id; pruned tokens: that id iff the distance is strictly below alpha * d_c, else -1) and written out.
 constexpr int kScanTile = kListBlock * 8;   // cluster sizes scanned per step of part 2
 constexpr int kNoLabel = 0x7fffffff;
-constexpr int kListsMaxN = 2048;
+constexpr int kListsMaxN = 1024;
 
 template <typename T>
 __global__ void __launch_bounds__(kListBlock) k_lists(const __grid_constant__ Batch bt, int spin_limit) {
