@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
 // 1.1 until the accumulator is complete, 2.0 in the epilogue, 1.1 for the tickets.
 constexpr int kAsnRing = 192 * 1024;                 // (with more of it the next kernels' CTAs find no room beside this one and crowd on a few SMs)
 constexpr int kAsnSmem = 1024 + kAsnRing;
-constexpr int kAsnMostCols = TMEM_COLS, kAsnLeastCols = 64;
+constexpr int kAsnMostCols = TMEM_COLS, kAsnLeastCols = 128;   // (with 64 as least, DBDPC and merge of 2977 keys 60.3 us, 59.6 with 128, 61.3 with 256)
 
 // a / b for a below 2^22 and b > 0 (the compiler's division is three times as long, from a cold instruction cache)
 __device__ __forceinline__ int div_small(int a, int b) {
