@@ -79,6 +79,10 @@ struct Shared {
 };
 
 enum { MODE_GRAM = 0, MODE_ASSIGN = 1, MODE_SPREAD = 2 };
+// The largest-distance pass runs into the power limit: its warps sleep while they wait (ten layers of 7290 keys, one pass after another:
+// 232 -> 218 us; a pass by itself 198 -> 203).  The other passes are bound by how soon a wait ends (16 images of 2916 tokens 247 ->
+// 256 us with all waits asleep).
+constexpr bool sleeps(int mode) { return mode == MODE_SPREAD; }
 
 // The largest-distance pass needs every unordered pair once: tiles that lie wholly below the diagonal
 // are left out (by the producer, the MMA issuer and the epilogue alike).
@@ -148,7 +152,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
   __syncwarp();
   if (lane * 4 < HALF) reinterpret_cast<float4 *>(rn_col)[lane] = r4;
   __syncwarp();
-  if (!mbar_wait_warp(acc_full, parity)) return false;
+  if (!mbar_wait_warp<sleeps(MODE)>(acc_full, parity)) return false;
   tc_fence_after();
   unsigned long long rowsum = 0ull;
   float bd = 3.0f, bc = -4.0f;                  // distance to the nearest centre of the tile (<= 2) and its cosine
@@ -773,6 +777,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
   using PC = PairCfg<MODE, EW>;
   constexpr int PSTAGES = PC::STAGES, SLABS = PC::SLABS, PSTAGE_BYTES = PC::STAGE_BYTES;
   constexpr size_t PRING = PC::RING;
+  constexpr bool ASLEEP = sleeps(MODE);
   constexpr int LIST = MODE == MODE_ASSIGN ? MODE_ASSIGN : MODE_GRAM;   // how the tiles of an image are listed
   TL_SCOPE(bt.img[0], MODE == MODE_GRAM ? 4 : 6);
   extern __shared__ uint8_t smem_raw[];
@@ -848,7 +853,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
         for (int ks = 0; ks < nslab; ks += SLABS, ++it) {
           const int s = it % PSTAGES;
           const int n = min(SLABS, nslab - ks);      // K-slabs of this stage
-          if (!mbar_wait(&sh.empty[s], ((it / PSTAGES) & 1) ^ 1)) { ok = false; break; }
+          if (!mbar_wait<ASLEEP>(&sh.empty[s], ((it / PSTAGES) & 1) ^ 1)) { ok = false; break; }
           uint8_t *a_dst = ring + (size_t)s * PSTAGE_BYTES, *b_dst = a_dst + SLABS * A_BYTES;
           if (leader) mbar_arrive_expect_tx(&sh.full[s], (uint32_t)n * 4u * A_BYTES);   // the bytes of both CTAs
           const uint32_t bar = map_to_rank(smem_u32(&sh.full[s]), 0);
@@ -876,7 +881,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
         int I, J, nrows, ncols;
         locate(item, b, I, J, nrows, ncols);
         const uint32_t a = tcount % PNACC;
-        if (!mbar_wait(&sh.acc_empty[a], ((tcount / PNACC) & 1) ^ 1)) { ok = false; break; }
+        if (!mbar_wait<ASLEEP>(&sh.acc_empty[a], ((tcount / PNACC) & 1) ^ 1)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * PBN;
         // kind::f16, fp32 accumulate, bf16 x bf16, both operands K-major, M = 256 over the pair, N = this tile's width
@@ -884,7 +889,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
         for (int ks = 0; ks < nslab; ks += SLABS, ++it) {
           const int s = it % PSTAGES;
           const int n = min(SLABS, nslab - ks);
-          if (!mbar_wait(&sh.full[s], (it / PSTAGES) & 1)) { ok = false; break; }
+          if (!mbar_wait<ASLEEP>(&sh.full[s], (it / PSTAGES) & 1)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_addr = smem_u32(ring + (size_t)s * PSTAGE_BYTES);
           const uint64_t da = smem_desc(a_addr), db = smem_desc(a_addr + SLABS * A_BYTES);
@@ -905,7 +910,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
       if (!ok) atomicExch(&sh.abort, 1);
     }
     // whatever way the loop ended, no MMA may still be running when the tensor memory is given back
-    if (lane == 0 && !mbar_wait(&sh.done, 0)) atomicExch(&sh.abort, 1);
+    if (lane == 0 && !mbar_wait<ASLEEP>(&sh.done, 0)) atomicExch(&sh.abort, 1);
   } else {
     // ---------------- epilogue (each CTA for its 128 rows) ----------------
     const int ew = warp - 2;

@@ -29,6 +29,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
       : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
+// The same, but the thread may sleep for up to 20 us in it: wakes later, takes no power meanwhile.
+__device__ __forceinline__ bool mbar_try_wait_asleep(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(20000u) : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -42,9 +52,10 @@ static __device__ __noinline__ bool mbar_wait_slow(uint64_t *bar, uint32_t parit
     if ((i & 255u) == 255u && global_ns() - t0 > kWaitNs) return false;
   }
 }
+template <bool ASLEEP = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   for (int i = 0; i < 64; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
+    if (ASLEEP ? mbar_try_wait_asleep(bar, parity) : mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow(bar, parity);
 }
 
@@ -91,9 +102,10 @@ static __device__ __noinline__ void land_copies(uint64_t *bars, int n) {
 
 // Wait of a whole warp: one lane polls (32 lanes spinning on one barrier word get in the way of the
 // copy engine that has to update it), the result is shared.
+template <bool ASLEEP = false>
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
   int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait<ASLEEP>(bar, parity) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
