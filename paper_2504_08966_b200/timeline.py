@@ -22,7 +22,7 @@ from . import build as pact_build
 from . import workloads
 
 KERNELS = {0: "k_qsum", 1: "k_tokens", 2: "k_scores", 3: "k_select", 4: "k_tiles_umma<gram>", 5: "k_centers",
-           6: "k_tiles_umma<assign>", 7: "  k_select: threshold known", 8: "k_members / k_lists", 9: "k_merge",
+           6: "k_tiles_pair<assign>", 7: "  k_select: threshold known", 8: "k_members / k_lists", 9: "k_merge",
            10: "  k_centers: rows staged", 11: "  k_centers: sweeps done", 12: "  k_center_keys: start",
            13: "  members: labels read", 14: "  members: offsets known", 15: "  k_merge: records read"}
 # the same slots in a step of one cluster per image
@@ -52,12 +52,14 @@ def main(name: str = "single_image") -> None:
     torch.cuda.synchronize()
     buf.zero_()
     torch.cuda.synchronize()
+    for i in range(9):                        # (one after another, as a server replays them; what is printed is the last)
+        graphs[(i + 1) % 3].launch()
     before = ctx.launch_count()
-    graphs[0].launch()
+    graphs[1].launch()
     torch.cuda.synchronize()
     names = {**KERNELS, **SMALL} if ctx.launch_count() - before == 4 else KERNELS
     a = buf.cpu().numpy().reshape(SLOTS, CTAS, 2)
-    t0 = a[a > 0].min()
+    t0 = a[0][a[0] > 0].min()
     print(f"{name}: one graph replay, first image of the batch; microseconds from the first CTA start")
     print(f"{'kernel / point':34s} {'CTAs':>5s}   start min / median / max      end min / median / max")
     for k in range(SLOTS):
