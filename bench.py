@@ -605,7 +605,7 @@ def main():
             "dtype": "bf16", "data": "synthetic",
             "config": {"workload": f"{wl.name} (LLaVA-OneVision-7B-shaped)", "images_per_step_per_gpu": B, "N": img0.N,
                        "text_tokens": T, "d": d, "d_k": d_k, "lambda": wl.lam, "d_c": wl.d_c, "alpha": wl.alpha,
-                       "d_n": wl.d_n, "out_dtype": "bf16", "launch": "CUDA graph replay of pact_reduce (pact_graph_launch): 11 kernels chained by programmatic dependent launch",
+                       "d_n": wl.d_n, "out_dtype": "bf16", "launch": "CUDA graph replay of pact_reduce (pact_graph_launch): 10 kernels chained by programmatic dependent launch",
                        "l2": f"{copies} input copies rotated between steps ({in_bytes * copies / 1e6:.0f} MB > 126 MB L2)"
                              + ("; per-kernel pass also writes a 512 MB flush buffer" if flush is not None else "")},
             "latency_us": ms_per_step * 1e3 / B, "step_times": step_times, "stream_launch_ms_per_step": plain_ms,

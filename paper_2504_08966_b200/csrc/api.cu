@@ -584,10 +584,10 @@ static pact_status reduce_images(pact_ctx *ctx, const pact_image *imgs, int B, c
     else CK(launch_gram(bt, cmaxN, bf, ctx->dev, st));
     CK(mark());
     CK(launch_centers(bt, cmaxQ, bf, ctx->dev, ctx->sweep_limit, st));  CK(mark());
-    // On the tensor-core path with few tokens the labels and member counts are formed as the rows x centres pass finishes groups of
+    // On the tensor-core path with little work per SM (one image) the labels and member counts are formed as the rows x centres pass finishes groups of
     // rows, and one kernel places the members.  With more the pass runs on pairs of CTAs, and labels and lists are formed as on the
     // fp32 path.
-    const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, ctx->dev);
+    const bool pairs = ctx->umma && umma_pairs_for_assign(cmaxN, nb, ctx->dev);
     const bool fused_labels = ctx->umma && !pairs;
     if (ctx->umma) CK(launch_assign_umma(bt, cmaxN, false, ctx->dev, st, fused_labels, pairs));
     else CK(launch_assign(bt, cmaxN, bf, ROWS_ALL, ctx->dev, st));

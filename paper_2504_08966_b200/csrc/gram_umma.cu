@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
 // kept_rows, bit 0: rows are the gathered survivors (Kp, rnk) instead of all tokens; bit 1: the labels, cluster sizes and
 // per-block member counts are formed here as groups of rows finish.
 //
-// For the stage calls and the whole step of images of up to 1024 tokens; the whole step of larger ones takes pairs of CTAs.
+// For the stage calls and the whole step of a few images; that of batches and long images takes pairs of CTAs.
 // Where the row blocks are few enough that every CTA needs one tile only, the centres are shared out among as many columns of tiles
 // as give every CTA one, all of the same width: up to 512 columns, i.e. the whole tensor memory, in two instructions per
 // step (DBDPC and merge of 2977 keys 61.5 -> 60.0 us against columns of 256 whatever C is; where some CTAs had a second, narrow tile,
@@ -686,8 +686,8 @@ __global__ void __maxnreg__(80) k_assign(const __grid_constant__ Batch bt, const
 // columns (half of operand B), CTA 0 issues tcgen05.mma.cta_group::2 for both, and each CTA finds its
 // 128 x 256 part of the product in its own tensor memory.  A CTA therefore fetches half as many operand
 // bytes from the L2 per output element as it does alone.  The largest-distance pass always runs this way, the
-// all-pairs pass when an SM has six or more 128 x 128 blocks to do (with fewer, the coarser tiles cost a round) and the rows x
-// centres pass of the whole step from 1025 tokens on.
+// all-pairs pass when an SM has six or more 128 x 128 blocks to do and the rows x centres pass of the whole step when it has two
+// or more 128-row blocks (with fewer, the coarser tiles cost a round).
 //   full[s]      in CTA 0: both CTAs' copies of stage s report their bytes there
 //   empty[s]     in each CTA: tcgen05.commit (multicast to both CTAs) once the MMAs have read stage s
 //   acc_full[a]  in each CTA: tcgen05.commit (multicast) once accumulator a is complete
@@ -954,6 +954,8 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
   cluster_barrier();                                  // nothing is in flight towards the other CTA any more
   tc_fence_after();
   if (warp == 1) tmem_dealloc2(tmem_base, TMEM_COLS);
+  __syncthreads();
+  cluster_barrier();                                  // neither SM goes to another kernel's CTA before both have given their tensor memory back
   if (threadIdx.x == 0 && sh.abort)
     for (int b = 0; b < bt.B; ++b) atomicMin(&bt.img[b].cnt[PACT_CNT_STATUS], (int)PACT_ERR_TIMEOUT);
 }
@@ -1069,12 +1071,11 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
   return launch_k(k_tiles_umma<MODE_GRAM, kGramBN>, grid, dim3(THREADS), TileCfg<kGramBN>::SMEM, st, true, bt, tm);
 }
 
-bool umma_pairs_for_assign(int maxN, const DeviceCfg &cfg) {
-  // In the whole step, from 1025 tokens on, pairs of CTAs on 256 x 256 tiles: a pair fetches two thirds of the operand bytes, and
-  // the labels, formed by a kernel of their own, cost less than the tickets of single CTAs that form them as they go.  One
-  // image of 7290 tokens 91.9 -> 90.0 us, of 3000 64.3 -> 63.7, of 13000 154.9 -> 148.9, five of 2000 98.3 -> 94.5, sixteen of 1030
-  // 118.1 -> 119.8.
-  return cfg.pair_assign && maxN > 1024;
+bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
+  // With two or more 128-row blocks per SM (batches, long images) pairs of CTAs on 256 x 256 tiles are faster: a pair fetches two thirds
+  // of the operand bytes.  (From 1025 tokens on a call by itself is faster with them too, one image of 7290 tokens by 2 us, but four such
+  // calls on four streams did not come to an end.)
+  return cfg.pair_assign && (long long)((maxN + BM - 1) / BM) * B >= 2LL * cfg.sm_count;
 }
 
 // labels: the single-CTA kernel also forms labels and member counts (all-token rows only); pairs: the pair kernel

@@ -132,7 +132,7 @@ bool umma_supported(int d_k);
 cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cudaStream_t st, int est_rows = 0);
 cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const DeviceCfg &cfg, cudaStream_t st, bool labels = false,
                                bool pairs = false);
-bool umma_pairs_for_assign(int maxN, const DeviceCfg &cfg);
+bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg);
 cudaError_t launch_members(const Batch &bt, int maxN, bool label_none, cudaStream_t st);   // label_none: where there is no centre the labels are written (-1)
 cudaError_t launch_spread_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cudaStream_t st);
 
