@@ -22,7 +22,7 @@ from . import build as pact_build
 from . import workloads
 
 KERNELS = {0: "k_qsum", 1: "k_tokens", 2: "k_scores", 3: "k_select", 4: "k_tiles_umma<gram>", 5: "k_centers",
-           6: "k_tiles_pair<assign>", 7: "  k_select: threshold known", 8: "k_members / k_lists", 9: "k_merge",
+           6: "k_assign / pair<assign>", 7: "  k_select: threshold known", 8: "k_members / k_lists", 9: "k_merge",
            10: "  k_centers: rows staged", 11: "  k_centers: sweeps done", 12: "  k_center_keys: start",
            13: "  members: labels read", 14: "  members: offsets known", 15: "  k_merge: records read"}
 # the same slots in a step of one cluster per image
