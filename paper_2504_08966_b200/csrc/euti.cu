@@ -461,7 +461,8 @@ __global__ void __launch_bounds__(kTokThreads, 2) k_tokens(const __grid_constant
     // One buffer per warp until k_qsum is done, all of them from then on: with more from the start this stream leaves k_qsum a
     // third of the memory rate and the logits begin late (16 images of 2916 tokens: at 37 us), with none the memory
     // idles towards the end of k_qsum.
-    if (lane == 0) issue_row();
+    // (A launch without norms asks for no row: nobody would wait for it, and the CTA could end with the copy under way.)
+    if (lane == 0 && (what & kTokNorms)) issue_row();
     bool all = false;
     int slot = 0, b = 0, dealt = 0;                     // buffer that is next; rows of the units before
     uint32_t par = 0;                                   // parity of each buffer's barrier

@@ -68,3 +68,37 @@ def test_a_planted_trigger_is_found():
         assert early != body and _too_early(early) == want
     body = next(b for _, n, b in KERNELS if n == "k_scores")
     assert _too_early(body.replace("pdl_wait();", ";", 1)) == ["return"]
+
+
+def _headers(body, at):
+    """The statement at this place from its start, and the head of every block around it."""
+    heads, i = [body[max(body.rfind(c, 0, at) for c in "{};") + 1:at]], at
+    while True:
+        depth, i = 0, i - 1
+        while i >= 0 and (depth or body[i] != "{"):
+            depth += {"}": 1, "{": -1}.get(body[i], 0)
+            i -= 1
+        if i < 0:
+            return heads
+        begin = i                                          # a head ends at its brace and may hold the semicolons of a for
+        depth = 0
+        while begin > 0 and (depth or body[begin - 1] not in "{};"):
+            begin -= 1
+            depth += {")": 1, "(": -1}.get(body[begin], 0)
+        heads.append(body[begin:i])
+
+
+def _not_asked_for(body, call, bit):
+    """Calls of `call` that are reached in a launch without the part `bit` of the token pass."""
+    return [m.start() for m in re.finditer(re.escape(call), body) if not any(f"what & {bit}" in h for h in _headers(body, m.start()))]
+
+
+def test_the_token_pass_asks_for_no_copies_that_it_does_not_wait_for():
+    """A launch without norms (or without logits) has no wait for rows (or keys)."""
+    body = next(b for _, n, b in KERNELS if n == "k_tokens")
+    for call, wait, bit in (("issue_row();", "mbar_wait_warp(&s_rbar", "kTokNorms"), ("issue_keys(u0", "mbar_wait_warp_unless(&s_abort, &s_kbar", "kTokLogits"), ("issue_keys(mu", "mbar_wait_warp_unless(&s_abort, &s_kbar", "kTokLogits")):
+        assert call in body and wait in body
+        assert not _not_asked_for(body, call, bit), call
+        assert not _not_asked_for(body, wait, bit), wait
+    bare = body.replace("if (lane == 0 && (what & kTokNorms)) issue_row();", "if (lane == 0) issue_row();")
+    assert bare != body and len(_not_asked_for(bare, "issue_row();", "kTokNorms")) == 1
