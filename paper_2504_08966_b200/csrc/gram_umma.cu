@@ -692,8 +692,10 @@ __global__ void __maxnreg__(80) k_assign(const __grid_constant__ Batch bt, const
 //   empty[s]     in each CTA: tcgen05.commit (multicast to both CTAs) once the MMAs have read stage s
 //   acc_full[a]  in each CTA: tcgen05.commit (multicast) once accumulator a is complete
 //   acc_empty[a] in CTA 0: the epilogue warps of both CTAs arrive there
-// Every wait is bounded as in the single-CTA kernel; the CTAs leave together through a cluster barrier, after
-// which nothing is in flight towards either's shared memory.
+// Every mbarrier wait is bounded as in the single-CTA kernel.  Without a bound are the cluster barriers (both CTAs of a cluster run at once, and every
+// way through the kernel passes all four) and the allocation and deallocation, which are the pair's together: each lies between two cluster barriers,
+// so that neither CTA asks before the other one runs and neither leaves, and its SM goes to another stream's kernel, before
+// both have their tensor memory back.  The allocation finds it free: no SM has two CTAs with tensor memory (kAloneOnSm).
 constexpr int PBN = 256;                              // tile width of the pair kernel
 constexpr int PNACC = TMEM_COLS / PBN;
 constexpr int PMAX_STAGES = 5;
@@ -758,6 +760,11 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t *bar) {
                ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
 }
 
+// A CTA that holds tensor memory must not wait for another one that wants some on its SM, which clusters would: every kernel with tensor memory takes
+// more than half of an SM's 228 KB of shared memory, so that there is no other.
+static_assert(PairCfg<MODE_GRAM, 16>::SMEM > kAloneOnSm && PairCfg<MODE_ASSIGN, 8>::SMEM > kAloneOnSm && PairCfg<MODE_SPREAD, 8>::SMEM > kAloneOnSm &&
+              TileCfg<128>::SMEM > kAloneOnSm && TileCfg<256>::SMEM > kAloneOnSm && kAsnSmem > kAloneOnSm, "one CTA with tensor memory per SM");
+
 template <int EW> struct SharedPair {
   uint64_t full[PMAX_STAGES], empty[PMAX_STAGES], acc_full[PNACC], acc_empty[PNACC];
   uint64_t done;                                   // every MMA of the pair is complete (signalled in both CTAs)
@@ -795,10 +802,15 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
     sh.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // The allocation takes tensor memory of both SMs: it may only be asked for once the other CTA is known to run there.  (Without
+  // this barrier, and with an exit that did not wait for the other CTA's deallocation, calls on four streams did not come to an end;
+  // within one stream no other kernel with tensor memory is next to this one.)
+  __syncthreads();
+  cluster_barrier();
   if (warp == 1) tmem_alloc2(&sh.tmem_base, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  cluster_barrier();                                  // both CTAs' barriers exist before either is signalled
+  cluster_barrier();                                  // both CTAs' barriers and tensor memory exist before either is used
   tc_fence_after();
   const uint32_t tmem_base = sh.tmem_base;
   pdl_wait();
@@ -1073,8 +1085,8 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
 
 bool umma_pairs_for_assign(int maxN, int B, const DeviceCfg &cfg) {
   // With two or more 128-row blocks per SM (batches, long images) pairs of CTAs on 256 x 256 tiles are faster: a pair fetches two thirds
-  // of the operand bytes.  (From 1025 tokens on a call by itself is faster with them too, one image of 7290 tokens by 2 us, but four such
-  // calls on four streams did not come to an end.)
+  // of the operand bytes.  (From 1025 tokens on a call by itself is faster with them too, one image of 7290 tokens by 2 us; but four such
+  // calls on four streams did not come to an end while a pair asked for tensor memory before both of its CTAs ran and left one by one.)
   return cfg.pair_assign && (long long)((maxN + BM - 1) / BM) * B >= 2LL * cfg.sm_count;
 }
 

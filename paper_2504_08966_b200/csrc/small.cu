@@ -703,6 +703,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
 namespace {
 
 static_assert(sizeof(SmallShared<__nv_bfloat16>) + kSmDynUmma <= 227 * 1024 && sizeof(SmallShared<float>) + kSmDynF64 <= 227 * 1024, "shared memory of an SM");
+static_assert(kSmDynUmma > kAloneOnSm, "one CTA with tensor memory per SM");
 static_assert(4 * sizeof(F64Group) <= kSmDynF64 - 1024, "double-precision tiles");
 static_assert((size_t)kSmallMaxN * (kSmMaxW / 4 + 1) * 16 + kSmallMaxN * 8 <= kSmDynF64 - 1024, "adjacency of the survivors");
 static_assert(kSmMaxHeads * (kSmallMaxN / kMinPiece) * 8 <= kSmDynF64 - 1024 && kSmMaxW * kSmallMaxN <= kSmDynF64 - 1024, "softmax pieces, member table");

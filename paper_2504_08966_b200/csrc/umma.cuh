@@ -6,6 +6,8 @@
 
 namespace pact {
 
+constexpr size_t kAloneOnSm = 114 * 1024;   // a CTA with more dynamic shared memory than this has its SM to itself among its like
+
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols) : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
