@@ -14,6 +14,7 @@
 //            range order, so the result does not depend on timing.
 #include "kernels.cuh"
 #include "labels.cuh"
+#include "merge_ranges.h"
 #include "tma.cuh"
 
 namespace pact {
@@ -387,11 +388,8 @@ __global__ void __launch_bounds__(256) k_list_clear(const __grid_constant__ Batc
 // warp instructions per 512 bytes and with them 83 us; with bulk copies a thread only adds, and from the end of the lists to
 // the end of the last CTA it is 75 us, 5.0 TB/s.  One image of 7290 tokens, 53 MB that mostly lie in the L2: 17 us.
 constexpr int kMrgThreads = 128;
-constexpr int kMrgCtasPerSm = 8;
-constexpr int kMrgRanges = 296;                     // most ranges per image (sizes the scratch)
 constexpr int kMrgRingBytes = 24 * 1024;            // rows in flight per CTA when an SM has eight, more when it has fewer
 constexpr int kMrgRingMost = 192 * 1024;
-constexpr int kMrgWhole = 24;                       // items past its end that a range goes on for a cluster
 constexpr int kMrgMaxHalf = 32;                     // rows in a half ring
 
 template <typename T, typename O, int VPL>
@@ -490,7 +488,7 @@ __global__ void __launch_bounds__(kMrgThreads, kMrgCtasPerSm) k_merge(const __gr
         p[1] = make_float4(acc[v][4], acc[v][5], acc[v][6], acc[v][7]);
       }
     const int x0 = first / per, x1 = (first + size - 1) / per;
-    int32_t *ticket = &im.cticket[x0 * 8 + sl];     // (at most one cluster goes on after a range; a range has eight members or more)
+    int32_t *ticket = &im.cticket[x0 * 8 + sl];     // (at most one cluster goes on after a range; a range has kMrgLeast places or more)
     __threadfence();
     __syncthreads();
     if (t == 0) s_last = (atomicAdd(ticket, 1) == x1 - x0);
@@ -620,20 +618,6 @@ cudaError_t launch_lists(const Batch &bt, int maxN, bool bf16, bool from_best, i
   return e != cudaSuccess ? e : launch_members(bt, maxN, false, st);
 }
 
-// items per range: 24 (with 16: 2.5 us more of 16 images of 2916 tokens, 2 us of three of 2309; with 48 as much), 12 where
-// that leaves an SM less than two CTAs, 8 where 12 does (the tickets of cut clusters need eight): the rows of a range follow one
-// another, 40 ns each where a CTA has the SM to itself.  No more than eight rounds of CTAs over the GPU, and no more ranges than
-// the scratch has room for.  (16 for all small calls: 729 tokens 47.8 us, 46.3 with 8; 1300 57.4, 55.9 with 12, 57.8 with 8.)
-static int merge_per(int n_items, int slices, int B, int sm_count) {
-  const long long most = 8LL * kMrgCtasPerSm * sm_count;
-  long long r = (n_items + 23) / 24;
-  if (r * slices * B < 2 * sm_count) r = (n_items + 11) / 12;
-  if (r * slices * B < 2 * sm_count) r = (n_items + 7) / 8;
-  if (r * slices * B > most) r = most / ((long long)slices * B);
-  if (r > kMrgRanges) r = kMrgRanges;
-  if (r < 1) r = 1;
-  return (int)((n_items + r - 1) / r);
-}
 size_t merge_scratch_rows() { return 2 * kMrgRanges; }
 
 template <typename T, typename O, int VPL>
@@ -642,11 +626,8 @@ static cudaError_t launch_merge_v(const Batch &bt, int n_items, int slices, cons
   const long long per_sm = ((long long)ranges * slices * bt.B + cfg.sm_count - 1) / cfg.sm_count;
   int ring = per_sm >= kMrgCtasPerSm ? kMrgRingBytes : (int)(kMrgCtasPerSm * kMrgRingBytes / per_sm);
   if (ring > kMrgRingMost) ring = kMrgRingMost;
-  // One round of CTAs: the longest range counts, so only clusters that leave it within what the ring holds at once stay
-  // whole, and no more than kMrgWhole items past its end (as many rows as a cut costs; 900 tokens of a video 49.8 -> 45.4 us, 729 of a
-  // photo 46.7 -> 46.3).  Several rounds: the bytes count.
   const int row = ((bt.d / 8 + slices - 1) / slices) * 8 * (int)sizeof(T), most = 2 * kMrgMaxHalf, room = (ring / row < most ? ring / row : most) - per;
-  const int whole = per_sm > kMrgCtasPerSm ? per : room < 8 ? 8 : room > kMrgWhole ? kMrgWhole : room;
+  const int whole = merge_whole(per, per_sm, room);
   return launch_k(k_merge<T, O, VPL>, dim3(ranges * slices, bt.B), dim3(kMrgThreads), (size_t)ring, st, true, bt, per, whole, slices, ring);
 }
 
