@@ -121,7 +121,7 @@ template <int MODE> __device__ __forceinline__ void tile_at(int t, int ntm, int 
 // applies the mode's arithmetic; arrive() is called once the accumulator has been read.  skip: the warp only
 // waits and releases (a block below the diagonal of the all-pairs pass).  Returns false when the wait ran out.
 template <int MODE, int HALF, typename Arrive>
-__device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int tmi, int cbase, bool skip, int nrows,
+__device__ __forceinline__ bool epi_tile(const ImgDesc &im, int tmi, int cbase, bool skip, int nrows,
                                          int ncols, uint32_t taddr, uint64_t *acc_full, uint32_t parity, float *rn_col,
                                          uint32_t *tr, int lane, int qd, int &band, float &mx, Arrive arrive) {
   // inverse norms of this warp's columns and of this lane's row (in flight while the MMAs run)
@@ -136,8 +136,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
   }
   const int row = tmi * BM + qd * 32 + lane;
   const bool row_ok = row < nrows;
-  const bool kept_space = MODE == MODE_GRAM || (MODE == MODE_ASSIGN && kept_rows);
-  float rni = row_ok ? (kept_space ? im.rnk[row] : im.rn[row]) : 0.f;
+  float rni = row_ok ? (MODE == MODE_GRAM ? im.rnk[row] : im.rn[row]) : 0.f;
   if (MODE == MODE_GRAM) {
     // the all-pairs pass multiplies the two inverse norms first; a vanishing key (inverse norm at
     // its clamp, 1e20) takes 0 here so that the product stays finite: dot product 0, distance 1
@@ -262,7 +261,7 @@ __device__ __forceinline__ bool epi_tile(const ImgDesc &im, int kept_rows, int t
     if (MODE == MODE_GRAM) atomicAdd(&im.rho_fix[row], rowsum);
     else if (MODE == MODE_ASSIGN && bd <= 2.0f) {
       const unsigned long long pk = ((unsigned long long)__float_as_uint(bd) << 32) | (unsigned)bi;
-      atomicMin(&im.best[kept_rows ? im.kept_idx[row] : row], pk);
+      atomicMin(&im.best[row], pk);
     }
   }
   return true;
@@ -396,7 +395,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tiles_umma(const __grid_constant
       const uint32_t a = tcount % NACC;
       const int cbase = tni * BN + half * HALF;     // first column of this warp
       const uint32_t taddr = tmem_base + a * BN + half * HALF + ((uint32_t)(qd * 32) << 16);
-      ok = epi_tile<MODE, HALF>(im, 0, tmi, cbase, false, nrows, ncols, taddr, &sh.acc_full[a], (tcount / NACC) & 1,
+      ok = epi_tile<MODE, HALF>(im, tmi, cbase, false, nrows, ncols, taddr, &sh.acc_full[a], (tcount / NACC) & 1,
                                 rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive(&sh.acc_empty[a]); });
       if (!ok) break;
       ++tcount;
@@ -780,7 +779,7 @@ template <int EW> struct SharedPair {
 // with J >= I are listed, and of the tile (I, I) the block (2 I + 1, 2 I) lies below the diagonal: computed, not used.
 template <int MODE, int EW>
 __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(const __grid_constant__ Batch bt,
-                                                                              const __grid_constant__ TmapSet tm, int kept_rows) {
+                                                                              const __grid_constant__ TmapSet tm) {
   using PC = PairCfg<MODE, EW>;
   constexpr int PSTAGES = PC::STAGES, SLABS = PC::SLABS, PSTAGE_BYTES = PC::STAGE_BYTES;
   constexpr size_t PRING = PC::RING;
@@ -824,7 +823,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
       int nr, nc;
       if (MODE == MODE_GRAM) { nr = *ib.q_ptr; nc = nr; }
       else if (MODE == MODE_SPREAD) { nr = ib.N; nc = ib.N; }
-      else { nr = (kept_rows & 1) ? *ib.q_ptr : ib.N; nc = *ib.C_ptr; }
+      else { nr = ib.N; nc = *ib.C_ptr; }
       s_rows[b] = nr;
       s_cols[b] = nc;
       s_first[b] = first;
@@ -951,7 +950,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
       const uint32_t taddr = tmem_base + a * PBN + half * PC::COLS + ((uint32_t)(qd * 32) << 16);
       const uint32_t rel = map_to_rank(smem_u32(&sh.acc_empty[a]), 0);
       int band = 0;
-      ok = epi_tile<MODE, PC::COLS>(im, kept_rows, R, cbase, skip, nrows, ncols, taddr, &sh.acc_full[a], (tcount / PNACC) & 1,
+      ok = epi_tile<MODE, PC::COLS>(im, R, cbase, skip, nrows, ncols, taddr, &sh.acc_full[a], (tcount / PNACC) & 1,
                                     rn_col, tr, lane, qd, band, mx, [&]() { mbar_arrive_remote(rel); });
       if (MODE == MODE_GRAM && band) atomicAdd(&im.cnt[PACT_CNT_BAND_DC], band);
       if (!ok) break;
@@ -998,14 +997,14 @@ bool umma_supported(int d_k) { return d_k % BK == 0; }
 
 namespace {
 template <int MODE, int EW>
-cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, int kept_rows, const DeviceCfg &cfg, cudaStream_t st) {
+cudaError_t launch_pair(const Batch &bt, const TmapSet &tm, long long tiles, const DeviceCfg &cfg, cudaStream_t st) {
   using PC = PairCfg<MODE, EW>;
   long long P = cfg.sm_count / 2;                     // one pair per two SMs
   if (P > tiles * bt.B) P = tiles * bt.B;
   if (P < 1) P = 1;
   LaunchOpt opt;
   opt.cluster = 2;
-  return launch_opt(opt, k_tiles_pair<MODE, EW>, dim3((unsigned)(2 * P)), dim3(PC::THREADS), PC::SMEM, st, bt, tm, kept_rows);
+  return launch_opt(opt, k_tiles_pair<MODE, EW>, dim3((unsigned)(2 * P)), dim3(PC::THREADS), PC::SMEM, st, bt, tm);
 }
 
 // can clusters of two CTAs of this kernel be launched at all?
@@ -1076,7 +1075,7 @@ cudaError_t launch_gram_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, cu
   const long long nq = (est_rows + BM - 1) / BM;
   if (cfg.pair_gram && nq * (nq + 1) / 2 * bt.B >= 6LL * cfg.sm_count) {
     const long long n2 = (maxN + 2 * BM - 1) / (2 * BM);
-    return launch_pair<MODE_GRAM, 16>(bt, tm, n2 * (n2 + 1) / 2, 0, cfg, st);
+    return launch_pair<MODE_GRAM, 16>(bt, tm, n2 * (n2 + 1) / 2, cfg, st);
   }
   const long long nb = (maxN + BM - 1) / BM;
   dim3 grid(umma_grid_x(nb * (nb + 1) / 2, bt.B, cfg.sm_count), bt.B);
@@ -1102,7 +1101,7 @@ cudaError_t launch_assign_umma(const Batch &bt, int maxN, bool kept_rows, const 
     for (int b = 0; b < bt.B; ++b)
       if (!rows_map(bt.img[b], &tm.a[b]) || !encode_rows(cfg, &tm.b[b], bt.img[b].Kcen, bt.img[b].Np, bt.d_k, bt.d_k)) return cudaErrorInvalidValue;
     const long long pt = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
-    return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, 0, cfg, st);
+    return launch_pair<MODE_ASSIGN, 8>(bt, tm, pt, cfg, st);
   }
   AssignMaps tm;
   for (int b = 0; b < bt.B; ++b) {
@@ -1126,7 +1125,7 @@ cudaError_t launch_spread_umma(const Batch &bt, int maxN, const DeviceCfg &cfg, 
   }
   if (cfg.pair_spread) {
     const long long ptiles = (long long)((maxN + 2 * BM - 1) / (2 * BM)) * ((maxN + PBN - 1) / PBN);
-    return launch_pair<MODE_SPREAD, 8>(bt, tm, ptiles, 0, cfg, st);
+    return launch_pair<MODE_SPREAD, 8>(bt, tm, ptiles, cfg, st);
   }
   const long long tiles = (long long)((maxN + BM - 1) / BM) * ((maxN + kWideBN - 1) / kWideBN);
   dim3 grid(umma_grid_x(tiles, bt.B, cfg.sm_count), bt.B);
