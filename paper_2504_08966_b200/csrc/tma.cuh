@@ -3,6 +3,8 @@
 #pragma once
 #include <stdint.h>
 
+#include <cuda/annotated_ptr>
+
 #include "../../include/pact.h"
 
 namespace pact {
@@ -68,8 +70,10 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-// Loads that say what the L2 is to do with their lines: the policies that createpolicy.fractional makes for all of the lines.
-constexpr uint64_t kEvictNormal = 0x1000000000000000ull, kEvictFirst = 0x12F0000000000000ull;   // (first: the first to be replaced)
+// Loads that say what the L2 is to do with their lines.  The policies are the words of CUDA's access properties, known when the kernels are
+// compiled; made by createpolicy in the kernels they would take two registers where the token pass already spills some.
+constexpr uint64_t kEvictNormal = static_cast<uint64_t>(cuda::access_property(cuda::access_property::normal{}));
+constexpr uint64_t kEvictFirst = static_cast<uint64_t>(cuda::access_property(cuda::access_property::streaming{}));   // (the first to be replaced)
 __device__ __forceinline__ void bulk_load_hint(void *dst, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy) : "memory");

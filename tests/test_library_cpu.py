@@ -104,3 +104,10 @@ def test_product_does_not_import_the_oracle():
                 text = open(os.path.join(dirpath, f)).read()
                 assert not re.search(r"^\s*(from|import)\s+oracle", text, flags=re.M), f
                 assert "pact_oracle" not in text and "oracle/" not in text, f
+
+
+def test_cache_policies_are_made_by_cuda():
+    """The encoding of an L2 policy is CUDA's own: no 64-bit word of one stands in the source."""
+    csrc = os.path.join(ROOT, "paper_2504_08966_b200", "csrc")
+    for f in os.listdir(csrc):
+        assert not re.findall(r"0x1[02-6][0-9A-Fa-f]0{13}", open(os.path.join(csrc, f)).read()), f
