@@ -1340,8 +1340,9 @@ static cudaError_t launch_qsum(const Batch &bt, const DeviceCfg &cfg, cudaStream
   opt.cluster = 1;
   while (opt.cluster < kQPartRows && ncg * bt.B * opt.cluster * 2 <= 3 * cfg.sm_count) opt.cluster *= 2;
   const dim3 grid(ncg * opt.cluster, bt.B), block(kQsumThreads);
-  // nothing reads the queries again: where they are many they leave the L2 first (three images with 28 heads, 37 MB: 93.7 -> 92.2
-  // us; 16 images of four heads, 48 MB: 251.5 -> 249.8; 7.5 MB of one image: no difference)
+  // Nothing reads the queries again: where they are many they leave the L2 first.  Whole steps with new inputs each, kept and marked:
+  // 40 MB 99.6 and 98.4 us, eight images of 48 MB together 269.8 and 267.9, of 24 MB 154.7 and 154.2, of 16 MB 116.4 and 116.3, one
+  // of 6 to 30 MB the same within 0.3; scores and split alone gain 0.7 to 1.2 us from 10 MB on.
   long long rows = 0;
   for (int b = 0; b < bt.B; ++b) rows += bt.img[b].N;
   const uint64_t policy = rows * bt.n_qcols * (long long)sizeof(T) > (16ll << 20) ? kEvictFirst : kEvictNormal;
@@ -1354,7 +1355,7 @@ template <typename T> static TokCfg tokens_config(const Batch &bt, const DeviceC
   return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, cfg.sm_count, cfg.smem_optin - kTokReserve);
 }
 template <typename T>
-static cudaError_t launch_tokens(const Batch &bt, bool scores_only, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
+static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
   const TokCfg tc = tokens_config<T>(bt, cfg);
   if (rpp) *rpp = tc.rpp;
   const bool group = bt.n_qh / bt.n_kvh >= kGroupHeads;
@@ -1364,11 +1365,12 @@ static cudaError_t launch_tokens(const Batch &bt, bool scores_only, int what, bo
   for (int b = 0; b < bt.B; ++b) tokens += N[b] = bt.img[b].N;
   TokUnits un;
   const int grid = tokens_units(N, bt.B, tc.rpp, cfg.sm_count, un);
-  // Hidden states that the merge will not find in the L2 in any case (a call with more than 72 MB of them, scores as a stage of
-  // their own) leave it first, so that queries, keys and what the kernels hand to one another stay: 16 images of 2916 tokens (334
-  // MB) 254.6 -> 249.4 us with all of them marked, 253.1 with the first 72 MB kept; scores and split of 7290 tokens 27.9 ->
-  // 27.3; one image of 7290 (52 MB) the other way, 94.3 -> 96.5.
-  const uint64_t policy = scores_only || tokens * bt.d * (long long)sizeof(T) > (72ll << 20) ? kEvictFirst : kEvictNormal;
+  // Hidden states of which the merge will find too little in the L2 in any case leave it first, so that queries, keys and what the kernels
+  // hand to one another stay.  Whole steps with new inputs each, kept and marked: one image of 75 MB 135.3 and 136.5 us, 82 MB 140.5 and 141.0, 90
+  // MB 151.5 and 150.7, 130 MB 213.1 and 208.3, 40 MB 82.9 and 85.5; four images of 75 MB together 99.8 and 99.9, 90 MB 114.7 and
+  // 113.7.  Scores as a stage of their own cross there too (scores and split up to 52 MB the same, 100 MB 45.2 and 43.0), and up to there a program
+  // that goes on to the merge finds them again (five stages of 36 MB 94.4 and 97.6).
+  const uint64_t policy = tokens * bt.d * (long long)sizeof(T) > (80ll << 20) ? kEvictFirst : kEvictNormal;
   return launch_k(kernel, dim3(grid), dim3(kTokThreads), tok_smem_launch(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, un, policy, what);
 }
 
@@ -1381,7 +1383,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
   int rpp = 0;
-  e = launch_tokens<T>(bt, mode == 1, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
+  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
   if (e != cudaSuccess) return e;
   for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
     // (a part without visual tokens may still bring text rows, which k_merge copies)
@@ -1391,7 +1393,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
     part.img[0].N = feed->end[k] - first;
     part.img[0].vis_start += first;
     part.img[0].nrm += first;
-    if ((e = launch_tokens<T>(part, false, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
+    if ((e = launch_tokens<T>(part, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
   }
   if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;
