@@ -144,7 +144,8 @@ const char *pact_status_string(pact_status s);
 const char *pact_last_cuda_error(const pact_ctx *ctx);
 
 /* Bounds of the device-side waits (Algorithm 2's centre selection is resolved in sweeps over two bit masks,
- * and the member lists of Eq. 10 of up to 1024 tokens on fp32 keys are built behind one barrier between CTAs).  When a bound is reached the
+ * and some of the member lists of Eq. 10 are built behind one barrier between CTAs: those of a whole step of up to 1024 tokens per image on keys that the
+ * tensor cores do not take, i.e. fp32, or bf16 whose width is no multiple of 64, unless it is small enough for one cluster).  When a bound is reached the
  * kernel stops waiting, writes PACT_ERR_TIMEOUT to counters[PACT_CNT_STATUS] of the image and carries on
  * within bounds; the call itself still returns PACT_OK and the outputs of that image are not valid.
  * barrier_polls: polls of the member-list barrier; center_sweeps: sweeps of the centre selection (rows that are

@@ -79,9 +79,9 @@ struct Shared {
 };
 
 enum { MODE_GRAM = 0, MODE_ASSIGN = 1, MODE_SPREAD = 2 };
-// The largest-distance pass runs into the power limit: its warps sleep while they wait (ten layers of 7290 keys, one pass after another:
-// 232 -> 218 us; a pass by itself 198 -> 203).  The other passes are bound by how soon a wait ends (16 images of 2916 tokens 247 ->
-// 256 us with all waits asleep).
+// The largest-distance pass runs into the power limit: its warps sleep while they wait.  Ten layers of 7290 keys, awake and asleep: one pass after
+// another for 0.3 s 228 and 221 us, for 2 ms 193 and 187, a pass by itself after a pause of 5 ms 209 and 198; three layers 72 and 69, one 32.4 and
+// 31.6 by themselves.  The other passes are bound by how soon a wait ends (16 images of 2916 tokens 247 -> 256 us with all waits asleep).
 constexpr bool sleeps(int mode) { return mode == MODE_SPREAD; }
 
 // The largest-distance pass needs every unordered pair once: tiles that lie wholly below the diagonal

@@ -45,9 +45,10 @@ __device__ __forceinline__ float4 ld_cg_f4(const float *p) {
 //   member_off is the exclusive prefix sum of csize.  It writes its record there; the first member of a
 //   cluster also writes P', the size and its logarithm for the cluster's output row.
 // The parts are separated by a barrier over the blocks of the image (all blocks must be resident: cooperative launch).
-// For the whole step of up to kListsMaxN tokens on the double-precision tiles.  k_label_counts and k_members do the same for all others:
-// DBDPC and merge of 900 tokens 46.6 -> 43.8 us, of 7290 113.3 -> 109.4, one fp32 image of 1100 57.7 -> 53.7.  (Here a token looks up
-// its cluster in the sorted block, and the counts of the blocks before its own come in one trip to the L2 after the other.)
+// For the whole step of up to kListsMaxN tokens on the double-precision tiles, which has ten kernels with it and eleven without; that number is
+// what it is kept for.  k_label_counts and k_members do the same for all others, and would be faster here too: one fp32 image of 680 tokens (d_k 128) 49.7 us
+// with k_lists and 45.7 with these two, of 1024 56.6 and 52.4, four of 800 72.4 and 68.4, bf16 with d_k 160, 1000 tokens, 65.1 and 62.0.  (Here a token
+// looks up its cluster in the sorted block, and the counts of the blocks before its own come in one trip to the L2 after the other.)
 // The labels are first formed here from the nearest-centre pass (survivors: cluster id of the nearest centre, a centre its own
 // id; pruned tokens: that id iff the distance is strictly below alpha * d_c, else -1) and written out.
 constexpr int kScanTile = kListBlock * 8;   // cluster sizes scanned per step of part 2
