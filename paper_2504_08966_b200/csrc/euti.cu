@@ -1355,7 +1355,7 @@ template <typename T> static TokCfg tokens_config(const Batch &bt, const DeviceC
   return tokens_config(total, bt.d * (int)sizeof(T), bt.d_k * (int)sizeof(T), bt.n_qcols, bt.n_qh / bt.n_kvh, cfg.sm_count, cfg.smem_optin - kTokReserve);
 }
 template <typename T>
-static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
+static cudaError_t launch_tokens(const Batch &bt, bool scores_only, int what, bool pdl, const DeviceCfg &cfg, cudaStream_t st, int *rpp) {
   const TokCfg tc = tokens_config<T>(bt, cfg);
   if (rpp) *rpp = tc.rpp;
   const bool group = bt.n_qh / bt.n_kvh >= kGroupHeads;
@@ -1366,11 +1366,13 @@ static cudaError_t launch_tokens(const Batch &bt, int what, bool pdl, const Devi
   TokUnits un;
   const int grid = tokens_units(N, bt.B, tc.rpp, cfg.sm_count, un);
   // Hidden states of which the merge will find too little in the L2 in any case leave it first, so that queries, keys and what the kernels
-  // hand to one another stay.  Whole steps with new inputs each, kept and marked: one image of 75 MB 135.3 and 136.5 us, 82 MB 140.5 and 141.0, 90
-  // MB 151.5 and 150.7, 130 MB 213.1 and 208.3, 40 MB 82.9 and 85.5; four images of 75 MB together 99.8 and 99.9, 90 MB 114.7 and
-  // 113.7.  Scores as a stage of their own cross there too (scores and split up to 52 MB the same, 100 MB 45.2 and 43.0), and up to there a program
-  // that goes on to the merge finds them again (five stages of 36 MB 94.4 and 97.6).
-  const uint64_t policy = tokens * bt.d * (long long)sizeof(T) > (80ll << 20) ? kEvictFirst : kEvictNormal;
+  // hand to one another stay.  Whole steps with new inputs each, kept and marked: one image of 40 MB 82.9 and 85.5 us, 75 MB 135.3 and 136.5, 82 MB 140.5
+  // and 141.0, 90 MB 151.5 and 150.7, 130 MB 213.1 and 208.3; four images of 75 MB together 99.8 and 99.9, 90 MB 114.7 and 113.7.
+  // Scores as a stage of their own: nobody knows whether a merge follows.  Scores and split alone, over and over on two or three buffers, gain from
+  // about 32 MB on (30 MB 21.3 and 21.3 us, 38 MB 24.2 and 22.7, 52 MB 27.8 and 25.7; on new inputs the same, 52 MB 28.1 and 28.1, 100 MB 45.2 and
+  // 43.0); five stages with new inputs lose (18 MB 80.8 and 82.1, 36 MB 94.4 and 97.6, 52 MB 111.6 and 114.8, 100 MB 182.9 and 180.5).
+  const long long kept = scores_only ? 32ll << 20 : 80ll << 20;
+  const uint64_t policy = tokens * bt.d * (long long)sizeof(T) > kept ? kEvictFirst : kEvictNormal;
   return launch_k(kernel, dim3(grid), dim3(kTokThreads), tok_smem_launch(tc, bt.d_k * (int)sizeof(T), bt.n_qcols), st, pdl, bt, tc, un, policy, what);
 }
 
@@ -1383,7 +1385,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
   if (e != cudaSuccess) return e;
   if (mark && (e = mark(mark_arg)) != cudaSuccess) return e;
   int rpp = 0;
-  e = launch_tokens<T>(bt, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
+  e = launch_tokens<T>(bt, mode == 1, (mode != 1 ? kTokInit : 0) | (feed ? 0 : kTokNorms) | kTokLogits, true, cfg, st, &rpp);
   if (e != cudaSuccess) return e;
   for (int k = 0, first = 0; feed && k < kFeedParts; first = feed->end[k++]) {
     // (a part without visual tokens may still bring text rows, which k_merge copies)
@@ -1393,7 +1395,7 @@ static cudaError_t launch_euti_t(const Batch &bt, int maxN, int mode, const Devi
     part.img[0].N = feed->end[k] - first;
     part.img[0].vis_start += first;
     part.img[0].nrm += first;
-    if ((e = launch_tokens<T>(part, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
+    if ((e = launch_tokens<T>(part, false, kTokNorms, false, cfg, st, nullptr)) != cudaSuccess) return e;
   }
   if (rpp_out) *rpp_out = rpp;
   if (mode == 2) return cudaSuccess;
