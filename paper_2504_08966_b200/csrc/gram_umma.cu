@@ -794,6 +794,7 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
 
+  cluster_arrive();                                   // this CTA runs
   if (threadIdx.x == 0) {
     for (int s = 0; s < PSTAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
     for (int a = 0; a < PNACC; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], 2 * EW); }
@@ -801,15 +802,15 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
     sh.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
   // The allocation takes tensor memory of both SMs: it may only be asked for once the other CTA is known to run there.  (Without
   // this barrier, and with an exit that did not wait for the other CTA's deallocation, calls on four streams did not come to an end;
   // within one stream no other kernel with tensor memory is next to this one.)
-  __syncthreads();
-  cluster_barrier();
+  cluster_wait();
   if (warp == 1) tmem_alloc2(&sh.tmem_base, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  cluster_barrier();                                  // both CTAs' barriers and tensor memory exist before either is used
+  cluster_arrive();                                   // this CTA's barriers and tensor memory exist
   tc_fence_after();
   const uint32_t tmem_base = sh.tmem_base;
   pdl_wait();
@@ -832,6 +833,8 @@ __global__ void __launch_bounds__(PairCfg<MODE, EW>::THREADS, 1) k_tiles_pair(co
     s_first[bt.B] = first;
   }
   __syncthreads();
+  cluster_wait();                                     // the other CTA's too: from here on either may signal and write there
+  tc_fence_after();
   const int total = s_first[bt.B];
   const int P = gridDim.x >> 1, pr = blockIdx.x >> 1;
   const int nslab = bt.d_k / BK;

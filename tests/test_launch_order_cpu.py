@@ -108,7 +108,7 @@ def _pair_steps(body):
     """Barriers of the whole cluster, collective allocations and deallocations of a pair's tensor memory and returns, in order; those inside a
     block, i.e. not on every way through the kernel, in brackets (returns of lambdas aside)."""
     depth, steps = -1, []                                  # (the body's own brace comes first)
-    for m in re.finditer(r"[{}]|\bcluster_barrier\(\)|\btmem_alloc2\(|\btmem_dealloc2\(|\breturn\b", body):
+    for m in re.finditer(r"[{}]|\bcluster_(?:barrier|arrive|wait)\(\)|\btmem_alloc2\(|\btmem_dealloc2\(|\breturn\b", body):
         tok = m.group(0).rstrip("()")
         depth += {"{": 1, "}": -1}.get(tok, 0)
         if tok not in "{}" and (depth == 0 or tok != "return"):
@@ -120,7 +120,7 @@ def test_pairs_of_ctas_ask_for_tensor_memory_between_cluster_barriers():
     """A CTA may ask for tensor memory of its pair only once the other one runs, and leave only when both have theirs back."""
     pairs = [(n, b) for _, n, b in KERNELS if "tmem_alloc2(" in b]
     assert [n for n, _ in pairs] == ["k_tiles_pair"]
-    want = ["cluster_barrier", "tmem_alloc2", "cluster_barrier", "cluster_barrier", "tmem_dealloc2", "cluster_barrier"]
+    want = ["cluster_arrive", "cluster_wait", "tmem_alloc2", "cluster_arrive", "cluster_wait", "cluster_barrier", "tmem_dealloc2", "cluster_barrier"]
     for _, body in pairs:
         assert _pair_steps(body) == want
         assert _pair_steps(body.replace("pdl_wait();", "if (rank) return; pdl_wait();", 1)) != want
