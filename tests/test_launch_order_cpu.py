@@ -124,3 +124,10 @@ def test_pairs_of_ctas_ask_for_tensor_memory_between_cluster_barriers():
     for _, body in pairs:
         assert _pair_steps(body) == want
         assert _pair_steps(body.replace("pdl_wait();", "if (rank) return; pdl_wait();", 1)) != want
+
+
+def test_every_kernel_that_is_launched_is_found():
+    """No kernel of the sources escapes the checks above, those least that read ahead of their wait."""
+    declared = {m for f in FILES for m in re.findall(r"\b(?:launch_k|launch_opt|launch_coop)\(\s*(?:\w+,\s*)?(k_\w+)", _read(f))}
+    assert {"k_assign", "k_label_counts", "k_list_clear"} <= {name for _, name, _ in KERNELS}
+    assert len(declared) > 10 and declared <= {name for _, name, _ in KERNELS}
